@@ -61,12 +61,8 @@ struct Workspace {
   int32_t* big_list = nullptr;
   int32_t* hset = nullptr;     // fanouts above kWideMax: the sampler's per-warp hash sets
   int64_t hset_elems = 0;
-  int32_t* q_cells = nullptr;  // default frontier's dedup queue (internal.h, DedupBufs)
-  int32_t* q_cnt = nullptr;
-  int32_t* q_off = nullptr;
-  int32_t* q_dense = nullptr;
-  int32_t* q_next = nullptr;
-  int32_t q_chunks_cap = 0;
+  int32_t* q_dense = nullptr;  // default frontier's dedup queue and its counters (internal.h, DedupBufs)
+  int32_t* q_ctl = nullptr;
   int32_t* big_n = nullptr;
   int32_t* tmp_id = nullptr;
   int32_t* tmp_pos = nullptr;

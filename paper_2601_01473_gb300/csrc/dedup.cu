@@ -28,14 +28,17 @@ constexpr int kIlp = 4;  // independent elements per thread in the streaming pas
 
 // Places every sampled edge of minibatch j at soff[cell] + rank (cell and
 // rank were recorded while sampling), building the sampled bucket: (id, edge
-// index) pairs, or packed 4-byte entries edge index << 12 | tile-local id.
+// index) pairs, or packed 4-byte entries edge index << 12 | tile-local id.  It
+// also empties the queue of the cell kernels that follow.
 __global__ void __launch_bounds__(kThreads)
 dedup_scatter_kernel(const int32_t* __restrict__ nbr, const int32_t* __restrict__ ecnt,
                      int64_t ecap, const int32_t* __restrict__ scell,
                      const int32_t* __restrict__ srank, const int32_t* __restrict__ soff,
-                     int2* __restrict__ sb, bool packed, const int32_t* status) {
+                     int2* __restrict__ sb, bool packed, int32_t* __restrict__ q_ctl,
+                     const int32_t* status) {
   grid_dep_wait();
   if (failed(status)) return;
+  if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x < 2) q_ctl[threadIdx.x] = 0;
   const int32_t j = blockIdx.y;
   const int64_t E = ecnt[j];
   const int64_t o = (int64_t)j * ecap;
@@ -563,7 +566,8 @@ cudaError_t launch_dedup(const HopArgs& a, const DedupBufs& d, int num_sms, cuda
   cudaError_t e = cells_scan(d.scnt, d.soff, ncells, d.flat_scratch, d.scan_scratch, a.status, st);
   if (e != cudaSuccess) return e;
   dedup_scatter_kernel<<<egrid, kThreads, 0, st>>>(d.nbr, d.ecnt, a.ecap, d.scell, d.srank,
-                                                   d.soff, d.sb, a.sb_packed, a.status);
+                                                   d.soff, d.sb, a.sb_packed, d.q_ctl,
+                                                   a.status);
 
   CellArgs c;
   c.tm = tm;

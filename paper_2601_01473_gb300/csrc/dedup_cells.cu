@@ -14,17 +14,16 @@
 // Work layout.  Cells are small on average, but the entries concentrate in
 // the larger cells of the tiles that hold the graph's hubs (at rmat100m's hop
 // 3, cells of more than 32 entries hold over half of them), so:
-//   - a lane kernel walks all cells in chunks of 256 taken from a counter, a
+//   - a lane kernel walks all cells in chunks of up to 256 taken from a counter, a
 //     warp over 32 consecutive cells at a time; a cell of at most 8 entries
 //     is resolved by its own thread: its entries become keys (tile-local id
 //     << 1 | sampled) in registers, carried with their rows or edge indices
 //     through a 5- or 19-comparator sorting network, and swept once -- equal
 //     ids are adjacent with the frontier entry first, so the first entry of
 //     each id is its frontier twin or the new id's first occurrence;
-//   - larger cells with samples are queued in cell order (each chunk's cells
-//     in order at the start of its own range; a scan and a copy concatenate
-//     the ranges) and resolved one warp per cell on bitmaps over the tile,
-//     where every rank is a popcount over per-word prefix counts.
+//   - larger cells with samples are queued (each chunk appends its cells in
+//     order) and resolved one warp per cell on bitmaps over the tile, where
+//     every rank is a popcount over per-word prefix counts.
 // The sampled bucket is either (id, edge index) pairs or, when the hop's
 // edge indices fit 20 bits, packed words edge index << 12 | tile-local id
 // (the kernels' kPacked).
@@ -61,11 +60,9 @@ struct CellsArgs {
   int32_t* nfcnt;
   int2* tmp;     // per cell at fcell_off + soff: next-frontier entries, local ranks
   int32_t* col;  // H x ecap
-  int32_t* q_cells;  // per chunk of kChunkCells cells: its queued cells, at the chunk's start
-  int32_t* q_cnt;    // per chunk: how many
-  int32_t* q_off;    // exclusive scan of q_cnt (nchunks + 1)
-  int32_t* q_dense;  // the queue, in cell order
-  int32_t* q_next;   // the lane kernel's next chunk (zero between launches)
+  int32_t* q_dense;  // the queue of larger cells
+  int32_t* q_len;    // its length
+  int32_t* q_next;   // the lane kernel's next chunk
   const int32_t* status;
 };
 
@@ -187,116 +184,72 @@ __device__ __forceinline__ void thread_cell(const CellsArgs& a, int64_t cell, co
 }
 
 // Walks every cell, a warp over 32 consecutive cells at a time.  Warps take
-// chunks of kChunkCells cells from a counter (cells differ widely in cost, so
-// fixed ranges would leave warps idle); each appends its queued cells (with
-// samples and more than kLaneMax entries) in order at the start of the
-// chunk's range of q_cells (q_cnt[chunk] of them).
-constexpr int kChunkCells = kDedupChunkCells;
-constexpr int kChunkBatches = kChunkCells / 32;
-
-// Batches [b_lo, b_hi) of one chunk.
-template <bool kPacked>
-__device__ __forceinline__ void lane_chunk(const CellsArgs& a, int lane, int64_t b_lo,
-                                           int64_t b_hi, int32_t chunk) {
-  int32_t queued = 0;
-  // the lane's cell (t, j), advanced by 32 cells per batch
-  int32_t t = (int32_t)((uint32_t)((b_lo << 5) + lane) / (uint32_t)a.H);  // cells < 2^31
-  int32_t j = (int32_t)((b_lo << 5) + lane) - t * a.H;
-  for (int64_t b = b_lo; b < b_hi; ++b) {
-    const int64_t cell = (b << 5) + lane;
-    const bool has = cell < a.ncells;
-    CellFacts c{0, 0, 0, 0, 0, 0};
-    if (has) c = cell_facts(a, cell, t, j);
-    for (j += 32; j >= a.H; j -= a.H) ++t;
-    const int32_t n = c.fn + c.sn;
-    if (has && c.fn > 0) a.adj_flags[a.tile_adj_block[c.t]] = 1;
-    if (has && c.sn == 0) {  // nothing sampled: the compaction copies the frontier cell
-      a.newcnt[cell] = 0;
-      a.nfcnt[cell] = c.fn;
-    }
-    const unsigned qm = __ballot_sync(kFull, has && c.sn > 0 && n > kLaneMax);
-    if ((qm >> lane) & 1u)
-      a.q_cells[(b_lo << 5) + queued + __popc(qm & ((1u << lane) - 1u))] = (int32_t)cell;
-    queued += __popc(qm);
-    // the warp takes the 4-entry network unless one of its cells needs 8
-    const bool mine = has && c.sn > 0 && n <= kLaneMax;
-    if (__any_sync(kFull, mine && n > 4)) {
-      if (mine) thread_cell<kPacked, 8>(a, cell, c);
-    } else if (mine) {
-      thread_cell<kPacked, 4>(a, cell, c);
-    }
-  }
-  if (lane == 0) a.q_cnt[chunk] = queued;
-}
+// chunks of `batches` x 32 cells from a counter (cells differ widely in cost,
+// so fixed ranges would leave warps idle); a chunk's queued cells (with
+// samples and more than kLaneMax entries) are collected in shared memory and
+// appended to the queue with one atomic, so the queue follows the order in
+// which chunks finish, near enough to cell order for the tile kernel to find
+// neighbouring cells' offsets and col lines in L2.
+//
+// Bound by the latency of a cell's dependent loads (offsets, then entries,
+// then stores), so a chunk may not be long where cells are few: the launch
+// gives every resident warp a chunk before it makes chunks longer, up to
+// kChunkBatches, where the counter's atomics stop mattering.  Measured with
+// chunks of always 256 cells and the queue put in cell order by two more
+// kernels, then like this: one minibatch of 1024 on 10M nodes (5.7k cells)
+// 411 -> 333 us per hyperbatch, 16 of them (91k cells) 800 -> 736 us; at 1.6M
+// cells, where chunks stay at 256 cells, 5.37 -> 5.36 ms with its layers.
+constexpr int kChunkBatches = 8;
 
 template <bool kPacked>
-__global__ void __launch_bounds__(kThreads, 6) dedup_lane_kernel(CellsArgs a) {
+__global__ void __launch_bounds__(kThreads, 6) dedup_lane_kernel(CellsArgs a, int32_t batches) {
   grid_dep_wait();
   if (failed(a.status)) return;
+  __shared__ int32_t queue_s[kWarps][kChunkBatches * 32];
   const int lane = lane_id();
-  const int64_t nbatch = (a.ncells + 31) >> 5;
-  const int32_t nchunks = (int32_t)((a.ncells + kChunkCells - 1) / kChunkCells);
+  int32_t* queue = queue_s[threadIdx.x >> 5];
+  const int32_t nbatch = (int32_t)((a.ncells + 31) >> 5);
+  const int32_t nchunks = (nbatch + batches - 1) / batches;
   for (;;) {
     int32_t chunk = 0;
     if (lane == 0) chunk = atomicAdd(a.q_next, 1);
     chunk = __shfl_sync(kFull, chunk, 0);
     if (chunk >= nchunks) break;
-    lane_chunk<kPacked>(a, lane, (int64_t)chunk * kChunkBatches,
-                        min((int64_t)(chunk + 1) * kChunkBatches, nbatch), chunk);
-  }
-}
-
-// The queue in cell order: q_off = the exclusive scan of the chunks' counts
-// (one CTA, four counts per thread and round; it also rewinds the lane
-// kernel's chunk counter) ...
-__global__ void __launch_bounds__(1024) queue_offsets_kernel(const int32_t* q_cnt, int32_t nw,
-                                                             int32_t* q_off, int32_t* q_next,
-                                                             const int32_t* status) {
-  grid_dep_wait();
-  if (threadIdx.x == 0) *q_next = 0;
-  if (failed(status)) return;
-  __shared__ int32_t wsum[32];
-  __shared__ int32_t carry;
-  if (threadIdx.x == 0) carry = 0;
-  __syncthreads();
-  const int lane = lane_id(), w = threadIdx.x >> 5;
-  for (int32_t base = 0; base < nw; base += 4096) {
-    const int32_t i = base + 4 * (int32_t)threadIdx.x;
-    int32_t v[4];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) v[k] = i + k < nw ? q_cnt[i + k] : 0;
-    const int32_t mine = v[0] + v[1] + v[2] + v[3];
-    const int32_t incl = warp_incl_scan(mine);
-    if (lane == 31) wsum[w] = incl;
-    __syncthreads();
-    if (w == 0) {
-      const int32_t t = wsum[lane];
-      wsum[lane] = warp_incl_scan(t) - t;
+    const int32_t b_lo = chunk * batches, b_hi = min(b_lo + batches, nbatch);
+    int32_t queued = 0;
+    // the lane's cell (t, j), advanced by 32 cells per batch (cells < 2^31)
+    int32_t t = (int32_t)(((uint32_t)b_lo * 32u + (uint32_t)lane) / (uint32_t)a.H);
+    int32_t j = (int32_t)((uint32_t)b_lo * 32u + (uint32_t)lane - (uint32_t)t * (uint32_t)a.H);
+    for (int32_t b = b_lo; b < b_hi; ++b) {
+      const int64_t cell = ((int64_t)b << 5) + lane;
+      const bool has = cell < a.ncells;
+      CellFacts c{0, 0, 0, 0, 0, 0};
+      if (has) c = cell_facts(a, cell, t, j);
+      for (j += 32; j >= a.H; j -= a.H) ++t;
+      const int32_t n = c.fn + c.sn;
+      if (has && c.fn > 0) a.adj_flags[a.tile_adj_block[c.t]] = 1;
+      if (has && c.sn == 0) {  // nothing sampled: the compaction copies the frontier cell
+        a.newcnt[cell] = 0;
+        a.nfcnt[cell] = c.fn;
+      }
+      const unsigned qm = __ballot_sync(kFull, has && c.sn > 0 && n > kLaneMax);
+      if ((qm >> lane) & 1u) queue[queued + __popc(qm & ((1u << lane) - 1u))] = (int32_t)cell;
+      queued += __popc(qm);
+      // the warp takes the 4-entry network unless one of its cells needs 8
+      const bool mine = has && c.sn > 0 && n <= kLaneMax;
+      if (__any_sync(kFull, mine && n > 4)) {
+        if (mine) thread_cell<kPacked, 8>(a, cell, c);
+      } else if (mine) {
+        thread_cell<kPacked, 4>(a, cell, c);
+      }
     }
-    __syncthreads();
-    int32_t run = carry + wsum[w] + incl - mine;
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      if (i + k < nw) q_off[i + k] = run;
-      run += v[k];
-    }
-    __syncthreads();
-    if (threadIdx.x == 1023) carry = run;
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) q_off[nw] = carry;
-}
-
-// ... then each chunk's run copied to q_dense[q_off[chunk] ...).
-__global__ void __launch_bounds__(kThreads) queue_compact_kernel(CellsArgs a, int32_t nw) {
-  grid_dep_wait();
-  if (failed(a.status)) return;
-  const int lane = lane_id();
-  const int64_t nwarps = (int64_t)gridDim.x * kWarps;
-  for (int64_t r = blockIdx.x * (int64_t)kWarps + (threadIdx.x >> 5); r < nw; r += nwarps) {
-    const int64_t src = r * kChunkCells;
-    const int32_t dst = a.q_off[r], cnt = a.q_off[r + 1] - dst;
-    for (int32_t i = lane; i < cnt; i += 32) a.q_dense[dst + i] = a.q_cells[src + i];
+    if (queued == 0) continue;  // warp-uniform
+    int32_t at = 0;
+    if (lane == 0) at = atomicAdd(a.q_len, queued);
+    at = __shfl_sync(kFull, at, 0);
+    __syncwarp();
+    for (int32_t i = lane; i < queued; i += 32) a.q_dense[at + i] = queue[i];
+    __syncwarp();
   }
 }
 
@@ -373,7 +326,7 @@ struct TileResolver {
 // (mark, resolve).  Each warp loads the next queued cell's offsets while it
 // resolves the current one.
 template <bool kPacked>
-__global__ void __launch_bounds__(kThreads, 5) dedup_tile_kernel(CellsArgs a, int32_t nw) {
+__global__ void __launch_bounds__(kThreads, 5) dedup_tile_kernel(CellsArgs a) {
   grid_dep_wait();
   if (failed(a.status)) return;
   __shared__ __align__(16) uint32_t D_s[kWarps][kTileWords];
@@ -385,7 +338,7 @@ __global__ void __launch_bounds__(kThreads, 5) dedup_tile_kernel(CellsArgs a, in
   uint32_t* N = N_s[warp];
   uint32_t* P = P_s[warp];
   uint32_t* C = C_s[warp];
-  const int32_t total = a.q_off[nw];
+  const int32_t total = *a.q_len;
   const int32_t nwarps = (int32_t)gridDim.x * kWarps;
   int32_t q = (int32_t)blockIdx.x * kWarps + warp;
   int32_t cell = q < total ? a.q_dense[q] : 0;
@@ -481,27 +434,23 @@ CellsArgs cells_args(const HopArgs& h, const DedupBufs& d) {
   a.nfcnt = d.nfcnt;
   a.tmp = d.tmp;
   a.col = d.col;
-  a.q_cells = d.q_cells;
-  a.q_cnt = d.q_cnt;
-  a.q_off = d.q_off;
   a.q_dense = d.q_dense;
-  a.q_next = d.q_next;
+  a.q_len = d.q_ctl;
+  a.q_next = d.q_ctl + 1;
   a.status = h.status;
   return a;
 }
 
 template <bool kPacked>
-cudaError_t launch_cells(const CellsArgs& a, int32_t q_chunks_cap, int num_sms, cudaStream_t st) {
+cudaError_t launch_cells(const CellsArgs& a, int num_sms, cudaStream_t st) {
   const int grid = resident_grid((const void*)dedup_lane_kernel<kPacked>, kThreads, num_sms);
-  const int64_t nw = (a.ncells + kChunkCells - 1) / kChunkCells;  // chunks
-  if (nw > q_chunks_cap) return cudaErrorInvalidValue;
-  dedup_lane_kernel<kPacked><<<grid, kThreads, 0, st>>>(a);
-  queue_offsets_kernel<<<1, 1024, 0, st>>>(a.q_cnt, (int32_t)nw, a.q_off, a.q_next, a.status);
-  queue_compact_kernel<<<resident_grid((const void*)queue_compact_kernel, kThreads, num_sms),
-                         kThreads, 0, st>>>(a, (int32_t)nw);
+  const int64_t nbatch = (a.ncells + 31) / 32;
+  int64_t batches = nbatch / ((int64_t)grid * kWarps);
+  batches = batches < 1 ? 1 : batches > kChunkBatches ? kChunkBatches : batches;
+  dedup_lane_kernel<kPacked><<<grid, kThreads, 0, st>>>(a, (int32_t)batches);
   dedup_tile_kernel<kPacked><<<resident_grid((const void*)dedup_tile_kernel<kPacked>, kThreads,
                                              num_sms),
-                               kThreads, 0, st>>>(a, (int32_t)nw);
+                               kThreads, 0, st>>>(a);
   return cudaGetLastError();
 }
 
@@ -510,8 +459,7 @@ cudaError_t launch_cells(const CellsArgs& a, int32_t q_chunks_cap, int num_sms, 
 cudaError_t launch_dedup_cells(const HopArgs& h, const DedupBufs& d, int num_sms,
                                cudaStream_t st) {
   const CellsArgs a = cells_args(h, d);
-  return h.sb_packed ? launch_cells<true>(a, d.q_chunks_cap, num_sms, st)
-                     : launch_cells<false>(a, d.q_chunks_cap, num_sms, st);
+  return h.sb_packed ? launch_cells<true>(a, num_sms, st) : launch_cells<false>(a, num_sms, st);
 }
 
 }  // namespace agnes

@@ -173,8 +173,6 @@ constexpr int kDedupSmallMax = 32;
 // by one thread each; larger cells with samples are queued (q_dense), so the
 // queue holds at most (entries) / (kDedupLaneMax + 1) cells.
 constexpr int kDedupLaneMax = 8;
-// The lane kernel's unit of dynamically scheduled work: 256 consecutive cells.
-constexpr int kDedupChunkCells = 256;
 
 struct DedupBufs {
   const int32_t* nbr;       // H x ecap sampled ids (packed: rank << 12 | tile-local id)
@@ -189,16 +187,10 @@ struct DedupBufs {
   int32_t* big_list;        // cells with more than kDedupSmallMax entries
   int32_t* big_n;           // their count
   // default frontier: the queue of cells with samples and more than
-  // kDedupLaneMax entries: per chunk of kDedupChunkCells cells a run in
-  // q_cells (T*H), the runs' counts and offsets (q_chunks_cap,
-  // q_chunks_cap + 1), the queue in cell order (q_dense), and the lane
-  // kernel's chunk counter (q_next, zero between launches)
-  int32_t* q_cells;
-  int32_t* q_cnt;
-  int32_t* q_off;
+  // kDedupLaneMax entries, and {its length, the lane kernel's next chunk},
+  // which the scatter clears
   int32_t* q_dense;
-  int32_t* q_next;
-  int32_t q_chunks_cap;
+  int32_t* q_ctl;
   const int32_t* fb_id;     // current frontier bucket
   const int32_t* fb_pos;
   const int32_t* fcell_off;
@@ -241,7 +233,7 @@ cudaError_t launch_dedup_compact(const HopArgs& a, const DedupBufs& d, int num_s
 // The default frontier's resolution of one hop's cells (launch_dedup calls
 // it in place of the sampled frontier's cell kernels): newcnt, nfcnt, col
 // with local new-id ranks, the next frontier cells in tmp, the touched-block
-// flags; it builds and uses the queue in q_cells / q_cnt / q_off / q_dense.
+// flags; it builds and uses the queue in q_dense / q_ctl.
 cudaError_t launch_dedup_cells(const HopArgs& a, const DedupBufs& d, int num_sms,
                                cudaStream_t st);
 

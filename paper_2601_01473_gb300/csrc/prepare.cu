@@ -59,11 +59,8 @@ void free_workspace(Workspace* w) {
   cudaFree(w->sb);
   cudaFree(w->tmp);
   cudaFree(w->big_list);
-  cudaFree(w->q_cells);
   cudaFree(w->hset);
-  cudaFree(w->q_cnt);
-  cudaFree(w->q_off);
-  cudaFree(w->q_next);
+  cudaFree(w->q_ctl);
   cudaFree(w->q_dense);
   cudaFree(w->big_n);
   cudaFree(w->tmp_id);
@@ -162,11 +159,7 @@ static agnes_status ensure_workspace(agnes_ctx* ctx, int32_t H, int32_t B, const
   WA(w.tmp, rows + edges);
   WA(w.big_list, (rows + edges) / (kDedupSmallMax + 1) + 1);
   WA(w.big_n, 1);
-  w.q_chunks_cap = (int32_t)((cells + kDedupChunkCells - 1) / kDedupChunkCells);
-  WA(w.q_cells, cells);
-  WA(w.q_cnt, w.q_chunks_cap);
-  WA(w.q_off, w.q_chunks_cap + 1);
-  WA(w.q_next, 1);
+  WA(w.q_ctl, 2);
   WA(w.q_dense, (rows + edges) / (kDedupLaneMax + 1) + 1);
   w.hset_elems = 0;
   for (int h = 0; h < K; ++h) {
@@ -208,7 +201,6 @@ static agnes_status ensure_workspace(agnes_ctx* ctx, int32_t H, int32_t B, const
       cudaMemset(w.side_scratch, 0, sizeof(int64_t) * s4) != cudaSuccess ||
       cudaMemset(w.fcnt, 0, sizeof(int32_t) * cells) != cudaSuccess ||
       cudaMemset(w.scnt, 0, sizeof(int32_t) * cells) != cudaSuccess ||
-      cudaMemset(w.q_next, 0, sizeof(int32_t)) != cudaSuccess ||
       cudaMemset(w.flat_scratch, 0, sizeof(uint64_t) * w.flat_elems) != cudaSuccess) {
     free_workspace(&w);
     set_err(ctx, "cudaMemset failed");
@@ -402,13 +394,8 @@ static agnes_status enqueue_hyperbatch(agnes_ctx* ctx, const int32_t* fanouts, i
     d.sb = w.sb;
     d.tmp = w.tmp;
     d.big_list = w.big_list;
-    d.q_cells = w.q_cells;
-    d.q_cnt = w.q_cnt;
-    d.q_off = w.q_off;
     d.q_dense = w.q_dense;
-    d.q_next = w.q_next;
-    d.q_chunks_cap = w.q_chunks_cap;
-
+    d.q_ctl = w.q_ctl;
     d.big_n = w.big_n;
     d.fb_id = w.fb_id[cur];
     d.fb_pos = w.fb_pos[cur];
