@@ -112,6 +112,8 @@ __device__ __forceinline__ bool load_cell(const CellArgs& a, int64_t cell, Cell*
 // Cells with more than 32 entries go to the big-cell list.
 constexpr int kCellThreads = 128;  // threads per CTA of the cells kernel
 constexpr int kCompactIlp = 2;     // bucket entries per thread and round of the compaction (4 and 8 measured slower)
+constexpr int kCompactOversplit = 2;    // the compaction's (group, slice) items per resident CTA
+constexpr int kCompactMaxSlices = 256;
 constexpr int kGroupCells = kCellThreads;
 constexpr int kSlotCap = 1024;
 constexpr int kSmallMax = kDedupSmallMax;
@@ -458,6 +460,7 @@ dedup_fix_col_kernel(int32_t* __restrict__ col, const int32_t* __restrict__ ecnt
 
 struct CompactArgs {
   int64_t ncells;
+  int32_t slices;  // CTAs per group of kGroupCells cells
   int32_t H;
   int64_t capK;
   const int32_t* fb_id;
@@ -488,7 +491,10 @@ __global__ void __launch_bounds__(kCellThreads) dedup_compact_kernel(CompactArgs
   __shared__ int32_t s_row[kGroupCells];   // j * capK + |dst_h| + newbase
   const int tid = threadIdx.x;
   const int64_t ngroups = (a.ncells + kGroupCells - 1) / kGroupCells;
-  for (int64_t grp = blockIdx.x; grp < ngroups; grp += gridDim.x) {
+  const int64_t nitems = ngroups * a.slices;
+  for (int64_t item = blockIdx.x; item < nitems; item += gridDim.x) {
+    const int64_t grp = item / a.slices;
+    const int32_t slice = (int32_t)(item - grp * a.slices);
     const int64_t c0 = grp * kGroupCells;
     const int64_t cell = c0 + tid;
     const int64_t last = min(a.ncells, c0 + kGroupCells);
@@ -506,7 +512,8 @@ __global__ void __launch_bounds__(kCellThreads) dedup_compact_kernel(CompactArgs
     __syncthreads();
     const int32_t k0 = s_nfo[0], k1 = s_nfo[last - c0];
     // kCompactIlp entries per thread and round: their loads in flight before the stores
-    for (int32_t kb = k0 + tid; kb < k1; kb += kCompactIlp * kCellThreads) {
+    constexpr int kRound = kCompactIlp * kCellThreads;
+    for (int32_t kb = k0 + slice * kRound + tid; kb < k1; kb += a.slices * kRound) {
       int32_t cl[kCompactIlp], r[kCompactIlp], id[kCompactIlp], pos[kCompactIlp];
       bool in[kCompactIlp];
 #pragma unroll
@@ -657,8 +664,11 @@ cudaError_t launch_dedup_compact(const HopArgs& a, const DedupBufs& d, int num_s
   k.nfb_pos = d.nfb_pos;
   k.nodes = d.nodes;
   k.status = a.status;
-  dedup_compact_kernel<<<resident_grid((const void*)dedup_compact_kernel, kCellThreads, num_sms),
-                         kCellThreads, 0, st>>>(k);
+  const int grid = resident_grid((const void*)dedup_compact_kernel, kCellThreads, num_sms);
+  const int64_t ngroups = (ncells + kGroupCells - 1) / kGroupCells;
+  const int64_t slices = (kCompactOversplit * (int64_t)grid + ngroups - 1) / ngroups;
+  k.slices = (int32_t)(slices > kCompactMaxSlices ? kCompactMaxSlices : slices);
+  dedup_compact_kernel<<<grid, kCellThreads, 0, st>>>(k);
   return cudaGetLastError();
 }
 
