@@ -482,7 +482,12 @@ struct CompactArgs {
 // Writes the next frontier bucket in cell order: a cell without samples is
 // copied from the current bucket, any other from its tmp entries, where a new
 // node (x = -(1 + r)) gets its output row j * capK + |dst_h| + newbase + r and
-// its id is appended to the minibatch's node list.
+// its id is appended to the minibatch's node list.  A group of kGroupCells
+// cells is shared by `slices` CTAs, each taking every slices-th round of its
+// entries: small graphs have few groups with many entries each, and the
+// entries' loads are latency-bound, so they need every SM (8 minibatches of
+// 500 at [25, 10] on 250k nodes: 446 -> 349 us a hyperbatch; two items per
+// resident CTA, where four cost 3% and eight 5% on 10M nodes).
 __global__ void __launch_bounds__(kCellThreads) dedup_compact_kernel(CompactArgs a) {
   grid_dep_wait();
   if (failed(a.status)) return;
