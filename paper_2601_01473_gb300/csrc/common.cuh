@@ -115,6 +115,20 @@ __device__ __forceinline__ T warp_sum(T x) {
   return x;
 }
 
+// *count += the number of the n blocks b (tiles [first_tile[b],
+// first_tile[b + 1])) with an entry in the bucket whose cell offsets are
+// cell_off (H cells per tile); the whole grid takes part.
+__device__ __forceinline__ void count_touched(const int32_t* __restrict__ cell_off, int32_t H,
+                                              const int32_t* __restrict__ first_tile, int64_t n,
+                                              int64_t* __restrict__ count) {
+  int32_t local = 0;
+  for (int64_t b = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; b < n;
+       b += (int64_t)gridDim.x * blockDim.x)
+    local += cell_off[(int64_t)first_tile[b + 1] * H] > cell_off[(int64_t)first_tile[b] * H];
+  local = warp_sum(local);
+  if (lane_id() == 0 && local) atomicAdd((unsigned long long*)count, (unsigned long long)local);
+}
+
 __device__ __forceinline__ bool failed(const int32_t* status) {
   return *(volatile const int32_t*)status != 0;
 }

@@ -47,10 +47,15 @@ struct Workspace {
   int32_t* nfcnt = nullptr;
   int32_t* newcnt = nullptr;
   int32_t* newbase = nullptr;
+  // the sizes, statistics and status the host reads back, one device block
+  // laid out like h_back (Back); the pointers below it are into it
+  void* back = nullptr;
+  int32_t* status = nullptr;
   int32_t* nsz = nullptr;   // (K+1) x H: |dst_h| (h < K), |src_{K-1}| (h = K)
-  int32_t* srcsz = nullptr; // K x H: |src_h|
-  int32_t* noutbase = nullptr;  // T*H: sampled frontier: per-minibatch scan of next-frontier counts
   int32_t* ecnt = nullptr;  // K x H
+  int32_t* srcsz = nullptr; // K x H: |src_h|
+  int64_t* stats = nullptr; // K+1
+  int32_t* noutbase = nullptr;  // T*H: sampled frontier: per-minibatch scan of next-frontier counts
   int64_t* indptr[AGNES_MAX_HOPS] = {nullptr};
   int32_t* col[AGNES_MAX_HOPS] = {nullptr};
   int32_t* nbr = nullptr;
@@ -71,21 +76,17 @@ struct Workspace {
   uint64_t* flat_scratch = nullptr;  // single-pass scans of the cell counts (zero between scans)
   int64_t flat_elems = 0;
   void* feats_out = nullptr;
-  uint8_t* adj_flags = nullptr;
-  uint8_t* feat_flags = nullptr;
-  int64_t* stats = nullptr;  // K+1
   int64_t* scan_scratch = nullptr;
   int64_t* side_scratch = nullptr;  // scans on the side stream
-  int32_t* status = nullptr;
   unsigned long long* distinct = nullptr;
   uint64_t* key = nullptr;  // sampling key {seed, first minibatch id}
 
-  // pinned host readback: [status][nsz (K+1)H][ecnt KH][srcsz KH] then int64 stats (K+1)
-  void* h_back = nullptr;
-  size_t h_back_bytes = 0;
+  void* h_back = nullptr;  // pinned copy of back
+  size_t back_bytes = 0;   // a multiple of 8
 };
 
-// Host view of the readback buffer.
+// The readback block: [status][nsz (K+1)H][ecnt KH][srcsz KH], then int64
+// stats (K+1).
 struct Back {
   int32_t* status;
   int32_t* nsz;
@@ -94,17 +95,23 @@ struct Back {
   int64_t* stats;
 };
 
-inline Back back_of(Workspace& w) {
+inline size_t back_stats_offset(int32_t K, int32_t H) {
+  const size_t n32 = 1 + (size_t)(K + 1) * H + 2 * (size_t)K * H;
+  return (n32 * sizeof(int32_t) + 7) & ~(size_t)7;
+}
+
+inline Back back_at(void* base, int32_t K, int32_t H) {
   Back b;
-  int32_t* p = (int32_t*)w.h_back;
-  b.status = p;
-  b.nsz = p + 1;
-  b.ecnt = b.nsz + (size_t)(w.K + 1) * w.H;
-  b.srcsz = b.ecnt + (size_t)w.K * w.H;
-  size_t off32 = 1 + (size_t)(w.K + 1) * w.H + 2 * (size_t)w.K * w.H + 1;
-  b.stats = (int64_t*)((char*)w.h_back + ((off32 * sizeof(int32_t) + 7) & ~(size_t)7));
+  b.status = (int32_t*)base;
+  b.nsz = b.status + 1;
+  b.ecnt = b.nsz + (size_t)(K + 1) * H;
+  b.srcsz = b.ecnt + (size_t)K * H;
+  b.stats = (int64_t*)((char*)base + back_stats_offset(K, H));
   return b;
 }
+
+// Host view of a finished hyperbatch's sizes.
+inline Back back_of(const Workspace& w) { return back_at(w.h_back, w.K, w.H); }
 
 }  // namespace agnes
 

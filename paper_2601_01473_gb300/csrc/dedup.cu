@@ -64,8 +64,6 @@ struct CellArgs {
   const int32_t* fcell_off;
   const int2* sb;            // sampled bucket: (id, edge index)
   const int32_t* soff;
-  const int32_t* tile_adj_block;
-  uint8_t* adj_flags;
   int32_t* newcnt;           // per cell: new ids
   int32_t* nfcnt;            // per cell: next-frontier entries
   int2* tmp;                 // per cell at fcell_off + soff: next-frontier entries, local ranks
@@ -153,7 +151,6 @@ __global__ void __launch_bounds__(kCellThreads) dedup_cells_kernel(CellArgs a) {
     const int n = c.fn + c.sn;
     const bool staged = valid && c.sn > 0 && n <= kSmallMax;
     if (valid) {
-      if (c.fn > 0) a.adj_flags[a.tile_adj_block[c.t]] = 1;
       if (n > kSmallMax) {
         a.big_list[atomicAdd(a.big_n, 1)] = (int32_t)my_cell;
       } else if (c.sn == 0) {
@@ -575,7 +572,8 @@ cudaError_t launch_dedup(const HopArgs& a, const DedupBufs& d, int num_sms, cuda
   int gx = (num_sms * 8 + a.H - 1) / a.H;
   if (gx < 1) gx = 1;
   const dim3 egrid(gx, a.H);
-  cudaError_t e = cells_scan(d.scnt, d.soff, ncells, d.flat_scratch, d.scan_scratch, a.status, st);
+  cudaError_t e =
+      flat_scan(d.scnt, d.soff, ncells, true, nullptr, true, d.flat_scratch, a.status, st);
   if (e != cudaSuccess) return e;
   dedup_scatter_kernel<<<egrid, kThreads, 0, st>>>(d.nbr, d.ecnt, a.ecap, d.scell, d.srank,
                                                    d.soff, d.sb, a.sb_packed, d.q_ctl,
@@ -592,8 +590,6 @@ cudaError_t launch_dedup(const HopArgs& a, const DedupBufs& d, int num_sms, cuda
   c.fcell_off = d.fcell_off;
   c.sb = d.sb;
   c.soff = d.soff;
-  c.tile_adj_block = d.tile_adj_block;
-  c.adj_flags = d.adj_flags;
   c.newcnt = d.newcnt;
   c.nfcnt = d.nfcnt;
   c.tmp = d.tmp;
@@ -628,23 +624,21 @@ cudaError_t launch_dedup(const HopArgs& a, const DedupBufs& d, int num_sms, cuda
     nst = d.side;
     nscratch = d.side_scratch;
   }
-  e = col_scan(d.newcnt, d.newbase, a.T, a.H, d.nsz_prev, d.srcsz, nscratch, a.status, nst);
+  e = col_scan(d.newcnt, d.newbase, a.T, a.H, d.nsz_prev, d.srcsz,
+               d.frontier_sampled ? nullptr : d.nsz_next, nscratch, a.status, nst);
   if (e != cudaSuccess) return e;
   if (d.side && (e = cudaEventRecord(d.ready, d.side)) != cudaSuccess) return e;
   dedup_fix_col_kernel<<<egrid, kThreads, 0, nst>>>(d.col, d.ecnt, a.ecap, d.scell, d.newbase,
                                                     d.nsz_prev, a.status);
   if (d.frontier_sampled) {
-    e = col_scan(d.nfcnt, d.noutbase, a.T, a.H, nullptr, d.nsz_next, d.scan_scratch, a.status,
-                 st);
+    e = col_scan(d.nfcnt, d.noutbase, a.T, a.H, nullptr, d.nsz_next, nullptr, d.scan_scratch,
+                 a.status, st);
     if (e != cudaSuccess) return e;
   }
-  e = cells_scan(d.nfcnt, d.nfcell_off, ncells, d.flat_scratch, d.scan_scratch, a.status, st);
+  e = flat_scan(d.nfcnt, d.nfcell_off, ncells, true, nullptr, false, d.flat_scratch, a.status,
+                st);
   if (e != cudaSuccess) return e;
   if (d.side && (e = cudaStreamWaitEvent(st, d.ready, 0)) != cudaSuccess) return e;
-  if (!d.frontier_sampled) {
-    e = cudaMemcpyAsync(d.nsz_next, d.srcsz, sizeof(int32_t) * a.H, cudaMemcpyDeviceToDevice, st);
-    if (e != cudaSuccess) return e;
-  }
   return cudaGetLastError();
 }
 

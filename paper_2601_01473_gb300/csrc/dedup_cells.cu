@@ -54,8 +54,6 @@ struct CellsArgs {
   const int2* sb;  // sampled bucket: (id, edge index in the minibatch), or packed 4-byte
                    // entries edge index << 12 | tile-local id (the kernels' kPacked)
   const int32_t* soff;
-  const int32_t* tile_adj_block;
-  uint8_t* adj_flags;
   int32_t* newcnt;
   int32_t* nfcnt;
   int2* tmp;     // per cell at fcell_off + soff: next-frontier entries, local ranks
@@ -227,7 +225,6 @@ __global__ void __launch_bounds__(kThreads, 6) dedup_lane_kernel(CellsArgs a, in
       if (has) c = cell_facts(a, cell, t, j);
       for (j += 32; j >= a.H; j -= a.H) ++t;
       const int32_t n = c.fn + c.sn;
-      if (has && c.fn > 0) a.adj_flags[a.tile_adj_block[c.t]] = 1;
       if (has && c.sn == 0) {  // nothing sampled: the compaction copies the frontier cell
         a.newcnt[cell] = 0;
         a.nfcnt[cell] = c.fn;
@@ -428,8 +425,6 @@ CellsArgs cells_args(const HopArgs& h, const DedupBufs& d) {
   a.fcell_off = d.fcell_off;
   a.sb = d.sb;
   a.soff = d.soff;
-  a.tile_adj_block = d.tile_adj_block;
-  a.adj_flags = d.adj_flags;
   a.newcnt = d.newcnt;
   a.nfcnt = d.nfcnt;
   a.tmp = d.tmp;

@@ -116,15 +116,13 @@ load_feat_blocks_kernel(const uint4* __restrict__ host, int64_t host_vecs,
   }
 }
 
-__global__ void mark_kernel(const int32_t* __restrict__ cell_off, int32_t T, int32_t H,
-                            const int32_t* __restrict__ map, uint8_t* __restrict__ flags,
-                            const int32_t* status) {
+__global__ void __launch_bounds__(kThreads)
+count_touched_kernel(const int32_t* __restrict__ cell_off, int32_t H,
+                     const int32_t* __restrict__ first_tile, int64_t n,
+                     int64_t* __restrict__ count, const int32_t* status) {
   grid_dep_wait();
   if (failed(status)) return;
-  const int64_t ncells = (int64_t)T * H;
-  for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < ncells;
-       c += (int64_t)gridDim.x * blockDim.x)
-    if (cell_off[c + 1] > cell_off[c]) flags[map[(uint32_t)c / (uint32_t)H]] = 1;
+  count_touched(cell_off, H, first_tile, n, count);
 }
 
 // Requests per feature block: counts[tile_feat_block[t]] += entries of tile t.
@@ -204,17 +202,6 @@ __global__ void mark_runs_kernel(const int32_t* __restrict__ cell_off, int32_t T
   for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < T;
        t += (int64_t)gridDim.x * blockDim.x)
     if (cell_off[(t + 1) * H] > cell_off[t * H]) need[tile_adj_start[t]] = 1;
-}
-
-__global__ void count_flags_kernel(const uint8_t* __restrict__ flags, int64_t n,
-                                   int64_t* __restrict__ count) {
-  grid_dep_wait();
-  int64_t local = 0;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x)
-    local += flags[i] != 0;
-  local = warp_sum(local);
-  if (lane_id() == 0 && local) atomicAdd((unsigned long long*)count, (unsigned long long)local);
 }
 
 // One warp per tile: union of the tile's cells over all minibatches.
@@ -559,12 +546,12 @@ cudaError_t launch_gather_staged_rows(const void* staging, int64_t row_bytes, co
   return cudaGetLastError();
 }
 
-cudaError_t launch_mark_count(const int32_t* cell_off, int32_t T, int32_t H, const int32_t* map,
-                              uint8_t* flags, int64_t n_flags, int64_t* count,
-                              const int32_t* status, cudaStream_t st) {
-  if (cell_off && map)
-    mark_kernel<<<1184, 256, 0, st>>>(cell_off, T, H, map, flags, status);
-  count_flags_kernel<<<256, 256, 0, st>>>(flags, n_flags, count);
+cudaError_t launch_count_touched(const int32_t* cell_off, int32_t H, const int32_t* first_tile,
+                                 int64_t n, int64_t* count, const int32_t* status,
+                                 cudaStream_t st) {
+  const int64_t blocks = (n + kThreads - 1) / kThreads;
+  count_touched_kernel<<<(unsigned)std::min<int64_t>(blocks, 1184), kThreads, 0, st>>>(
+      cell_off, H, first_tile, n, count, status);
   return cudaGetLastError();
 }
 

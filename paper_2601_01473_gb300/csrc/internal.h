@@ -29,34 +29,23 @@ cudaError_t seg_scan(const InT* in, int64_t in_stride, OutT* out, int64_t out_st
 
 // Single-pass exclusive scan of n int32 values (decoupled look-back): out[i]
 // = sum of in[i'] for i' < i; with write_end out[n] = the total; total_out
-// (if non-null) gets it too.  in and out 16-byte aligned
-// (flat_scan_supported).  scratch needs flat_scan_scratch_elems(n) uint64s,
+// (if non-null) gets it too; with clear the counts are left zero.  in and out
+// are 16-byte aligned.  scratch needs flat_scan_scratch_elems(n) uint64s,
 // zero before first use (the scan leaves it zero again).  Scans sharing a
 // scratch must be ordered on one stream.
 int64_t flat_scan_scratch_elems(int64_t max_n);
-bool flat_scan_supported(const int32_t* in, const int32_t* out);
-cudaError_t flat_scan(const int32_t* in, int32_t* out, int64_t n, bool write_end,
-                      int32_t* total_out, uint64_t* scratch, int32_t* status, cudaStream_t st);
-
-// Exclusive scan of n int32 cell counts into out (n + 1 entries, the total
-// last): single pass where flat_scratch is given and the arrays allow it,
-// else the three-phase seg_scan with scan_scratch.
-inline cudaError_t cells_scan(const int32_t* in, int32_t* out, int64_t n, uint64_t* flat_scratch,
-                              int64_t* scan_scratch, int32_t* status, cudaStream_t st) {
-  if (flat_scratch && flat_scan_supported(in, out))
-    return flat_scan(in, out, n, true, nullptr, flat_scratch, status, st);
-  return seg_scan<int32_t, int32_t>(in, 0, out, 0, nullptr, n, 1, n, true, nullptr, scan_scratch,
-                                    status, st);
-}
+cudaError_t flat_scan(int32_t* in, int32_t* out, int64_t n, bool write_end, int32_t* total_out,
+                      bool clear, uint64_t* scratch, int32_t* status, cudaStream_t st);
 
 // Exclusive scan down each column of a row-major [rows x cols] matrix:
 // out[r*cols + c] = sum of in[r'*cols + c] over r' < r (coalesced along
 // rows).  total_out[c] (if non-null) = column total + add_in[c] (add_in may be
-// null).  scratch needs col_scan_scratch_elems(rows, cols) int64s.
+// null), and so does total_out2[c].  scratch needs
+// col_scan_scratch_elems(rows, cols) int64s.
 int64_t col_scan_scratch_elems(int64_t rows, int32_t cols);
 cudaError_t col_scan(const int32_t* in, int32_t* out, int64_t rows, int32_t cols,
-                     const int32_t* add_in, int32_t* total_out, int64_t* scratch,
-                     const int32_t* status, cudaStream_t st);
+                     const int32_t* add_in, int32_t* total_out, int32_t* total_out2,
+                     int64_t* scratch, const int32_t* status, cudaStream_t st);
 
 // ---- blocks.cu -------------------------------------------------------------
 struct BlockTables {
@@ -102,7 +91,7 @@ struct HopArgs {
   int64_t ecap;      // edge capacity per minibatch at this hop
   int32_t k;         // fanout
   int32_t hop;       // 1-based
-  const uint64_t* key;  // device: {seed, first minibatch id} (launch_set_key)
+  const uint64_t* key;  // device: {seed, first minibatch id}
   int32_t* status;
   // fanouts above kWideMax: per-warp hash sets of chosen positions, 2^hset_log2
   // int32 entries each, for the hset_grid CTAs of the sampler
@@ -125,20 +114,20 @@ constexpr int64_t kPackedEdgeMax = (int64_t)1 << 20;
 // 1 GiB); returns the int32 entries to allocate (0 when k <= kWideMax).
 int64_t huge_fanout_tables(int32_t k, int num_sms, int32_t* log2, int32_t* grid);
 
-// Writes the sampling key {seed, first minibatch id} to device memory ahead
-// of a hyperbatch (one 1-thread kernel: the arguments travel with the launch).
-cudaError_t launch_set_key(uint64_t* key, uint64_t seed, uint64_t first_gid, cudaStream_t st);
-
 cudaError_t launch_bucket_targets(int32_t* nodes, int64_t capK, int32_t H, int32_t B, int32_t N,
                                   const int32_t* tile_first, const int32_t* chunk_tile, int32_t T,
                                   int32_t* fcnt, int32_t* fcell_off, int32_t* tmp_id,
                                   int32_t* tmp_pos, int32_t* fb_id, int32_t* fb_pos,
-                                  int64_t* scan_scratch, uint64_t* flat_scratch, int32_t* status,
-                                  int num_sms, cudaStream_t st);
+                                  uint64_t* flat_scratch, int32_t* status, int num_sms,
+                                  cudaStream_t st);
 
+// The frontier's edge counts per dst (cnt), and in *touched the number of
+// topology blocks holding a frontier node: of the n_runs block starts, those
+// whose tiles [run_first_tile[r], run_first_tile[r + 1]) have an entry.
 cudaError_t launch_sample_count(const HopArgs& a, const int32_t* fb_id, const int32_t* fb_pos,
-                                const int32_t* fcell_off, int32_t* cnt, int num_sms,
-                                cudaStream_t st);
+                                const int32_t* fcell_off, int32_t* cnt,
+                                const int32_t* run_first_tile, int64_t n_runs, int64_t* touched,
+                                int num_sms, cudaStream_t st);
 
 // Which frontier cells to sample and, for streamed topology, where their
 // edge lists are (gbuf == nullptr: the edges are read from HopArgs::indices).
@@ -179,7 +168,7 @@ struct DedupBufs {
   const int32_t* ecnt;      // H edge counts
   const int32_t* scell;     // H x ecap: cell of each sampled id
   const int32_t* srank;     // H x ecap: its rank within the cell (not packed)
-  const int32_t* scnt;      // T*H per-cell counts of sampled ids
+  int32_t* scnt;            // T*H per-cell counts of sampled ids (left zero)
   int32_t* soff;            // T*H+1
   int2* sb;                 // bucketed (sampled id, edge index in the minibatch), or packed
                             // 4-byte entries edge index << 12 | tile-local id (sb_packed)
@@ -207,10 +196,8 @@ struct DedupBufs {
   bool frontier_sampled;    // next frontier = distinct sampled ids (Algorithm 1's N_out)
   int32_t* nodes;           // H x capK
   int32_t* col;             // H x ecap
-  const int32_t* tile_adj_block;
-  uint8_t* adj_flags;       // per topology block: touched at this hop
   int64_t* scan_scratch;
-  uint64_t* flat_scratch = nullptr;  // flat_scan_scratch_elems(T*H), or null
+  uint64_t* flat_scratch = nullptr;  // flat_scan_scratch_elems(T*H)
   // If side is set, the new-id scan (into newbase, with side_scratch) and the
   // col fix-up (which needs only newbase, col and scell) run on it, forked
   // from st through the event fork; st waits for the scan through the event
@@ -232,8 +219,7 @@ cudaError_t launch_dedup_compact(const HopArgs& a, const DedupBufs& d, int num_s
 // ---- dedup_cells.cu --------------------------------------------------------
 // The default frontier's resolution of one hop's cells (launch_dedup calls
 // it in place of the sampled frontier's cell kernels): newcnt, nfcnt, col
-// with local new-id ranks, the next frontier cells in tmp, the touched-block
-// flags; it builds and uses the queue in q_dense / q_ctl.
+// with local new-id ranks, the next frontier cells in tmp; it builds and uses the queue in q_dense / q_ctl.
 cudaError_t launch_dedup_cells(const HopArgs& a, const DedupBufs& d, int num_sms,
                                cudaStream_t st);
 
@@ -298,11 +284,11 @@ cudaError_t launch_load_feat_blocks(const void* host_dev, int64_t host_bytes, co
                                     const unsigned long long* dst, int32_t njobs,
                                     int64_t block_bytes, int num_sms, cudaStream_t st);
 
-// Marks flags[map[t]] for every tile t whose cells (t, 0..H-1) in cell_off
-// hold an entry, then counts set flags into *count (int64).
-cudaError_t launch_mark_count(const int32_t* cell_off, int32_t T, int32_t H, const int32_t* map,
-                              uint8_t* flags, int64_t n_flags, int64_t* count,
-                              const int32_t* status, cudaStream_t st);
+// *count += the number of the n blocks whose tiles [first_tile[b],
+// first_tile[b + 1]) hold an entry of the bucket with offsets cell_off.
+cudaError_t launch_count_touched(const int32_t* cell_off, int32_t H, const int32_t* first_tile,
+                                 int64_t n, int64_t* count, const int32_t* status,
+                                 cudaStream_t st);
 
 // Topology cache bookkeeping for one hop's frontier bucket: acc[run] +=
 // requests of the block run's tiles; cached += requests on tiles whose

@@ -23,11 +23,44 @@ using namespace agnes;
 
 namespace agnes {
 namespace {
-__global__ void fill_i32_kernel(int32_t* p, int64_t n, int32_t v) {
+// A hyperbatch's start, one launch: the targets into the node lists (unless
+// targets is null: they were copied from host memory), the sampling key, and
+// the readback block cleared but for the targets' frontier sizes.  What a node
+// of the sequence costs a small hyperbatch is its place in the chain (about 3 us
+// each): with this, one copy of the readback block instead of five, counters
+// that their scan clears and block statistics taken from the bucket's offsets,
+// a request of 16 targets went from 168 to 150 us and 1 x 1024 targets at
+// [15, 10, 5] from 289 to 272 us.
+struct BeginArgs {
+  const int32_t* targets;  // H x B
+  int32_t* nodes;          // H x capK
+  int64_t capK;
+  int32_t H, B;
+  uint64_t* key;
+  uint64_t seed, first_gid;
+  int32_t* back;
+  int64_t back_words;
+  int32_t* fcnt;  // targets' cell counters, cleared
+  int64_t cells;
+};
+
+__global__ void __launch_bounds__(256) begin_kernel(BeginArgs a) {
   grid_dep_wait();
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x)
-    p[i] = v;
+  const int64_t i0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  if (i0 == 0) {
+    a.key[0] = a.seed;
+    a.key[1] = a.first_gid;
+  }
+  // word 0 is the status; words 1 .. H are |dst_0| of every minibatch
+  for (int64_t i = i0; i < a.back_words; i += stride) a.back[i] = i >= 1 && i <= a.H ? a.B : 0;
+  for (int64_t i = i0; i < a.cells; i += stride) a.fcnt[i] = 0;
+  if (!a.targets) return;
+  const int64_t n = (int64_t)a.H * a.B;
+  for (int64_t i = i0; i < n; i += stride) {
+    const int64_t j = i / a.B;
+    a.nodes[j * a.capK + (i - j * a.B)] = a.targets[i];
+  }
 }
 }  // namespace
 }  // namespace agnes
@@ -45,10 +78,8 @@ void free_workspace(Workspace* w) {
   cudaFree(w->nfcnt);
   cudaFree(w->newcnt);
   cudaFree(w->newbase);
-  cudaFree(w->nsz);
-  cudaFree(w->srcsz);
+  cudaFree(w->back);
   cudaFree(w->noutbase);
-  cudaFree(w->ecnt);
   for (int h = 0; h < AGNES_MAX_HOPS; ++h) {
     cudaFree(w->indptr[h]);
     cudaFree(w->col[h]);
@@ -69,12 +100,8 @@ void free_workspace(Workspace* w) {
   cudaFree(w->fbd);
   cudaFree(w->flat_scratch);
   cudaFree(w->feats_out);
-  cudaFree(w->adj_flags);
-  cudaFree(w->feat_flags);
-  cudaFree(w->stats);
   cudaFree(w->scan_scratch);
   cudaFree(w->side_scratch);
-  cudaFree(w->status);
   cudaFree(w->distinct);
   cudaFree(w->key);
   if (w->h_back) cudaFreeHost(w->h_back);
@@ -112,8 +139,6 @@ static agnes_status ensure_workspace(agnes_ctx* ctx, int32_t H, int32_t B, const
   const int64_t cells = T * H;
   const int64_t rows = (int64_t)H * w.capK;
   const int64_t edges = (int64_t)H * w.ecap_max;
-  const int64_t nb = ctx->bt.n_blocks;
-  const int64_t nfb = ctx->bt.n_feat_blocks;
   int64_t scratch = scan_scratch_elems(1, cells);
   const int64_t s2 = scan_scratch_elems(1, ctx->N);
   const int64_t s3 = scan_scratch_elems(H, w.cap_prev_max);
@@ -144,10 +169,19 @@ static agnes_status ensure_workspace(agnes_ctx* ctx, int32_t H, int32_t B, const
   WA(w.nfcnt, cells);
   WA(w.newcnt, cells);
   WA(w.newbase, cells);
-  WA(w.nsz, (int64_t)(K + 1) * H);
-  WA(w.srcsz, (int64_t)K * H);
+  w.back_bytes = back_stats_offset(K, H) + sizeof(int64_t) * (size_t)(K + 1);
+  {
+    uint8_t* p = nullptr;
+    WA(p, (int64_t)w.back_bytes);
+    w.back = p;
+    const Back b = back_at(p, K, H);
+    w.status = b.status;
+    w.nsz = b.nsz;
+    w.ecnt = b.ecnt;
+    w.srcsz = b.srcsz;
+    w.stats = b.stats;
+  }
   WA(w.noutbase, cells);
-  WA(w.ecnt, (int64_t)K * H);
   for (int h = 0; h < K; ++h) {
     WA(w.indptr[h], (int64_t)H * (cap[h] + 1));
     WA(w.col[h], (int64_t)H * cap[h] * fan[h]);
@@ -179,18 +213,12 @@ static agnes_status ensure_workspace(agnes_ctx* ctx, int32_t H, int32_t B, const
     WA(f, rows * ctx->row_bytes);
     w.feats_out = f;
   }
-  WA(w.adj_flags, (int64_t)K * nb);
-  WA(w.feat_flags, nfb);
-  WA(w.stats, K + 1);
   WA(w.scan_scratch, scratch);
   WA(w.side_scratch, s4);
-  WA(w.status, 1);
   WA(w.distinct, 1);
   WA(w.key, 2);
 #undef WA
-  w.h_back_bytes = sizeof(int32_t) * (1 + (size_t)(K + 1) * H + 2 * (size_t)K * H + 1) +
-                   sizeof(int64_t) * (K + 2);
-  if (cudaMallocHost(&w.h_back, w.h_back_bytes) != cudaSuccess) {
+  if (cudaMallocHost(&w.h_back, w.back_bytes) != cudaSuccess) {
     cudaGetLastError();
     w.h_back = nullptr;
     free_workspace(&w);
@@ -199,9 +227,10 @@ static agnes_status ensure_workspace(agnes_ctx* ctx, int32_t H, int32_t B, const
   }
   if (cudaMemset(w.scan_scratch, 0, sizeof(int64_t) * scratch) != cudaSuccess ||
       cudaMemset(w.side_scratch, 0, sizeof(int64_t) * s4) != cudaSuccess ||
-      cudaMemset(w.fcnt, 0, sizeof(int32_t) * cells) != cudaSuccess ||
       cudaMemset(w.scnt, 0, sizeof(int32_t) * cells) != cudaSuccess ||
-      cudaMemset(w.flat_scratch, 0, sizeof(uint64_t) * w.flat_elems) != cudaSuccess) {
+      cudaMemset(w.flat_scratch, 0, sizeof(uint64_t) * w.flat_elems) != cudaSuccess ||
+      // the hyperbatch may run on a stream that does not wait for this one
+      cudaStreamSynchronize(cudaStreamLegacy) != cudaSuccess) {
     free_workspace(&w);
     set_err(ctx, "cudaMemset failed");
     return AGNES_ECUDA;
@@ -289,8 +318,7 @@ void drop_launch_graph(agnes_ctx::LaunchGraph* g) {
   g->n_marks = 0;
 }
 
-// Enqueues one hyperbatch on st whose targets are already in w.nodes and whose
-// sampling key is in w.key: the bucketing of the targets, K hops of sampling
+// Enqueues one hyperbatch on st behind its begin_kernel: the bucketing of the targets, K hops of sampling
 // and dedup, the feature gather, the statistics and the size read-back.
 // mark_flags is cudaEventRecordExternal while the sequence is being captured,
 // so the phase events become event-record nodes of the graph; *n_marks gets
@@ -313,17 +341,9 @@ static agnes_status enqueue_hyperbatch(agnes_ctx* ctx, const int32_t* fanouts, i
   };
 
   mark();
-  CK(ctx, cudaMemsetAsync(w.status, 0, sizeof(int32_t), st));
-  CK(ctx, cudaMemsetAsync(w.fcnt, 0, sizeof(int32_t) * cells, st));
-  CK(ctx, cudaMemsetAsync(w.adj_flags, 0, (size_t)K * ctx->bt.n_blocks, st));
-  CK(ctx, cudaMemsetAsync(w.feat_flags, 0, (size_t)ctx->bt.n_feat_blocks, st));
-  CK(ctx, cudaMemsetAsync(w.stats, 0, sizeof(int64_t) * (K + 1), st));
-  fill_i32_kernel<<<(H + 255) / 256, 256, 0, st>>>(w.nsz, H, B);
-  CK(ctx, cudaGetLastError());
   CK(ctx, launch_bucket_targets(w.nodes, w.capK, H, B, (int32_t)ctx->N, ctx->bt.tile_first,
                                 ctx->bt.chunk_tile, T, w.fcnt, w.fcell_off[0], w.tmp_id, w.tmp_pos,
-                                w.fb_id[0], w.fb_pos[0], w.scan_scratch, w.flat_scratch, w.status,
-                                nsm, st));
+                                w.fb_id[0], w.fb_pos[0], w.flat_scratch, w.status, nsm, st));
   int cur = 0;
   for (int h = 0; h < K; ++h) {
     mark();
@@ -350,11 +370,11 @@ static agnes_status enqueue_hyperbatch(agnes_ctx* ctx, const int32_t* fanouts, i
     a.sb_packed = !frontier_sampled && a.ecap <= kPackedEdgeMax;
     int32_t* nsz_prev = w.nsz + (int64_t)h * H;
     int32_t* ecnt = w.ecnt + (int64_t)h * H;
-    CK(ctx, launch_sample_count(a, w.fb_id[cur], w.fb_pos[cur], w.fcell_off[cur], w.cnt, nsm, st));
+    CK(ctx, launch_sample_count(a, w.fb_id[cur], w.fb_pos[cur], w.fcell_off[cur], w.cnt,
+                                ctx->bt.run_first_tile, ctx->bt.n_starts, w.stats + h, nsm, st));
     CK(ctx, (seg_scan<int32_t, int64_t>(w.cnt, cap[h], w.indptr[h], cap[h] + 1, nsz_prev, 0, H,
                                          cap[h], true, ecnt, w.scan_scratch, w.status, st)));
     mark();
-    CK(ctx, cudaMemsetAsync(w.scnt, 0, sizeof(int32_t) * cells, st));
     // the previous hop's col fix-up still reads scell and newbase
     if (h > 0) {
       CK(ctx, cudaEventRecord(ctx->aux_join, ctx->aux));
@@ -413,8 +433,6 @@ static agnes_status enqueue_hyperbatch(agnes_ctx* ctx, const int32_t* fanouts, i
     d.frontier_sampled = frontier_sampled;
     d.nodes = w.nodes;
     d.col = w.col[h];
-    d.tile_adj_block = ctx->bt.tile_adj_block;
-    d.adj_flags = w.adj_flags + (int64_t)h * ctx->bt.n_blocks;
     d.scan_scratch = w.scan_scratch;
     d.flat_scratch = w.flat_scratch;
     d.side = ctx->aux;
@@ -423,17 +441,12 @@ static agnes_status enqueue_hyperbatch(agnes_ctx* ctx, const int32_t* fanouts, i
     d.side_scratch = w.side_scratch;
     CK(ctx, launch_dedup(a, d, nsm, st));
     if (h + 1 == K) {
-      // blocks touched by the hyperbatch (the statistics), on the side stream
-      // beside the last compaction: feature blocks from the final bucket's
-      // offsets, topology blocks from the flags the dedup of each hop set
+      // feature blocks touched by the hyperbatch, on the side stream beside the
+      // last compaction (each hop's count kernel counted the topology blocks)
       CK(ctx, cudaEventRecord(ctx->aux_fork, st));
       CK(ctx, cudaStreamWaitEvent(ctx->aux, ctx->aux_fork, 0));
-      CK(ctx, launch_mark_count(w.fcell_off[1 - cur], T, H, ctx->bt.tile_feat_block, w.feat_flags,
-                                ctx->bt.n_feat_blocks, w.stats + K, w.status, ctx->aux));
-      for (int hh = 0; hh < K; ++hh)
-        CK(ctx, launch_mark_count(nullptr, T, H, nullptr,
-                                  w.adj_flags + (int64_t)hh * ctx->bt.n_blocks, ctx->bt.n_blocks,
-                                  w.stats + hh, w.status, ctx->aux));
+      CK(ctx, launch_count_touched(w.fcell_off[1 - cur], H, ctx->bt.fblock_first_tile,
+                                   ctx->bt.n_feat_blocks, w.stats + K, w.status, ctx->aux));
     }
     CK(ctx, launch_dedup_compact(a, d, nsm, st));
     cur = 1 - cur;
@@ -450,17 +463,24 @@ static agnes_status enqueue_hyperbatch(agnes_ctx* ctx, const int32_t* fanouts, i
   // the last hop's col fix-up and the statistics ran beside its compaction
   CK(ctx, cudaEventRecord(ctx->aux_join, ctx->aux));
   CK(ctx, cudaStreamWaitEvent(st, ctx->aux_join, 0));
-  const Back b = back_of(w);
-  CK(ctx, cudaMemcpyAsync(b.status, w.status, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
-  CK(ctx, cudaMemcpyAsync(b.nsz, w.nsz, sizeof(int32_t) * (K + 1) * H, cudaMemcpyDeviceToHost, st));
-  CK(ctx, cudaMemcpyAsync(b.ecnt, w.ecnt, sizeof(int32_t) * K * H, cudaMemcpyDeviceToHost, st));
-  CK(ctx, cudaMemcpyAsync(b.srcsz, w.srcsz, sizeof(int32_t) * K * H, cudaMemcpyDeviceToHost, st));
-  CK(ctx, cudaMemcpyAsync(b.stats, w.stats, sizeof(int64_t) * (K + 1), cudaMemcpyDeviceToHost, st));
+  CK(ctx, cudaMemcpyAsync(w.h_back, w.back, w.back_bytes, cudaMemcpyDeviceToHost, st));
   if (ctx->topo.cache)
     CK(ctx, cudaMemcpyAsync(ctx->topo.h_cached, ctx->topo.d_cached, sizeof(unsigned long long),
                             cudaMemcpyDeviceToHost, st));
   *n_marks = ph;
   return AGNES_OK;
+}
+
+// Whether a kernel on `device` can read p: its own device memory or managed
+// memory.
+static bool device_can_read(const void* p, int device) {
+  cudaPointerAttributes attr;
+  if (cudaPointerGetAttributes(&attr, p) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return attr.type == cudaMemoryTypeManaged ||
+         (attr.type == cudaMemoryTypeDevice && attr.device == device);
 }
 
 // Whether work enqueued on st is being captured (by the caller's own graph
@@ -692,15 +712,33 @@ agnes_status agnes_prepare_hyperbatch(agnes_ctx* ctx, const int32_t* targets, in
     rc = update_topology_cache(ctx, st);
     if (rc != AGNES_OK) return rc;
   }
-  CK(ctx, cudaMemcpy2DAsync(w.nodes, sizeof(int32_t) * w.capK, targets, sizeof(int32_t) * B,
-                            sizeof(int32_t) * B, H, cudaMemcpyDefault, st));
-  CK(ctx, launch_set_key(w.key, seed, first_minibatch_id, st));
+  BeginArgs b;
+  b.targets = device_can_read(targets, ctx->device) ? targets : nullptr;
+  if (!b.targets)
+    CK(ctx, cudaMemcpy2DAsync(w.nodes, sizeof(int32_t) * w.capK, targets, sizeof(int32_t) * B,
+                              sizeof(int32_t) * B, H, cudaMemcpyDefault, st));
+  b.nodes = w.nodes;
+  b.capK = w.capK;
+  b.H = H;
+  b.B = B;
+  b.key = w.key;
+  b.seed = seed;
+  b.first_gid = first_minibatch_id;
+  b.back = (int32_t*)w.back;
+  b.back_words = (int64_t)(w.back_bytes / sizeof(int32_t));
+  b.fcnt = w.fcnt;
+  b.cells = ctx->bt.T * H;
+  begin_kernel<<<resident_grid((const void*)begin_kernel, 256, ctx->num_sms), 256, 0, st>>>(b);
+  CK(ctx, cudaGetLastError());
   int n_marks = 0;
   if (resident && ctx->lg.mode != AGNES_LAUNCH_DIRECT && !capturing)
     rc = launch_graphed(ctx, fanouts, K, cap, ring, st, &n_marks);
   else
     rc = enqueue_hyperbatch(ctx, fanouts, K, cap, ring, cudaEventRecordDefault, st, &n_marks);
-  if (rc != AGNES_OK) return rc;
+  if (rc != AGNES_OK) {
+    w.valid = false;  // a sequence cut short may have left counters set: start from a new one
+    return rc;
+  }
   // inside a caller's capture nothing has run yet: the caller orders its
   // replays, and there are no phase times to read
   if (!capturing) CK(ctx, cudaEventRecord(ctx->done, st));

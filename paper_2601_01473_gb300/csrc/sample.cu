@@ -174,15 +174,19 @@ targets_sort_kernel(const int32_t* __restrict__ fcell_off, int64_t ncells, int32
 // Per frontier entry i (bucket order): the node's count of sampled edges
 // min(deg, k) at its minibatch position (for the edge offsets' scan), and
 // (first edge, degree) in fbd[i] for the fill, which then reads them
-// coalesced instead of the offsets at random.
+// coalesced instead of the offsets at random.  Also the hop's count of touched
+// topology blocks.
 template <typename OffT>
 __global__ void __launch_bounds__(kThreads)
 sample_count_kernel(const int32_t* __restrict__ fb_id, const int32_t* __restrict__ fb_pos,
                     const int32_t* total_ptr, const OffT* __restrict__ off, int64_t capK,
                     int64_t cap_prev, int32_t k, int32_t* __restrict__ cnt,
-                    longlong2* __restrict__ fbd, const int32_t* status) {
+                    longlong2* __restrict__ fbd, const int32_t* __restrict__ cell_off, int32_t H,
+                    const int32_t* __restrict__ run_first_tile, int64_t n_runs,
+                    int64_t* __restrict__ touched, const int32_t* status) {
   grid_dep_wait();
   if (failed(status)) return;
+  count_touched(cell_off, H, run_first_tile, n_runs, touched);
   const int64_t total = *total_ptr;
   const uint32_t capk32 = (uint32_t)capK;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total;
@@ -529,13 +533,15 @@ cudaError_t launch_bucket_targets(int32_t* nodes, int64_t capK, int32_t H, int32
                                   const int32_t* tile_first, const int32_t* chunk_tile, int32_t T,
                                   int32_t* fcnt, int32_t* fcell_off, int32_t* tmp_id,
                                   int32_t* tmp_pos, int32_t* fb_id, int32_t* fb_pos,
-                                  int64_t* scan_scratch, uint64_t* flat_scratch, int32_t* status,
-                                  int num_sms, cudaStream_t st) {
+                                  uint64_t* flat_scratch, int32_t* status, int num_sms,
+                                  cudaStream_t st) {
   const TileMap tm{tile_first, chunk_tile, T};
   const int64_t ncells = (int64_t)T * H;
   const int grid = resident_grid((const void*)targets_count_kernel, kThreads, num_sms);
   targets_count_kernel<<<grid, kThreads, 0, st>>>(nodes, capK, H, B, N, tm, fcnt, status);
-  cudaError_t e = cells_scan(fcnt, fcell_off, ncells, flat_scratch, scan_scratch, status, st);
+  // the scatter counts fcnt back down to zero
+  cudaError_t e =
+      flat_scan(fcnt, fcell_off, ncells, true, nullptr, false, flat_scratch, status, st);
   if (e != cudaSuccess) return e;
   targets_scatter_kernel<<<resident_grid((const void*)targets_scatter_kernel, kThreads, num_sms),
                            kThreads, 0, st>>>(nodes, capK, H, B, N, tm, fcnt, fcell_off,
@@ -546,33 +552,25 @@ cudaError_t launch_bucket_targets(int32_t* nodes, int64_t capK, int32_t H, int32
   return cudaGetLastError();
 }
 
-static __global__ void set_key_kernel(uint64_t* key, uint64_t seed, uint64_t first_gid) {
-  grid_dep_wait();
-  key[0] = seed;
-  key[1] = first_gid;
-}
-
-cudaError_t launch_set_key(uint64_t* key, uint64_t seed, uint64_t first_gid, cudaStream_t st) {
-  set_key_kernel<<<1, 1, 0, st>>>(key, seed, first_gid);
-  return cudaGetLastError();
-}
-
 cudaError_t launch_sample_count(const HopArgs& a, const int32_t* fb_id, const int32_t* fb_pos,
-                                const int32_t* fcell_off, int32_t* cnt, int num_sms,
-                                cudaStream_t st) {
+                                const int32_t* fcell_off, int32_t* cnt,
+                                const int32_t* run_first_tile, int64_t n_runs, int64_t* touched,
+                                int num_sms, cudaStream_t st) {
   const int32_t* total = fcell_off + (int64_t)a.T * a.H;
   if (a.offsets_bits == 32)
     sample_count_kernel<int32_t><<<resident_grid((const void*)sample_count_kernel<int32_t>,
                                                  kThreads, num_sms),
                                    kThreads, 0, st>>>(
         fb_id, fb_pos, total, (const int32_t*)a.offsets, a.capK, a.cap_prev, a.k, cnt,
-        reinterpret_cast<longlong2*>(a.fbd), a.status);
+        reinterpret_cast<longlong2*>(a.fbd), fcell_off, a.H, run_first_tile, n_runs, touched,
+        a.status);
   else
     sample_count_kernel<int64_t><<<resident_grid((const void*)sample_count_kernel<int64_t>,
                                                  kThreads, num_sms),
                                    kThreads, 0, st>>>(
         fb_id, fb_pos, total, (const int64_t*)a.offsets, a.capK, a.cap_prev, a.k, cnt,
-        reinterpret_cast<longlong2*>(a.fbd), a.status);
+        reinterpret_cast<longlong2*>(a.fbd), fcell_off, a.H, run_first_tile, n_runs, touched,
+        a.status);
   return cudaGetLastError();
 }
 

@@ -218,13 +218,16 @@ col_reduce_kernel(const int32_t* __restrict__ in, int64_t rows, int32_t cols,
 __global__ void __launch_bounds__(kThreads)
 col_partials_kernel(int64_t* __restrict__ partial, int64_t chunks, int32_t cols,
                     const int32_t* __restrict__ add_in, int32_t* __restrict__ total_out,
-                    const int32_t* status) {
+                    int32_t* __restrict__ total_out2, const int32_t* status) {
   grid_dep_wait();
   if (status && failed(status)) return;
   const int32_t c = blockIdx.x;
   const int64_t carry = cta_scan_inplace(partial + c, chunks, cols, false);
-  if (threadIdx.x == 0 && total_out)
-    total_out[c] = (int32_t)carry + (add_in ? add_in[c] : 0);
+  if (threadIdx.x == 0) {
+    const int32_t total = (int32_t)carry + (add_in ? add_in[c] : 0);
+    if (total_out) total_out[c] = total;
+    if (total_out2) total_out2[c] = total;
+  }
 }
 
 __global__ void __launch_bounds__(128)
@@ -273,9 +276,8 @@ __device__ __forceinline__ unsigned long long flag_load(const unsigned long long
 }
 
 __global__ void __launch_bounds__(kThreads)
-flat_scan_kernel(const int32_t* __restrict__ in, int32_t* __restrict__ out, int64_t n,
-                 bool write_end, int32_t* total_out, unsigned long long* scratch,
-                 int32_t* status) {
+flat_scan_kernel(int32_t* __restrict__ in, int32_t* __restrict__ out, int64_t n, bool write_end,
+                 int32_t* total_out, bool clear, unsigned long long* scratch, int32_t* status) {
   grid_dep_wait();
   // no early return on a failed status: every CTA takes its tile and counts
   // itself finished, so the scratch is left zero for the next scan
@@ -308,6 +310,17 @@ flat_scan_kernel(const int32_t* __restrict__ in, int32_t* __restrict__ out, int6
   } else {
 #pragma unroll
     for (int k = 0; k < kFlatItems; ++k) v[k] = i0 + k < n ? in[i0 + k] : 0;
+  }
+  if (clear) {  // the counts start from zero next time, without a memset of their own
+    if (i0 + kFlatItems <= n) {
+      int4* p = reinterpret_cast<int4*>(in + i0);
+#pragma unroll
+      for (int q = 0; q < kFlatItems / 4; ++q) p[q] = make_int4(0, 0, 0, 0);
+    } else {
+#pragma unroll
+      for (int k = 0; k < kFlatItems; ++k)
+        if (i0 + k < n) in[i0 + k] = 0;
+    }
   }
   int64_t mine = 0;
 #pragma unroll
@@ -394,14 +407,15 @@ int64_t col_scan_scratch_elems(int64_t rows, int32_t cols) {
 }
 
 cudaError_t col_scan(const int32_t* in, int32_t* out, int64_t rows, int32_t cols,
-                     const int32_t* add_in, int32_t* total_out, int64_t* scratch,
-                     const int32_t* status, cudaStream_t st) {
+                     const int32_t* add_in, int32_t* total_out, int32_t* total_out2,
+                     int64_t* scratch, const int32_t* status, cudaStream_t st) {
   if (rows <= 0 || cols <= 0) return cudaSuccess;
   const int64_t chunks = (rows + kColRows - 1) / kColRows;
   const dim3 grid((unsigned)chunks, (unsigned)((cols + 127) / 128));
   int64_t* partial = scratch + kTicketElems;  // leave the seg_scan tickets untouched
   col_reduce_kernel<<<grid, 128, 0, st>>>(in, rows, cols, partial, status);
-  col_partials_kernel<<<cols, kThreads, 0, st>>>(partial, chunks, cols, add_in, total_out, status);
+  col_partials_kernel<<<cols, kThreads, 0, st>>>(partial, chunks, cols, add_in, total_out, total_out2,
+                                                  status);
   col_down_kernel<<<grid, 128, 0, st>>>(in, out, rows, cols, partial, status);
   return cudaGetLastError();
 }
@@ -438,17 +452,14 @@ int64_t flat_scan_scratch_elems(int64_t max_n) {
   return 2 + (max_n + kFlatTile - 1) / kFlatTile + 1;
 }
 
-bool flat_scan_supported(const int32_t* in, const int32_t* out) {
-  return (uintptr_t)in % 16 == 0 && (uintptr_t)out % 16 == 0;
-}
-
-cudaError_t flat_scan(const int32_t* in, int32_t* out, int64_t n, bool write_end,
-                      int32_t* total_out, uint64_t* scratch, int32_t* status, cudaStream_t st) {
-  if (!flat_scan_supported(in, out)) return cudaErrorInvalidValue;
+cudaError_t flat_scan(int32_t* in, int32_t* out, int64_t n, bool write_end, int32_t* total_out,
+                      bool clear, uint64_t* scratch, int32_t* status, cudaStream_t st) {
+  if ((uintptr_t)in % 16 != 0 || (uintptr_t)out % 16 != 0) return cudaErrorInvalidValue;
   const int64_t ntiles = n > 0 ? (n + kFlatTile - 1) / kFlatTile : 1;
   if (ntiles > 0x7fffffff) return cudaErrorInvalidValue;
   flat_scan_kernel<<<(unsigned)ntiles, kThreads, 0, st>>>(
-      in, out, n, write_end, total_out, reinterpret_cast<unsigned long long*>(scratch), status);
+      in, out, n, write_end, total_out, clear, reinterpret_cast<unsigned long long*>(scratch),
+      status);
   return cudaGetLastError();
 }
 
