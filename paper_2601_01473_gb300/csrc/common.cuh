@@ -117,13 +117,14 @@ __device__ __forceinline__ T warp_sum(T x) {
 
 // *count += the number of the n blocks b (tiles [first_tile[b],
 // first_tile[b + 1])) with an entry in the bucket whose cell offsets are
-// cell_off (H cells per tile); the whole grid takes part.
-__device__ __forceinline__ void count_touched(const int32_t* __restrict__ cell_off, int32_t H,
+// cell_off (H cells per tile); every thread of the grid takes part, as thread
+// i0 of `stride`.
+__device__ __forceinline__ void count_touched(int64_t i0, int64_t stride,
+                                              const int32_t* __restrict__ cell_off, int32_t H,
                                               const int32_t* __restrict__ first_tile, int64_t n,
                                               int64_t* __restrict__ count) {
   int32_t local = 0;
-  for (int64_t b = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; b < n;
-       b += (int64_t)gridDim.x * blockDim.x)
+  for (int64_t b = i0; b < n; b += stride)
     local += cell_off[(int64_t)first_tile[b + 1] * H] > cell_off[(int64_t)first_tile[b] * H];
   local = warp_sum(local);
   if (lane_id() == 0 && local) atomicAdd((unsigned long long*)count, (unsigned long long)local);
@@ -131,6 +132,12 @@ __device__ __forceinline__ void count_touched(const int32_t* __restrict__ cell_o
 
 __device__ __forceinline__ bool failed(const int32_t* status) {
   return *(volatile const int32_t*)status != 0;
+}
+
+// The same for a whole CTA: one answer for all its threads, for kernels with
+// barriers in which another CTA may record a failure meanwhile.
+__device__ __forceinline__ bool cta_failed(const int32_t* status) {
+  return __syncthreads_or(failed(status)) != 0;
 }
 
 // Programmatic dependent launch: a kernel launched ahead of its predecessor's

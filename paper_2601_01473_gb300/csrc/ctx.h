@@ -71,8 +71,7 @@ struct Workspace {
   int32_t* big_n = nullptr;
   int32_t* tmp_id = nullptr;
   int32_t* tmp_pos = nullptr;
-  int32_t* cnt = nullptr;
-  int64_t* fbd = nullptr;  // 2 per frontier entry: (first edge, degree)
+  uint64_t* indptr_scratch = nullptr;  // flags of the indptr scan (zero between hops)
   uint64_t* flat_scratch = nullptr;  // single-pass scans of the cell counts (zero between scans)
   int64_t flat_elems = 0;
   void* feats_out = nullptr;

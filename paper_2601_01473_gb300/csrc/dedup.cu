@@ -29,16 +29,26 @@ constexpr int kIlp = 4;  // independent elements per thread in the streaming pas
 // Places every sampled edge of minibatch j at soff[cell] + rank (cell and
 // rank were recorded while sampling), building the sampled bucket: (id, edge
 // index) pairs, or packed 4-byte entries edge index << 12 | tile-local id.  It
-// also empties the queue of the cell kernels that follow.
+// also empties the queue of the cell kernels that follow, clears the indptr
+// scan's flags and counts the topology blocks the frontier touches.
 __global__ void __launch_bounds__(kThreads)
 dedup_scatter_kernel(const int32_t* __restrict__ nbr, const int32_t* __restrict__ ecnt,
                      int64_t ecap, const int32_t* __restrict__ scell,
                      const int32_t* __restrict__ srank, const int32_t* __restrict__ soff,
                      int2* __restrict__ sb, bool packed, int32_t* __restrict__ q_ctl,
-                     const int32_t* status) {
+                     unsigned long long* __restrict__ clear, int64_t n_clear,
+                     const int32_t* __restrict__ fcell_off, int32_t H,
+                     const int32_t* __restrict__ run_first_tile, int64_t n_runs,
+                     int64_t* __restrict__ touched, const int32_t* status) {
   grid_dep_wait();
+  const int64_t i0 =
+      ((int64_t)blockIdx.y * gridDim.x + blockIdx.x) * blockDim.x + threadIdx.x;
+  const int64_t threads = (int64_t)gridDim.x * gridDim.y * blockDim.x;
+  // whatever the status: the next hop or hyperbatch relies on it
+  for (int64_t i = i0; i < n_clear; i += threads) clear[i] = 0;
+  if (i0 < 2) q_ctl[i0] = 0;
   if (failed(status)) return;
-  if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x < 2) q_ctl[threadIdx.x] = 0;
+  count_touched(i0, threads, fcell_off, H, run_first_tile, n_runs, touched);
   const int32_t j = blockIdx.y;
   const int64_t E = ecnt[j];
   const int64_t o = (int64_t)j * ecap;
@@ -577,7 +587,11 @@ cudaError_t launch_dedup(const HopArgs& a, const DedupBufs& d, int num_sms, cuda
   if (e != cudaSuccess) return e;
   dedup_scatter_kernel<<<egrid, kThreads, 0, st>>>(d.nbr, d.ecnt, a.ecap, d.scell, d.srank,
                                                    d.soff, d.sb, a.sb_packed, d.q_ctl,
-                                                   a.status);
+                                                   reinterpret_cast<unsigned long long*>(
+                                                       d.indptr_scratch),
+                                                   indptr_scratch_elems(a.H, a.cap_prev),
+                                                   d.fcell_off, a.H, d.run_first_tile, d.n_runs,
+                                                   d.touched, a.status);
 
   CellArgs c;
   c.tm = tm;

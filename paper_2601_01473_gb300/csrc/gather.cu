@@ -122,7 +122,8 @@ count_touched_kernel(const int32_t* __restrict__ cell_off, int32_t H,
                      int64_t* __restrict__ count, const int32_t* status) {
   grid_dep_wait();
   if (failed(status)) return;
-  count_touched(cell_off, H, first_tile, n, count);
+  count_touched(blockIdx.x * (int64_t)blockDim.x + threadIdx.x, (int64_t)gridDim.x * blockDim.x,
+                cell_off, H, first_tile, n, count);
 }
 
 // Requests per feature block: counts[tile_feat_block[t]] += entries of tile t.

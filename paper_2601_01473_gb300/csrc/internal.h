@@ -102,9 +102,6 @@ struct HopArgs {
   // id): the default frontier with ecap <= kPackedEdgeMax; the sampler then
   // records rank << 12 | tile-local id per edge (no rank array)
   bool sb_packed = false;
-  // per frontier entry (bucket order): its node's first edge and degree, two
-  // int64 each, written by the count kernel and read by the fill
-  int64_t* fbd = nullptr;
 };
 
 constexpr int64_t kPackedEdgeMax = (int64_t)1 << 20;
@@ -121,13 +118,14 @@ cudaError_t launch_bucket_targets(int32_t* nodes, int64_t capK, int32_t H, int32
                                   uint64_t* flat_scratch, int32_t* status, int num_sms,
                                   cudaStream_t st);
 
-// The frontier's edge counts per dst (cnt), and in *touched the number of
-// topology blocks holding a frontier node: of the n_runs block starts, those
-// whose tiles [run_first_tile[r], run_first_tile[r + 1]) have an entry.
-cudaError_t launch_sample_count(const HopArgs& a, const int32_t* fb_id, const int32_t* fb_pos,
-                                const int32_t* fcell_off, int32_t* cnt,
-                                const int32_t* run_first_tile, int64_t n_runs, int64_t* touched,
-                                int num_sms, cudaStream_t st);
+// The hop's edge offsets: minibatch j's indptr (nsz[j] + 1 entries at
+// j * (cap_prev + 1)) from the degrees of its dst list (nsz[j] ids at
+// nodes + j * capK) and its edge count ecnt[j].  scratch: indptr_scratch_elems uint64s, zero on entry (launch_dedup's scatter
+// clears them).
+int64_t indptr_scratch_elems(int32_t H, int64_t cap_prev);
+cudaError_t launch_sample_indptr(const HopArgs& a, const int32_t* nodes, const int32_t* nsz,
+                                 int64_t* indptr, int32_t* ecnt, uint64_t* scratch, int num_sms,
+                                 cudaStream_t st);
 
 // Which frontier cells to sample and, for streamed topology, where their
 // edge lists are (gbuf == nullptr: the edges are read from HopArgs::indices).
@@ -180,6 +178,13 @@ struct DedupBufs {
   // which the scatter clears
   int32_t* q_dense;
   int32_t* q_ctl;
+  uint64_t* indptr_scratch;  // launch_sample_indptr's, cleared by the scatter
+  // *touched += the topology blocks holding a frontier node: of the n_runs
+  // block starts, those whose tiles [run_first_tile[r], run_first_tile[r + 1])
+  // have an entry (the scatter counts them)
+  const int32_t* run_first_tile;
+  int64_t n_runs;
+  int64_t* touched;
   const int32_t* fb_id;     // current frontier bucket
   const int32_t* fb_pos;
   const int32_t* fcell_off;

@@ -1,8 +1,8 @@
 // prepare.cu -- agnes_prepare_hyperbatch: one hyperbatch (Algorithm 1,
 // Sec. 3.5) on the caller's stream:
 //   bucket the targets by (tile, minibatch)                   [sample.cu]
-//   for each hop: count min(deg, k) per frontier entry, scan to indptr,
-//                 sample in bucket order                      [sample.cu, scan.cu]
+//   for each hop: scan min(deg, k) of the dst lists to indptr, sample in
+//                 bucket order                                [sample.cu]
 //                 bucket the samples, dedup + relabel, carry the bucket
 //                                                             [dedup.cu]
 //   gather the final bucket's rows block by block             [gather_hbm.cu]
@@ -96,8 +96,7 @@ void free_workspace(Workspace* w) {
   cudaFree(w->big_n);
   cudaFree(w->tmp_id);
   cudaFree(w->tmp_pos);
-  cudaFree(w->cnt);
-  cudaFree(w->fbd);
+  cudaFree(w->indptr_scratch);
   cudaFree(w->flat_scratch);
   cudaFree(w->feats_out);
   cudaFree(w->scan_scratch);
@@ -141,10 +140,8 @@ static agnes_status ensure_workspace(agnes_ctx* ctx, int32_t H, int32_t B, const
   const int64_t edges = (int64_t)H * w.ecap_max;
   int64_t scratch = scan_scratch_elems(1, cells);
   const int64_t s2 = scan_scratch_elems(1, ctx->N);
-  const int64_t s3 = scan_scratch_elems(H, w.cap_prev_max);
   const int64_t s4 = col_scan_scratch_elems(T, H);
   if (s2 > scratch) scratch = s2;
-  if (s3 > scratch) scratch = s3;
   if (s4 > scratch) scratch = s4;
 
 #define WA(p, n)                                                                             \
@@ -204,8 +201,8 @@ static agnes_status ensure_workspace(agnes_ctx* ctx, int32_t H, int32_t B, const
   if (w.hset_elems > 0) WA(w.hset, w.hset_elems);
   WA(w.tmp_id, (int64_t)H * B);
   WA(w.tmp_pos, (int64_t)H * B);
-  WA(w.cnt, (int64_t)H * w.cap_prev_max);
-  WA(w.fbd, 2 * (int64_t)H * w.cap_prev_max);
+  const int64_t indptr_elems = indptr_scratch_elems(H, w.cap_prev_max);
+  WA(w.indptr_scratch, indptr_elems);
   w.flat_elems = flat_scan_scratch_elems(cells);
   WA(w.flat_scratch, w.flat_elems);
   {
@@ -227,6 +224,7 @@ static agnes_status ensure_workspace(agnes_ctx* ctx, int32_t H, int32_t B, const
   }
   if (cudaMemset(w.scan_scratch, 0, sizeof(int64_t) * scratch) != cudaSuccess ||
       cudaMemset(w.side_scratch, 0, sizeof(int64_t) * s4) != cudaSuccess ||
+      cudaMemset(w.indptr_scratch, 0, sizeof(uint64_t) * indptr_elems) != cudaSuccess ||
       cudaMemset(w.scnt, 0, sizeof(int32_t) * cells) != cudaSuccess ||
       cudaMemset(w.flat_scratch, 0, sizeof(uint64_t) * w.flat_elems) != cudaSuccess ||
       // the hyperbatch may run on a stream that does not wait for this one
@@ -364,16 +362,13 @@ static agnes_status enqueue_hyperbatch(agnes_ctx* ctx, const int32_t* fanouts, i
     a.key = w.key;
     a.status = w.status;
     a.hset = w.hset;
-    a.fbd = w.fbd;
     huge_fanout_tables(fanouts[h], nsm, &a.hset_log2, &a.hset_grid);
     const bool frontier_sampled = ctx->frontier_mode == AGNES_FRONTIER_SAMPLED && h + 1 < K;
     a.sb_packed = !frontier_sampled && a.ecap <= kPackedEdgeMax;
     int32_t* nsz_prev = w.nsz + (int64_t)h * H;
     int32_t* ecnt = w.ecnt + (int64_t)h * H;
-    CK(ctx, launch_sample_count(a, w.fb_id[cur], w.fb_pos[cur], w.fcell_off[cur], w.cnt,
-                                ctx->bt.run_first_tile, ctx->bt.n_starts, w.stats + h, nsm, st));
-    CK(ctx, (seg_scan<int32_t, int64_t>(w.cnt, cap[h], w.indptr[h], cap[h] + 1, nsz_prev, 0, H,
-                                         cap[h], true, ecnt, w.scan_scratch, w.status, st)));
+    CK(ctx, launch_sample_indptr(a, w.nodes, nsz_prev, w.indptr[h], ecnt, w.indptr_scratch, nsm,
+                                 st));
     mark();
     // the previous hop's col fix-up still reads scell and newbase
     if (h > 0) {
@@ -416,6 +411,10 @@ static agnes_status enqueue_hyperbatch(agnes_ctx* ctx, const int32_t* fanouts, i
     d.big_list = w.big_list;
     d.q_dense = w.q_dense;
     d.q_ctl = w.q_ctl;
+    d.indptr_scratch = w.indptr_scratch;
+    d.run_first_tile = ctx->bt.run_first_tile;
+    d.n_runs = ctx->bt.n_starts;
+    d.touched = w.stats + h;
     d.big_n = w.big_n;
     d.fb_id = w.fb_id[cur];
     d.fb_pos = w.fb_pos[cur];
@@ -442,7 +441,7 @@ static agnes_status enqueue_hyperbatch(agnes_ctx* ctx, const int32_t* fanouts, i
     CK(ctx, launch_dedup(a, d, nsm, st));
     if (h + 1 == K) {
       // feature blocks touched by the hyperbatch, on the side stream beside the
-      // last compaction (each hop's count kernel counted the topology blocks)
+      // last compaction (each hop's scatter counted the topology blocks)
       CK(ctx, cudaEventRecord(ctx->aux_fork, st));
       CK(ctx, cudaStreamWaitEvent(ctx->aux, ctx->aux_fork, 0));
       CK(ctx, launch_count_touched(w.fcell_off[1 - cur], H, ctx->bt.fblock_first_tile,

@@ -16,9 +16,7 @@
 // draws slot s's candidate in parallel and the k-step collision resolution
 // runs over warp shuffles.  Above 32 a warp takes 32 slots at a time,
 // checking each candidate against the earlier chunks' choices (in shared
-// memory up to kWideMax, in a hash set in global memory beyond).  The count
-// kernel's (first edge, degree) per frontier entry lets the fill read them
-// coalesced.
+// memory up to kWideMax, in a hash set in global memory beyond).
 #include "common.cuh"
 #include "internal.h"
 
@@ -171,34 +169,142 @@ targets_sort_kernel(const int32_t* __restrict__ fcell_off, int64_t ncells, int32
 
 // ---- sampling --------------------------------------------------------------------
 
-// Per frontier entry i (bucket order): the node's count of sampled edges
-// min(deg, k) at its minibatch position (for the edge offsets' scan), and
-// (first edge, degree) in fbd[i] for the fill, which then reads them
-// coalesced instead of the offsets at random.  Also the hop's count of touched
-// topology blocks.
+// Edge offsets of one hop: indptr of every minibatch's dst list, the exclusive
+// scan of min(deg(nodes[i]), k) with the total at the end (also ecnt[j]).
+//
+// One pass (Merrill & Garland's decoupled look-back, 2016, per minibatch): a
+// CTA takes the next (tile of kIndptrTile dst rows, minibatch) pair from a
+// counter, tile-major, reads the rows' degrees, publishes the tile's sum and
+// walks back over its minibatch's earlier tiles until it meets an inclusive
+// prefix.  Pairs are taken in order, so a CTA waits only on pairs of CTAs that
+// are already running, and every wait is bounded.  Reading the degrees here in
+// dst order replaces a kernel that counted in bucket order, its scattered
+// counts, and the two passes over them: 16 x 1024 targets at [15, 10, 5] on 10M
+// nodes 653 -> 638 us a hyperbatch, 1 x 1024 272 -> 256 us.
+//
+// Scratch (uint64, zero on entry; the hop's scatter clears it): [0] the
+// counter, [1 + j * tiles + t] flag of minibatch j's tile t = state << 62 |
+// value, state 1 = the tile's sum, 2 = the inclusive prefix through it.
+constexpr int kIndptrItems = 8;
+constexpr int kIndptrTile = kThreads * kIndptrItems;
+constexpr unsigned long long kFlagAgg = 1ull << 62;
+constexpr unsigned long long kFlagInc = 2ull << 62;
+constexpr unsigned long long kFlagVal = (1ull << 62) - 1;
+constexpr int kIndptrSpinLimit = 1 << 20;
+
+struct IndptrArgs {
+  const int32_t* nodes;  // minibatch j's dst ids at j * capK
+  const int32_t* nsz;    // H: |dst|
+  const void* offsets;
+  bool off32;
+  int64_t capK, cap_prev;
+  int32_t H, k, tiles;  // tiles: ceil(cap_prev / kIndptrTile)
+  int64_t* indptr;
+  int32_t* ecnt;
+  unsigned long long* scratch;
+  int32_t* status;
+};
+
 template <typename OffT>
-__global__ void __launch_bounds__(kThreads)
-sample_count_kernel(const int32_t* __restrict__ fb_id, const int32_t* __restrict__ fb_pos,
-                    const int32_t* total_ptr, const OffT* __restrict__ off, int64_t capK,
-                    int64_t cap_prev, int32_t k, int32_t* __restrict__ cnt,
-                    longlong2* __restrict__ fbd, const int32_t* __restrict__ cell_off, int32_t H,
-                    const int32_t* __restrict__ run_first_tile, int64_t n_runs,
-                    int64_t* __restrict__ touched, const int32_t* status) {
+__global__ void __launch_bounds__(kThreads) sample_indptr_kernel(IndptrArgs a) {
   grid_dep_wait();
-  if (failed(status)) return;
-  count_touched(cell_off, H, run_first_tile, n_runs, touched);
-  const int64_t total = *total_ptr;
-  const uint32_t capk32 = (uint32_t)capK;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    const int32_t v = fb_id[i];
-    const uint32_t g = (uint32_t)fb_pos[i];
-    const uint32_t j = g / capk32;
-    const uint32_t pos = g - j * capk32;
-    const int64_t base = (int64_t)__ldg(off + v);
-    const int64_t d = (int64_t)__ldg(off + v + 1) - base;
-    cnt[j * cap_prev + pos] = (int32_t)(d < k ? d : k);
-    fbd[i] = make_longlong2(base, d);
+  if (cta_failed(a.status)) return;
+  __shared__ int32_t s_ticket;
+  __shared__ int32_t warp_tot[kWarps];
+  __shared__ int64_t s_excl;
+  const int tid = threadIdx.x, lane = lane_id(), warp = tid >> 5;
+  // pairs up to the longest minibatch's last tile
+  int32_t longest = 0;
+  for (int32_t j = tid; j < a.H; j += kThreads) longest = max(longest, a.nsz[j]);
+  longest = __reduce_max_sync(0xffffffffu, longest);
+  if (lane == 0) warp_tot[warp] = longest;
+  __syncthreads();
+  for (int w = 0; w < kWarps; ++w) longest = max(longest, warp_tot[w]);
+  const int32_t pairs = max(1, (longest + kIndptrTile - 1) / kIndptrTile) * a.H;  // < 2^31
+  const OffT* off = (const OffT*)a.offsets;
+  for (;;) {
+    __syncthreads();  // the shared words are rewritten
+    if (tid == 0) s_ticket = (int32_t)atomicAdd(a.scratch, 1ull);
+    __syncthreads();
+    const int32_t ticket = s_ticket;
+    if (ticket >= pairs) break;
+    const int32_t t = ticket / a.H, j = ticket - t * a.H;
+    const int32_t len = a.nsz[j];
+    const int32_t begin = t * kIndptrTile;
+    if (begin >= len && t > 0) continue;
+    unsigned long long* flags = a.scratch + 1 + (int64_t)j * a.tiles;
+    // a warp's 256 rows as eight coalesced 32-wide slices
+    const int32_t* nodes = a.nodes + (int64_t)j * a.capK;
+    const int32_t wbase = begin + warp * (32 * kIndptrItems);
+    int32_t v[kIndptrItems], c[kIndptrItems];
+#pragma unroll
+    for (int q = 0; q < kIndptrItems; ++q) {
+      const int32_t i = wbase + 32 * q + lane;
+      v[q] = i < len ? nodes[i] : -1;
+    }
+#pragma unroll
+    for (int q = 0; q < kIndptrItems; ++q) {
+      c[q] = 0;
+      if (v[q] >= 0) {
+        const int64_t d = (int64_t)__ldg(off + v[q] + 1) - (int64_t)__ldg(off + v[q]);
+        c[q] = (int32_t)(d < a.k ? d : a.k);
+      }
+    }
+    int32_t sum = 0;  // exclusive within the warp, slice by slice (a tile's edges < 2^31)
+#pragma unroll
+    for (int q = 0; q < kIndptrItems; ++q) {
+      const int32_t incl = warp_incl_scan(c[q]);
+      c[q] = sum + incl - c[q];
+      sum += __shfl_sync(0xffffffffu, incl, 31);
+    }
+    if (lane == 0) warp_tot[warp] = sum;
+    __syncthreads();
+    if (warp == 0) {
+      const int32_t w = lane < kWarps ? warp_tot[lane] : 0;
+      const int32_t wi = warp_incl_scan(w);
+      const int64_t agg = __shfl_sync(0xffffffffu, wi, kWarps - 1);
+      if (lane < kWarps) warp_tot[lane] = wi - w;
+      int64_t excl = 0;
+      if (t > 0) {
+        if (lane == 0) atomicExch(flags + t, kFlagAgg | (unsigned long long)agg);
+        for (int32_t p = t - 1;; p -= 32) {
+          const int32_t idx = p - lane;  // lane 0 the nearest predecessor
+          unsigned long long f = kFlagInc;  // before tile 0: an inclusive prefix of 0
+          if (idx >= 0) {
+            f = *(const volatile unsigned long long*)(flags + idx);
+            for (int spin = 0; (f >> 62) == 0; ++spin) {
+              if (spin == kIndptrSpinLimit) {
+                atomicOr(a.status, kErrWaitTimeout);
+                f = kFlagInc;
+                break;
+              }
+              __nanosleep(32);
+              f = *(const volatile unsigned long long*)(flags + idx);
+            }
+          }
+          const unsigned inc = __ballot_sync(0xffffffffu, (f >> 62) == 2);
+          const int stop = inc ? __ffs(inc) - 1 : 31;  // lanes 0 .. stop contribute
+          excl += warp_sum(lane <= stop ? (int64_t)(f & kFlagVal) : (int64_t)0);
+          if (inc) break;
+        }
+      }
+      if (lane == 0) {
+        atomicExch(flags + t, kFlagInc | (unsigned long long)(excl + agg));
+        s_excl = excl;
+        if (begin + kIndptrTile >= len) {  // the minibatch's last tile
+          a.indptr[(int64_t)j * (a.cap_prev + 1) + len] = excl + agg;
+          a.ecnt[j] = (int32_t)(excl + agg);
+        }
+      }
+    }
+    __syncthreads();
+    const int64_t base = s_excl + warp_tot[warp];
+    int64_t* indptr = a.indptr + (int64_t)j * (a.cap_prev + 1);
+#pragma unroll
+    for (int q = 0; q < kIndptrItems; ++q) {
+      const int32_t i = wbase + 32 * q + lane;
+      if (i < len) indptr[i] = base + c[q];
+    }
   }
 }
 
@@ -220,7 +326,8 @@ struct FillArgs {
   int32_t* srank;  // per edge: its rank within the cell
   const int32_t* fb_id;
   const int32_t* fb_pos;
-  const longlong2* fbd;  // per frontier entry: (first edge, degree) of its node
+  const void* offsets;
+  bool off32;
   const int64_t* indptr;
   const int32_t* indices;
   int32_t* nbr;
@@ -244,6 +351,22 @@ struct Key {
 __device__ __forceinline__ Key load_key(const uint64_t* key) {
   const uint64_t seed = __ldg(key);
   return Key{(uint32_t)seed, (uint32_t)(seed >> 32), __ldg(key + 1)};
+}
+
+// First edge and degree of node v.  Entries are walked in bucket order, so
+// neighbouring lanes' offsets share cache lines.
+__device__ __forceinline__ longlong2 first_and_degree(const FillArgs& a, int32_t v) {
+  int64_t lo, hi;
+  if (a.off32) {
+    const int32_t* off = (const int32_t*)a.offsets + v;
+    lo = __ldg(off);
+    hi = __ldg(off + 1);
+  } else {
+    const int64_t* off = (const int64_t*)a.offsets + v;
+    lo = __ldg(off);
+    hi = __ldg(off + 1);
+  }
+  return make_longlong2(lo, hi - lo);
 }
 
 // Where the sampler reads neighbour entries.
@@ -340,7 +463,7 @@ __global__ void __launch_bounds__(kThreads, 8) sample_fill_kernel(FillArgs a) {
     if (live) {
       v = a.fb_id[i];
       g = (uint32_t)a.fb_pos[i];
-      bd = a.fbd[i];
+      bd = first_and_degree(a, v);
     }
     const int64_t base = bd.x, d = bd.y;
     const uint32_t j = g / capk32;
@@ -392,7 +515,7 @@ __global__ void __launch_bounds__(kThreads) sample_fill_wide_kernel(FillArgs a) 
     const uint32_t g = (uint32_t)a.fb_pos[i];
     const uint32_t j = g / capk32;
     const uint32_t pos = g - j * capk32;
-    const longlong2 bd = a.fbd[i];
+    const longlong2 bd = first_and_degree(a, v);
     const int64_t base = bd.x, d = bd.y;
     const int64_t ebase = a.indptr[j * (a.cap_prev + 1) + pos];
     if (d <= a.k) {
@@ -476,7 +599,7 @@ __global__ void __launch_bounds__(kThreads) sample_fill_huge_kernel(FillArgs a) 
     const uint32_t g = (uint32_t)a.fb_pos[i];
     const uint32_t j = g / capk32;
     const uint32_t pos = g - j * capk32;
-    const longlong2 bd = a.fbd[i];
+    const longlong2 bd = first_and_degree(a, v);
     const int64_t base = bd.x, d = bd.y;
     const int64_t ebase = a.indptr[j * (a.cap_prev + 1) + pos];
     if (d <= a.k) {
@@ -552,25 +675,36 @@ cudaError_t launch_bucket_targets(int32_t* nodes, int64_t capK, int32_t H, int32
   return cudaGetLastError();
 }
 
-cudaError_t launch_sample_count(const HopArgs& a, const int32_t* fb_id, const int32_t* fb_pos,
-                                const int32_t* fcell_off, int32_t* cnt,
-                                const int32_t* run_first_tile, int64_t n_runs, int64_t* touched,
-                                int num_sms, cudaStream_t st) {
-  const int32_t* total = fcell_off + (int64_t)a.T * a.H;
-  if (a.offsets_bits == 32)
-    sample_count_kernel<int32_t><<<resident_grid((const void*)sample_count_kernel<int32_t>,
-                                                 kThreads, num_sms),
-                                   kThreads, 0, st>>>(
-        fb_id, fb_pos, total, (const int32_t*)a.offsets, a.capK, a.cap_prev, a.k, cnt,
-        reinterpret_cast<longlong2*>(a.fbd), fcell_off, a.H, run_first_tile, n_runs, touched,
-        a.status);
+int64_t indptr_scratch_elems(int32_t H, int64_t cap_prev) {
+  return 1 + H * ((cap_prev + kIndptrTile - 1) / kIndptrTile);
+}
+
+cudaError_t launch_sample_indptr(const HopArgs& a, const int32_t* nodes, const int32_t* nsz,
+                                 int64_t* indptr, int32_t* ecnt, uint64_t* scratch, int num_sms,
+                                 cudaStream_t st) {
+  IndptrArgs p;
+  p.nodes = nodes;
+  p.nsz = nsz;
+  p.offsets = a.offsets;
+  p.off32 = a.offsets_bits == 32;
+  p.capK = a.capK;
+  p.cap_prev = a.cap_prev;
+  p.H = a.H;
+  p.k = a.k;
+  p.tiles = (int32_t)((a.cap_prev + kIndptrTile - 1) / kIndptrTile);
+  p.indptr = indptr;
+  p.ecnt = ecnt;
+  p.scratch = reinterpret_cast<unsigned long long*>(scratch);
+  p.status = a.status;
+  const void* kernel = p.off32 ? (const void*)sample_indptr_kernel<int32_t>
+                               : (const void*)sample_indptr_kernel<int64_t>;
+  const int64_t pairs = (int64_t)p.tiles * a.H;  // at most H * ceil(cap / tile) < 2^31
+  const int resident = resident_grid(kernel, kThreads, num_sms);
+  const int grid = (int)(pairs < resident ? pairs : resident);
+  if (p.off32)
+    sample_indptr_kernel<int32_t><<<grid, kThreads, 0, st>>>(p);
   else
-    sample_count_kernel<int64_t><<<resident_grid((const void*)sample_count_kernel<int64_t>,
-                                                 kThreads, num_sms),
-                                   kThreads, 0, st>>>(
-        fb_id, fb_pos, total, (const int64_t*)a.offsets, a.capK, a.cap_prev, a.k, cnt,
-        reinterpret_cast<longlong2*>(a.fbd), fcell_off, a.H, run_first_tile, n_runs, touched,
-        a.status);
+    sample_indptr_kernel<int64_t><<<grid, kThreads, 0, st>>>(p);
   return cudaGetLastError();
 }
 
@@ -611,7 +745,8 @@ cudaError_t launch_sample_fill(const HopArgs& a, const int32_t* fb_id, const int
   f.srank = srank;
   f.fb_id = fb_id;
   f.fb_pos = fb_pos;
-  f.fbd = reinterpret_cast<const longlong2*>(a.fbd);
+  f.offsets = a.offsets;
+  f.off32 = a.offsets_bits == 32;
   f.indptr = indptr;
   f.indices = a.indices;
   f.nbr = nbr;

@@ -492,9 +492,6 @@ cudaError_t seg_scan(const InT* in, int64_t in_stride, OutT* out, int64_t out_st
 template cudaError_t seg_scan<int32_t, int32_t>(const int32_t*, int64_t, int32_t*, int64_t,
                                                 const int32_t*, int64_t, int32_t, int64_t, bool,
                                                 int32_t*, int64_t*, const int32_t*, cudaStream_t);
-template cudaError_t seg_scan<int32_t, int64_t>(const int32_t*, int64_t, int64_t*, int64_t,
-                                                const int32_t*, int64_t, int32_t, int64_t, bool,
-                                                int32_t*, int64_t*, const int32_t*, cudaStream_t);
 template cudaError_t seg_scan<uint8_t, int32_t>(const uint8_t*, int64_t, int32_t*, int64_t,
                                                 const int32_t*, int64_t, int32_t, int64_t, bool,
                                                 int32_t*, int64_t*, const int32_t*, cudaStream_t);
