@@ -224,10 +224,7 @@ agnes_status agnes_set_frontier_mode(agnes_ctx* ctx, int32_t mode);
  *   every block of the previous one has exited, and first waits for its
  *   writes to become visible), so each launch overlaps the previous kernel's
  *   completion.
- * In every mode, work off the critical chain (each hop's new-id scan and col
- * fix-up, the touched-block statistics) runs on a side stream the ctx owns,
- * forked from and joined back into the caller's stream within the call's
- * work.  Results are identical in every mode.  A caller stream that is itself being
+ * Results are identical in every mode.  A caller stream that is itself being
  * captured, and the host-resident modes (whose calls read sizes back
  * mid-sequence), always take the direct path.  Errors: EINVAL. */
 #define AGNES_LAUNCH_DIRECT 0

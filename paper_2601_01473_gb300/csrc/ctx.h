@@ -76,7 +76,7 @@ struct Workspace {
   int64_t flat_elems = 0;
   void* feats_out = nullptr;
   int64_t* scan_scratch = nullptr;
-  int64_t* side_scratch = nullptr;  // scans on the side stream
+  int32_t* cols_scratch = nullptr;  // column scans' chunk sums
   unsigned long long* distinct = nullptr;
   uint64_t* key = nullptr;  // sampling key {seed, first minibatch id}
 
@@ -150,13 +150,6 @@ struct agnes_ctx {
   cudaEvent_t ev[agnes::kEventRing][agnes::kMaxPhases + 1] = {{nullptr}};
   bool ev_created = false;
   uint64_t ws_gen = 0;  // bumped whenever the workspace is reallocated
-  // side stream of a hyperbatch: each hop's new-id scan and col fix-up run on
-  // it (forked after the cells are resolved; the compaction waits for the
-  // scan through aux_ready; joined before the next hop's sampling), and the
-  // touched-block statistics (forked before the last compaction, joined
-  // before the size read-back)
-  cudaStream_t aux = nullptr;
-  cudaEvent_t aux_fork = nullptr, aux_join = nullptr, aux_ready = nullptr;
 
   // The resident path's launch sequence, captured once per hyperbatch shape
   // and replayed as one CUDA graph launch (agnes_set_launch_mode).
@@ -177,8 +170,8 @@ struct agnes_ctx {
 
   // Hyperbatches in flight (agnes_set_pipeline_depth): with a depth of d > 1
   // the ctx keeps d - 1 more sets of the per-hyperbatch state -- workspace,
-  // launch graph, completion and side-stream events, side stream, its own
-  // internal stream and the fetch state -- and rotates them with the active
+  // launch graph, completion event, its own internal
+  // stream and the fetch state -- and rotates them with the active
   // set at every prepare, so consecutive hyperbatches use the sets in turn
   // and run on their internal streams, overlapping.  The active set (the
   // fields above and pipe_st) always belongs to the last prepare; spares[0]
@@ -191,8 +184,7 @@ struct agnes_ctx {
     agnes::Workspace ws;
     LaunchGraph lg;
     uint64_t ws_gen = 0;
-    cudaEvent_t done = nullptr, aux_fork = nullptr, aux_join = nullptr, aux_ready = nullptr;
-    cudaStream_t aux = nullptr;
+    cudaEvent_t done = nullptr;
     cudaStream_t pipe_st = nullptr;
     int cur = 0;
     bool prepared = false, synced = false;

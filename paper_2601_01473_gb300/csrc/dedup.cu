@@ -12,7 +12,7 @@
 // next hop's frontier bucket (D | new in ascending id); after the scans, a
 // fix-up pass and a compaction pass turn the local ranks into final indices.
 // The bucket is carried from hop to hop and never rebuilt.  This file holds
-// the scatter, the scans, the fix-up and the compaction, and the cell kernels
+// the scatter, the compaction with the fix-up, and the cell kernels
 // of the sampled frontier; the default frontier's cells are resolved in
 // dedup_cells.cu.
 #include "common.cuh"
@@ -433,37 +433,7 @@ __global__ void __launch_bounds__(kThreads) dedup_big_kernel(CellArgs a) {
   }
 }
 
-// ---- fix-up and compaction (after the scans) --------------------------------------
-
-// col[e] = -(1 + r) becomes the new node's index in src_h:
-// |dst_h| + (new ids of the minibatch in earlier tiles) + r.
-__global__ void __launch_bounds__(kThreads)
-dedup_fix_col_kernel(int32_t* __restrict__ col, const int32_t* __restrict__ ecnt, int64_t ecap,
-                     const int32_t* __restrict__ scell, const int32_t* __restrict__ newbase,
-                     const int32_t* __restrict__ nsz_prev, const int32_t* status) {
-  grid_dep_wait();
-  if (failed(status)) return;
-  const int32_t j = blockIdx.y;
-  const int64_t E = ecnt[j];
-  const int64_t o = (int64_t)j * ecap;
-  const int32_t base = nsz_prev[j];
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t e0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e0 < E;
-       e0 += kIlp * stride) {  // kIlp edges per thread: their base loads in flight together
-    int32_t v[kIlp], cell[kIlp], nb[kIlp];
-#pragma unroll
-    for (int k = 0; k < kIlp; ++k) {
-      const int64_t e = e0 + k * stride;
-      v[k] = e < E ? col[o + e] : 0;
-      cell[k] = e < E ? scell[o + e] : 0;
-    }
-#pragma unroll
-    for (int k = 0; k < kIlp; ++k) nb[k] = v[k] < 0 ? newbase[cell[k]] : 0;
-#pragma unroll
-    for (int k = 0; k < kIlp; ++k)
-      if (v[k] < 0) col[o + e0 + k * stride] = base + nb[k] + (-1 - v[k]);
-  }
-}
+// ---- compaction and fix-up (after the scans) --------------------------------------
 
 struct CompactArgs {
   int64_t ncells;
@@ -483,8 +453,43 @@ struct CompactArgs {
   int32_t* nfb_id;
   int32_t* nfb_pos;
   int32_t* nodes;
+  // the col fix-up: H x ecap edges, ecnt[j] of minibatch j's, fix_ctas CTAs each
+  int32_t* col;
+  const int32_t* ecnt;
+  int64_t ecap;
+  const int32_t* scell;
+  int32_t fix_ctas;
+  // the last hop's count of touched feature blocks (n_feat_blocks 0: none)
+  const int32_t* fblock_first_tile;
+  int64_t n_feat_blocks;
+  int64_t* feat_touched;
   const int32_t* status;
 };
+
+// col[e] = -(1 + r) becomes the new node's index in src_h:
+// |dst_h| + (new ids of the minibatch in earlier tiles) + r.  kIlp edges per
+// thread: their base loads in flight together.
+__device__ __forceinline__ void fix_col(const CompactArgs& a, int32_t j, int32_t part) {
+  const int64_t E = a.ecnt[j];
+  int32_t* col = a.col + (int64_t)j * a.ecap;
+  const int32_t* scell = a.scell + (int64_t)j * a.ecap;
+  const int32_t base = a.nsz_prev[j];
+  const int64_t stride = (int64_t)a.fix_ctas * kCellThreads;
+  for (int64_t e0 = (int64_t)part * kCellThreads + threadIdx.x; e0 < E; e0 += kIlp * stride) {
+    int32_t v[kIlp], cell[kIlp], nb[kIlp];
+#pragma unroll
+    for (int k = 0; k < kIlp; ++k) {
+      const int64_t e = e0 + k * stride;
+      v[k] = e < E ? col[e] : 0;
+      cell[k] = e < E ? scell[e] : 0;
+    }
+#pragma unroll
+    for (int k = 0; k < kIlp; ++k) nb[k] = v[k] < 0 ? a.newbase[cell[k]] : 0;
+#pragma unroll
+    for (int k = 0; k < kIlp; ++k)
+      if (v[k] < 0) col[e0 + k * stride] = base + nb[k] + (-1 - v[k]);
+  }
+}
 
 // Writes the next frontier bucket in cell order: a cell without samples is
 // copied from the current bucket, any other from its tmp entries, where a new
@@ -495,6 +500,8 @@ struct CompactArgs {
 // entries' loads are latency-bound, so they need every SM (8 minibatches of
 // 500 at [25, 10] on 250k nodes: 446 -> 349 us a hyperbatch; two items per
 // resident CTA, where four cost 3% and eight 5% on 10M nodes).
+// The col fix-up needs the same scans and nothing else, so the CTAs take it on
+// afterwards in the same launch.
 __global__ void __launch_bounds__(kCellThreads) dedup_compact_kernel(CompactArgs a) {
   grid_dep_wait();
   if (failed(a.status)) return;
@@ -572,6 +579,14 @@ __global__ void __launch_bounds__(kCellThreads) dedup_compact_kernel(CompactArgs
     }
     __syncthreads();
   }
+  const int64_t nfix = (int64_t)a.H * a.fix_ctas;
+  for (int64_t f = blockIdx.x; f < nfix; f += gridDim.x) {
+    const int32_t j = (int32_t)(f / a.fix_ctas);
+    fix_col(a, j, (int32_t)(f - (int64_t)j * a.fix_ctas));
+  }
+  if (a.n_feat_blocks > 0)
+    count_touched(blockIdx.x * (int64_t)kCellThreads + tid, (int64_t)gridDim.x * kCellThreads,
+                  a.nfcell_off, a.H, a.fblock_first_tile, a.n_feat_blocks, a.feat_touched);
 }
 
 }  // namespace
@@ -626,39 +641,13 @@ cudaError_t launch_dedup(const HopArgs& a, const DedupBufs& d, int num_sms, cuda
   // tile-major [T x H] count matrix; totals give the next frontier sizes
   // |src_h| = |dst_h| + new ids; the next frontier is src_h, or (sampled
   // frontier) the distinct sampled ids, numbered by their own column scan.
-  // With a side stream, the new-id scan and the col fix-up (which needs only
-  // its result) run there, beside the scans of the next-frontier counts; the
-  // side stream has its own scan scratch, and the compaction waits for the
-  // new-id offsets.
-  cudaStream_t nst = st;
-  int64_t* nscratch = d.scan_scratch;
-  if (d.side) {
-    if ((e = cudaEventRecord(d.fork, st)) != cudaSuccess) return e;
-    if ((e = cudaStreamWaitEvent(d.side, d.fork, 0)) != cudaSuccess) return e;
-    nst = d.side;
-    nscratch = d.side_scratch;
-  }
-  e = col_scan(d.newcnt, d.newbase, a.T, a.H, d.nsz_prev, d.srcsz,
-               d.frontier_sampled ? nullptr : d.nsz_next, nscratch, a.status, nst);
+  const ColumnScan scans[2] = {
+      {d.newcnt, d.newbase, d.nsz_prev, {d.srcsz, d.frontier_sampled ? nullptr : d.nsz_next}},
+      {d.nfcnt, d.noutbase, nullptr, {d.nsz_next, nullptr}}};
+  e = cell_scans(a.T, a.H, d.nfcnt, d.nfcell_off, d.flat_scratch, scans,
+                 d.frontier_sampled ? 2 : 1, d.cols_scratch, a.status, st);
   if (e != cudaSuccess) return e;
-  if (d.side && (e = cudaEventRecord(d.ready, d.side)) != cudaSuccess) return e;
-  dedup_fix_col_kernel<<<egrid, kThreads, 0, nst>>>(d.col, d.ecnt, a.ecap, d.scell, d.newbase,
-                                                    d.nsz_prev, a.status);
-  if (d.frontier_sampled) {
-    e = col_scan(d.nfcnt, d.noutbase, a.T, a.H, nullptr, d.nsz_next, nullptr, d.scan_scratch,
-                 a.status, st);
-    if (e != cudaSuccess) return e;
-  }
-  e = flat_scan(d.nfcnt, d.nfcell_off, ncells, true, nullptr, false, d.flat_scratch, a.status,
-                st);
-  if (e != cudaSuccess) return e;
-  if (d.side && (e = cudaStreamWaitEvent(st, d.ready, 0)) != cudaSuccess) return e;
-  return cudaGetLastError();
-}
 
-cudaError_t launch_dedup_compact(const HopArgs& a, const DedupBufs& d, int num_sms,
-                                 cudaStream_t st) {
-  const int64_t ncells = (int64_t)a.T * a.H;
   CompactArgs k;
   k.ncells = ncells;
   k.H = a.H;
@@ -676,8 +665,16 @@ cudaError_t launch_dedup_compact(const HopArgs& a, const DedupBufs& d, int num_s
   k.nfb_id = d.nfb_id;
   k.nfb_pos = d.nfb_pos;
   k.nodes = d.nodes;
+  k.col = d.col;
+  k.ecnt = d.ecnt;
+  k.ecap = a.ecap;
+  k.scell = d.scell;
+  k.fblock_first_tile = d.fblock_first_tile;
+  k.n_feat_blocks = d.n_feat_blocks;
+  k.feat_touched = d.feat_touched;
   k.status = a.status;
   const int grid = resident_grid((const void*)dedup_compact_kernel, kCellThreads, num_sms);
+  k.fix_ctas = grid / a.H > 1 ? grid / a.H : 1;
   const int64_t ngroups = (ncells + kGroupCells - 1) / kGroupCells;
   const int64_t slices = (kCompactOversplit * (int64_t)grid + ngroups - 1) / ngroups;
   k.slices = (int32_t)(slices > kCompactMaxSlices ? kCompactMaxSlices : slices);

@@ -116,16 +116,6 @@ load_feat_blocks_kernel(const uint4* __restrict__ host, int64_t host_vecs,
   }
 }
 
-__global__ void __launch_bounds__(kThreads)
-count_touched_kernel(const int32_t* __restrict__ cell_off, int32_t H,
-                     const int32_t* __restrict__ first_tile, int64_t n,
-                     int64_t* __restrict__ count, const int32_t* status) {
-  grid_dep_wait();
-  if (failed(status)) return;
-  count_touched(blockIdx.x * (int64_t)blockDim.x + threadIdx.x, (int64_t)gridDim.x * blockDim.x,
-                cell_off, H, first_tile, n, count);
-}
-
 // Requests per feature block: counts[tile_feat_block[t]] += entries of tile t.
 __global__ void count_requests_kernel(const int32_t* __restrict__ cell_off, int32_t T, int32_t H,
                                       const int32_t* __restrict__ tile_map,
@@ -544,15 +534,6 @@ cudaError_t launch_gather_staged_rows(const void* staging, int64_t row_bytes, co
                                                         wpref, doff, addr, (int32_t)rpb, cache_lo,
                                                         cache_hi, o, status);
 #undef AGNES_GSR
-  return cudaGetLastError();
-}
-
-cudaError_t launch_count_touched(const int32_t* cell_off, int32_t H, const int32_t* first_tile,
-                                 int64_t n, int64_t* count, const int32_t* status,
-                                 cudaStream_t st) {
-  const int64_t blocks = (n + kThreads - 1) / kThreads;
-  count_touched_kernel<<<(unsigned)std::min<int64_t>(blocks, 1184), kThreads, 0, st>>>(
-      cell_off, H, first_tile, n, count, status);
   return cudaGetLastError();
 }
 

@@ -38,14 +38,22 @@ cudaError_t flat_scan(int32_t* in, int32_t* out, int64_t n, bool write_end, int3
                       bool clear, uint64_t* scratch, int32_t* status, cudaStream_t st);
 
 // Exclusive scan down each column of a row-major [rows x cols] matrix:
-// out[r*cols + c] = sum of in[r'*cols + c] over r' < r (coalesced along
-// rows).  total_out[c] (if non-null) = column total + add_in[c] (add_in may be
-// null), and so does total_out2[c].  scratch needs
-// col_scan_scratch_elems(rows, cols) int64s.
-int64_t col_scan_scratch_elems(int64_t rows, int32_t cols);
-cudaError_t col_scan(const int32_t* in, int32_t* out, int64_t rows, int32_t cols,
-                     const int32_t* add_in, int32_t* total_out, int32_t* total_out2,
-                     int64_t* scratch, const int32_t* status, cudaStream_t st);
+// out[r*cols + c] = sum of in[r'*cols + c] over r' < r; total[i][c] (where
+// non-null) = the column's total + add_in[c] (add_in may be null).
+struct ColumnScan {
+  const int32_t* in;
+  int32_t* out;
+  const int32_t* add_in;
+  int32_t* total[2];
+};
+
+// The flat_scan of rows * cols counts into offsets (rows * cols + 1 entries)
+// and up to two column scans of [rows x cols] matrices, in two launches.
+// flat_scratch as for flat_scan; scratch: cell_scans_scratch_elems int32s.
+int64_t cell_scans_scratch_elems(int64_t rows, int32_t cols);
+cudaError_t cell_scans(int64_t rows, int32_t cols, int32_t* counts, int32_t* offsets,
+                       uint64_t* flat_scratch, const ColumnScan* scans, int32_t nscans,
+                       int32_t* scratch, int32_t* status, cudaStream_t st);
 
 // ---- blocks.cu -------------------------------------------------------------
 struct BlockTables {
@@ -201,25 +209,20 @@ struct DedupBufs {
   bool frontier_sampled;    // next frontier = distinct sampled ids (Algorithm 1's N_out)
   int32_t* nodes;           // H x capK
   int32_t* col;             // H x ecap
-  int64_t* scan_scratch;
-  uint64_t* flat_scratch = nullptr;  // flat_scan_scratch_elems(T*H)
-  // If side is set, the new-id scan (into newbase, with side_scratch) and the
-  // col fix-up (which needs only newbase, col and scell) run on it, forked
-  // from st through the event fork; st waits for the scan through the event
-  // ready, and the caller joins side back before anything rewrites scell,
-  // newbase or the hop's col.
-  cudaStream_t side = nullptr;
-  cudaEvent_t fork = nullptr, ready = nullptr;
-  int64_t* side_scratch = nullptr;  // col_scan_scratch_elems(T, H) int64
+  int32_t* cols_scratch;    // cell_scans_scratch_elems(T, H) int32s
+  uint64_t* flat_scratch;   // flat_scan_scratch_elems(T*H)
+  // the last hop: *feat_touched += the feature blocks holding a gathered
+  // node, of the n_feat_blocks with tiles fblock_first_tile[b] .. [b + 1] - 1
+  const int32_t* fblock_first_tile = nullptr;
+  int64_t n_feat_blocks = 0;
+  int64_t* feat_touched = nullptr;
 };
 
-// One hop's dedup up to the next-frontier offsets (nfcell_off, nsz_next) and
-// the new-id offsets (newbase): scatter, cells, big cells, scans, col fix-up.
+// One hop's dedup: scatter, cells, the scans of their counts (nfcell_off,
+// newbase, nsz_next, srcsz), then the compaction with the col fix-up: the next
+// frontier bucket (nfb_id / nfb_pos), the new nodes' ids in the node lists,
+// and the final col.
 cudaError_t launch_dedup(const HopArgs& a, const DedupBufs& d, int num_sms, cudaStream_t st);
-// Then the compaction: the next frontier bucket (nfb_id / nfb_pos) and the
-// new nodes' ids in the node lists.
-cudaError_t launch_dedup_compact(const HopArgs& a, const DedupBufs& d, int num_sms,
-                                 cudaStream_t st);
 
 // ---- dedup_cells.cu --------------------------------------------------------
 // The default frontier's resolution of one hop's cells (launch_dedup calls
@@ -288,12 +291,6 @@ cudaError_t launch_gather_staged_rows(const void* staging, int64_t row_bytes, co
 cudaError_t launch_load_feat_blocks(const void* host_dev, int64_t host_bytes, const int32_t* blk,
                                     const unsigned long long* dst, int32_t njobs,
                                     int64_t block_bytes, int num_sms, cudaStream_t st);
-
-// *count += the number of the n blocks whose tiles [first_tile[b],
-// first_tile[b + 1]) hold an entry of the bucket with offsets cell_off.
-cudaError_t launch_count_touched(const int32_t* cell_off, int32_t H, const int32_t* first_tile,
-                                 int64_t n, int64_t* count, const int32_t* status,
-                                 cudaStream_t st);
 
 // Topology cache bookkeeping for one hop's frontier bucket: acc[run] +=
 // requests of the block run's tiles; cached += requests on tiles whose

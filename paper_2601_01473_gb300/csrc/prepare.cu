@@ -6,7 +6,6 @@
 //                 bucket the samples, dedup + relabel, carry the bucket
 //                                                             [dedup.cu]
 //   gather the final bucket's rows block by block             [gather_hbm.cu]
-//   count the blocks touched (the paper's block-wise I/Os)   [gather.cu]
 // Everything is sized for the worst case up front (per-minibatch capacities
 // cap_h = min(N, B * prod(1 + k))), so no kernel's launch waits on a count
 // from the device and the host synchronises only when a view is fetched.
@@ -100,7 +99,7 @@ void free_workspace(Workspace* w) {
   cudaFree(w->flat_scratch);
   cudaFree(w->feats_out);
   cudaFree(w->scan_scratch);
-  cudaFree(w->side_scratch);
+  cudaFree(w->cols_scratch);
   cudaFree(w->distinct);
   cudaFree(w->key);
   if (w->h_back) cudaFreeHost(w->h_back);
@@ -140,9 +139,7 @@ static agnes_status ensure_workspace(agnes_ctx* ctx, int32_t H, int32_t B, const
   const int64_t edges = (int64_t)H * w.ecap_max;
   int64_t scratch = scan_scratch_elems(1, cells);
   const int64_t s2 = scan_scratch_elems(1, ctx->N);
-  const int64_t s4 = col_scan_scratch_elems(T, H);
   if (s2 > scratch) scratch = s2;
-  if (s4 > scratch) scratch = s4;
 
 #define WA(p, n)                                                                             \
   do {                                                                                       \
@@ -211,7 +208,7 @@ static agnes_status ensure_workspace(agnes_ctx* ctx, int32_t H, int32_t B, const
     w.feats_out = f;
   }
   WA(w.scan_scratch, scratch);
-  WA(w.side_scratch, s4);
+  WA(w.cols_scratch, cell_scans_scratch_elems(T, H));
   WA(w.distinct, 1);
   WA(w.key, 2);
 #undef WA
@@ -223,7 +220,6 @@ static agnes_status ensure_workspace(agnes_ctx* ctx, int32_t H, int32_t B, const
     return AGNES_ENOMEM;
   }
   if (cudaMemset(w.scan_scratch, 0, sizeof(int64_t) * scratch) != cudaSuccess ||
-      cudaMemset(w.side_scratch, 0, sizeof(int64_t) * s4) != cudaSuccess ||
       cudaMemset(w.indptr_scratch, 0, sizeof(uint64_t) * indptr_elems) != cudaSuccess ||
       cudaMemset(w.scnt, 0, sizeof(int32_t) * cells) != cudaSuccess ||
       cudaMemset(w.flat_scratch, 0, sizeof(uint64_t) * w.flat_elems) != cudaSuccess ||
@@ -242,10 +238,6 @@ void swap_hyperbatch_state(agnes_ctx* ctx, agnes_ctx::Spare& o) {
   std::swap(ctx->lg, o.lg);
   std::swap(ctx->ws_gen, o.ws_gen);
   std::swap(ctx->done, o.done);
-  std::swap(ctx->aux_fork, o.aux_fork);
-  std::swap(ctx->aux_join, o.aux_join);
-  std::swap(ctx->aux_ready, o.aux_ready);
-  std::swap(ctx->aux, o.aux);
   std::swap(ctx->pipe_st, o.pipe_st);
   std::swap(ctx->cur, o.cur);
   std::swap(ctx->prepared, o.prepared);
@@ -261,10 +253,6 @@ static agnes_status make_one_spare(agnes_ctx* ctx, agnes_ctx::Spare& o) {
   if (o.done) return AGNES_OK;
   const unsigned f = cudaEventDisableTiming;
   if (cudaEventCreateWithFlags(&o.done, f) != cudaSuccess ||
-      cudaEventCreateWithFlags(&o.aux_fork, f) != cudaSuccess ||
-      cudaEventCreateWithFlags(&o.aux_join, f) != cudaSuccess ||
-      cudaEventCreateWithFlags(&o.aux_ready, f) != cudaSuccess ||
-      cudaStreamCreateWithFlags(&o.aux, cudaStreamNonBlocking) != cudaSuccess ||
       cudaStreamCreateWithFlags(&o.pipe_st, cudaStreamNonBlocking) != cudaSuccess) {
     cudaGetLastError();
     set_err(ctx, "creating a further hyperbatch's events or streams failed");
@@ -297,10 +285,6 @@ void free_spare_state(agnes_ctx* ctx) {
     o.lg.cap = nullptr;
     free_workspace(&o.ws);
     if (o.done) cudaEventDestroy(o.done);
-    if (o.aux_fork) cudaEventDestroy(o.aux_fork);
-    if (o.aux_join) cudaEventDestroy(o.aux_join);
-    if (o.aux_ready) cudaEventDestroy(o.aux_ready);
-    if (o.aux) cudaStreamDestroy(o.aux);
     if (o.pipe_st) cudaStreamDestroy(o.pipe_st);
     const int32_t mode = o.lg.mode;
     o = agnes_ctx::Spare();
@@ -370,11 +354,6 @@ static agnes_status enqueue_hyperbatch(agnes_ctx* ctx, const int32_t* fanouts, i
     CK(ctx, launch_sample_indptr(a, w.nodes, nsz_prev, w.indptr[h], ecnt, w.indptr_scratch, nsm,
                                  st));
     mark();
-    // the previous hop's col fix-up still reads scell and newbase
-    if (h > 0) {
-      CK(ctx, cudaEventRecord(ctx->aux_join, ctx->aux));
-      CK(ctx, cudaStreamWaitEvent(st, ctx->aux_join, 0));
-    }
     if (ctx->topo.on) {
       rc = fill_streamed(ctx, a, cur, h, st);
       if (rc != AGNES_OK) return rc;
@@ -432,22 +411,14 @@ static agnes_status enqueue_hyperbatch(agnes_ctx* ctx, const int32_t* fanouts, i
     d.frontier_sampled = frontier_sampled;
     d.nodes = w.nodes;
     d.col = w.col[h];
-    d.scan_scratch = w.scan_scratch;
+    d.cols_scratch = w.cols_scratch;
     d.flat_scratch = w.flat_scratch;
-    d.side = ctx->aux;
-    d.fork = ctx->aux_fork;
-    d.ready = ctx->aux_ready;
-    d.side_scratch = w.side_scratch;
-    CK(ctx, launch_dedup(a, d, nsm, st));
     if (h + 1 == K) {
-      // feature blocks touched by the hyperbatch, on the side stream beside the
-      // last compaction (each hop's scatter counted the topology blocks)
-      CK(ctx, cudaEventRecord(ctx->aux_fork, st));
-      CK(ctx, cudaStreamWaitEvent(ctx->aux, ctx->aux_fork, 0));
-      CK(ctx, launch_count_touched(w.fcell_off[1 - cur], H, ctx->bt.fblock_first_tile,
-                                   ctx->bt.n_feat_blocks, w.stats + K, w.status, ctx->aux));
+      d.fblock_first_tile = ctx->bt.fblock_first_tile;
+      d.n_feat_blocks = ctx->bt.n_feat_blocks;
+      d.feat_touched = w.stats + K;
     }
-    CK(ctx, launch_dedup_compact(a, d, nsm, st));
+    CK(ctx, launch_dedup(a, d, nsm, st));
     cur = 1 - cur;
   }
   mark(true);
@@ -459,9 +430,6 @@ static agnes_status enqueue_hyperbatch(agnes_ctx* ctx, const int32_t* fanouts, i
                           w.fcell_off[cur] + cells, w.feats_out, w.status, nsm, st));
   }
   mark(true);
-  // the last hop's col fix-up and the statistics ran beside its compaction
-  CK(ctx, cudaEventRecord(ctx->aux_join, ctx->aux));
-  CK(ctx, cudaStreamWaitEvent(st, ctx->aux_join, 0));
   CK(ctx, cudaMemcpyAsync(w.h_back, w.back, w.back_bytes, cudaMemcpyDeviceToHost, st));
   if (ctx->topo.cache)
     CK(ctx, cudaMemcpyAsync(ctx->topo.h_cached, ctx->topo.d_cached, sizeof(unsigned long long),
@@ -495,9 +463,8 @@ static bool stream_capturing(cudaStream_t st) {
 }
 
 // Turns every kernel-to-kernel link of the captured chain (an edge whose
-// source has no other successor and whose destination no other predecessor;
-// fork and join edges of the side stream stay as they are) into a
-// programmatic one from the programmatic port: the kernels trigger nothing
+// source has no other successor and whose destination no other predecessor)
+// into a programmatic one from the programmatic port: the kernels trigger nothing
 // early, so the next kernel is launched as soon as every block of its
 // predecessor has exited, and its blocks wait at their first statement
 // (grid_dep_wait) for the predecessor's writes to become visible; the launch

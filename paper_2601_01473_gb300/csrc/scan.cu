@@ -1,10 +1,9 @@
-// scan.cu -- segmented exclusive scans (reduce / scan-of-partials / downsweep).
+// scan.cu -- exclusive scans.
 //
-// Used for every prefix sum on the path: the per-minibatch indptr of a hop,
-// the cell offsets of the bucket matrix, the per-minibatch offsets of the new
-// nodes of each (tile, minibatch) cell, and the tile compaction at load time.
-// Three launches per scan and no inter-block waiting, so no kernel ever spins
-// on another block's progress.
+// The cell offsets of the bucket matrix (single pass), the per-minibatch
+// offsets of the new nodes of each (tile, minibatch) cell (column scans), and
+// the segmented scan of the tile compaction at load time and of the staged
+// rows (two launches, no waiting between blocks).
 #include <mutex>
 #include <unordered_map>
 
@@ -193,63 +192,6 @@ scan_down_kernel(const InT* __restrict__ in, int64_t in_stride, OutT* __restrict
   }
 }
 
-// ---- column scan of a row-major [rows x cols] matrix ----------------------------
-constexpr int kColRows = 16;  // rows per chunk
-
-__global__ void __launch_bounds__(128)
-col_reduce_kernel(const int32_t* __restrict__ in, int64_t rows, int32_t cols,
-                  int64_t* __restrict__ partial, const int32_t* status) {
-  grid_dep_wait();
-  if (status && failed(status)) return;
-  const int32_t c = blockIdx.y * 128 + threadIdx.x;
-  if (c >= cols) return;
-  const int64_t r0 = (int64_t)blockIdx.x * kColRows;
-  const int64_t r1 = min(rows, r0 + kColRows);
-  int32_t v[kColRows];
-#pragma unroll
-  for (int k = 0; k < kColRows; ++k) v[k] = r0 + k < r1 ? in[(r0 + k) * cols + c] : 0;
-  int64_t sum = 0;
-#pragma unroll
-  for (int k = 0; k < kColRows; ++k) sum += v[k];
-  partial[(int64_t)blockIdx.x * cols + c] = sum;
-}
-
-// One CTA per column: exclusive scan of its chunk partials (strided by cols).
-__global__ void __launch_bounds__(kThreads)
-col_partials_kernel(int64_t* __restrict__ partial, int64_t chunks, int32_t cols,
-                    const int32_t* __restrict__ add_in, int32_t* __restrict__ total_out,
-                    int32_t* __restrict__ total_out2, const int32_t* status) {
-  grid_dep_wait();
-  if (status && failed(status)) return;
-  const int32_t c = blockIdx.x;
-  const int64_t carry = cta_scan_inplace(partial + c, chunks, cols, false);
-  if (threadIdx.x == 0) {
-    const int32_t total = (int32_t)carry + (add_in ? add_in[c] : 0);
-    if (total_out) total_out[c] = total;
-    if (total_out2) total_out2[c] = total;
-  }
-}
-
-__global__ void __launch_bounds__(128)
-col_down_kernel(const int32_t* __restrict__ in, int32_t* __restrict__ out, int64_t rows,
-                int32_t cols, const int64_t* __restrict__ partial, const int32_t* status) {
-  grid_dep_wait();
-  if (status && failed(status)) return;
-  const int32_t c = blockIdx.y * 128 + threadIdx.x;
-  if (c >= cols) return;
-  const int64_t r0 = (int64_t)blockIdx.x * kColRows;
-  const int64_t r1 = min(rows, r0 + kColRows);
-  int64_t run = partial[(int64_t)blockIdx.x * cols + c];
-  int32_t v[kColRows];
-#pragma unroll
-  for (int k = 0; k < kColRows; ++k) v[k] = r0 + k < r1 ? in[(r0 + k) * cols + c] : 0;
-#pragma unroll
-  for (int k = 0; k < kColRows; ++k) {
-    if (r0 + k < r1) out[(r0 + k) * cols + c] = (int32_t)run;
-    run += v[k];
-  }
-}
-
 // ---- single-pass flat scan (decoupled look-back) ----------------------------------
 //
 // Merrill & Garland's single-pass prefix scan (2016): every CTA takes the next
@@ -275,17 +217,16 @@ __device__ __forceinline__ unsigned long long flag_load(const unsigned long long
   return *(const volatile unsigned long long*)p;
 }
 
-__global__ void __launch_bounds__(kThreads)
-flat_scan_kernel(int32_t* __restrict__ in, int32_t* __restrict__ out, int64_t n, bool write_end,
-                 int32_t* total_out, bool clear, unsigned long long* scratch, int32_t* status) {
-  grid_dep_wait();
+__device__ __forceinline__ void flat_scan_cta(int32_t* __restrict__ in, int32_t* __restrict__ out,
+                                              int64_t n, int64_t ntiles, bool write_end,
+                                              int32_t* total_out, bool clear,
+                                              unsigned long long* scratch, int32_t* status) {
   // no early return on a failed status: every CTA takes its tile and counts
   // itself finished, so the scratch is left zero for the next scan
   __shared__ int64_t s_tile, s_excl;
   __shared__ int64_t warp_tot[kThreads / 32];
   __shared__ bool s_last;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int64_t ntiles = (int64_t)gridDim.x;
   unsigned long long* flags = scratch + 2;
   if (tid == 0) {
     const int64_t t = (int64_t)atomicAdd(scratch, 1ull);
@@ -400,23 +341,209 @@ flat_scan_kernel(int32_t* __restrict__ in, int32_t* __restrict__ out, int64_t n,
   }
 }
 
-}  // namespace
-
-int64_t col_scan_scratch_elems(int64_t rows, int32_t cols) {
-  return kTicketElems + ((rows + kColRows - 1) / kColRows) * (int64_t)cols;
+__global__ void __launch_bounds__(kThreads)
+flat_scan_kernel(int32_t* __restrict__ in, int32_t* __restrict__ out, int64_t n, bool write_end,
+                 int32_t* total_out, bool clear, unsigned long long* scratch, int32_t* status) {
+  grid_dep_wait();
+  flat_scan_cta(in, out, n, gridDim.x, write_end, total_out, clear, scratch, status);
 }
 
-cudaError_t col_scan(const int32_t* in, int32_t* out, int64_t rows, int32_t cols,
-                     const int32_t* add_in, int32_t* total_out, int32_t* total_out2,
-                     int64_t* scratch, const int32_t* status, cudaStream_t st) {
-  if (rows <= 0 || cols <= 0) return cudaSuccess;
-  const int64_t chunks = (rows + kColRows - 1) / kColRows;
-  const dim3 grid((unsigned)chunks, (unsigned)((cols + 127) / 128));
-  int64_t* partial = scratch + kTicketElems;  // leave the seg_scan tickets untouched
-  col_reduce_kernel<<<grid, 128, 0, st>>>(in, rows, cols, partial, status);
-  col_partials_kernel<<<cols, kThreads, 0, st>>>(partial, chunks, cols, add_in, total_out, total_out2,
-                                                  status);
-  col_down_kernel<<<grid, 128, 0, st>>>(in, out, rows, cols, partial, status);
+// ---- the scans between a hop's cells and its compaction -----------------------------
+//
+// The flat scan of the next frontier's cell counts, and exclusive scans down
+// the columns of row-major [rows x cols] count matrices (one or two), in two
+// launches: the first holds the flat scan's CTAs and the CTAs that sum the
+// matrices' chunks of rows; in the second, each CTA adds up the sums of the
+// chunks before its own and writes its chunk's prefixes.  Both are latency-
+// bound (a few MB at most), so what counts is launches and dependent loads:
+// the column scan used to be three launches on a side stream beside the flat
+// scan, with an event to fork and one to join (16 x 1024 targets at [15, 10, 5]
+// on 10M nodes: 638 -> 623 us a hyperbatch, the col fix-up moved into the
+// compaction's launch; 128 x 1024 with three layers 5.27 -> 5.26 ms).
+//
+// A CTA covers `width` columns (the power of two from cols up, at most
+// kColWidth) and kThreads / width groups of `depth` rows; depth grows with
+// rows so that a column has at most kColChunks chunks, whose sums the second
+// launch reads again in every CTA.
+constexpr int kColWidth = 128;
+constexpr int kColBatch = 16;  // rows whose loads are in flight together
+constexpr int kColChunks = 256;
+
+struct ColShape {
+  int64_t rows;
+  int32_t cols, width, depth, chunks, col_blocks;
+};
+
+ColShape col_shape(int64_t rows, int32_t cols) {
+  ColShape s;
+  s.rows = rows;
+  s.cols = cols;
+  s.width = 1;
+  while (s.width < cols && s.width < kColWidth) s.width *= 2;
+  const int64_t groups = kThreads / s.width;
+  int64_t depth = (rows + groups * kColChunks - 1) / (groups * kColChunks);
+  depth = (depth + kColBatch - 1) / kColBatch * kColBatch;
+  s.depth = (int32_t)depth;
+  s.chunks = (int32_t)((rows + groups * depth - 1) / (groups * depth));
+  s.col_blocks = (cols + s.width - 1) / s.width;
+  return s;
+}
+
+// Sum of rows [r0, r1) of column c.
+__device__ __forceinline__ int32_t col_sum(const int32_t* __restrict__ in, int32_t cols, int32_t c,
+                                           int64_t r0, int64_t r1) {
+  int32_t sum = 0;
+  for (int64_t r = r0; r < r1; r += kColBatch) {
+    int32_t v[kColBatch];
+#pragma unroll
+    for (int k = 0; k < kColBatch; ++k) v[k] = r + k < r1 ? in[(r + k) * cols + c] : 0;
+#pragma unroll
+    for (int k = 0; k < kColBatch; ++k) sum += v[k];
+  }
+  return sum;
+}
+
+// One CTA's block b of a matrix: its chunk, and the thread's group and column
+// (c >= cols: none).
+struct ColPlace {
+  int32_t chunk, group, groups, c;
+  int64_t r0, r1;
+};
+
+__device__ __forceinline__ ColPlace col_place(const ColShape& s, int32_t b) {
+  ColPlace p;
+  p.groups = kThreads / s.width;
+  p.group = (int32_t)threadIdx.x / s.width;
+  p.chunk = b / s.col_blocks;
+  p.c = (b - p.chunk * s.col_blocks) * s.width + (int32_t)threadIdx.x % s.width;
+  p.r0 = min(s.rows, ((int64_t)p.chunk * p.groups + p.group) * s.depth);
+  p.r1 = min(s.rows, p.r0 + s.depth);
+  return p;
+}
+
+// Exclusive prefix of v over the groups of the thread's column, and the
+// column's total; s_v is kThreads words.
+__device__ __forceinline__ int32_t group_excl(int32_t* s_v, int32_t v, int32_t width,
+                                              int32_t group, int32_t groups, int32_t* total) {
+  const int tid = threadIdx.x;
+  __syncthreads();
+  s_v[tid] = v;
+  __syncthreads();
+  for (int d = 1; d < groups; d <<= 1) {  // inclusive scan over the groups
+    const int32_t x = group >= d ? s_v[tid - d * width] : 0;
+    __syncthreads();
+    s_v[tid] += x;
+    __syncthreads();
+  }
+  *total = s_v[(groups - 1) * width + tid % width];
+  return s_v[tid] - v;
+}
+
+struct ColScan {
+  const int32_t* in;
+  int32_t* out;
+  const int32_t* add_in;  // cols, or null
+  int32_t* total[2];      // cols, or null
+  int32_t* partial;       // chunks x cols
+};
+
+struct CellScansArgs {
+  int32_t* flat_in;
+  int32_t* flat_out;
+  int64_t flat_n;
+  int32_t flat_tiles;
+  unsigned long long* flat_scratch;
+  int32_t* status;
+  ColShape shape;
+  int32_t col_ctas;  // CTAs per matrix
+  ColScan m[2];
+};
+
+__global__ void __launch_bounds__(kThreads) cell_scans_kernel(CellScansArgs a) {
+  grid_dep_wait();
+  if ((int32_t)blockIdx.x < a.flat_tiles) {
+    flat_scan_cta(a.flat_in, a.flat_out, a.flat_n, a.flat_tiles, true, nullptr, false,
+                  a.flat_scratch, a.status);
+    return;
+  }
+  if (cta_failed(a.status)) return;
+  __shared__ int32_t s_v[kThreads];
+  int32_t b = (int32_t)blockIdx.x - a.flat_tiles;
+  const int32_t which = b / a.col_ctas;
+  b -= which * a.col_ctas;
+  const ColScan& m = a.m[which];
+  const ColPlace p = col_place(a.shape, b);
+  const bool has = p.c < a.shape.cols;
+  const int32_t sum = has ? col_sum(m.in, a.shape.cols, p.c, p.r0, p.r1) : 0;
+  int32_t total;
+  group_excl(s_v, sum, a.shape.width, p.group, p.groups, &total);
+  if (has && p.group == 0) m.partial[(int64_t)p.chunk * a.shape.cols + p.c] = total;
+}
+
+__global__ void __launch_bounds__(kThreads) cell_scans_down_kernel(CellScansArgs a) {
+  grid_dep_wait();
+  if (failed(a.status)) return;
+  __shared__ int32_t s_v[kThreads];
+  int32_t b = (int32_t)blockIdx.x;
+  const int32_t which = b / a.col_ctas;
+  b -= which * a.col_ctas;
+  const ColScan& m = a.m[which];
+  const ColPlace p = col_place(a.shape, b);
+  const int32_t cols = a.shape.cols;
+  const bool has = p.c < cols;
+  // the chunks before this one, a contiguous share per group
+  const int32_t share = (p.chunk + p.groups - 1) / p.groups;
+  const int32_t s0 = min(p.chunk, p.group * share);
+  const int32_t before =
+      has ? col_sum(m.partial, cols, p.c, s0, min(p.chunk, s0 + share)) : 0;
+  const int32_t sum = has ? col_sum(m.in, cols, p.c, p.r0, p.r1) : 0;
+  int32_t base, total;
+  group_excl(s_v, before, a.shape.width, p.group, p.groups, &base);
+  int32_t run = base + group_excl(s_v, sum, a.shape.width, p.group, p.groups, &total);
+  if (!has) return;
+  if (p.chunk == a.shape.chunks - 1 && p.group == 0) {
+    const int32_t t = base + total + (m.add_in ? m.add_in[p.c] : 0);
+    if (m.total[0]) m.total[0][p.c] = t;
+    if (m.total[1]) m.total[1][p.c] = t;
+  }
+  for (int64_t r = p.r0; r < p.r1; r += kColBatch) {
+    int32_t v[kColBatch];
+#pragma unroll
+    for (int k = 0; k < kColBatch; ++k) v[k] = r + k < p.r1 ? m.in[(r + k) * cols + p.c] : 0;
+#pragma unroll
+    for (int k = 0; k < kColBatch; ++k) {
+      if (r + k < p.r1) m.out[(r + k) * cols + p.c] = run;
+      run += v[k];
+    }
+  }
+}
+
+}  // namespace
+
+int64_t cell_scans_scratch_elems(int64_t rows, int32_t cols) {
+  return 2 * (int64_t)col_shape(rows, cols).chunks * cols;
+}
+
+cudaError_t cell_scans(int64_t rows, int32_t cols, int32_t* counts, int32_t* offsets,
+                       uint64_t* flat_scratch, const ColumnScan* scans, int32_t nscans,
+                       int32_t* scratch, int32_t* status, cudaStream_t st) {
+  CellScansArgs a;
+  a.flat_in = counts;
+  a.flat_out = offsets;
+  a.flat_n = rows * cols;
+  a.flat_tiles = (int32_t)((a.flat_n + kFlatTile - 1) / kFlatTile);
+  a.flat_scratch = reinterpret_cast<unsigned long long*>(flat_scratch);
+  a.status = status;
+  a.shape = col_shape(rows, cols);
+  a.col_ctas = a.shape.chunks * a.shape.col_blocks;
+  for (int32_t i = 0; i < 2; ++i) {
+    const ColumnScan& c = scans[i < nscans ? i : 0];
+    a.m[i] = ColScan{c.in, c.out, c.add_in, {c.total[0], c.total[1]},
+                     scratch + (int64_t)i * a.shape.chunks * cols};
+  }
+  const unsigned cta = (unsigned)(a.col_ctas * nscans);
+  cell_scans_kernel<<<(unsigned)a.flat_tiles + cta, kThreads, 0, st>>>(a);
+  cell_scans_down_kernel<<<cta, kThreads, 0, st>>>(a);
   return cudaGetLastError();
 }
 
