@@ -63,28 +63,6 @@ __device__ __forceinline__ uint4 philox4x32_10(uint4 c, uint2 k) {
 
 __device__ __forceinline__ int lane_id() { return threadIdx.x & 31; }
 
-// counters[idx] += 1 for every active lane, one atomic per distinct idx.
-__device__ __forceinline__ void warp_agg_inc(int32_t* counters, int64_t idx, bool active) {
-  const unsigned mask = __ballot_sync(0xffffffffu, active);
-  if (!active) return;
-  const unsigned peers = __match_any_sync(mask, (unsigned long long)idx);
-  const int leader = __ffs(peers) - 1;
-  if (lane_id() == leader) atomicAdd(counters + idx, __popc(peers));
-}
-
-// Takes one slot per active lane from counters[idx] by counting it down;
-// returns a slot in [0, count) distinct among all takers of idx.  After every
-// counted item has taken its slot the counter is back at zero.
-__device__ __forceinline__ int32_t warp_agg_take(int32_t* counters, int64_t idx, unsigned mask) {
-  const unsigned peers = __match_any_sync(mask, (unsigned long long)idx);
-  const int leader = __ffs(peers) - 1;
-  const int lane = lane_id();
-  int32_t old = 0;
-  if (lane == leader) old = atomicSub(counters + idx, __popc(peers));
-  old = __shfl_sync(peers, old, leader);
-  return old - 1 - __popc(peers & ((1u << lane) - 1u));
-}
-
 // Adds one per active lane to counters[idx] (one atomic per distinct idx) and
 // returns this lane's rank among all additions to idx: the counter's value
 // before it plus its rank among the warp's peers.

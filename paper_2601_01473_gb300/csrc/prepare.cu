@@ -39,8 +39,6 @@ struct BeginArgs {
   uint64_t seed, first_gid;
   int32_t* back;
   int64_t back_words;
-  int32_t* fcnt;  // targets' cell counters, cleared
-  int64_t cells;
 };
 
 __global__ void __launch_bounds__(256) begin_kernel(BeginArgs a) {
@@ -53,7 +51,6 @@ __global__ void __launch_bounds__(256) begin_kernel(BeginArgs a) {
   }
   // word 0 is the status; words 1 .. H are |dst_0| of every minibatch
   for (int64_t i = i0; i < a.back_words; i += stride) a.back[i] = i >= 1 && i <= a.H ? a.B : 0;
-  for (int64_t i = i0; i < a.cells; i += stride) a.fcnt[i] = 0;
   if (!a.targets) return;
   const int64_t n = (int64_t)a.H * a.B;
   for (int64_t i = i0; i < n; i += stride) {
@@ -221,6 +218,7 @@ static agnes_status ensure_workspace(agnes_ctx* ctx, int32_t H, int32_t B, const
   }
   if (cudaMemset(w.scan_scratch, 0, sizeof(int64_t) * scratch) != cudaSuccess ||
       cudaMemset(w.indptr_scratch, 0, sizeof(uint64_t) * indptr_elems) != cudaSuccess ||
+      cudaMemset(w.fcnt, 0, sizeof(int32_t) * cells) != cudaSuccess ||
       cudaMemset(w.scnt, 0, sizeof(int32_t) * cells) != cudaSuccess ||
       cudaMemset(w.flat_scratch, 0, sizeof(uint64_t) * w.flat_elems) != cudaSuccess ||
       // the hyperbatch may run on a stream that does not wait for this one
@@ -692,9 +690,10 @@ agnes_status agnes_prepare_hyperbatch(agnes_ctx* ctx, const int32_t* targets, in
   b.first_gid = first_minibatch_id;
   b.back = (int32_t*)w.back;
   b.back_words = (int64_t)(w.back_bytes / sizeof(int32_t));
-  b.fcnt = w.fcnt;
-  b.cells = ctx->bt.T * H;
-  begin_kernel<<<resident_grid((const void*)begin_kernel, 256, ctx->num_sms), 256, 0, st>>>(b);
+  const int64_t most = b.back_words > (int64_t)H * B ? b.back_words : (int64_t)H * B;
+  const int64_t ctas = (most + 255) / 256;
+  const int resident_ctas = resident_grid((const void*)begin_kernel, 256, ctx->num_sms);
+  begin_kernel<<<(unsigned)(ctas < resident_ctas ? ctas : resident_ctas), 256, 0, st>>>(b);
   CK(ctx, cudaGetLastError());
   int n_marks = 0;
   if (resident && ctx->lg.mode != AGNES_LAUNCH_DIRECT && !capturing)

@@ -29,9 +29,12 @@ constexpr int kWarps = kThreads / 32;
 
 // ---- bucketing of the targets ------------------------------------------------
 
+// Counts the targets per (tile, minibatch) cell; rank[i] = the target's place
+// among its cell's (the order of arrival).
 __global__ void __launch_bounds__(kThreads)
 targets_count_kernel(const int32_t* __restrict__ nodes, int64_t capK, int32_t H, int32_t B,
-                     int32_t N, TileMap tm, int32_t* __restrict__ fcnt, int32_t* status) {
+                     int32_t N, TileMap tm, int32_t* __restrict__ fcnt,
+                     int32_t* __restrict__ rank, int32_t* status) {
   grid_dep_wait();
   const int64_t total = (int64_t)H * B;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
@@ -50,120 +53,65 @@ targets_count_kernel(const int32_t* __restrict__ nodes, int64_t capK, int32_t H,
         cell = (int64_t)tile_of(tm, v) * H + j;
       }
     }
-    warp_agg_inc(fcnt, cell, active);
+    const unsigned mask = __ballot_sync(0xffffffffu, active);
+    if (active) rank[i] = warp_agg_add(fcnt, cell, mask);
   }
 }
 
+// Every target to its cell's slots, in order of arrival.
 __global__ void __launch_bounds__(kThreads)
 targets_scatter_kernel(const int32_t* __restrict__ nodes, int64_t capK, int32_t H, int32_t B,
-                       int32_t N, TileMap tm, int32_t* __restrict__ fcnt,
-                       const int32_t* __restrict__ fcell_off, int32_t* __restrict__ tmp_id,
+                       TileMap tm, const int32_t* __restrict__ fcell_off,
+                       const int32_t* __restrict__ rank, int32_t* __restrict__ tmp_id,
                        int32_t* __restrict__ tmp_pos, const int32_t* status) {
   grid_dep_wait();
   if (failed(status)) return;
   const int64_t total = (int64_t)H * B;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t i0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) & ~31ll; i0 < total;
-       i0 += stride) {
-    const int64_t i = i0 + lane_id();
-    bool active = i < total;
-    int32_t v = 0, j = 0;
-    int64_t cell = 0;
-    if (active) {
-      j = (int32_t)(i / B);
-      v = nodes[j * capK + (i - (int64_t)j * B)];
-      active = v >= 0 && v < N;
-      if (active) cell = (int64_t)tile_of(tm, v) * H + j;
-    }
-    const unsigned mask = __ballot_sync(0xffffffffu, active);
-    if (active) {
-      const int32_t slot = fcell_off[cell] + warp_agg_take(fcnt, cell, mask);
-      tmp_id[slot] = v;
-      tmp_pos[slot] = (int32_t)(j * capK + (i - (int64_t)j * B));
-    }
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += stride) {
+    const int32_t j = (int32_t)(i / B);
+    const int64_t pos = j * capK + (i - (int64_t)j * B);
+    const int32_t v = nodes[pos];
+    const int32_t slot = fcell_off[(int64_t)tile_of(tm, v) * H + j] + rank[i];
+    tmp_id[slot] = v;
+    tmp_pos[slot] = (int32_t)pos;
   }
 }
 
 // Orders each cell's targets by id and flags a target repeated within a
-// minibatch.  A warp scans 32 consecutive cells and skips empty ones; a cell
-// of at most 32 targets is ranked in registers (each lane counts the smaller
-// ids), a bigger one by popcount ranks in a bitmap over its tile.
+// minibatch: a thread per slot counts the smaller ids of its cell.  Neighbouring
+// slots share a cell, so its ids are read from L1, and the work is spread over
+// the whole grid however few cells hold the targets.  A cell with more entries
+// than a tile has ids repeats one, and is not walked.  (A warp per 32 cells,
+// sorting them one after another, took 5 us of a hyperbatch of 16 x 1024 targets
+// on 10M nodes, 623 -> 619 us.)
 __global__ void __launch_bounds__(kThreads)
-targets_sort_kernel(const int32_t* __restrict__ fcell_off, int64_t ncells, int32_t H, TileMap tm,
-                    const int32_t* __restrict__ tmp_id, const int32_t* __restrict__ tmp_pos,
-                    int32_t* __restrict__ fb_id, int32_t* __restrict__ fb_pos, int32_t* status) {
+targets_place_kernel(const int32_t* __restrict__ fcell_off, int64_t total, int64_t capK, int32_t H,
+                     TileMap tm, const int32_t* __restrict__ tmp_id,
+                     const int32_t* __restrict__ tmp_pos, int32_t* __restrict__ fb_id,
+                     int32_t* __restrict__ fb_pos, int32_t* status) {
   grid_dep_wait();
   if (failed(status)) return;
-  __shared__ uint32_t bits_s[kWarps][kTileWords];
-  __shared__ int32_t pref_s[kWarps][kTileWords];
-  const int warp = threadIdx.x >> 5, lane = lane_id();
-  uint32_t* bits = bits_s[warp];
-  int32_t* pref = pref_s[warp];
-  const int64_t nchunks = (ncells + 31) / 32;
-  const int64_t nwarps = (int64_t)gridDim.x * kWarps;
-  for (int64_t ch = blockIdx.x * (int64_t)kWarps + warp; ch < nchunks; ch += nwarps) {
-    const int64_t my_cell = ch * 32 + lane;
-    int32_t my_o = 0, my_n = 0;
-    if (my_cell < ncells) {
-      my_o = fcell_off[my_cell];
-      my_n = fcell_off[my_cell + 1] - my_o;
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < total; s += stride) {
+    const int32_t v = tmp_id[s];
+    const int32_t pos = tmp_pos[s];
+    const int64_t cell = (int64_t)tile_of(tm, v) * H + (uint32_t)pos / (uint32_t)capK;
+    const int32_t o = fcell_off[cell], e = fcell_off[cell + 1];
+    if (e - o > kTileSpan) {
+      atomicOr(status, kErrTargetDup);
+      continue;
     }
-    unsigned todo = __ballot_sync(0xffffffffu, my_n > 0);
-    while (todo) {
-      const int k = __ffs(todo) - 1;
-      todo &= todo - 1u;
-      const int32_t o = __shfl_sync(0xffffffffu, my_o, k);
-      const int32_t n = __shfl_sync(0xffffffffu, my_n, k);
-      if (n <= 32) {
-        const bool act = lane < n;
-        const int32_t v = act ? tmp_id[o + lane] : 0x7fffffff;
-        const int32_t p = act ? tmp_pos[o + lane] : 0;
-        const unsigned amask = n >= 32 ? 0xffffffffu : ((1u << n) - 1u);
-        const unsigned peers = __match_any_sync(0xffffffffu, v);  // every lane takes part
-        if (act && __popc(peers & amask) > 1) atomicOr(status, kErrTargetDup);
-        int32_t r = 0;
-        for (int q = 0; q < n; ++q) r += __shfl_sync(0xffffffffu, v, q) < v;
-        if (act) {
-          fb_id[o + r] = v;
-          fb_pos[o + r] = p;
-        }
-        continue;
-      }
-      const int32_t t = (int32_t)((ch * 32 + k) / H);
-      const int32_t base = tm.tile_first[t];
-      const int32_t words = (tm.tile_first[t + 1] - base + 31) >> 5;
-      for (int w = lane; w < words; w += 32) bits[w] = 0;
-      __syncwarp();
-      for (int32_t i = lane; i < n; i += 32) {
-        const int32_t lu = tmp_id[o + i] - base;
-        const uint32_t bit = 1u << (lu & 31);
-        if (atomicOr(&bits[lu >> 5], bit) & bit) atomicOr(status, kErrTargetDup);
-      }
-      __syncwarp();
-      int32_t c[4], sum = 0;
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const int w = lane * 4 + q;
-        c[q] = w < words ? __popc(bits[w]) : 0;
-        sum += c[q];
-      }
-      int32_t run = warp_incl_scan(sum) - sum;
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        pref[lane * 4 + q] = run;
-        run += c[q];
-      }
-      __syncwarp();
-      for (int32_t i = lane; i < n; i += 32) {
-        const int32_t v = tmp_id[o + i];
-        const int32_t lu = v - base;
-        const int32_t w = lu >> 5;
-        const int32_t r = pref[w] + __popc(bits[w] & ((1u << (lu & 31)) - 1u));
-        fb_id[o + r] = v;
-        fb_pos[o + r] = tmp_pos[o + i];
-      }
-      __syncwarp();
+    int32_t smaller = 0, same = 0;
+#pragma unroll 4
+    for (int32_t q = o; q < e; ++q) {
+      const int32_t u = tmp_id[q];
+      smaller += u < v;
+      same += u == v;
     }
+    if (same > 1) atomicOr(status, kErrTargetDup);
+    fb_id[o + smaller] = v;
+    fb_pos[o + smaller] = pos;
   }
 }
 
@@ -660,18 +608,23 @@ cudaError_t launch_bucket_targets(int32_t* nodes, int64_t capK, int32_t H, int32
                                   cudaStream_t st) {
   const TileMap tm{tile_first, chunk_tile, T};
   const int64_t ncells = (int64_t)T * H;
-  const int grid = resident_grid((const void*)targets_count_kernel, kThreads, num_sms);
-  targets_count_kernel<<<grid, kThreads, 0, st>>>(nodes, capK, H, B, N, tm, fcnt, status);
-  // the scatter counts fcnt back down to zero
+  const int64_t total = (int64_t)H * B;
+  // a thread per target, on at most the resident CTAs
+  auto grid = [&](const void* kernel) {
+    const int64_t ctas = (total + kThreads - 1) / kThreads;
+    const int resident = resident_grid(kernel, kThreads, num_sms);
+    return (unsigned)(ctas < resident ? ctas : resident);
+  };
+  int32_t* rank = fb_id;  // free until the bucket is written
+  targets_count_kernel<<<grid((const void*)targets_count_kernel), kThreads, 0, st>>>(
+      nodes, capK, H, B, N, tm, fcnt, rank, status);
   cudaError_t e =
-      flat_scan(fcnt, fcell_off, ncells, true, nullptr, false, flat_scratch, status, st);
+      flat_scan(fcnt, fcell_off, ncells, true, nullptr, true, flat_scratch, status, st);
   if (e != cudaSuccess) return e;
-  targets_scatter_kernel<<<resident_grid((const void*)targets_scatter_kernel, kThreads, num_sms),
-                           kThreads, 0, st>>>(nodes, capK, H, B, N, tm, fcnt, fcell_off,
-                                                    tmp_id, tmp_pos, status);
-  targets_sort_kernel<<<resident_grid((const void*)targets_sort_kernel, kThreads, num_sms),
-                        kThreads, 0, st>>>(fcell_off, ncells, H, tm, tmp_id, tmp_pos,
-                                                 fb_id, fb_pos, status);
+  targets_scatter_kernel<<<grid((const void*)targets_scatter_kernel), kThreads, 0, st>>>(
+      nodes, capK, H, B, tm, fcell_off, rank, tmp_id, tmp_pos, status);
+  targets_place_kernel<<<grid((const void*)targets_place_kernel), kThreads, 0, st>>>(
+      fcell_off, total, capK, H, tm, tmp_id, tmp_pos, fb_id, fb_pos, status);
   return cudaGetLastError();
 }
 
