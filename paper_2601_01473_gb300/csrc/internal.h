@@ -231,10 +231,14 @@ cudaError_t launch_dedup(const HopArgs& a, const DedupBufs& d, int num_sms, cuda
 cudaError_t launch_dedup_cells(const HopArgs& a, const DedupBufs& d, int num_sms,
                                cudaStream_t st);
 
+// ---- gather_hbm.cu ---------------------------------------------------------
+// Gathers the rows of a bucket of *total entries (row id at feats + id *
+// row_bytes, feats_bytes in all) to out + pos * row_bytes, byte for byte.
+cudaError_t launch_gather(const void* feats, int64_t feats_bytes, int64_t row_bytes,
+                          const int32_t* fb_id, const int32_t* fb_pos, const int32_t* total,
+                          void* out, const int32_t* status, int num_sms, cudaStream_t st);
+
 // ---- gather.cu -------------------------------------------------------------
-cudaError_t launch_gather(const void* feats, int64_t row_bytes, const int32_t* fb_id,
-                          const int32_t* fb_pos, const int32_t* total, void* out,
-                          const int32_t* status, int num_sms, cudaStream_t st);
 
 // Gathers the rows of a batch of feature blocks held in HBM copies: the
 // batch's blocks are touched[0 .. nb) (ascending), block touched[p] starts at

@@ -28,8 +28,8 @@ namespace {
 // of the sequence costs a small hyperbatch is its place in the chain (about 3 us
 // each): with this, one copy of the readback block instead of five, counters
 // that their scan clears and block statistics taken from the bucket's offsets,
-// a request of 16 targets went from 168 to 150 us and 1 x 1024 targets at
-// [15, 10, 5] from 289 to 272 us.
+// 1 x 1024 targets at [15, 10, 5] went from 289 to 272 us and 16 x 1024 from 671
+// to 653.
 struct BeginArgs {
   const int32_t* targets;  // H x B
   int32_t* nodes;          // H x capK
@@ -424,7 +424,7 @@ static agnes_status enqueue_hyperbatch(agnes_ctx* ctx, const int32_t* fanouts, i
     rc = gather_streamed(ctx, cur, st);
     if (rc != AGNES_OK) return rc;
   } else {
-    CK(ctx, launch_gather(ctx->features, ctx->row_bytes, w.fb_id[cur], w.fb_pos[cur],
+    CK(ctx, launch_gather(ctx->features, ctx->N * ctx->row_bytes, ctx->row_bytes, w.fb_id[cur], w.fb_pos[cur],
                           w.fcell_off[cur] + cells, w.feats_out, w.status, nsm, st));
   }
   mark(true);
