@@ -5,23 +5,34 @@
 //
 //   out_i = ReLU(W_self x_i + W_neigh mean_{(i,u) in hop} x_u + b).
 //
-// Two kernels.  The dst rows of minibatch j form ceil(|dst_h| / 128) tiles of
-// 128 rows (the MMA's M).
-//  1. sage_agg_kernel (HBM-bound gather): for every row, the mean of its
-//     neighbours' rows in fp32, written with the row itself as the update's
-//     input A = [x_i | mean_i] in fp16 -- each tile as the exact image of a
-//     tcgen05 K-major, no-swizzle shared-memory operand (8-row x 16-byte core
-//     matrices, the 16 row groups of one 16-byte K slice after one another).
-//     No shared memory and no barriers, so it runs at full occupancy.
-//  2. sage_gemm_kernel (persistent, warp-specialised, one CTA per SM): W is
-//     loaded into shared memory once; a producer lane moves A tiles into a
-//     ring of shared-memory stages with cp.async.bulk (mbarrier transaction
-//     counts); an MMA lane issues each tile's tcgen05.mma chain (M = 128,
-//     N = d_out, K = 16 each) into one of two TMEM accumulators; four
-//     epilogue warps read the accumulator back with tcgen05.ld, add the bias,
-//     apply ReLU and store -- overlapped with the next tile's copy and MMA.
-// Every mbarrier wait is bounded; on timeout the kernel records an error,
-// frees its tensor memory and returns.
+// One persistent, warp-specialised kernel, one CTA per SM.  The dst rows of
+// minibatch j form ceil(|dst_h| / R) tiles of R rows, R = 128 (the MMA's M) or
+// less where that gives every SM a tile.  Per tile of a CTA:
+//   index warps     stage the tile's indptr and neighbour positions (one
+//                   contiguous run of col) in a ring of shared-memory slots, so
+//                   that the chain indptr -> col -> row costs the producers one
+//                   trip to memory per round of neighbours, not three;
+//   producer warps  form the update's input A = [x_i | mean_i]: an item (row,
+//                   8-feature chunk) per thread, its neighbours' chunks summed
+//                   in fp32 with several loads in flight, rounded to fp16 into
+//                   a stage of the shared-memory ring laid out as a tcgen05
+//                   K-major operand;
+//   the MMA warp    issues the tile's tcgen05.mma chain (M = 128, N = d_out,
+//                   K = 16 each) into one of two TMEM accumulators;
+//   epilogue warps  read the accumulator back with tcgen05.ld, add the bias,
+//                   apply ReLU and store.  They load W into shared memory first.
+// All stages overlap.  Every mbarrier wait is bounded; on timeout the kernel
+// records an error, frees its tensor memory and returns.
+//
+// Bound by the neighbour rows' loads and the instructions that sum them (61% of
+// the issue slots, the tensor pipe nearly idle), so most warps are producers.
+// Measured against a gather kernel that wrote A to memory and a GEMM that read
+// it back: 24 x 8192 rows of up to 15 neighbours, d_in = d_out = 128 in fp16,
+// 241 -> 160 us a call; 128 x 1024 targets at [15, 10, 5] on 40M nodes with
+// three layers 5.25 -> 4.35 ms.  On the way there: lanes over rows instead of
+// over a row's chunks kept the L1 data pipe 81% busy (a quarter warp's loads
+// touched 8 lines) and gained nothing; 16 producer warps instead of 24 cost 8%
+// of that model, 8 neighbours in flight instead of 5 cost 11% (registers).
 #include <cuda_fp16.h>
 
 #include "../../include/agnes.h"
@@ -32,16 +43,33 @@ namespace agnes {
 
 namespace {
 
-constexpr int kM = 128;              // dst rows per tile (the MMA's M)
+constexpr int kM = 128;              // dst rows per tile at most (the MMA's M)
 constexpr int kWaitIters = 1 << 24;  // mbarrier polls before giving up (~1 s)
-constexpr int kAggThreads = 256;
-constexpr int kGemmThreads = 256;    // warp 0 producer, warp 1 MMA, warps 4-7 epilogue
+// warps: 0-3 epilogue, 4 MMA, then the index warps, then the producers
+constexpr int kMmaWarp = 4;
+constexpr int kIdxWarps = 2;
+constexpr int kIdxWarp0 = kMmaWarp + 1;
+constexpr int kProdWarp0 = kIdxWarp0 + kIdxWarps;
+constexpr int kProdWarps = 24;
+constexpr int kSageThreads = 32 * (kProdWarp0 + kProdWarps);
 constexpr int kBarBytes = 128;       // mbarriers + TMEM address slot
-// Every GEMM CTA asks for at least this much shared memory, so no two CTAs
+// Index slots: row, validity and col facts of a tile, its indptr relative to
+// the tile's first edge, and up to idx_cap neighbour positions.
+constexpr int kIdxSlots = 3;
+constexpr int kIdxCapMax = 4096;
+constexpr int kMaxStages = 3;
+struct IdxHead {
+  int32_t i0, rows, j, staged;
+  const int32_t* col;  // the tile's first edge's neighbour position, in global memory
+  int64_t pad;
+  int32_t ptr[kM + 4];
+};
+static_assert(sizeof(IdxHead) % 16 == 0, "the slots stay 16-byte aligned");
+// Every CTA asks for at least this much shared memory, so no two CTAs
 // share an SM (and its 512 tensor-memory columns).
 constexpr size_t kSageMinSmem = 120 * 1024;
 
-constexpr int32_t kSageTimeout = 1;  // error word bits
+constexpr int32_t kSageTimeout = 1;  // error word
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
   return (uint32_t)__cvta_generic_to_shared(p);
@@ -53,12 +81,27 @@ __host__ __device__ __forceinline__ uint32_t kmajor_off(int r, int k, int rows) 
   return (uint32_t)((((k >> 3) * (rows >> 3)) + (r >> 3)) * 128 + (r & 7) * 16 + (k & 7) * 2);
 }
 
+// Byte offset of the 16-byte chunk c (elements 8 c .. 8 c + 7) of row r in a
+// K-major operand of kM rows with 128-byte swizzle: blocks of 64 elements
+// (kM rows of 128 bytes each), a row's eight chunks permuted by the row.
+__device__ __forceinline__ uint32_t swizzled_off(int r, int c) {
+  return (uint32_t)((c >> 3) * (kM * 128) + r * 128 + (((c & 7) ^ (r & 7)) << 4));
+}
+
 // tcgen05 shared-memory matrix descriptor, no swizzle: start address, the
 // byte distance between core matrices adjacent in K (leading) and in M/N
 // (stride), and the fixed version bits 46-48 = 0b001.
 __device__ __forceinline__ uint64_t smem_desc(uint32_t addr, uint32_t lbo, uint32_t sbo) {
   return (uint64_t)((addr & 0x3FFFF) >> 4) | ((uint64_t)((lbo & 0x3FFFF) >> 4) << 16) |
          ((uint64_t)((sbo & 0x3FFFF) >> 4) << 32) | (1ull << 46);
+}
+
+// The same for an operand with 128-byte swizzle (bits 61-63 = 2), its atoms of
+// 8 rows x 128 bytes 1024 bytes apart; a K step within an atom starts 32 bytes
+// on (the leading distance is not used).
+__device__ __forceinline__ uint64_t smem_desc_swizzled(uint32_t addr) {
+  return (uint64_t)((addr & 0x3FFFF) >> 4) | (1ull << 16) | ((uint64_t)(1024 >> 4) << 32) |
+         (1ull << 46) | (2ull << 61);
 }
 
 // Instruction descriptor of kind::f16: fp32 accumulator (bits 4-5 = 1), fp16
@@ -93,38 +136,23 @@ __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
 
-__device__ __forceinline__ void mbar_arrive_tx(uint32_t bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes)
-               : "memory");
-}
-
 // Waits for the phase with the given parity to complete; false after
-// kWaitIters polls.
+// kWaitIters tries.  try_wait suspends the thread for a while in hardware, so
+// waiting warps leave the shared-memory pipe to the others.
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
   for (int it = 0; it < kWaitIters; ++it) {
     uint32_t done;
     asm volatile(
         "{\n\t.reg .pred p;\n\t"
-        "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
         "selp.u32 %0, 1, 0, p;\n\t}"
         : "=r"(done)
         : "r"(bar), "r"(parity)
         : "memory");
     if (done) return true;
-    if (it >= 32) __nanosleep(64);
+    if (it >= 64) __nanosleep(64);
   }
   return false;
-}
-
-// Bulk copy of `bytes` (a multiple of 16, both addresses 16-byte aligned)
-// from global memory into shared memory, completing a transaction on bar.
-__device__ __forceinline__ void bulk_g2s(uint32_t dst, const void* src, uint32_t bytes,
-                                         uint32_t bar) {
-  asm volatile(
-      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::
-          "r"(dst),
-      "l"(src), "r"(bytes), "r"(bar)
-      : "memory");
 }
 
 // 8 consecutive features of a row as raw 16-byte vectors (one for fp16, two
@@ -143,20 +171,41 @@ __device__ __forceinline__ Chunk<T> load_chunk(const T* row, int c) {
   return ch;
 }
 
-__device__ __forceinline__ void add_chunk(const Chunk<__half>& ch, float* acc) {
+// Sums of the 8 features of a chunk as four pairs, added with the packed fp32
+// add (each half rounded as by a single one).
+struct Sum8 {
+  uint64_t p[4];
+};
+
+__device__ __forceinline__ uint64_t pair(float a, float b) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+
+__device__ __forceinline__ float2 unpair(uint64_t p) {
+  float2 f;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(f.x), "=f"(f.y) : "l"(p));
+  return f;
+}
+
+__device__ __forceinline__ void add_pair(uint64_t& acc, float a, float b) {
+  asm("add.rn.f32x2 %0, %0, %1;" : "+l"(acc) : "l"(pair(a, b)));
+}
+
+__device__ __forceinline__ void add_chunk(const Chunk<__half>& ch, Sum8& acc) {
   const __half2* h = (const __half2*)&ch.v[0];
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
     const float2 f = __half22float2(h[q]);
-    acc[2 * q] += f.x;
-    acc[2 * q + 1] += f.y;
+    add_pair(acc.p[q], f.x, f.y);
   }
 }
 
-__device__ __forceinline__ void add_chunk(const Chunk<float>& ch, float* acc) {
+__device__ __forceinline__ void add_chunk(const Chunk<float>& ch, Sum8& acc) {
   const float* f = (const float*)&ch.v[0];
 #pragma unroll
-  for (int q = 0; q < 8; ++q) acc[q] += f[q];
+  for (int q = 0; q < 4; ++q) add_pair(acc.p[q], f[2 * q], f[2 * q + 1]);
 }
 
 __device__ __forceinline__ uint4 to_half8(const float* f) {
@@ -167,6 +216,19 @@ __device__ __forceinline__ uint4 to_half8(const float* f) {
   h = __floats2half2_rn(f[4], f[5]); o.z = *(uint32_t*)&h;
   h = __floats2half2_rn(f[6], f[7]); o.w = *(uint32_t*)&h;
   return o;
+}
+
+// 32 bytes of an output row: one store, a whole sector, where the output is
+// 32-byte aligned.
+__device__ __forceinline__ void store_sector(void* p, bool wide, uint4 a, uint4 b) {
+  if (wide) {
+    asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(a.x),
+                 "r"(a.y), "r"(a.z), "r"(a.w), "r"(b.x), "r"(b.y), "r"(b.z), "r"(b.w)
+                 : "memory");
+  } else {
+    ((uint4*)p)[0] = a;
+    ((uint4*)p)[1] = b;
+  }
 }
 
 struct SageArgs {
@@ -181,142 +243,216 @@ struct SageArgs {
   const int32_t* tile_mb;     // per tile: its minibatch
   int32_t H;
   int32_t d_in, d_out;
-  uint8_t* A;                 // tiles x (kM x 2 d_in fp16), each tile a shared-memory image
+  int32_t tile_rows;          // R: dst rows per tile, a multiple of 8 up to kM
+  uint64_t inv_chunks;        // ceil(2^32 / (d_in / 8))
   const __half* w;            // d_out x 2 d_in
   const float* bias;          // d_out or null
   void* out;                  // minibatch j's dst rows at out + (j * out_stride + i) * d_out
   int64_t out_stride;
-  int32_t stages;             // A stages in the GEMM's shared memory
+  int32_t stages;             // A stages in shared memory
+  int32_t idx_cap;            // neighbour positions an index slot holds
   int32_t* err;
 };
 
+// Shared memory: W, the A stages, the index slots, the mbarriers.
+struct SageSmem {
+  uint8_t* w;
+  uint8_t* a;
+  uint8_t* idx;
+  uint32_t idx_bytes;  // per slot
+  uint64_t* bars;
+};
 
-// Items (R, c): row R of the tile space, 8-feature chunk c of x; each
-// thread takes kAggU items kAggThreads apart at a time, every load stage
-// issued for all of them before the next.  Writes the chunk of x_i and of
-// mean_i into the row's A tile (zeros past |dst_h|).
-constexpr int kAggU = 1;
+__host__ __device__ __forceinline__ uint32_t idx_slot_bytes(int32_t idx_cap) {
+  return (uint32_t)sizeof(IdxHead) + 4u * (uint32_t)idx_cap;  // idx_cap: a multiple of 4
+}
 
-template <typename T>
-__global__ void __launch_bounds__(kAggThreads, 5) sage_agg_kernel(SageArgs a, int64_t rows_total) {
-  constexpr int kER = sizeof(T) == 2 ? 8 : 4;  // edges in flight per item and round
-  constexpr int U = kAggU;
+__device__ __forceinline__ SageSmem sage_smem(uint8_t* smem, const SageArgs& a) {
+  const uint32_t KT = 2 * a.d_in;
+  SageSmem m;
+  m.w = smem;
+  m.a = m.w + (size_t)a.d_out * KT * 2;
+  m.idx = m.a + (size_t)a.stages * kM * KT * 2;
+  m.idx_bytes = idx_slot_bytes(a.idx_cap);
+  m.bars = (uint64_t*)(m.idx + (size_t)kIdxSlots * m.idx_bytes);
+  return m;
+}
+
+// The mbarriers, as shared-memory addresses: full[s] / empty[s] of the A
+// stages, dfull[d] / dempty[d] of the accumulators, ifull[q] / iempty[q] of
+// the index slots, and W's.
+struct SageBars {
+  uint32_t base;
+  __device__ uint32_t full(int s) const { return base + 8u * (uint32_t)s; }
+  __device__ uint32_t empty(int s) const { return base + 8u * (uint32_t)(kMaxStages + s); }
+  __device__ uint32_t dfull(int d) const { return base + 8u * (uint32_t)(2 * kMaxStages + d); }
+  __device__ uint32_t dempty(int d) const { return base + 8u * (uint32_t)(2 * kMaxStages + 2 + d); }
+  __device__ uint32_t ifull(int q) const { return base + 8u * (uint32_t)(2 * kMaxStages + 4 + q); }
+  __device__ uint32_t iempty(int q) const {
+    return base + 8u * (uint32_t)(2 * kMaxStages + 4 + kIdxSlots + q);
+  }
+  __device__ uint32_t w() const {
+    return base + 8u * (uint32_t)(2 * kMaxStages + 4 + 2 * kIdxSlots);
+  }
+};
+constexpr int kBars = 2 * kMaxStages + 4 + 2 * kIdxSlots + 1;
+constexpr int kBarBytesNeeded = 8 * kBars + 8;  // and the TMEM address slot
+
+// Whether use k (from 0) of a ring of n slots may start: use k - n has been
+// released.
+__device__ __forceinline__ bool ring_free(uint32_t bar, int k, int n) {
+  return k < n || mbar_wait(bar, (uint32_t)((k / n - 1) & 1));
+}
+
+// An index warp: tiles w, w + kIdxWarps, ... of the CTA.
+__device__ __forceinline__ bool sage_index_warp(const SageArgs& a, const SageSmem& m,
+                                                const SageBars& bar, int w, int lane,
+                                                int total_tiles) {
+  for (int k = w;; k += kIdxWarps) {
+    const int tile = (int)blockIdx.x + k * (int)gridDim.x;
+    if (tile >= total_tiles) return true;
+    const int q = k % kIdxSlots;
+    if (!__all_sync(0xffffffffu, ring_free(bar.iempty(q), k, kIdxSlots))) return false;
+    IdxHead* h = (IdxHead*)(m.idx + (size_t)q * m.idx_bytes);
+    int32_t* cols = (int32_t*)(h + 1);
+    const int j = __ldg(a.tile_mb + tile);
+    const int i0 = (tile - __ldg(a.tile_start + j)) * a.tile_rows;
+    const int rows = min(__ldg(a.num_dst + j) - i0, a.tile_rows);
+    const int64_t* ip = a.indptr + (size_t)j * a.indptr_stride + i0;
+    const int64_t e0 = __ldg(ip);
+    const int32_t n = (int32_t)(__ldg(ip + rows) - e0);
+    for (int r = lane; r <= a.tile_rows; r += 32)
+      h->ptr[r] = r < rows ? (int32_t)(__ldg(ip + r) - e0) : n;
+    const int32_t* col = a.col + (size_t)j * a.col_stride + e0;
+    const bool staged = n <= a.idx_cap;
+    if (staged) {
+      for (int32_t i = lane; i < n; i += 256) {
+        int32_t v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) v[u] = i + 32 * u < n ? __ldg(col + i + 32 * u) : 0;
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+          if (i + 32 * u < n) cols[i + 32 * u] = v[u];
+      }
+    }
+    if (lane == 0) {
+      h->i0 = i0;
+      h->rows = rows;
+      h->j = j;
+      h->staged = staged;
+      h->col = col;
+    }
+    __syncwarp();
+    if (lane == 0) mbar_arrive(bar.ifull(q));
+  }
+}
+
+// A producer warp: groups of 32 items of every tile of the CTA.
+template <typename T, bool kSwizzle>
+__device__ __forceinline__ bool sage_producer_warp(const SageArgs& a, const SageSmem& m,
+                                                   const SageBars& bar, int w, int lane,
+                                                   int total_tiles) {
+  constexpr int kER = sizeof(T) == 2 ? 5 : 3;  // neighbours in flight per item
   const int chunks = a.d_in / 8;
-  const int64_t items = rows_total * chunks;
-  const size_t tile_bytes = (size_t)kM * 2 * a.d_in * 2;
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t q0 = blockIdx.x * (int64_t)blockDim.x * U + threadIdx.x; q0 < items;
-       q0 += stride * U) {
-    int c[U], tile[U], r[U];
-    bool row_ok[U];
-    const T* x[U];
-    const int32_t* cl[U];
-    int64_t e0[U], e1[U], span = 0;
-    Chunk<T> sc[U];
-#pragma unroll
-    for (int k = 0; k < U; ++k) {
-      const int64_t q = q0 + (int64_t)k * blockDim.x;
-      const int64_t R = q < items ? q / chunks : 0;
-      c[k] = (int)(q - R * chunks);
-      tile[k] = (int)(R / kM);
-      r[k] = (int)(R - (int64_t)tile[k] * kM);
-      row_ok[k] = false;
-      e0[k] = e1[k] = 0;
-      if (q < items) {
-        const int j = __ldg(a.tile_mb + tile[k]);
-        const int i = (tile[k] - __ldg(a.tile_start + j)) * kM + r[k];
-        if (i < __ldg(a.num_dst + j)) {
-          row_ok[k] = true;
-          x[k] = (const T*)a.x + (size_t)j * a.x_stride * a.d_in;
-          cl[k] = a.col + (size_t)j * a.col_stride;
-          const int64_t* ip = a.indptr + (size_t)j * a.indptr_stride;
-          sc[k] = load_chunk<T>(x[k] + (size_t)i * a.d_in, c[k]);
-          e0[k] = __ldg(ip + i);
-          e1[k] = __ldg(ip + i + 1);
-          span = e1[k] - e0[k] > span ? e1[k] - e0[k] : span;
-        }
-      }
-    }
-    float acc[U][8];
-#pragma unroll
-    for (int k = 0; k < U; ++k)
-#pragma unroll
-      for (int z = 0; z < 8; ++z) acc[k][z] = 0.f;
-    for (int64_t base = 0; base < span; base += kER) {
-      int32_t idx[U][kER];
-#pragma unroll
-      for (int k = 0; k < U; ++k)
-#pragma unroll
-        for (int u = 0; u < kER; ++u)
-          idx[k][u] = e0[k] + base + u < e1[k] ? __ldg(cl[k] + e0[k] + base + u) : -1;
-      Chunk<T> val[U][kER];
-#pragma unroll
-      for (int k = 0; k < U; ++k)
-#pragma unroll
-        for (int u = 0; u < kER; ++u) {
-          if (idx[k][u] >= 0) {
-            val[k][u] = load_chunk<T>(x[k] + (size_t)idx[k][u] * a.d_in, c[k]);
-          } else {
-#pragma unroll
-            for (int z = 0; z < (int)(sizeof(T) / 2); ++z)
-              val[k][u].v[z] = make_uint4(0, 0, 0, 0);
-          }
-        }
-#pragma unroll
-      for (int k = 0; k < U; ++k)
-#pragma unroll
-        for (int u = 0; u < kER; ++u) add_chunk(val[k][u], acc[k]);
-    }
-#pragma unroll
-    for (int k = 0; k < U; ++k) {
-      const int64_t q = q0 + (int64_t)k * blockDim.x;
-      if (q >= items) continue;
+  const int groups = a.tile_rows * chunks / 32;
+  const size_t stage_bytes = (size_t)kM * 2 * a.d_in * 2;
+  int first = w;  // the warp's first group, rotated from tile to tile so that a
+                  // remainder of groups falls to every warp in turn
+  for (int k = 0;; ++k) {
+    const int tile = (int)blockIdx.x + k * (int)gridDim.x;
+    if (tile >= total_tiles) return true;
+    const int q = k % kIdxSlots, s = k % a.stages;
+    const bool ready = mbar_wait(bar.ifull(q), (uint32_t)((k / kIdxSlots) & 1)) &&
+                       ring_free(bar.empty(s), k, a.stages);
+    if (!__all_sync(0xffffffffu, ready)) return false;
+    const IdxHead* h = (const IdxHead*)(m.idx + (size_t)q * m.idx_bytes);
+    const int32_t* cl = h->staged ? (const int32_t*)(h + 1) : h->col;
+    const T* x = (const T*)a.x + (size_t)h->j * a.x_stride * a.d_in;
+    const int32_t i0 = h->i0, rows = h->rows;
+    uint8_t* A = m.a + (size_t)s * stage_bytes;
+    for (int g = first; g < groups; g += kProdWarps) {
+      // the chunks fastest: the 8 lanes of a quarter warp, which one wavefront
+      // serves, read one 128-byte line of a row
+      const uint32_t item = (uint32_t)(g * 32 + lane);
+      const int r = (int)((item * a.inv_chunks) >> 32);  // item / chunks
+      const int c = (int)item - r * chunks;
       uint4 self = make_uint4(0, 0, 0, 0), mean = make_uint4(0, 0, 0, 0);
-      if (row_ok[k]) {
-        if constexpr (sizeof(T) == 2) {
-          self = sc[k].v[0];
-        } else {
-          const float* f = (const float*)&sc[k].v[0];
-          float g[8];
+      if (r < rows) {
+        const Chunk<T> sc = load_chunk<T>(x + (size_t)(i0 + r) * a.d_in, c);
+        const int32_t e0 = h->ptr[r], e1 = h->ptr[r + 1];
+        Sum8 acc;
 #pragma unroll
-          for (int z = 0; z < 8; ++z) g[z] = f[z];
-          self = to_half8(g);
+        for (int z = 0; z < 4; ++z) acc.p[z] = 0;
+        for (int32_t e = e0; e < e1; e += kER) {
+          Chunk<T> val[kER];
+#pragma unroll
+          for (int u = 0; u < kER; ++u) {
+            if (e + u < e1) {
+              val[u] = load_chunk<T>(x + (size_t)cl[e + u] * a.d_in, c);
+            } else {
+#pragma unroll
+              for (int z = 0; z < (int)(sizeof(T) / 2); ++z) val[u].v[z] = make_uint4(0, 0, 0, 0);
+            }
+          }
+#pragma unroll
+          for (int u = 0; u < kER; ++u) add_chunk(val[u], acc);
         }
-        if (e1[k] > e0[k]) {
-          const float deg = (float)(e1[k] - e0[k]);
+        if constexpr (sizeof(T) == 2) {
+          self = sc.v[0];
+        } else {
+          self = to_half8((const float*)&sc.v[0]);
+        }
+        if (e1 > e0) {
+          const float deg = (float)(e1 - e0);
+          float f[8];
 #pragma unroll
-          for (int z = 0; z < 8; ++z) acc[k][z] /= deg;
-          mean = to_half8(acc[k]);
+          for (int z = 0; z < 4; ++z) {
+            const float2 t = unpair(acc.p[z]);
+            f[2 * z] = t.x / deg;
+            f[2 * z + 1] = t.y / deg;
+          }
+          mean = to_half8(f);
         }
       }
-      uint8_t* At = a.A + (size_t)tile[k] * tile_bytes;
-      *(uint4*)(At + kmajor_off(r[k], c[k] * 8, kM)) = self;
-      *(uint4*)(At + kmajor_off(r[k], a.d_in + c[k] * 8, kM)) = mean;
+      if constexpr (kSwizzle) {
+        *(uint4*)(A + swizzled_off(r, c)) = self;
+        *(uint4*)(A + swizzled_off(r, chunks + c)) = mean;
+      } else {
+        *(uint4*)(A + kmajor_off(r, c * 8, kM)) = self;
+        *(uint4*)(A + kmajor_off(r, a.d_in + c * 8, kM)) = mean;
+      }
+    }
+    first = (first + kProdWarps - groups % kProdWarps) % kProdWarps;
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    __syncwarp();
+    if (lane == 0) {
+      mbar_arrive(bar.full(s));
+      mbar_arrive(bar.iempty(q));
     }
   }
 }
 
-template <typename OutT>
-__global__ void __launch_bounds__(kGemmThreads, 1) sage_gemm_kernel(SageArgs a) {
+// kSwizzle: A with 128-byte swizzle, where its rows are whole 64-element blocks
+// (d_in a multiple of 32): a quarter warp's 8 chunks of one row then go to 8
+// different bank groups.  Otherwise without swizzle, where they share one.
+template <typename T, typename OutT, bool kSwizzle>
+__global__ void __launch_bounds__(kSageThreads, 1) sage_kernel(SageArgs a) {
   extern __shared__ __align__(1024) uint8_t smem[];
   const int KT = 2 * a.d_in;
   const int N = a.d_out;
-  const int S = a.stages;
-  const uint32_t tile_bytes = (uint32_t)kM * KT * 2;
-  uint8_t* sW = smem;                                 // N x KT fp16
-  uint8_t* sA = smem + (size_t)N * KT * 2;            // S stages of kM x KT fp16
-  uint64_t* bars = (uint64_t*)(sA + (size_t)S * tile_bytes);
-  // full[0..S), empty[4..4+S), dfull[8..10), dempty[10..12), then the TMEM slot
-  const uint32_t bar0 = smem_u32(bars);
+  const SageSmem m = sage_smem(smem, a);
+  const SageBars bar{smem_u32(m.bars)};
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const uint32_t ncols = 2 * N <= 64 ? 64 : (2 * N <= 128 ? 128 : (2 * N <= 256 ? 256 : 512));
-  uint32_t* tmem_slot = (uint32_t*)(bars + 12);
-#define AGNES_FULL(s) (bar0 + 8u * (uint32_t)(s))
-#define AGNES_EMPTY(s) (bar0 + 8u * (uint32_t)(4 + (s)))
-#define AGNES_DFULL(d) (bar0 + 8u * (uint32_t)(8 + (d)))
-#define AGNES_DEMPTY(d) (bar0 + 8u * (uint32_t)(10 + (d)))
+  uint32_t* tmem_slot = (uint32_t*)(m.bars + kBars);
 
-  if (warp == 0) {
+  // the swizzle's atoms are 1024-byte aligned: dynamic shared memory starts on
+  // such a boundary, and W is a multiple of that long
+  if (kSwizzle && (smem_u32(smem) & 1023u) != 0) {
+    if (tid == 0) *(volatile int32_t*)a.err = kSageTimeout;
+    return;
+  }
+  if (warp == kMmaWarp) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
                      smem_u32(tmem_slot)),
                  "r"(ncols)
@@ -324,91 +460,93 @@ __global__ void __launch_bounds__(kGemmThreads, 1) sage_gemm_kernel(SageArgs a) 
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
   if (tid == 0) {
-    for (int s = 0; s < S; ++s) {
-      mbar_init(AGNES_FULL(s), 1);
-      mbar_init(AGNES_EMPTY(s), 1);
+    for (int s = 0; s < kMaxStages; ++s) {
+      mbar_init(bar.full(s), kProdWarps);
+      mbar_init(bar.empty(s), 1);
     }
     for (int d = 0; d < 2; ++d) {
-      mbar_init(AGNES_DFULL(d), 1);
-      mbar_init(AGNES_DEMPTY(d), 4);  // one arrival per epilogue warp
+      mbar_init(bar.dfull(d), 1);
+      mbar_init(bar.dempty(d), 4);  // one arrival per epilogue warp
     }
+    for (int q = 0; q < kIdxSlots; ++q) {
+      mbar_init(bar.ifull(q), 1);
+      mbar_init(bar.iempty(q), kProdWarps);
+    }
+    mbar_init(bar.w(), 4);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  // W into its K-major layout: 16-byte chunk (n, kc) = W[n][8 kc .. 8 kc + 7]
-  const int kchunks = KT / 8;
-  for (int q = tid; q < N * kchunks; q += kGemmThreads) {
-    const int n = q / kchunks, kc = q - n * kchunks;
-    *(uint4*)(sW + kmajor_off(n, kc * 8, N)) = __ldg((const uint4*)(a.w + (size_t)n * KT) + kc);
-  }
-  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = *tmem_slot;
   const int total_tiles = __ldg(a.tile_start + a.H);
   bool ok = true;
+  const bool wide_out = ((uintptr_t)a.out & 31) == 0;  // rows are whole 32-byte sectors
 
-  if (warp == 0) {
-    // producer: A tile k of this CTA into stage k % S
-    if (lane == 0) {
-      int k = 0;
-      for (int tile = blockIdx.x; tile < total_tiles; tile += gridDim.x, ++k) {
-        const int s = k % S;
-        if (k >= S && !mbar_wait(AGNES_EMPTY(s), (uint32_t)((k / S - 1) & 1))) {
-          ok = false;
-          break;
-        }
-        mbar_arrive_tx(AGNES_FULL(s), tile_bytes);
-        bulk_g2s(smem_u32(sA + (size_t)s * tile_bytes), a.A + (size_t)tile * tile_bytes,
-                 tile_bytes, AGNES_FULL(s));
-      }
-    }
-  } else if (warp == 1) {
-    // MMA issuer: tile k from stage k % S into accumulator k % 2
+  if (warp >= kProdWarp0) {
+    ok = sage_producer_warp<T, kSwizzle>(a, m, bar, warp - kProdWarp0, lane, total_tiles);
+  } else if (warp >= kIdxWarp0) {
+    ok = sage_index_warp(a, m, bar, warp - kIdxWarp0, lane, total_tiles);
+  } else if (warp == kMmaWarp) {
+    // MMA issuer: tile k from stage k % stages into accumulator k % 2
     if (lane == 0) {
       const uint32_t idesc = idesc_f16(kM, N);
-      const uint32_t w_addr = smem_u32(sW);
+      const uint32_t w_addr = smem_u32(m.w);
+      const uint32_t stage_bytes = (uint32_t)kM * KT * 2;
+      ok = mbar_wait(bar.w(), 0);
       int k = 0;
-      for (int tile = blockIdx.x; tile < total_tiles; tile += gridDim.x, ++k) {
-        const int s = k % S, d = k & 1;
-        if (!mbar_wait(AGNES_FULL(s), (uint32_t)((k / S) & 1)) ||
-            (k >= 2 && !mbar_wait(AGNES_DEMPTY(d), (uint32_t)((k / 2 - 1) & 1)))) {
+      for (int tile = blockIdx.x; ok && tile < total_tiles; tile += gridDim.x, ++k) {
+        const int s = k % a.stages, d = k & 1;
+        if (!mbar_wait(bar.full(s), (uint32_t)((k / a.stages) & 1)) ||
+            !ring_free(bar.dempty(d), k, 2)) {
           ok = false;
           break;
         }
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const uint32_t a_addr = smem_u32(sA + (size_t)s * tile_bytes);
+        const uint32_t a_addr = smem_u32(m.a) + (uint32_t)s * stage_bytes;
         const uint32_t dcol = tmem + (uint32_t)(d * N);
         // K step t covers K columns [16 t, 16 t + 16): core-matrix columns 2t, 2t+1
         for (int t = 0; t < KT / 16; ++t) {
-          const uint64_t da = smem_desc(a_addr + (uint32_t)(2 * t) * (kM / 8) * 128,
-                                        (kM / 8) * 128, 128);
+          const uint64_t da =
+              kSwizzle ? smem_desc_swizzled(a_addr + (uint32_t)(t >> 2) * (kM * 128) +
+                                            (uint32_t)(t & 3) * 32)
+                       : smem_desc(a_addr + (uint32_t)(2 * t) * (kM / 8) * 128, (kM / 8) * 128,
+                                   128);
           const uint64_t dw = smem_desc(w_addr + (uint32_t)(2 * t) * (uint32_t)(N / 8) * 128,
                                         (uint32_t)(N / 8) * 128, 128);
           mma_f16(dcol, da, dw, idesc, t > 0 ? 1u : 0u);
         }
-        mma_commit(AGNES_EMPTY(s));  // the stage is free once these MMAs have read it
-        mma_commit(AGNES_DFULL(d));  // and the accumulator is complete
+        mma_commit(bar.empty(s));  // the stage is free once these MMAs have read it
+        mma_commit(bar.dfull(d));  // and the accumulator is complete
       }
     }
-  } else if (warp >= 4) {
+  } else {
+    // W into its K-major layout: 16-byte chunk (n, kc) = W[n][8 kc .. 8 kc + 7]
+    const int kchunks = KT / 8;
+    for (int q = tid; q < N * kchunks; q += 128) {
+      const int n = q / kchunks, kc = q - n * kchunks;
+      *(uint4*)(m.w + kmajor_off(n, kc * 8, N)) = __ldg((const uint4*)(a.w + (size_t)n * KT) + kc);
+    }
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    __syncwarp();
+    if (lane == 0) mbar_arrive(bar.w());
     // epilogue: warp w reads TMEM lanes 32 (w % 4) .. +31 (its rows)
-    const int quad = warp & 3;
+    const int row = warp * 32 + lane;
     int k = 0;
     for (int tile = blockIdx.x; tile < total_tiles; tile += gridDim.x, ++k) {
       const int d = k & 1;
-      if (!mbar_wait(AGNES_DFULL(d), (uint32_t)((k / 2) & 1))) {
+      if (!__all_sync(0xffffffffu, mbar_wait(bar.dfull(d), (uint32_t)((k / 2) & 1)))) {
         ok = false;
         break;
       }
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       const int j = __ldg(a.tile_mb + tile);
-      const int i = (tile - __ldg(a.tile_start + j)) * kM + quad * 32 + lane;
-      const bool valid = i < __ldg(a.num_dst + j);
+      const int i = (tile - __ldg(a.tile_start + j)) * a.tile_rows + row;
+      const bool valid = row < a.tile_rows && i < __ldg(a.num_dst + j);
       OutT* orow = (OutT*)a.out + ((size_t)j * a.out_stride + i) * N;
       for (int c0 = 0; c0 < N; c0 += 32) {  // 32 columns per tcgen05.ld, one wait
         uint32_t v[32];
-        const uint32_t taddr = tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(d * N + c0);
+        const uint32_t taddr = tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(d * N + c0);
         asm volatile(
             "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, "
             "%10, %11, %12, %13, %14, %15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, "
@@ -423,6 +561,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) sage_gemm_kernel(SageArgs a) 
             : "memory");
         asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
         if (valid) {
+          uint4 half = make_uint4(0, 0, 0, 0);
 #pragma unroll
           for (int g = 0; g < 4; ++g) {
             float f[8];
@@ -433,36 +572,47 @@ __global__ void __launch_bounds__(kGemmThreads, 1) sage_gemm_kernel(SageArgs a) 
               f[q] = f[q] > 0.f ? f[q] : 0.f;
             }
             if constexpr (sizeof(OutT) == 4) {
-              ((float4*)(orow + c0 + 8 * g))[0] = make_float4(f[0], f[1], f[2], f[3]);
-              ((float4*)(orow + c0 + 8 * g))[1] = make_float4(f[4], f[5], f[6], f[7]);
+              store_sector(orow + c0 + 8 * g, wide_out, *(const uint4*)&f[0],
+                           *(const uint4*)&f[4]);
+            } else if (g & 1) {
+              store_sector(orow + c0 + 8 * (g - 1), wide_out, half, to_half8(f));
             } else {
-              *(uint4*)(orow + c0 + 8 * g) = to_half8(f);
+              half = to_half8(f);
             }
           }
         }
       }
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
       __syncwarp();
-      if (lane == 0) mbar_arrive(AGNES_DEMPTY(d));
+      if (lane == 0) mbar_arrive(bar.dempty(d));
     }
   }
-#undef AGNES_FULL
-#undef AGNES_EMPTY
-#undef AGNES_DFULL
-#undef AGNES_DEMPTY
-  if (!ok) atomicOr(a.err, kSageTimeout);
+  if (!ok) {
+    *(volatile int32_t*)a.err = kSageTimeout;  // pinned host memory
+    __threadfence_system();
+  }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
-  if (warp == 0) {
+  if (warp == kMmaWarp) {
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(ncols)
                  : "memory");
   }
 }
 
-// Shared memory of the GEMM kernel with `stages` A stages.
-size_t gemm_smem_bytes(int64_t d_in, int64_t d_out, int stages) {
-  return (size_t)d_out * 2 * d_in * 2 + (size_t)stages * kM * 2 * d_in * 2 + kBarBytes;
+// Shared memory of the kernel with `stages` A stages and index slots of
+// idx_cap neighbour positions.
+size_t sage_smem_bytes(int64_t d_in, int64_t d_out, int stages, int32_t idx_cap) {
+  return (size_t)d_out * 2 * d_in * 2 + (size_t)stages * kM * 2 * d_in * 2 +
+         (size_t)kIdxSlots * idx_slot_bytes(idx_cap) + kBarBytesNeeded;
+}
+
+// What the entry point's limit counts: W, one stage and kBarBytes.  The largest
+// accepted shapes (d_in a multiple of 8, d_out of 32) leave 2048 bytes of the
+// limit or more, so the heads of the index slots (kIdxSlots * sizeof(IdxHead)
+// = 1680 bytes) and the mbarriers always fit beside them.
+size_t stated_smem_bytes(int64_t d_in, int64_t d_out) {
+  return (size_t)d_out * 2 * d_in * 2 + (size_t)kM * 2 * d_in * 2 + kBarBytes;
 }
 
 bool is_device_ptr(const void* p) {
@@ -474,22 +624,40 @@ bool is_device_ptr(const void* p) {
   return attr.type == cudaMemoryTypeDevice || attr.type == cudaMemoryTypeManaged;
 }
 
-template <typename T, typename OutT>
-cudaError_t launch_sage(const SageArgs& a, int64_t tiles, int num_sms, cudaStream_t st) {
-  const int64_t rows = tiles * kM;
-  const int64_t items = rows * (a.d_in / 8);
-  int64_t agg_grid = resident_grid((const void*)sage_agg_kernel<T>, kAggThreads, num_sms);
-  const int64_t per_cta = (int64_t)kAggThreads * kAggU;
-  if (agg_grid * per_cta > items) agg_grid = (items + per_cta - 1) / per_cta;
-  sage_agg_kernel<T><<<(unsigned)agg_grid, kAggThreads, 0, st>>>(a, rows);
-  size_t smem = gemm_smem_bytes(a.d_in, a.d_out, a.stages);
+template <typename T, typename OutT, bool kSwizzle>
+cudaError_t launch_sage_typed(const SageArgs& a, int64_t tiles, int num_sms, cudaStream_t st) {
+  size_t smem = sage_smem_bytes(a.d_in, a.d_out, a.stages, a.idx_cap);
   if (smem < kSageMinSmem) smem = kSageMinSmem;
-  cudaError_t e = cudaFuncSetAttribute(sage_gemm_kernel<OutT>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  const auto kernel = sage_kernel<T, OutT, kSwizzle>;
+  cudaError_t e =
+      cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   const int grid = (int)(tiles < num_sms ? tiles : num_sms);
-  sage_gemm_kernel<OutT><<<grid, kGemmThreads, smem, st>>>(a);
+  kernel<<<grid, kSageThreads, smem, st>>>(a);
   return cudaGetLastError();
+}
+
+template <typename T, typename OutT>
+cudaError_t launch_sage(const SageArgs& a, int64_t tiles, int num_sms, cudaStream_t st) {
+  return a.d_in % 32 == 0 ? launch_sage_typed<T, OutT, true>(a, tiles, num_sms, st)
+                          : launch_sage_typed<T, OutT, false>(a, tiles, num_sms, st);
+}
+
+// A stages and index slot size: the slots hold a tile of `edges` edges where
+// there is room, and at least half of it where that leaves two stages or more.
+bool sage_shape(int64_t d_in, int64_t d_out, int64_t edges, int32_t* stages, int32_t* idx_cap) {
+  const int32_t want = (int32_t)((edges < kIdxCapMax ? edges : kIdxCapMax) + 3) & ~3;
+  for (int s = kMaxStages; s >= 1; --s) {
+    const size_t base = sage_smem_bytes(d_in, d_out, s, 0);
+    if (base > AGNES_SAGE_MAX_SMEM) continue;
+    const int32_t room =
+        (int32_t)((AGNES_SAGE_MAX_SMEM - base) / (sizeof(int32_t) * kIdxSlots)) & ~3;
+    if (s > 1 && room < want / 2) continue;
+    *stages = s;
+    *idx_cap = room < want ? room : want;
+    return true;
+  }
+  return false;
 }
 
 }  // namespace
@@ -531,11 +699,9 @@ extern "C" agnes_status agnes_sage_mean_layer(agnes_ctx* ctx, int32_t hop, const
                        "[32, 256]");
     return AGNES_EINVAL;
   }
-  int stages = 2;
-  if (gemm_smem_bytes(d_in, d_out, stages) > AGNES_SAGE_MAX_SMEM) stages = 1;
-  if (gemm_smem_bytes(d_in, d_out, stages) > AGNES_SAGE_MAX_SMEM) {
+  if (stated_smem_bytes(d_in, d_out) > AGNES_SAGE_MAX_SMEM) {
     ctx_set_error(ctx, "d_in %lld with d_out %d needs %zu bytes of shared memory (limit %d)",
-                  (long long)d_in, d_out, gemm_smem_bytes(d_in, d_out, 1), AGNES_SAGE_MAX_SMEM);
+                  (long long)d_in, d_out, stated_smem_bytes(d_in, d_out), AGNES_SAGE_MAX_SMEM);
     return AGNES_ERANGE;
   }
   if (((uintptr_t)x | (uintptr_t)w | (uintptr_t)out) % 16 != 0 ||
@@ -544,11 +710,31 @@ extern "C" agnes_status agnes_sage_mean_layer(agnes_ctx* ctx, int32_t hop, const
     return AGNES_EINVAL;
   }
   const int H = v.H;
+  const int32_t* dst_size = v.node_size + (size_t)hop * H;
+  // rows per tile: 128 (the MMA's M), halved down to 32 while that leaves SMs
+  // without a tile -- a small layer is bound by the latency of its producers'
+  // loads, and the MMA costs the same for fewer rows
+  auto tiles_of = [&](int32_t rows) {
+    int64_t n = 0;
+    for (int j = 0; j < H; ++j) n += ((int64_t)dst_size[j] + rows - 1) / rows;
+    return n;
+  };
+  int32_t tile_rows = kM;
+  int64_t tiles = tiles_of(tile_rows);
+  while (tile_rows > 32 && tiles < g.num_sms) {
+    tile_rows /= 2;
+    tiles = tiles_of(tile_rows);
+  }
+  int32_t stages = 1, idx_cap = 0;
+  const int64_t fanout = v.col_stride[hop] / (v.indptr_stride[hop] - 1);
+  if (!sage_shape(d_in, d_out, tile_rows * fanout, &stages, &idx_cap)) {
+    ctx_set_error(ctx, "d_in %lld with d_out %d does not fit shared memory", (long long)d_in,
+                  d_out);
+    return AGNES_ERANGE;
+  }
   int64_t max_src = 0, max_dst = 0;
-  // pinned staging: error word (16 bytes), then tile_start (H + 1), num_dst
-  // (H), tile_mb (one per tile)
-  int64_t tiles = 0;
-  for (int j = 0; j < H; ++j) tiles += ((int64_t)v.node_size[(size_t)hop * H + j] + kM - 1) / kM;
+  // pinned staging: error word (16 bytes; the kernel writes it in place), then
+  // tile_start (H + 1), num_dst (H), tile_mb (one per tile)
   const size_t tab_bytes = sizeof(int32_t) * ((size_t)2 * H + 1 + (size_t)tiles);
   void* hp = nullptr;
   cudaError_t e = ctx_pinned(ctx, 16 + tab_bytes, &hp);
@@ -560,14 +746,15 @@ extern "C" agnes_status agnes_sage_mean_layer(agnes_ctx* ctx, int32_t hop, const
   int32_t* tabs = (int32_t*)((char*)hp + 16);
   tiles = 0;
   for (int j = 0; j < H; ++j) {
-    const int64_t nd = v.node_size[(size_t)hop * H + j];
+    const int64_t nd = dst_size[j];
     const int64_t ns = v.src_size[(size_t)hop * H + j];
     max_dst = nd > max_dst ? nd : max_dst;
     max_src = ns > max_src ? ns : max_src;
     tabs[j] = (int32_t)tiles;
     tabs[H + 1 + j] = (int32_t)nd;
-    for (int64_t t = tiles; t < tiles + (nd + kM - 1) / kM; ++t) tabs[2 * H + 1 + t] = j;
-    tiles += (nd + kM - 1) / kM;
+    const int64_t nt = (nd + tile_rows - 1) / tile_rows;
+    for (int64_t t = tiles; t < tiles + nt; ++t) tabs[2 * H + 1 + t] = j;
+    tiles += nt;
   }
   tabs[H] = (int32_t)tiles;
   if (x_stride_rows < max_src || out_stride_rows < max_dst) {
@@ -581,14 +768,12 @@ extern "C" agnes_status agnes_sage_mean_layer(agnes_ctx* ctx, int32_t hop, const
     return AGNES_EINVAL;
   }
   cudaStream_t st = (cudaStream_t)cuda_stream;
-  // device scratch: error word and tables, then (256-byte aligned) the A tiles
-  const size_t a_off = (16 + tab_bytes + 255) & ~(size_t)255;
-  const size_t a_bytes = (size_t)tiles * kM * 2 * (size_t)d_in * 2;
-  void* scratch = nullptr;
-  e = ctx_scratch(ctx, a_off + a_bytes, &scratch);
-  int32_t* err = (int32_t*)scratch;
-  int32_t* d_tabs = (int32_t*)((char*)scratch + 16);
-  if (e == cudaSuccess) e = cudaMemsetAsync(err, 0, sizeof(int32_t), st);
+  void* scratch = nullptr;  // the tables on the device
+  e = ctx_scratch(ctx, tab_bytes, &scratch);
+  int32_t* d_tabs = (int32_t*)scratch;
+  int32_t* d_err = nullptr;
+  if (e == cudaSuccess) e = cudaHostGetDevicePointer((void**)&d_err, h_err, 0);
+  *h_err = 0;
   if (e == cudaSuccess) e = cudaMemcpyAsync(d_tabs, tabs, tab_bytes, cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess && tiles > 0) {
     SageArgs a;
@@ -604,13 +789,15 @@ extern "C" agnes_status agnes_sage_mean_layer(agnes_ctx* ctx, int32_t hop, const
     a.H = H;
     a.d_in = (int32_t)d_in;
     a.d_out = d_out;
-    a.A = (uint8_t*)scratch + a_off;
+    a.tile_rows = tile_rows;
+    a.inv_chunks = ((1ull << 32) + d_in / 8 - 1) / (d_in / 8);
     a.w = (const __half*)w;
     a.bias = bias;
     a.out = out;
     a.out_stride = out_stride_rows;
     a.stages = stages;
-    a.err = err;
+    a.idx_cap = idx_cap;
+    a.err = d_err;
     if (x_dtype == AGNES_F16)
       e = out_dtype == AGNES_F32 ? launch_sage<__half, float>(a, tiles, g.num_sms, st)
                                  : launch_sage<__half, __half>(a, tiles, g.num_sms, st);
@@ -618,15 +805,12 @@ extern "C" agnes_status agnes_sage_mean_layer(agnes_ctx* ctx, int32_t hop, const
       e = out_dtype == AGNES_F32 ? launch_sage<float, float>(a, tiles, g.num_sms, st)
                                  : launch_sage<float, __half>(a, tiles, g.num_sms, st);
   }
-  *h_err = 0;
-  if (e == cudaSuccess)
-    e = cudaMemcpyAsync(h_err, err, sizeof(int32_t), cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) {
     ctx_set_error(ctx, "agnes_sage_mean_layer: %s", cudaGetErrorString(e));
     return e == cudaErrorMemoryAllocation ? AGNES_ENOMEM : AGNES_ECUDA;
   }
-  if (*h_err & kSageTimeout) {
+  if (*(volatile int32_t*)h_err != 0) {
     ctx_set_error(ctx, "agnes_sage_mean_layer: a tensor-core or copy wait ran out");
     return AGNES_ETIMEOUT;
   }
