@@ -122,6 +122,7 @@ constexpr int kCellThreads = 128;  // threads per CTA of the cells kernel
 constexpr int kCompactIlp = 2;     // bucket entries per thread and round of the compaction (4 and 8 measured slower)
 constexpr int kCompactOversplit = 2;    // the compaction's (group, slice) items per resident CTA
 constexpr int kCompactMaxSlices = 256;
+constexpr int kCompactRound = kCompactIlp * kCellThreads;
 constexpr int kGroupCells = kCellThreads;
 constexpr int kSlotCap = 1024;
 constexpr int kSmallMax = kDedupSmallMax;
@@ -531,8 +532,7 @@ __global__ void __launch_bounds__(kCellThreads) dedup_compact_kernel(CompactArgs
     __syncthreads();
     const int32_t k0 = s_nfo[0], k1 = s_nfo[last - c0];
     // kCompactIlp entries per thread and round: their loads in flight before the stores
-    constexpr int kRound = kCompactIlp * kCellThreads;
-    for (int32_t kb = k0 + slice * kRound + tid; kb < k1; kb += a.slices * kRound) {
+    for (int32_t kb = k0 + slice * kCompactRound + tid; kb < k1; kb += a.slices * kCompactRound) {
       int32_t cl[kCompactIlp], r[kCompactIlp], id[kCompactIlp], pos[kCompactIlp];
       bool in[kCompactIlp];
 #pragma unroll
@@ -594,9 +594,9 @@ __global__ void __launch_bounds__(kCellThreads) dedup_compact_kernel(CompactArgs
 cudaError_t launch_dedup(const HopArgs& a, const DedupBufs& d, int num_sms, cudaStream_t st) {
   const TileMap tm{a.tile_first, a.chunk_tile, a.T};
   const int64_t ncells = (int64_t)a.T * a.H;
-  int gx = (num_sms * 8 + a.H - 1) / a.H;
-  if (gx < 1) gx = 1;
-  const dim3 egrid(gx, a.H);
+  // CTAs per minibatch: eight per SM in all, no more than its edges fill
+  const int64_t gx = (num_sms * 8 + a.H - 1) / a.H, fill = (a.ecap + kThreads - 1) / kThreads;
+  const dim3 egrid((unsigned)(gx < fill ? gx : fill), (unsigned)a.H);
   cudaError_t e =
       flat_scan(d.scnt, d.soff, ncells, true, nullptr, true, d.flat_scratch, a.status, st);
   if (e != cudaSuccess) return e;
@@ -673,11 +673,19 @@ cudaError_t launch_dedup(const HopArgs& a, const DedupBufs& d, int num_sms, cuda
   k.n_feat_blocks = d.n_feat_blocks;
   k.feat_touched = d.feat_touched;
   k.status = a.status;
-  const int grid = resident_grid((const void*)dedup_compact_kernel, kCellThreads, num_sms);
-  k.fix_ctas = grid / a.H > 1 ? grid / a.H : 1;
+  const int resident = resident_grid((const void*)dedup_compact_kernel, kCellThreads, num_sms);
   const int64_t ngroups = (ncells + kGroupCells - 1) / kGroupCells;
-  const int64_t slices = (kCompactOversplit * (int64_t)grid + ngroups - 1) / ngroups;
+  const int64_t rounds =  // of all entries, if they were in one group
+      (a.H * (a.cap_prev + a.ecap) + kCompactRound - 1) / kCompactRound;
+  int64_t slices = (kCompactOversplit * (int64_t)resident + ngroups - 1) / ngroups;
+  if (slices > rounds) slices = rounds;
   k.slices = (int32_t)(slices > kCompactMaxSlices ? kCompactMaxSlices : slices);
+  const int64_t fix = (a.ecap + kIlp * kCellThreads - 1) / (kIlp * kCellThreads);
+  const int64_t fix_ctas = resident / a.H > 1 ? resident / a.H : 1;
+  k.fix_ctas = (int32_t)(fix < fix_ctas ? fix : fix_ctas);
+  const int64_t items = ngroups * k.slices, fixes = (int64_t)a.H * k.fix_ctas;
+  const int grid = fitted_grid((const void*)dedup_compact_kernel, kCellThreads, num_sms,
+                               items > fixes ? items : fixes);
   dedup_compact_kernel<<<grid, kCellThreads, 0, st>>>(k);
   return cudaGetLastError();
 }

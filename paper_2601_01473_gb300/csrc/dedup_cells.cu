@@ -437,14 +437,16 @@ CellsArgs cells_args(const HopArgs& h, const DedupBufs& d) {
 }
 
 template <bool kPacked>
-cudaError_t launch_cells(const CellsArgs& a, int num_sms, cudaStream_t st) {
-  const int grid = resident_grid((const void*)dedup_lane_kernel<kPacked>, kThreads, num_sms);
+cudaError_t launch_cells(const CellsArgs& a, int64_t entries, int num_sms, cudaStream_t st) {
   const int64_t nbatch = (a.ncells + 31) / 32;
+  const int grid = fitted_grid((const void*)dedup_lane_kernel<kPacked>, kThreads, num_sms,
+                               (nbatch + kWarps - 1) / kWarps);
   int64_t batches = nbatch / ((int64_t)grid * kWarps);
   batches = batches < 1 ? 1 : batches > kChunkBatches ? kChunkBatches : batches;
   dedup_lane_kernel<kPacked><<<grid, kThreads, 0, st>>>(a, (int32_t)batches);
-  dedup_tile_kernel<kPacked><<<resident_grid((const void*)dedup_tile_kernel<kPacked>, kThreads,
-                                             num_sms),
+  const int64_t queue = entries / (kLaneMax + 1);  // cells at most
+  dedup_tile_kernel<kPacked><<<fitted_grid((const void*)dedup_tile_kernel<kPacked>, kThreads,
+                                           num_sms, (queue + kWarps - 1) / kWarps),
                                kThreads, 0, st>>>(a);
   return cudaGetLastError();
 }
@@ -454,7 +456,9 @@ cudaError_t launch_cells(const CellsArgs& a, int num_sms, cudaStream_t st) {
 cudaError_t launch_dedup_cells(const HopArgs& h, const DedupBufs& d, int num_sms,
                                cudaStream_t st) {
   const CellsArgs a = cells_args(h, d);
-  return h.sb_packed ? launch_cells<true>(a, num_sms, st) : launch_cells<false>(a, num_sms, st);
+  const int64_t entries = h.H * (h.cap_prev + h.ecap);  // frontier and sampled, at most
+  return h.sb_packed ? launch_cells<true>(a, entries, num_sms, st)
+                     : launch_cells<false>(a, entries, num_sms, st);
 }
 
 }  // namespace agnes

@@ -62,8 +62,7 @@ gather_vec_kernel(const uint4* __restrict__ feats, const int32_t* __restrict__ f
 // entries and walks their R * vecs vectors as one range, lane after lane, with
 // U loads in flight per lane before their stores, so that neither a short row
 // (idle lanes) nor a row of 25 vectors (a nearly empty last round) costs
-// bandwidth (13 minibatches of 1000 targets, rows of 25 vectors: 264 -> 239 us a
-// hyperbatch against a warp per row).
+// bandwidth.
 template <int U>
 __global__ void __launch_bounds__(kThreads)
 gather_any_kernel(const uint4* __restrict__ feats, uint32_t vecs, int32_t R, uint64_t inv_vecs,
@@ -121,11 +120,10 @@ __device__ __forceinline__ uint4 load_within(uintptr_t p, uintptr_t lo, uintptr_
 // Rows whose size or addresses are not multiples of 16 bytes, but of E (4, 2 or
 // 1).  The output row is written as its aligned 16-byte vectors, the first and
 // last of them in part; the 16 source bytes of each come from the one or two
-// aligned vectors that hold them, shifted by bytes, so a load moves four times
-// the bytes of a word copy and more (8 minibatches of 500 targets, rows of 1204
-// bytes: 306 -> 277 us a hyperbatch against a copy by words, and 309 by bytes).
-// Ranges of R rows as in gather_any_kernel, `vecs` being the most vectors a row
-// can touch.
+// aligned vectors that hold them, shifted by bytes.  (Moving the row as E-byte
+// elements instead took 103 us for 190k rows of 1204 bytes, this 45: the
+// aligned loads move four times the bytes each.)  Ranges of R rows as in
+// gather_any_kernel, `vecs` being the most vectors a row can touch.
 template <int E, int U>
 __global__ void __launch_bounds__(kThreads)
 gather_shift_kernel(uintptr_t feats, uintptr_t feats_end, int64_t row_bytes, uint32_t vecs,
@@ -225,22 +223,26 @@ int32_t rows_per_range(int64_t vecs, int U) {
 
 uint64_t inverse_of(int64_t vecs) { return ((1ull << 32) + vecs - 1) / vecs; }
 
-int gather_grid(const void* kernel, int ctas_per_sm, int num_sms) {
-  const int g = resident_grid(kernel, kThreads, num_sms);
+// CTAs for at most max_total rows, per_warp of them a warp takes at a time.
+int gather_grid(const void* kernel, int ctas_per_sm, int num_sms, int64_t max_total,
+                int64_t per_warp) {
+  const int64_t per_cta = per_warp * (kThreads / 32);
+  const int g = fitted_grid(kernel, kThreads, num_sms, (max_total + per_cta - 1) / per_cta);
   return ctas_per_sm > 0 && g > ctas_per_sm * num_sms ? ctas_per_sm * num_sms : g;
 }
 
 template <int E>
 cudaError_t launch_gather_shift(const void* feats, int64_t feats_bytes, int64_t row_bytes,
                                 const int32_t* fb_id, const int32_t* fb_pos,
-                                const int32_t* total, void* out, const int32_t* status,
-                                int num_sms, cudaStream_t st) {
+                                const int32_t* total, int64_t max_total, void* out,
+                                const int32_t* status, int num_sms, cudaStream_t st) {
   constexpr int U = 3;
   const int64_t vecs = (row_bytes + 15 + 15) / 16;  // a row may start anywhere in a vector
+  const int32_t R = rows_per_range(vecs, U);
   const auto kernel = gather_shift_kernel<E, U>;
-  kernel<<<gather_grid((const void*)kernel, 0, num_sms), kThreads, 0, st>>>(
-      (uintptr_t)feats, (uintptr_t)feats + (uintptr_t)feats_bytes, row_bytes, (uint32_t)vecs,
-      rows_per_range(vecs, U), inverse_of(vecs), fb_id, fb_pos, total, (uintptr_t)out, status);
+  kernel<<<gather_grid((const void*)kernel, 0, num_sms, max_total, R), kThreads, 0, st>>>(
+      (uintptr_t)feats, (uintptr_t)feats + (uintptr_t)feats_bytes, row_bytes, (uint32_t)vecs, R,
+      inverse_of(vecs), fb_id, fb_pos, total, (uintptr_t)out, status);
   return cudaGetLastError();
 }
 
@@ -248,20 +250,23 @@ cudaError_t launch_gather_shift(const void* feats, int64_t feats_bytes, int64_t 
 
 cudaError_t launch_gather(const void* feats, int64_t feats_bytes, int64_t row_bytes,
                           const int32_t* fb_id, const int32_t* fb_pos, const int32_t* total,
-                          void* out, const int32_t* status, int num_sms, cudaStream_t st) {
+                          int64_t max_total, void* out, const int32_t* status, int num_sms,
+                          cudaStream_t st) {
   // what the row size and both addresses are multiples of
   const uint64_t align = (uint64_t)row_bytes | (uintptr_t)feats | (uintptr_t)out;
   if (align % 16 != 0) {
     const auto shift = align % 4 == 0   ? launch_gather_shift<4>
                        : align % 2 == 0 ? launch_gather_shift<2>
                                         : launch_gather_shift<1>;
-    return shift(feats, feats_bytes, row_bytes, fb_id, fb_pos, total, out, status, num_sms, st);
+    return shift(feats, feats_bytes, row_bytes, fb_id, fb_pos, total, max_total, out, status,
+                 num_sms, st);
   }
   const int64_t vecs = row_bytes / 16;
   const uint4* f = (const uint4*)feats;
   uint4* o = (uint4*)out;
+  const int32_t R = rows_per_range(vecs, kU);
 #define AGNES_GRID(KERNEL) \
-  gather_grid((const void*)KERNEL, kGatherCtasPerSm, num_sms), kThreads, 0, st
+  gather_grid((const void*)KERNEL, kGatherCtasPerSm, num_sms, max_total, R), kThreads, 0, st
   if (vecs == 8)
     gather_vec_kernel<8, kU><<<AGNES_GRID((gather_vec_kernel<8, kU>))>>>(f, fb_id, fb_pos, total,
                                                                          o, status);
@@ -273,8 +278,7 @@ cudaError_t launch_gather(const void* feats, int64_t feats_bytes, int64_t row_by
                                                                            o, status);
   else
     gather_any_kernel<kU><<<AGNES_GRID(gather_any_kernel<kU>)>>>(
-        f, (uint32_t)vecs, rows_per_range(vecs, kU), inverse_of(vecs), fb_id, fb_pos, total, o,
-        status);
+        f, (uint32_t)vecs, R, inverse_of(vecs), fb_id, fb_pos, total, o, status);
 #undef AGNES_GRID
   return cudaGetLastError();
 }

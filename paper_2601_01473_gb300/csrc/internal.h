@@ -13,6 +13,15 @@ namespace agnes {
 // kernel, so no CTA waits for a second wave.
 int resident_grid(const void* kernel, int threads, int num_sms);
 
+// The grid of a grid-stride kernel whose work fills at most `ctas` CTAs: no
+// more than that, and no more than are resident.  (A small hyperbatch's
+// launches are a few CTAs of work; starting and ending a thousand idle ones
+// costs each launch more than the work.)
+inline int fitted_grid(const void* kernel, int threads, int num_sms, int64_t ctas) {
+  const int resident = resident_grid(kernel, threads, num_sms);
+  return ctas < 1 ? 1 : ctas < resident ? (int)ctas : resident;
+}
+
 // Exclusive scan of nseg segments.  Segment s reads in[s*in_stride + i] for
 // i < len(s) and writes out[s*out_stride + i]; len(s) = d_len[s] when d_len is
 // non-null, else const_len.  With write_end, out[s*out_stride + len(s)] gets
@@ -232,11 +241,12 @@ cudaError_t launch_dedup_cells(const HopArgs& a, const DedupBufs& d, int num_sms
                                cudaStream_t st);
 
 // ---- gather_hbm.cu ---------------------------------------------------------
-// Gathers the rows of a bucket of *total entries (row id at feats + id *
+// Gathers the rows of a bucket of *total entries (max_total at most; row id at feats + id *
 // row_bytes, feats_bytes in all) to out + pos * row_bytes, byte for byte.
 cudaError_t launch_gather(const void* feats, int64_t feats_bytes, int64_t row_bytes,
                           const int32_t* fb_id, const int32_t* fb_pos, const int32_t* total,
-                          void* out, const int32_t* status, int num_sms, cudaStream_t st);
+                          int64_t max_total, void* out, const int32_t* status, int num_sms,
+                          cudaStream_t st);
 
 // ---- gather.cu -------------------------------------------------------------
 

@@ -424,8 +424,9 @@ static agnes_status enqueue_hyperbatch(agnes_ctx* ctx, const int32_t* fanouts, i
     rc = gather_streamed(ctx, cur, st);
     if (rc != AGNES_OK) return rc;
   } else {
-    CK(ctx, launch_gather(ctx->features, ctx->N * ctx->row_bytes, ctx->row_bytes, w.fb_id[cur], w.fb_pos[cur],
-                          w.fcell_off[cur] + cells, w.feats_out, w.status, nsm, st));
+    CK(ctx, launch_gather(ctx->features, ctx->N * ctx->row_bytes, ctx->row_bytes, w.fb_id[cur],
+                          w.fb_pos[cur], w.fcell_off[cur] + cells, H * w.capK, w.feats_out,
+                          w.status, nsm, st));
   }
   mark(true);
   CK(ctx, cudaMemcpyAsync(w.h_back, w.back, w.back_bytes, cudaMemcpyDeviceToHost, st));
@@ -691,9 +692,8 @@ agnes_status agnes_prepare_hyperbatch(agnes_ctx* ctx, const int32_t* targets, in
   b.back = (int32_t*)w.back;
   b.back_words = (int64_t)(w.back_bytes / sizeof(int32_t));
   const int64_t most = b.back_words > (int64_t)H * B ? b.back_words : (int64_t)H * B;
-  const int64_t ctas = (most + 255) / 256;
-  const int resident_ctas = resident_grid((const void*)begin_kernel, 256, ctx->num_sms);
-  begin_kernel<<<(unsigned)(ctas < resident_ctas ? ctas : resident_ctas), 256, 0, st>>>(b);
+  begin_kernel<<<fitted_grid((const void*)begin_kernel, 256, ctx->num_sms, (most + 255) / 256), 256,
+                 0, st>>>(b);
   CK(ctx, cudaGetLastError());
   int n_marks = 0;
   if (resident && ctx->lg.mode != AGNES_LAUNCH_DIRECT && !capturing)

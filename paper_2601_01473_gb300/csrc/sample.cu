@@ -609,11 +609,8 @@ cudaError_t launch_bucket_targets(int32_t* nodes, int64_t capK, int32_t H, int32
   const TileMap tm{tile_first, chunk_tile, T};
   const int64_t ncells = (int64_t)T * H;
   const int64_t total = (int64_t)H * B;
-  // a thread per target, on at most the resident CTAs
-  auto grid = [&](const void* kernel) {
-    const int64_t ctas = (total + kThreads - 1) / kThreads;
-    const int resident = resident_grid(kernel, kThreads, num_sms);
-    return (unsigned)(ctas < resident ? ctas : resident);
+  auto grid = [&](const void* kernel) {  // a thread per target
+    return fitted_grid(kernel, kThreads, num_sms, (total + kThreads - 1) / kThreads);
   };
   int32_t* rank = fb_id;  // free until the bucket is written
   targets_count_kernel<<<grid((const void*)targets_count_kernel), kThreads, 0, st>>>(
@@ -651,9 +648,7 @@ cudaError_t launch_sample_indptr(const HopArgs& a, const int32_t* nodes, const i
   p.status = a.status;
   const void* kernel = p.off32 ? (const void*)sample_indptr_kernel<int32_t>
                                : (const void*)sample_indptr_kernel<int64_t>;
-  const int64_t pairs = (int64_t)p.tiles * a.H;  // at most H * ceil(cap / tile) < 2^31
-  const int resident = resident_grid(kernel, kThreads, num_sms);
-  const int grid = (int)(pairs < resident ? pairs : resident);
+  const int grid = fitted_grid(kernel, kThreads, num_sms, (int64_t)p.tiles * a.H);
   if (p.off32)
     sample_indptr_kernel<int32_t><<<grid, kThreads, 0, st>>>(p);
   else
@@ -664,14 +659,17 @@ cudaError_t launch_sample_indptr(const HopArgs& a, const int32_t* nodes, const i
 template <int kSrc>
 static void launch_fill_typed(const FillArgs& f, int k, int huge_grid, int num_sms,
                               cudaStream_t st) {
+  const int64_t entries = f.H * f.cap_prev;  // at most
+  auto grid = [&](const void* kernel, int per_warp) {
+    const int64_t per_cta = (int64_t)kWarps * per_warp;
+    return fitted_grid(kernel, kThreads, num_sms, (entries + per_cta - 1) / per_cta);
+  };
   if (k <= 32)
-    sample_fill_kernel<kSrc><<<resident_grid((const void*)sample_fill_kernel<kSrc>, kThreads,
-                                             num_sms),
-                               kThreads, 0, st>>>(f);
+    sample_fill_kernel<kSrc>
+        <<<grid((const void*)sample_fill_kernel<kSrc>, 32 / k), kThreads, 0, st>>>(f);
   else if (k <= kWideMax)
-    sample_fill_wide_kernel<kSrc><<<resident_grid((const void*)sample_fill_wide_kernel<kSrc>,
-                                                  kThreads, num_sms),
-                                    kThreads, 0, st>>>(f);
+    sample_fill_wide_kernel<kSrc>
+        <<<grid((const void*)sample_fill_wide_kernel<kSrc>, 1), kThreads, 0, st>>>(f);
   else
     sample_fill_huge_kernel<kSrc><<<huge_grid, kThreads, 0, st>>>(f);
 }
