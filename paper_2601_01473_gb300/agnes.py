@@ -11,6 +11,7 @@ import ctypes
 import os
 from dataclasses import dataclass
 
+import numpy as np
 import torch
 
 _PKG = os.path.dirname(os.path.abspath(__file__))
@@ -174,12 +175,18 @@ def _check(rc: int, ctx=None):
         raise AgnesError(rc, msg.decode() if msg else "")
 
 
-def _stream_handle(stream) -> int | None:
-    if stream is None:
-        return torch.cuda.current_stream().cuda_stream or None
+def _stream_handle(stream, device=None) -> int | None:
+    if stream is None:  # the current stream of the device (None: the current one)
+        return torch.cuda.current_stream(device).cuda_stream or None
     if isinstance(stream, torch.cuda.Stream):
         return stream.cuda_stream or None
     return int(stream) or None
+
+
+def _int32_table(ptr: int, rows: int, cols: int):
+    """A copy of rows x cols int32 values in host memory."""
+    return np.frombuffer(bytearray(ctypes.string_at(ptr, 4 * rows * cols)),
+                         dtype=np.int32).reshape(rows, cols)
 
 
 class _CudaArray:
@@ -227,14 +234,9 @@ class HyperbatchView:
     def __init__(self, v: _HyperbatchView, device, tensors=None):
         K, H = v.K, v.H
         self.K, self.H = K, H
-        import numpy as np
-        sz = np.ctypeslib.as_array(ctypes.cast(v.node_size, ctypes.POINTER(ctypes.c_int32)),
-                                   shape=((K + 1) * H,)).reshape(K + 1, H).copy()
-        ed = np.ctypeslib.as_array(ctypes.cast(v.edges, ctypes.POINTER(ctypes.c_int32)),
-                                   shape=(K * H,)).reshape(K, H).copy()
-        ss = np.ctypeslib.as_array(ctypes.cast(v.src_size, ctypes.POINTER(ctypes.c_int32)),
-                                   shape=(K * H,)).reshape(K, H).copy()
-        self.node_size, self.edges, self.src_size = sz, ed, ss
+        self.node_size = _int32_table(v.node_size, K + 1, H)
+        self.edges = _int32_table(v.edges, K, H)
+        self.src_size = _int32_table(v.src_size, K, H)
         if tensors is None:  # wrappers of the ctx's output buffers
             tensors = ([_wrap(v.indptr[h], (H, v.indptr_stride[h]), torch.int64, device)
                         for h in range(K)],
@@ -245,15 +247,6 @@ class HyperbatchView:
                              _TORCH_OF[v.feat_dtype], device))
         self.indptr, self.col, self.nodes, self.feats = tensors
         self._tensors = tensors
-
-    @staticmethod
-    def _key(v: _HyperbatchView):
-        """What the buffer wrappers depend on: addresses, strides, shapes."""
-        K = v.K
-        return (K, v.H, v.nodes, v.nodes_stride, v.feats, v.feats_stride_rows, v.feat_dim,
-                v.feat_dtype, tuple(v.indptr[h] for h in range(K)),
-                tuple(v.indptr_stride[h] for h in range(K)), tuple(v.col[h] for h in range(K)),
-                tuple(v.col_stride[h] for h in range(K)))
 
     def view(self, j: int) -> "MinibatchView":
         hops = []
@@ -309,9 +302,8 @@ class Graph:
             raise ValueError(f"topology_io must be one of {sorted(FEATURE_IO)}")
         d.topology_io = FEATURE_IO[topology_io]
         ctx = ctypes.c_void_p()
-        with torch.cuda.device(self.device):
-            rc = lib().agnes_load_graph(ctypes.byref(d), device, _stream_handle(stream),
-                                        ctypes.byref(ctx))
+        rc = lib().agnes_load_graph(ctypes.byref(d), device, _stream_handle(stream, self.device),
+                                    ctypes.byref(ctx))
         _check(rc, None)
         self._ctx = ctx
         self._H = 0
@@ -343,10 +335,9 @@ class Graph:
         fan = (ctypes.c_int32 * len(fanouts))(*fanouts)
         H, B = targets.shape
         self._targets = targets  # keep alive until the copy has run
-        with torch.cuda.device(self.device):
-            rc = lib().agnes_prepare_hyperbatch(self._ctx, targets.data_ptr(), H, B, fan,
-                                                len(fanouts), seed & (2**64 - 1),
-                                                first_minibatch_id, _stream_handle(stream))
+        rc = lib().agnes_prepare_hyperbatch(self._ctx, targets.data_ptr(), H, B, fan, len(fanouts),
+                                            seed & (2**64 - 1), first_minibatch_id,
+                                            _stream_handle(stream, self.device))
         _check(rc, self._ctx)
         self._H, self._K = H, len(fanouts)
 
@@ -368,7 +359,7 @@ class Graph:
         workspace stays where it is (same hyperbatch shape)."""
         v = _HyperbatchView()
         _check(lib().agnes_fetch_hyperbatch(self._ctx, ctypes.byref(v)), self._ctx)
-        key = HyperbatchView._key(v)
+        key = bytes(v)  # every address, stride and shape
         cached = getattr(self, "_hv_cache", None)
         hv = HyperbatchView(v, self.device, cached[1] if cached and cached[0] == key else None)
         self._hv_cache = (key, hv._tensors)
