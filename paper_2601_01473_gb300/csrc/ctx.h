@@ -63,12 +63,10 @@ struct Workspace {
   int32_t* srank = nullptr;
   int2* sb = nullptr;
   int2* tmp = nullptr;
-  int32_t* big_list = nullptr;
   int32_t* hset = nullptr;     // fanouts above kWideMax: the sampler's per-warp hash sets
   int64_t hset_elems = 0;
-  int32_t* q_dense = nullptr;  // default frontier's dedup queue and its counters (internal.h, DedupBufs)
+  int32_t* q_dense = nullptr;  // dedup queue and its counters (internal.h, DedupBufs)
   int32_t* q_ctl = nullptr;
-  int32_t* big_n = nullptr;
   int32_t* tmp_id = nullptr;
   int32_t* tmp_pos = nullptr;
   uint64_t* indptr_scratch = nullptr;  // flags of the indptr scan (zero between hops)

@@ -1,13 +1,15 @@
-// dedup_cells.cu -- the default frontier's resolution of one hop's cells
-// (Algorithm 1: N^j_out <- N^j_out u Sample(j, ...); src_h = dst_h ++ new_h,
-// dst_{h+1} = src_h).  A cell (t, j) of the bucket matrix holds D, minibatch
-// j's frontier ids in tile t (ascending), and S, its sampled ids there.
-// Resolving it gives, with ranks local to the cell:
-//   newcnt / nfcnt   |S \ D| and |D u (S \ D)|;
+// dedup_cells.cu -- the resolution of one hop's cells (Algorithm 1: N^j_out <-
+// N^j_out u Sample(j, ...); src_h = dst_h ++ new_h; dst_{h+1} = src_h, or
+// with the sampled frontier the distinct sampled ids).  A cell (t, j) of the
+// bucket matrix holds D, minibatch j's frontier ids in tile t (ascending), and
+// S, its sampled ids there.  Resolving it gives, with ranks local to the cell:
+//   newcnt           |S \ D|;
+//   nfcnt            the next frontier cell's size, |D u S| or |S|;
 //   col[e]           the frontier twin's index in dst_h, or -(1 + r) for the
 //                    r-th smallest new id of the cell;
-//   tmp              the next frontier cell D u new in ascending id, a new id
-//                    with x = -(1 + r), a frontier id with its row;
+//   tmp              the next frontier cell in ascending id: D u S, a new id
+//                    with x = -(1 + r), a frontier id with its row; or S (the
+//                    kernels' kSampled), whose rows are their places;
 // dedup.cu's scans, col fix-up and compaction then turn the local ranks into
 // final indices (coalesced passes over edges and over the next bucket).
 //
@@ -24,6 +26,8 @@
 //   - larger cells with samples are queued (each chunk appends its cells in
 //     order) and resolved one warp per cell on bitmaps over the tile, where
 //     every rank is a popcount over per-word prefix counts.
+// The sampled frontier took an entry-parallel kernel and a bitmap kernel of its
+// own before: 16 x 1024 targets at [15, 10, 5] on 10M nodes 515 -> 437 us.
 // The sampled bucket is either (id, edge index) pairs or, when the hop's
 // edge indices fit 20 bits, packed words edge index << 12 | tile-local id
 // (the kernels' kPacked).
@@ -131,7 +135,7 @@ __device__ __forceinline__ void sort_net(int32_t (&k)[8], int32_t (&p)[8]) {
 
 // Resolves one cell with samples and at most W (4 or 8, kLaneMax at most)
 // entries in one thread.
-template <bool kPacked, int W>
+template <bool kPacked, bool kSampled, int W>
 __device__ __forceinline__ void thread_cell(const CellsArgs& a, int64_t cell, const CellFacts& c) {
   const int32_t n = c.fn + c.sn;
   const int32_t tb = __ldg(a.tile_first + c.t);
@@ -156,6 +160,7 @@ __device__ __forceinline__ void thread_cell(const CellsArgs& a, int64_t cell, co
   int32_t* col = a.col + (int64_t)c.j * a.ecap;
   int2* tmp = a.tmp + c.fo + c.so;
   int32_t prev = -1, cnt_new = 0, cnt_keep = 0, cur = 0;  // cur: col of the current id
+  int32_t kept = -1;  // kSampled: the last id kept
 #pragma unroll
   for (int q = 0; q < W; ++q) {
     if (key[q] != kNoKey) {
@@ -171,14 +176,18 @@ __device__ __forceinline__ void thread_cell(const CellsArgs& a, int64_t cell, co
           cur = x;
           ++cnt_new;
         }
-        tmp[cnt_keep++] = make_int2(tb + lu, x);
+        if constexpr (!kSampled) tmp[cnt_keep++] = make_int2(tb + lu, x);
       }
-      if (sampled) col[pay[q]] = cur;
+      if (sampled) {
+        col[pay[q]] = cur;
+        if (kSampled && lu != kept) tmp[cnt_keep++] = make_int2(tb + lu, 0);
+        kept = lu;
+      }
       prev = lu;
     }
   }
   a.newcnt[cell] = cnt_new;
-  a.nfcnt[cell] = c.fn + cnt_new;
+  a.nfcnt[cell] = cnt_keep;
 }
 
 // Walks every cell, a warp over 32 consecutive cells at a time.  Warps take
@@ -199,7 +208,7 @@ __device__ __forceinline__ void thread_cell(const CellsArgs& a, int64_t cell, co
 // cells, where chunks stay at 256 cells, 5.37 -> 5.36 ms with its layers.
 constexpr int kChunkBatches = 8;
 
-template <bool kPacked>
+template <bool kPacked, bool kSampled>
 __global__ void __launch_bounds__(kThreads, 6) dedup_lane_kernel(CellsArgs a, int32_t batches) {
   grid_dep_wait();
   if (failed(a.status)) return;
@@ -227,7 +236,7 @@ __global__ void __launch_bounds__(kThreads, 6) dedup_lane_kernel(CellsArgs a, in
       const int32_t n = c.fn + c.sn;
       if (has && c.sn == 0) {  // nothing sampled: the compaction copies the frontier cell
         a.newcnt[cell] = 0;
-        a.nfcnt[cell] = c.fn;
+        a.nfcnt[cell] = kSampled ? 0 : c.fn;
       }
       const unsigned qm = __ballot_sync(kFull, has && c.sn > 0 && n > kLaneMax);
       if ((qm >> lane) & 1u) queue[queued + __popc(qm & ((1u << lane) - 1u))] = (int32_t)cell;
@@ -235,9 +244,9 @@ __global__ void __launch_bounds__(kThreads, 6) dedup_lane_kernel(CellsArgs a, in
       // the warp takes the 4-entry network unless one of its cells needs 8
       const bool mine = has && c.sn > 0 && n <= kLaneMax;
       if (__any_sync(kFull, mine && n > 4)) {
-        if (mine) thread_cell<kPacked, 8>(a, cell, c);
+        if (mine) thread_cell<kPacked, kSampled, 8>(a, cell, c);
       } else if (mine) {
-        thread_cell<kPacked, 4>(a, cell, c);
+        thread_cell<kPacked, kSampled, 4>(a, cell, c);
       }
     }
     if (queued == 0) continue;  // warp-uniform
@@ -278,12 +287,17 @@ __device__ __forceinline__ void mark_entries(int32_t n, int lane, Get get, Put p
 //   N[w]   sampled ids, then the new ids S & ~D once both are marked;
 //   P[w]   frontier ids below word w << 16 | new ids below word w (each at
 //          most 4096, so the two halves add without carries);
-//   C[w]   new ids already entered in the next frontier cell.
+//   C[w]   new ids (kSampled: sampled ids) already entered in the next
+//          frontier cell;
+// and with kSampled S[w], the sampled ids, and PS[w], those below word w.
+template <bool kSampled>
 struct TileResolver {
   const uint32_t* D;
   const uint32_t* N;
   const uint32_t* P;
   uint32_t* C;
+  const uint32_t* S;
+  const uint32_t* PS;
   int2* tmp;            // the cell's next-frontier entries
   int32_t* col;         // the minibatch's col
   const int32_t* fpos;  // the cell's frontier rows
@@ -292,6 +306,7 @@ struct TileResolver {
   // Frontier entry i (sorted: i frontier ids lie below it) with tile-local id
   // v keeps its row; below it in the next cell also lie the new ids below v.
   __device__ __forceinline__ void frontier(int32_t i, int32_t v, int32_t row) const {
+    if constexpr (kSampled) return;
     const int32_t w = v >> 5;
     const uint32_t below = (1u << (v & 31)) - 1u;
     tmp[i + (int32_t)(P[w] & 0xffffu) + __popc(N[w] & below)] = make_int2(base + v, row);
@@ -312,8 +327,11 @@ struct TileResolver {
     } else {
       const int32_t rn = (int32_t)(pw & 0xffffu) + __popc(N[w] & below);  // new ids below
       col[e.y] = -1 - rn;
-      if ((atomicOr(C + w, bit) & bit) == 0u) tmp[rd + rn] = make_int2(base + v, -1 - rn);
+      if (!kSampled && (atomicOr(C + w, bit) & bit) == 0u)
+        tmp[rd + rn] = make_int2(base + v, -1 - rn);
     }
+    if (kSampled && (atomicOr(C + w, bit) & bit) == 0u)
+      tmp[(int32_t)PS[w] + __popc(S[w] & below)] = make_int2(base + v, 0);
   }
 };
 
@@ -322,7 +340,7 @@ struct TileResolver {
 // in flight together, and resolved from there; larger cells are walked twice
 // (mark, resolve).  Each warp loads the next queued cell's offsets while it
 // resolves the current one.
-template <bool kPacked>
+template <bool kPacked, bool kSampled>
 __global__ void __launch_bounds__(kThreads, 5) dedup_tile_kernel(CellsArgs a) {
   grid_dep_wait();
   if (failed(a.status)) return;
@@ -330,11 +348,15 @@ __global__ void __launch_bounds__(kThreads, 5) dedup_tile_kernel(CellsArgs a) {
   __shared__ __align__(16) uint32_t N_s[kWarps][kTileWords];
   __shared__ __align__(16) uint32_t P_s[kWarps][kTileWords];
   __shared__ __align__(16) uint32_t C_s[kWarps][kTileWords];
+  __shared__ __align__(16) uint32_t S_s[kSampled ? kWarps : 1][kTileWords];
+  __shared__ __align__(16) uint32_t PS_s[kSampled ? kWarps : 1][kTileWords];
   const int warp = threadIdx.x >> 5, lane = lane_id();
   uint32_t* D = D_s[warp];
   uint32_t* N = N_s[warp];
   uint32_t* P = P_s[warp];
   uint32_t* C = C_s[warp];
+  uint32_t* S = S_s[kSampled ? warp : 0];
+  uint32_t* PS = PS_s[kSampled ? warp : 0];
   const int32_t total = *a.q_len;
   const int32_t nwarps = (int32_t)gridDim.x * kWarps;
   int32_t q = (int32_t)blockIdx.x * kWarps + warp;
@@ -379,6 +401,17 @@ __global__ void __launch_bounds__(kThreads, 5) dedup_tile_kernel(CellsArgs a) {
     // N = S & ~D and the per-word prefix counts, both halves in one scan
     const uint4 d = reinterpret_cast<const uint4*>(D)[lane];
     uint4 nv = reinterpret_cast<const uint4*>(N)[lane];
+    int32_t kept = 0;  // kSampled: the cell's distinct sampled ids
+    if constexpr (kSampled) {
+      const uint32_t s0w = __popc(nv.x), s1w = __popc(nv.y), s2w = __popc(nv.z);
+      const uint32_t own = s0w + s1w + s2w + __popc(nv.w);
+      const uint32_t through = warp_incl_scan(own);
+      const uint32_t before = through - own;
+      reinterpret_cast<uint4*>(S)[lane] = nv;
+      reinterpret_cast<uint4*>(PS)[lane] =
+          make_uint4(before, before + s0w, before + s0w + s1w, before + s0w + s1w + s2w);
+      kept = (int32_t)through;  // on lane 31
+    }
     nv.x &= ~d.x;
     nv.y &= ~d.y;
     nv.z &= ~d.z;
@@ -394,11 +427,20 @@ __global__ void __launch_bounds__(kThreads, 5) dedup_tile_kernel(CellsArgs a) {
     reinterpret_cast<uint4*>(N)[lane] = nv;
     if (lane == 31) {
       a.newcnt[cell] = (int32_t)(incl & 0xffffu);
-      a.nfcnt[cell] = c.fn + (int32_t)(incl & 0xffffu);
+      a.nfcnt[cell] = kSampled ? kept : c.fn + (int32_t)(incl & 0xffffu);
     }
     __syncwarp();
-    const TileResolver r{D, N, P, C, a.tmp + c.fo + c.so, a.col + (int64_t)c.j * a.ecap, fpos,
-                         base, (int32_t)((int64_t)c.j * a.capK)};
+    const TileResolver<kSampled> r{D,
+                                   N,
+                                   P,
+                                   C,
+                                   S,
+                                   PS,
+                                   a.tmp + c.fo + c.so,
+                                   a.col + (int64_t)c.j * a.ecap,
+                                   fpos,
+                                   base,
+                                   (int32_t)((int64_t)c.j * a.capK)};
     if (small) {
       if (fv >= 0) r.frontier(lane, fv, fr);
       if (s0.x >= 0) r.sampled(s0);
@@ -436,18 +478,19 @@ CellsArgs cells_args(const HopArgs& h, const DedupBufs& d) {
   return a;
 }
 
-template <bool kPacked>
+template <bool kPacked, bool kSampled>
 cudaError_t launch_cells(const CellsArgs& a, int64_t entries, int num_sms, cudaStream_t st) {
   const int64_t nbatch = (a.ncells + 31) / 32;
-  const int grid = fitted_grid((const void*)dedup_lane_kernel<kPacked>, kThreads, num_sms,
-                               (nbatch + kWarps - 1) / kWarps);
+  const auto lane = dedup_lane_kernel<kPacked, kSampled>;
+  const int grid =
+      fitted_grid((const void*)lane, kThreads, num_sms, (nbatch + kWarps - 1) / kWarps);
   int64_t batches = nbatch / ((int64_t)grid * kWarps);
   batches = batches < 1 ? 1 : batches > kChunkBatches ? kChunkBatches : batches;
-  dedup_lane_kernel<kPacked><<<grid, kThreads, 0, st>>>(a, (int32_t)batches);
+  lane<<<grid, kThreads, 0, st>>>(a, (int32_t)batches);
   const int64_t queue = entries / (kLaneMax + 1);  // cells at most
-  dedup_tile_kernel<kPacked><<<fitted_grid((const void*)dedup_tile_kernel<kPacked>, kThreads,
-                                           num_sms, (queue + kWarps - 1) / kWarps),
-                               kThreads, 0, st>>>(a);
+  const auto tile = dedup_tile_kernel<kPacked, kSampled>;
+  tile<<<fitted_grid((const void*)tile, kThreads, num_sms, (queue + kWarps - 1) / kWarps),
+         kThreads, 0, st>>>(a);
   return cudaGetLastError();
 }
 
@@ -457,8 +500,12 @@ cudaError_t launch_dedup_cells(const HopArgs& h, const DedupBufs& d, int num_sms
                                cudaStream_t st) {
   const CellsArgs a = cells_args(h, d);
   const int64_t entries = h.H * (h.cap_prev + h.ecap);  // frontier and sampled, at most
-  return h.sb_packed ? launch_cells<true>(a, entries, num_sms, st)
-                     : launch_cells<false>(a, entries, num_sms, st);
+  const auto launch = h.sb_packed
+                          ? (d.frontier_sampled ? launch_cells<true, true>
+                                                : launch_cells<true, false>)
+                          : (d.frontier_sampled ? launch_cells<false, true>
+                                                : launch_cells<false, false>);
+  return launch(a, entries, num_sms, st);
 }
 
 }  // namespace agnes

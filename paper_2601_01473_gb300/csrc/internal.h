@@ -116,8 +116,8 @@ struct HopArgs {
   int32_t hset_log2 = 0;
   int32_t hset_grid = 0;
   // the sampled bucket holds 4-byte entries (edge index << 12 | tile-local
-  // id): the default frontier with ecap <= kPackedEdgeMax; the sampler then
-  // records rank << 12 | tile-local id per edge (no rank array)
+  // id): with ecap <= kPackedEdgeMax; the sampler then records
+  // rank << 12 | tile-local id per edge (no rank array)
   bool sb_packed = false;
 };
 
@@ -169,13 +169,9 @@ cudaError_t launch_sample_fill(const HopArgs& a, const int32_t* fb_id, const int
                                const FillRange& r, int num_sms, cudaStream_t st);
 
 // ---- dedup.cu --------------------------------------------------------------
-// Cells with more than this many entries (frontier + sampled) are resolved
-// on bitmaps, one warp each; the rest entry-parallel.  The big-cell list
-// therefore holds at most (entries) / (kDedupSmallMax + 1) cells.
-constexpr int kDedupSmallMax = 32;
-// With the default frontier, cells of at most this many entries are resolved
-// by one thread each; larger cells with samples are queued (q_dense), so the
-// queue holds at most (entries) / (kDedupLaneMax + 1) cells.
+// Cells of at most this many entries (frontier + sampled) are resolved by one
+// thread each; larger cells with samples are queued (q_dense), so the queue
+// holds at most (entries) / (kDedupLaneMax + 1) cells.
 constexpr int kDedupLaneMax = 8;
 
 struct DedupBufs {
@@ -188,9 +184,7 @@ struct DedupBufs {
   int2* sb;                 // bucketed (sampled id, edge index in the minibatch), or packed
                             // 4-byte entries edge index << 12 | tile-local id (sb_packed)
   int2* tmp;                // per cell: next-frontier entries with local ranks
-  int32_t* big_list;        // cells with more than kDedupSmallMax entries
-  int32_t* big_n;           // their count
-  // default frontier: the queue of cells with samples and more than
+  // the queue of cells with samples and more than
   // kDedupLaneMax entries, and {its length, the lane kernel's next chunk},
   // which the scatter clears
   int32_t* q_dense;
@@ -234,9 +228,9 @@ struct DedupBufs {
 cudaError_t launch_dedup(const HopArgs& a, const DedupBufs& d, int num_sms, cudaStream_t st);
 
 // ---- dedup_cells.cu --------------------------------------------------------
-// The default frontier's resolution of one hop's cells (launch_dedup calls
-// it in place of the sampled frontier's cell kernels): newcnt, nfcnt, col
-// with local new-id ranks, the next frontier cells in tmp; it builds and uses the queue in q_dense / q_ctl.
+// The resolution of one hop's cells: newcnt, nfcnt, col with local new-id
+// ranks, the next frontier cells in tmp; it builds and uses the queue in
+// q_dense / q_ctl.
 cudaError_t launch_dedup_cells(const HopArgs& a, const DedupBufs& d, int num_sms,
                                cudaStream_t st);
 

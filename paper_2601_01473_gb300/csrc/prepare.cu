@@ -85,11 +85,9 @@ void free_workspace(Workspace* w) {
   cudaFree(w->srank);
   cudaFree(w->sb);
   cudaFree(w->tmp);
-  cudaFree(w->big_list);
   cudaFree(w->hset);
   cudaFree(w->q_ctl);
   cudaFree(w->q_dense);
-  cudaFree(w->big_n);
   cudaFree(w->tmp_id);
   cudaFree(w->tmp_pos);
   cudaFree(w->indptr_scratch);
@@ -182,8 +180,6 @@ static agnes_status ensure_workspace(agnes_ctx* ctx, int32_t H, int32_t B, const
   WA(w.srank, edges);
   WA(w.sb, edges);
   WA(w.tmp, rows + edges);
-  WA(w.big_list, (rows + edges) / (kDedupSmallMax + 1) + 1);
-  WA(w.big_n, 1);
   WA(w.q_ctl, 2);
   WA(w.q_dense, (rows + edges) / (kDedupLaneMax + 1) + 1);
   w.hset_elems = 0;
@@ -346,7 +342,7 @@ static agnes_status enqueue_hyperbatch(agnes_ctx* ctx, const int32_t* fanouts, i
     a.hset = w.hset;
     huge_fanout_tables(fanouts[h], nsm, &a.hset_log2, &a.hset_grid);
     const bool frontier_sampled = ctx->frontier_mode == AGNES_FRONTIER_SAMPLED && h + 1 < K;
-    a.sb_packed = !frontier_sampled && a.ecap <= kPackedEdgeMax;
+    a.sb_packed = a.ecap <= kPackedEdgeMax;
     int32_t* nsz_prev = w.nsz + (int64_t)h * H;
     int32_t* ecnt = w.ecnt + (int64_t)h * H;
     CK(ctx, launch_sample_indptr(a, w.nodes, nsz_prev, w.indptr[h], ecnt, w.indptr_scratch, nsm,
@@ -385,14 +381,12 @@ static agnes_status enqueue_hyperbatch(agnes_ctx* ctx, const int32_t* fanouts, i
     d.soff = w.soff;
     d.sb = w.sb;
     d.tmp = w.tmp;
-    d.big_list = w.big_list;
     d.q_dense = w.q_dense;
     d.q_ctl = w.q_ctl;
     d.indptr_scratch = w.indptr_scratch;
     d.run_first_tile = ctx->bt.run_first_tile;
     d.n_runs = ctx->bt.n_starts;
     d.touched = w.stats + h;
-    d.big_n = w.big_n;
     d.fb_id = w.fb_id[cur];
     d.fb_pos = w.fb_pos[cur];
     d.fcell_off = w.fcell_off[cur];
