@@ -208,6 +208,17 @@ __device__ __forceinline__ void add_chunk(const Chunk<float>& ch, Sum8& acc) {
   for (int q = 0; q < 4; ++q) add_pair(acc.p[q], f[2 * q], f[2 * q + 1]);
 }
 
+// a / b rounded to nearest, for r = 1 / b rounded to nearest: the estimate
+// q = a r, corrected once by its exact remainder a - q b (Markstein, IBM J. Res.
+// Dev. 34, 1990).  The remainder is exact unless it underflows, where |a / b| is
+// below 2^-100 and fp16, what the quotient is rounded to next, keeps nothing of
+// it; where q is not finite the remainder is no number, and q is the quotient.
+__device__ __forceinline__ float quotient(float a, float b, float r) {
+  const float q = a * r;
+  const float rem = fmaf(-q, b, a);
+  return rem == rem ? fmaf(rem, r, q) : q;
+}
+
 __device__ __forceinline__ uint4 to_half8(const float* f) {
   uint4 o;
   __half2 h;
@@ -403,13 +414,13 @@ __device__ __forceinline__ bool sage_producer_warp(const SageArgs& a, const Sage
           self = to_half8((const float*)&sc.v[0]);
         }
         if (e1 > e0) {
-          const float deg = (float)(e1 - e0);
+          const float deg = (float)(e1 - e0), inv = __frcp_rn(deg);
           float f[8];
 #pragma unroll
           for (int z = 0; z < 4; ++z) {
             const float2 t = unpair(acc.p[z]);
-            f[2 * z] = t.x / deg;
-            f[2 * z + 1] = t.y / deg;
+            f[2 * z] = quotient(t.x, deg, inv);
+            f[2 * z + 1] = quotient(t.y, deg, inv);
           }
           mean = to_half8(f);
         }
