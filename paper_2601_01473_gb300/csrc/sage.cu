@@ -249,10 +249,13 @@ struct SageArgs {
   int64_t indptr_stride;
   const int32_t* col;
   int64_t col_stride;
+  // the tiles of more than kInlineH minibatches, in device memory (else null:
+  // SageTiles)
   const int32_t* tile_start;  // H + 1: first tile of each minibatch
   const int32_t* num_dst;     // H: |dst_h| per minibatch
   const int32_t* tile_mb;     // per tile: its minibatch
   int32_t H;
+  int32_t total_tiles;
   int32_t d_in, d_out;
   int32_t tile_rows;          // R: dst rows per tile, a multiple of 8 up to kM
   uint64_t inv_chunks;        // ceil(2^32 / (d_in / 8))
@@ -264,6 +267,41 @@ struct SageArgs {
   int32_t idx_cap;            // neighbour positions an index slot holds
   int32_t* err;
 };
+
+// The tiles of up to kInlineH minibatches travel with the launch: a tile's
+// minibatch is found by a search in the parameters, instead of in tables that a
+// copy would have to put on the device first (one layer of 300 to 18,000 rows:
+// 64-81 -> 60-71 us a call).
+constexpr int kInlineH = 256;
+struct SageTiles {
+  int32_t start[kInlineH + 1];  // first tile of each minibatch
+  int32_t dst[kInlineH];        // |dst_h| of each minibatch
+};
+
+// Tile `tile`: its minibatch, first dst row, and the rows from there on.
+struct SageTile {
+  int32_t j, i0, rows;
+};
+
+__device__ __forceinline__ SageTile sage_tile(const SageArgs& a, const SageTiles& t,
+                                              int32_t tile) {
+  SageTile r;
+  if (a.tile_mb) {
+    r.j = __ldg(a.tile_mb + tile);
+    r.i0 = (tile - __ldg(a.tile_start + r.j)) * a.tile_rows;
+    r.rows = __ldg(a.num_dst + r.j) - r.i0;
+  } else {
+    int32_t lo = 0, hi = a.H;  // the last minibatch that starts at or before the tile
+    while (hi - lo > 1) {
+      const int32_t mid = (lo + hi) >> 1;
+      if (t.start[mid] <= tile) lo = mid; else hi = mid;
+    }
+    r.j = lo;
+    r.i0 = (tile - t.start[lo]) * a.tile_rows;
+    r.rows = t.dst[lo] - r.i0;
+  }
+  return r;
+}
 
 // Shared memory: W, the A stages, the index slots, the mbarriers.
 struct SageSmem {
@@ -316,7 +354,8 @@ __device__ __forceinline__ bool ring_free(uint32_t bar, int k, int n) {
 }
 
 // An index warp: tiles w, w + kIdxWarps, ... of the CTA.
-__device__ __forceinline__ bool sage_index_warp(const SageArgs& a, const SageSmem& m,
+__device__ __forceinline__ bool sage_index_warp(const SageArgs& a, const SageTiles& tiles,
+                                                const SageSmem& m,
                                                 const SageBars& bar, int w, int lane,
                                                 int total_tiles) {
   for (int k = w;; k += kIdxWarps) {
@@ -326,9 +365,9 @@ __device__ __forceinline__ bool sage_index_warp(const SageArgs& a, const SageSme
     if (!__all_sync(0xffffffffu, ring_free(bar.iempty(q), k, kIdxSlots))) return false;
     IdxHead* h = (IdxHead*)(m.idx + (size_t)q * m.idx_bytes);
     int32_t* cols = (int32_t*)(h + 1);
-    const int j = __ldg(a.tile_mb + tile);
-    const int i0 = (tile - __ldg(a.tile_start + j)) * a.tile_rows;
-    const int rows = min(__ldg(a.num_dst + j) - i0, a.tile_rows);
+    const SageTile st = sage_tile(a, tiles, tile);
+    const int j = st.j, i0 = st.i0;
+    const int rows = min(st.rows, a.tile_rows);
     const int64_t* ip = a.indptr + (size_t)j * a.indptr_stride + i0;
     const int64_t e0 = __ldg(ip);
     const int32_t n = (int32_t)(__ldg(ip + rows) - e0);
@@ -447,7 +486,7 @@ __device__ __forceinline__ bool sage_producer_warp(const SageArgs& a, const Sage
 // (d_in a multiple of 32): a quarter warp's 8 chunks of one row then go to 8
 // different bank groups.  Otherwise without swizzle, where they share one.
 template <typename T, typename OutT, bool kSwizzle>
-__global__ void __launch_bounds__(kSageThreads, 1) sage_kernel(SageArgs a) {
+__global__ void __launch_bounds__(kSageThreads, 1) sage_kernel(SageArgs a, const __grid_constant__ SageTiles tiles) {
   extern __shared__ __align__(1024) uint8_t smem[];
   const int KT = 2 * a.d_in;
   const int N = a.d_out;
@@ -490,14 +529,14 @@ __global__ void __launch_bounds__(kSageThreads, 1) sage_kernel(SageArgs a) {
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = *tmem_slot;
-  const int total_tiles = __ldg(a.tile_start + a.H);
+  const int total_tiles = a.total_tiles;
   bool ok = true;
   const bool wide_out = ((uintptr_t)a.out & 31) == 0;  // rows are whole 32-byte sectors
 
   if (warp >= kProdWarp0) {
     ok = sage_producer_warp<T, kSwizzle>(a, m, bar, warp - kProdWarp0, lane, total_tiles);
   } else if (warp >= kIdxWarp0) {
-    ok = sage_index_warp(a, m, bar, warp - kIdxWarp0, lane, total_tiles);
+    ok = sage_index_warp(a, tiles, m, bar, warp - kIdxWarp0, lane, total_tiles);
   } else if (warp == kMmaWarp) {
     // MMA issuer: tile k from stage k % stages into accumulator k % 2
     if (lane == 0) {
@@ -551,10 +590,9 @@ __global__ void __launch_bounds__(kSageThreads, 1) sage_kernel(SageArgs a) {
         break;
       }
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      const int j = __ldg(a.tile_mb + tile);
-      const int i = (tile - __ldg(a.tile_start + j)) * a.tile_rows + row;
-      const bool valid = row < a.tile_rows && i < __ldg(a.num_dst + j);
-      OutT* orow = (OutT*)a.out + ((size_t)j * a.out_stride + i) * N;
+      const SageTile st = sage_tile(a, tiles, tile);
+      const bool valid = row < min(a.tile_rows, st.rows);
+      OutT* orow = (OutT*)a.out + ((size_t)st.j * a.out_stride + st.i0 + row) * N;
       for (int c0 = 0; c0 < N; c0 += 32) {  // 32 columns per tcgen05.ld, one wait
         uint32_t v[32];
         const uint32_t taddr = tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(d * N + c0);
@@ -636,22 +674,23 @@ bool is_device_ptr(const void* p) {
 }
 
 template <typename T, typename OutT, bool kSwizzle>
-cudaError_t launch_sage_typed(const SageArgs& a, int64_t tiles, int num_sms, cudaStream_t st) {
+cudaError_t launch_sage_typed(const SageArgs& a, const SageTiles& t, int num_sms,
+                              cudaStream_t st) {
   size_t smem = sage_smem_bytes(a.d_in, a.d_out, a.stages, a.idx_cap);
   if (smem < kSageMinSmem) smem = kSageMinSmem;
   const auto kernel = sage_kernel<T, OutT, kSwizzle>;
   cudaError_t e =
       cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  const int grid = (int)(tiles < num_sms ? tiles : num_sms);
-  kernel<<<grid, kSageThreads, smem, st>>>(a);
+  const int grid = a.total_tiles < num_sms ? a.total_tiles : num_sms;
+  kernel<<<grid, kSageThreads, smem, st>>>(a, t);
   return cudaGetLastError();
 }
 
 template <typename T, typename OutT>
-cudaError_t launch_sage(const SageArgs& a, int64_t tiles, int num_sms, cudaStream_t st) {
-  return a.d_in % 32 == 0 ? launch_sage_typed<T, OutT, true>(a, tiles, num_sms, st)
-                          : launch_sage_typed<T, OutT, false>(a, tiles, num_sms, st);
+cudaError_t launch_sage(const SageArgs& a, const SageTiles& t, int num_sms, cudaStream_t st) {
+  return a.d_in % 32 == 0 ? launch_sage_typed<T, OutT, true>(a, t, num_sms, st)
+                          : launch_sage_typed<T, OutT, false>(a, t, num_sms, st);
 }
 
 // A stages and index slot size: the slots hold a tile of `edges` edges where
@@ -744,9 +783,12 @@ extern "C" agnes_status agnes_sage_mean_layer(agnes_ctx* ctx, int32_t hop, const
     return AGNES_ERANGE;
   }
   int64_t max_src = 0, max_dst = 0;
-  // pinned staging: error word (16 bytes; the kernel writes it in place), then
-  // tile_start (H + 1), num_dst (H), tile_mb (one per tile)
-  const size_t tab_bytes = sizeof(int32_t) * ((size_t)2 * H + 1 + (size_t)tiles);
+  const bool inline_tiles = H <= kInlineH;
+  // pinned staging: error word (16 bytes; the kernel writes it in place), then,
+  // where the tiles do not travel with the launch, tile_start (H + 1), num_dst
+  // (H), tile_mb (one per tile)
+  const size_t tab_bytes =
+      inline_tiles ? 0 : sizeof(int32_t) * ((size_t)2 * H + 1 + (size_t)tiles);
   void* hp = nullptr;
   cudaError_t e = ctx_pinned(ctx, 16 + tab_bytes, &hp);
   if (e != cudaSuccess) {
@@ -755,19 +797,23 @@ extern "C" agnes_status agnes_sage_mean_layer(agnes_ctx* ctx, int32_t hop, const
   }
   int32_t* h_err = (int32_t*)hp;
   int32_t* tabs = (int32_t*)((char*)hp + 16);
+  SageTiles inl;
+  int32_t* starts = inline_tiles ? inl.start : tabs;
+  int32_t* dsts = inline_tiles ? inl.dst : tabs + H + 1;
   tiles = 0;
   for (int j = 0; j < H; ++j) {
     const int64_t nd = dst_size[j];
     const int64_t ns = v.src_size[(size_t)hop * H + j];
     max_dst = nd > max_dst ? nd : max_dst;
     max_src = ns > max_src ? ns : max_src;
-    tabs[j] = (int32_t)tiles;
-    tabs[H + 1 + j] = (int32_t)nd;
+    starts[j] = (int32_t)tiles;
+    dsts[j] = (int32_t)nd;
     const int64_t nt = (nd + tile_rows - 1) / tile_rows;
-    for (int64_t t = tiles; t < tiles + nt; ++t) tabs[2 * H + 1 + t] = j;
+    if (!inline_tiles)
+      for (int64_t t = tiles; t < tiles + nt; ++t) tabs[2 * H + 1 + t] = j;
     tiles += nt;
   }
-  tabs[H] = (int32_t)tiles;
+  starts[H] = (int32_t)tiles;
   if (x_stride_rows < max_src || out_stride_rows < max_dst) {
     ctx_set_error(ctx, "x_stride_rows must be >= %lld and out_stride_rows >= %lld",
                   (long long)max_src, (long long)max_dst);
@@ -780,12 +826,13 @@ extern "C" agnes_status agnes_sage_mean_layer(agnes_ctx* ctx, int32_t hop, const
   }
   cudaStream_t st = (cudaStream_t)cuda_stream;
   void* scratch = nullptr;  // the tables on the device
-  e = ctx_scratch(ctx, tab_bytes, &scratch);
+  if (!inline_tiles) e = ctx_scratch(ctx, tab_bytes, &scratch);
   int32_t* d_tabs = (int32_t*)scratch;
   int32_t* d_err = nullptr;
   if (e == cudaSuccess) e = cudaHostGetDevicePointer((void**)&d_err, h_err, 0);
   *h_err = 0;
-  if (e == cudaSuccess) e = cudaMemcpyAsync(d_tabs, tabs, tab_bytes, cudaMemcpyHostToDevice, st);
+  if (e == cudaSuccess && !inline_tiles)
+    e = cudaMemcpyAsync(d_tabs, tabs, tab_bytes, cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess && tiles > 0) {
     SageArgs a;
     a.x = x;
@@ -794,10 +841,11 @@ extern "C" agnes_status agnes_sage_mean_layer(agnes_ctx* ctx, int32_t hop, const
     a.indptr_stride = v.indptr_stride[hop];
     a.col = v.col[hop];
     a.col_stride = v.col_stride[hop];
-    a.tile_start = d_tabs;
-    a.num_dst = d_tabs + H + 1;
-    a.tile_mb = d_tabs + 2 * H + 1;
+    a.tile_start = inline_tiles ? nullptr : d_tabs;
+    a.num_dst = inline_tiles ? nullptr : d_tabs + H + 1;
+    a.tile_mb = inline_tiles ? nullptr : d_tabs + 2 * H + 1;
     a.H = H;
+    a.total_tiles = (int32_t)tiles;
     a.d_in = (int32_t)d_in;
     a.d_out = d_out;
     a.tile_rows = tile_rows;
@@ -810,11 +858,11 @@ extern "C" agnes_status agnes_sage_mean_layer(agnes_ctx* ctx, int32_t hop, const
     a.idx_cap = idx_cap;
     a.err = d_err;
     if (x_dtype == AGNES_F16)
-      e = out_dtype == AGNES_F32 ? launch_sage<__half, float>(a, tiles, g.num_sms, st)
-                                 : launch_sage<__half, __half>(a, tiles, g.num_sms, st);
+      e = out_dtype == AGNES_F32 ? launch_sage<__half, float>(a, inl, g.num_sms, st)
+                                 : launch_sage<__half, __half>(a, inl, g.num_sms, st);
     else
-      e = out_dtype == AGNES_F32 ? launch_sage<float, float>(a, tiles, g.num_sms, st)
-                                 : launch_sage<float, __half>(a, tiles, g.num_sms, st);
+      e = out_dtype == AGNES_F32 ? launch_sage<float, float>(a, inl, g.num_sms, st)
+                                 : launch_sage<float, __half>(a, inl, g.num_sms, st);
   }
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) {
