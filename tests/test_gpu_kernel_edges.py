@@ -133,6 +133,8 @@ def test_rows_of_any_width(cuda_device, dtype, dim, shift):
     (360, 32, torch.float32, [3], 2, 200),
     (224, 128, torch.float16, [12], 2, 500),    # one stage, few indices staged
     (64, 256, torch.float16, [300], 2, 60),     # more edges in a tile than are staged
+    (64, 64, torch.float16, [4], 256, 3),       # the most minibatches whose tiles travel along
+    (64, 64, torch.float16, [4], 257, 3),       # one more: tables on the device
 ])
 def test_sage_layer_shapes(cuda_device, d_in, d_out, dtype, fan, H, B):
     N = 30_000
