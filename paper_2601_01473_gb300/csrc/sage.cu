@@ -11,7 +11,9 @@
 //   index warps     stage the tile's indptr and neighbour positions (one
 //                   contiguous run of col) in a ring of shared-memory slots, so
 //                   that the chain indptr -> col -> row costs the producers one
-//                   trip to memory per round of neighbours, not three;
+//                   trip per round of neighbours, not three, and ask for the
+//                   tile's rows in L2 while they are at it, so that the trip ends
+//                   there;
 //   producer warps  form the update's input A = [x_i | mean_i]: an item (row,
 //                   8-feature chunk) per thread, its neighbours' chunks summed
 //                   in fp32 with several loads in flight, rounded to fp16 into
@@ -32,7 +34,10 @@
 // three layers 5.25 -> 4.35 ms.  On the way there: lanes over rows instead of
 // over a row's chunks kept the L1 data pipe 81% busy (a quarter warp's loads
 // touched 8 lines) and gained nothing; 16 producer warps instead of 24 cost 8%
-// of that model, 8 neighbours in flight instead of 5 cost 11% (registers).
+// of that model, 8 neighbours in flight instead of 5 cost 11% (registers).  The
+// rows asked for in L2 ahead: the model's outermost layer (3.4M rows, 16M
+// edges) 1.15 -> 1.01 ms, 5.2 TB/s; four or five index slots, further ahead,
+// lose that again.
 #include <cuda_fp16.h>
 
 #include "../../include/agnes.h"
@@ -353,7 +358,12 @@ __device__ __forceinline__ bool ring_free(uint32_t bar, int k, int n) {
   return k < n || mbar_wait(bar, (uint32_t)((k / n - 1) & 1));
 }
 
+__device__ __forceinline__ void prefetch_l2(const void* p) {
+  asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
+}
+
 // An index warp: tiles w, w + kIdxWarps, ... of the CTA.
+template <typename T>
 __device__ __forceinline__ bool sage_index_warp(const SageArgs& a, const SageTiles& tiles,
                                                 const SageSmem& m,
                                                 const SageBars& bar, int w, int lane,
@@ -375,6 +385,12 @@ __device__ __forceinline__ bool sage_index_warp(const SageArgs& a, const SageTil
       h->ptr[r] = r < rows ? (int32_t)(__ldg(ip + r) - e0) : n;
     const int32_t* col = a.col + (size_t)j * a.col_stride + e0;
     const bool staged = n <= a.idx_cap;
+    // the rows the tile reads -- its own, one after another, and its neighbours'
+    // -- on their way to L2, up to kIdxSlots tiles ahead of the producers
+    const uint32_t row_bytes = (uint32_t)a.d_in * (uint32_t)sizeof(T);
+    const char* x = (const char*)a.x + (size_t)j * a.x_stride * row_bytes;
+    for (uint32_t b = 128u * lane; b < (uint32_t)rows * row_bytes; b += 4096)
+      prefetch_l2(x + (size_t)i0 * row_bytes + b);
     if (staged) {
       for (int32_t i = lane; i < n; i += 256) {
         int32_t v[8];
@@ -382,7 +398,11 @@ __device__ __forceinline__ bool sage_index_warp(const SageArgs& a, const SageTil
         for (int u = 0; u < 8; ++u) v[u] = i + 32 * u < n ? __ldg(col + i + 32 * u) : 0;
 #pragma unroll
         for (int u = 0; u < 8; ++u)
-          if (i + 32 * u < n) cols[i + 32 * u] = v[u];
+          if (i + 32 * u < n) {
+            cols[i + 32 * u] = v[u];
+            const char* row = x + (size_t)v[u] * row_bytes;
+            for (uint32_t b = 0; b < row_bytes; b += 128) prefetch_l2(row + b);
+          }
       }
     }
     if (lane == 0) {
@@ -536,7 +556,7 @@ __global__ void __launch_bounds__(kSageThreads, 1) sage_kernel(SageArgs a, const
   if (warp >= kProdWarp0) {
     ok = sage_producer_warp<T, kSwizzle>(a, m, bar, warp - kProdWarp0, lane, total_tiles);
   } else if (warp >= kIdxWarp0) {
-    ok = sage_index_warp(a, tiles, m, bar, warp - kIdxWarp0, lane, total_tiles);
+    ok = sage_index_warp<T>(a, tiles, m, bar, warp - kIdxWarp0, lane, total_tiles);
   } else if (warp == kMmaWarp) {
     // MMA issuer: tile k from stage k % stages into accumulator k % 2
     if (lane == 0) {
