@@ -431,9 +431,10 @@ static agnes_status enqueue_hyperbatch(agnes_ctx* ctx, const int32_t* fanouts, i
   return AGNES_OK;
 }
 
-// Whether a kernel on `device` can read p: its own device memory or managed
-// memory.
+// Whether a kernel on `device` can read int32 values at p: its own device memory
+// or managed memory, aligned to them (a copy takes any address).
 static bool device_can_read(const void* p, int device) {
+  if ((uintptr_t)p % sizeof(int32_t) != 0) return false;
   cudaPointerAttributes attr;
   if (cudaPointerGetAttributes(&attr, p) != cudaSuccess) {
     cudaGetLastError();

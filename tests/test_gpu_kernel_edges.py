@@ -68,6 +68,23 @@ def test_hyperbatch_shapes(cuda_device, H, B, block):
     g.close()
 
 
+@pytest.mark.parametrize("shift", [1, 2])
+def test_targets_at_any_device_address(cuda_device, shift):
+    """Device targets that are not aligned to their four bytes go through a copy."""
+    block = 1 << 14
+    g, og, *_ = _graph(5000, 8, 16, 9, block)
+    t = _targets(5000, 2, 70, 9)
+    raw = torch.zeros(t.numel() * 4 + 8, dtype=torch.uint8, device=cuda_device)
+    raw[shift:shift + t.numel() * 4] = t.contiguous().view(torch.uint8).flatten().to(cuda_device)
+    g.prepare(t.to(cuda_device), [3, 2], 4, 0)
+    fan = (ctypes.c_int32 * 2)(3, 2)
+    stream = torch.cuda.current_stream().cuda_stream or None
+    assert lib().agnes_prepare_hyperbatch(g._ctx, raw.data_ptr() + shift, 2, 70, fan, 2, 5, 0,
+                                          stream) == 0
+    compare(g, og, t.numpy(), [3, 2], 5, 0, block, block)
+    g.close()
+
+
 @pytest.mark.parametrize("H,B,kind", [(1, 16, "dup"), (2, 100, "range"), (4, 64, "dup"),
                                       (1, 300, "dup"), (3, 200, "range"), (1, 5000, "dup")])
 def test_bad_targets_leave_no_counts_behind(cuda_device, H, B, kind):
