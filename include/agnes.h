@@ -210,8 +210,8 @@ agnes_status agnes_set_frontier_mode(agnes_ctx* ctx, int32_t mode);
 
 /* How agnes_prepare_hyperbatch issues its work when features and topology
  * are resident in HBM (set per ctx; takes effect at the next prepare).
- * AGNES_LAUNCH_DIRECT: every call launches the sequence (memsets, ~60
- *   kernels, the size read-back) on the caller's stream.
+ * AGNES_LAUNCH_DIRECT: every call launches the sequence (33 kernels at three
+ *   hops, the size read-back) on the caller's stream.
  * AGNES_LAUNCH_GRAPH: the sequence is captured into a CUDA graph on a
  *   private stream the first time a hyperbatch shape is seen (H, B, fanouts,
  *   frontier mode, profiling) and replayed as one graph launch on the
