@@ -430,8 +430,11 @@ agnes_status agnes_phase_times(agnes_ctx* ctx, int32_t ago, float* ms, int32_t n
  * tensor cores (tcgen05).  d_in is a multiple of 8, d_out a multiple of 32
  * in [32, 256], and W plus one 128-row tile of [x_i | mean_i] must fit
  * shared memory: 512*d_in + 4*d_in*d_out + 128 <= AGNES_SAGE_MAX_SMEM bytes
- * (ERANGE otherwise).  x, w and out are 16-byte aligned.  Waits for the hyperbatch
- * like agnes_fetch_hyperbatch, runs on cuda_stream and waits for it.
+ * (ERANGE otherwise).  x, w and out are 16-byte aligned.  out may share memory
+ * with x (a layer in place) or another input: the result is the same, formed in
+ * memory of the ctx's own (H * the largest |dst_h| rows) and copied from there.
+ * Waits for the hyperbatch like agnes_fetch_hyperbatch, runs on cuda_stream and
+ * waits for it.
  * Errors: EINVAL, ERANGE, ESTATE, ECUDA, ETIMEOUT (a tensor-core completion
  * wait ran out; the layer's output is then undefined). */
 #define AGNES_SAGE_MAX_SMEM 232448

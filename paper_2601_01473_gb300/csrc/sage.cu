@@ -670,6 +670,22 @@ __global__ void __launch_bounds__(kSageThreads, 1) sage_kernel(SageArgs a, const
   }
 }
 
+// The rows of every tile from a.out, where the layer put them, to where they
+// belong: a tile's rows are one contiguous run of row_vecs 16-byte vectors each in
+// both.
+__global__ void __launch_bounds__(256)
+sage_place_kernel(SageArgs a, const __grid_constant__ SageTiles tiles, int32_t row_vecs,
+                  uint4* __restrict__ out, int64_t out_stride) {
+  const uint4* from = (const uint4*)a.out;
+  for (int tile = blockIdx.x; tile < a.total_tiles; tile += gridDim.x) {
+    const SageTile t = sage_tile(a, tiles, tile);
+    const int32_t n = min(a.tile_rows, t.rows) * row_vecs;
+    const uint4* src = from + ((size_t)t.j * a.out_stride + t.i0) * row_vecs;
+    uint4* dst = out + ((size_t)t.j * out_stride + t.i0) * row_vecs;
+    for (int32_t q = threadIdx.x; q < n; q += blockDim.x) dst[q] = src[q];
+  }
+}
+
 // Shared memory of the kernel with `stages` A stages and index slots of
 // idx_cap neighbour positions.
 size_t sage_smem_bytes(int64_t d_in, int64_t d_out, int stages, int32_t idx_cap) {
@@ -692,6 +708,11 @@ bool is_device_ptr(const void* p) {
     return false;
   }
   return attr.type == cudaMemoryTypeDevice || attr.type == cudaMemoryTypeManaged;
+}
+
+// Whether [a, a + na) and [b, b + nb) share a byte (a null range has none).
+bool ranges_overlap(const void* a, size_t na, const void* b, size_t nb) {
+  return a && b && (uintptr_t)a < (uintptr_t)b + nb && (uintptr_t)b < (uintptr_t)a + na;
 }
 
 template <typename T, typename OutT, bool kSwizzle>
@@ -846,8 +867,26 @@ extern "C" agnes_status agnes_sage_mean_layer(agnes_ctx* ctx, int32_t hop, const
     return AGNES_EINVAL;
   }
   cudaStream_t st = (cudaStream_t)cuda_stream;
-  void* scratch = nullptr;  // the tables on the device
-  if (!inline_tiles) e = ctx_scratch(ctx, tab_bytes, &scratch);
+  // Tiles are stored while other CTAs still read the inputs, so an output that
+  // shares memory with any of them (a layer in place) is formed in scratch and
+  // placed once the kernel has read everything.
+  const size_t x_row = (size_t)d_in * (x_dtype == AGNES_F32 ? 4 : 2);
+  const size_t out_row = (size_t)d_out * (out_dtype == AGNES_F32 ? 4 : 2);
+  const size_t out_span = ((size_t)(H - 1) * out_stride_rows + max_dst) * out_row;
+  auto out_meets = [&](const void* p, size_t bytes) {
+    return ranges_overlap(out, out_span, p, bytes);
+  };
+  const bool staged =
+      out_meets(x, ((size_t)(H - 1) * x_stride_rows + max_src) * x_row) ||
+      out_meets(w, (size_t)d_out * 2 * d_in * sizeof(__half)) ||
+      out_meets(bias, (size_t)d_out * sizeof(float)) ||
+      out_meets(v.indptr[hop], (size_t)H * v.indptr_stride[hop] * sizeof(int64_t)) ||
+      out_meets(v.col[hop], (size_t)H * v.col_stride[hop] * sizeof(int32_t));
+  // the tables on the device, then the staged rows
+  const size_t tab_room = (tab_bytes + 255) & ~(size_t)255;
+  const size_t scratch_bytes = tab_room + (staged ? (size_t)H * max_dst * out_row : 0);
+  void* scratch = nullptr;
+  if (scratch_bytes > 0) e = ctx_scratch(ctx, scratch_bytes, &scratch);
   int32_t* d_tabs = (int32_t*)scratch;
   int32_t* d_err = nullptr;
   if (e == cudaSuccess) e = cudaHostGetDevicePointer((void**)&d_err, h_err, 0);
@@ -873,8 +912,8 @@ extern "C" agnes_status agnes_sage_mean_layer(agnes_ctx* ctx, int32_t hop, const
     a.inv_chunks = ((1ull << 32) + d_in / 8 - 1) / (d_in / 8);
     a.w = (const __half*)w;
     a.bias = bias;
-    a.out = out;
-    a.out_stride = out_stride_rows;
+    a.out = staged ? (char*)scratch + tab_room : out;
+    a.out_stride = staged ? max_dst : out_stride_rows;
     a.stages = stages;
     a.idx_cap = idx_cap;
     a.err = d_err;
@@ -884,6 +923,11 @@ extern "C" agnes_status agnes_sage_mean_layer(agnes_ctx* ctx, int32_t hop, const
     else
       e = out_dtype == AGNES_F32 ? launch_sage<float, float>(a, inl, g.num_sms, st)
                                  : launch_sage<float, __half>(a, inl, g.num_sms, st);
+    if (e == cudaSuccess && staged) {
+      sage_place_kernel<<<fitted_grid((const void*)sage_place_kernel, 256, g.num_sms, tiles), 256,
+                          0, st>>>(a, inl, (int32_t)(out_row / 16), (uint4*)out, out_stride_rows);
+      e = cudaGetLastError();
+    }
   }
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) {

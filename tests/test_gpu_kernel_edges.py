@@ -188,6 +188,40 @@ def test_sage_layer_output_16_byte_aligned(cuda_device):
     assert np.isfinite(ref.float().cpu().numpy()).all()
 
 
+@pytest.mark.parametrize("H,B,shift,out_dtype", [
+    (4, 2000, 0, torch.float16),    # out == x
+    (4, 2000, 3, torch.float16),    # three rows past x
+    (4, 2000, -5, torch.float16),   # five rows before it
+    (4, 2000, 0, torch.float32),    # wider rows over the same memory
+    (300, 20, 0, torch.float16),    # tiles in tables on the device
+])
+def test_sage_layer_in_place(cuda_device, H, B, shift, out_dtype):
+    """An output that shares memory with x holds what a separate one gets, and
+    rows past a minibatch's |dst_0| are not written."""
+    d = 64
+    g, *_ = _graph(20_000, 16, d, 9, 1 << 14)
+    g.prepare(_targets(20_000, H, B, 1).to(cuda_device), [6], 1, 0)
+    v = g.fetch_all()
+    w, b = _weights(d, d, 1, cuda_device)
+    ref = g.sage_mean_layer(0, v.feats, w, b, out_dtype=out_dtype)
+    rows, size = v.feats.shape[1], ref.element_size() // 2
+    buf = torch.empty(2 * v.feats.numel() + 16 * d, dtype=torch.float16, device=cuda_device)
+    x = buf[8 * d:8 * d + v.feats.numel()].view(v.feats.shape)
+    x.copy_(v.feats)
+    before = buf.clone()
+    first = (8 + shift) * d  # out's first element of buf
+    rc = lib().agnes_sage_mean_layer(g._ctx, 0, x.data_ptr(), 1, rows, d, w.data_ptr(),
+                                     b.data_ptr(), d, buf[first:].data_ptr(), int(out_dtype == torch.float16), rows,
+                                     ctypes.c_void_p(None))
+    assert rc == 0
+    want = before
+    for j in range(H):
+        at = first + j * rows * d * size
+        want[at:at + B * d * size] = ref[j, :B].view(torch.float16).flatten()
+    assert torch.equal(buf.view(torch.int16), want.view(torch.int16))
+    g.close()
+
+
 @pytest.mark.parametrize("dtype,fan", [(torch.float16, 45), (torch.float32, 45),
                                        (torch.float16, 3)])
 def test_sage_mean_is_the_rounded_quotient(cuda_device, dtype, fan):
