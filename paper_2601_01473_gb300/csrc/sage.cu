@@ -23,8 +23,8 @@
 //                   K = 16 each) into one of two TMEM accumulators;
 //   epilogue warps  read the accumulator back with tcgen05.ld, add the bias,
 //                   apply ReLU and store.  They load W into shared memory first.
-// All stages overlap.  Every mbarrier wait is bounded; on timeout the kernel
-// records an error, frees its tensor memory and returns.
+// All stages overlap.  Every mbarrier wait is bounded (a second, mbarrier.cuh); on
+// timeout the kernel records an error, frees its tensor memory and returns.
 //
 // Bound by the neighbour rows' loads and the instructions that sum them (61% of
 // the issue slots, the tensor pipe nearly idle), so most warps are producers.
@@ -44,13 +44,13 @@
 #include "../../include/agnes.h"
 #include "common.cuh"
 #include "internal.h"
+#include "mbarrier.cuh"
 
 namespace agnes {
 
 namespace {
 
 constexpr int kM = 128;              // dst rows per tile at most (the MMA's M)
-constexpr int kWaitIters = 1 << 24;  // mbarrier polls before giving up (~1 s)
 // warps: 0-3 epilogue, 4 MMA, then the index warps, then the producers
 constexpr int kMmaWarp = 4;
 constexpr int kIdxWarps = 2;
@@ -132,33 +132,6 @@ __device__ __forceinline__ void mma_commit(uint32_t bar) {
   asm volatile(
       "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar)
       : "memory");
-}
-
-__device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
-}
-
-__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
-}
-
-// Waits for the phase with the given parity to complete; false after
-// kWaitIters tries.  try_wait suspends the thread for a while in hardware, so
-// waiting warps leave the shared-memory pipe to the others.
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
-  for (int it = 0; it < kWaitIters; ++it) {
-    uint32_t done;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(done)
-        : "r"(bar), "r"(parity)
-        : "memory");
-    if (done) return true;
-    if (it >= 64) __nanosleep(64);
-  }
-  return false;
 }
 
 // 8 consecutive features of a row as raw 16-byte vectors (one for fp16, two
