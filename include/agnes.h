@@ -298,9 +298,10 @@ agnes_status agnes_fetch_hyperbatch(agnes_ctx* ctx, agnes_hyperbatch_view* out);
  * device memory of one) and d sets of internal streams, and consecutive
  * prepares use the sets in turn, each on its own internal stream that starts
  * when the caller's stream reaches the call and once the set's previous
- * hyperbatch (d prepares earlier) is done; the caller's stream is not made to
- * wait for the hyperbatch, so consecutive hyperbatches overlap (Sec. 3.4 (4):
- * one stage's latency hidden behind another's work).  Then: fetch, stats and
+ * hyperbatch (d prepares earlier) is done; the caller's stream waits (on the
+ * device) until the call's targets have been read, and so for that previous
+ * hyperbatch, but not for this one, so consecutive hyperbatches overlap
+ * (Sec. 3.4 (4): one stage's latency hidden behind another's work).  Then: fetch, stats and
  * counters wait for and describe the last prepared hyperbatch (host side, as
  * before); a stream that consumes the views on the device must first be
  * ordered with agnes_wait_hyperbatches; views stay valid until the d-th

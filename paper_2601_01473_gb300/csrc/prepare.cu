@@ -264,9 +264,10 @@ agnes_status make_spare_state(agnes_ctx* ctx, int32_t depth) {
   const unsigned f = cudaEventDisableTiming;
   if ((!ctx->pipe_st && cudaStreamCreateWithFlags(&ctx->pipe_st, cudaStreamNonBlocking) !=
                             cudaSuccess) ||
-      (!ctx->pipe_in && cudaEventCreateWithFlags(&ctx->pipe_in, f) != cudaSuccess)) {
+      (!ctx->pipe_in && cudaEventCreateWithFlags(&ctx->pipe_in, f) != cudaSuccess) ||
+      (!ctx->pipe_read && cudaEventCreateWithFlags(&ctx->pipe_read, f) != cudaSuccess)) {
     cudaGetLastError();
-    set_err(ctx, "creating the pipeline's stream or event failed");
+    set_err(ctx, "creating the pipeline's stream or events failed");
     return AGNES_ECUDA;
   }
   return AGNES_OK;
@@ -690,6 +691,12 @@ agnes_status agnes_prepare_hyperbatch(agnes_ctx* ctx, const int32_t* targets, in
   begin_kernel<<<fitted_grid((const void*)begin_kernel, 256, ctx->num_sms, (most + 255) / 256), 256,
                  0, st>>>(b);
   CK(ctx, cudaGetLastError());
+  if (pipelined) {
+    // the targets have been read by then: what the caller's stream does next
+    // may overwrite or free them
+    CK(ctx, cudaEventRecord(ctx->pipe_read, st));
+    CK(ctx, cudaStreamWaitEvent((cudaStream_t)cuda_stream, ctx->pipe_read, 0));
+  }
   int n_marks = 0;
   if (resident && ctx->lg.mode != AGNES_LAUNCH_DIRECT && !capturing)
     rc = launch_graphed(ctx, fanouts, K, cap, ring, st, &n_marks);

@@ -191,6 +191,37 @@ def test_pipeline_depth_matches_oracle_and_overlaps_safely(cuda_device, depth):
     g.close()
 
 
+@pytest.mark.parametrize("depth", [2, 3])
+def test_pipelined_targets_may_be_overwritten_after_the_call(cuda_device, depth):
+    """The caller's stream overwrites a prepare's targets right behind the
+    call, while the set they go to still runs an earlier hyperbatch: what was
+    there at the call is what is sampled."""
+    N, H, B, fan = 200_000, 64, 1024, [12, 6]
+    off, ind, feats = make(N, 20, seed=57, dim=64)
+    og = oracle.Graph(off.numpy(), ind.numpy(), feats.numpy())
+    g = load(off, ind, feats, ADJ, FEAT)
+    g.set_pipeline_depth(depth)
+    gen = torch.Generator().manual_seed(5)
+    tgts = [torch.stack([torch.randperm(N, generator=gen)[:B] for _ in range(H)]).to(torch.int32)
+            for _ in range(2)]
+    dev = [t.to(cuda_device) for t in tgts]
+    st = torch.cuda.Stream(cuda_device)
+    st.wait_stream(torch.cuda.current_stream())
+    buf = torch.empty_like(dev[0])
+    with torch.cuda.stream(st):
+        for s in range(2 * depth + 1):  # every set is in use when the last call comes
+            buf.copy_(dev[s % 2])
+            g.prepare(buf, fan, 7, 100 * s, st)
+        buf.copy_(dev[(s + 1) % 2])
+        for ago in range(depth):
+            v, a = g.fetch_earlier(ago), s - ago
+            for j in (0, H - 1):
+                r = oracle.sample_minibatch(og, tgts[a % 2][j].numpy(), fan, 7, 100 * a + j)
+                n = int(v.node_size[2, j])
+                assert np.array_equal(v.nodes[j, :n].cpu().numpy(), r["nodes"])
+    g.close()
+
+
 def test_pipeline_depth_two_needs_a_resident_graph(cuda_device):
     off, ind, feats = make(3000, 6, seed=52)
     dev = torch.device("cuda:0")
