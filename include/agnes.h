@@ -167,7 +167,8 @@ agnes_status agnes_load_graph(const agnes_graph_desc* desc, int device, void* cu
  * B targets each (Algorithm 1).
  *  targets   H*B int32 node ids, row j = minibatch j's targets (distinct
  *            within a row); host or device memory.  Host memory is copied
- *            inside the call (pinned memory makes that copy asynchronous).
+ *            inside the call (pinned memory makes that copy asynchronous:
+ *            it keeps its values until cuda_stream has come past the call).
  *  fanouts   K host int32 values, fanouts[0] for the targets' hop;
  *            1 <= fanouts[h] <= AGNES_MAX_FANOUT, 1 <= K <= AGNES_MAX_HOPS.
  *            A hop with a fanout above 1024 also uses ctx-owned device

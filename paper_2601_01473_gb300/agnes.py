@@ -7,6 +7,7 @@ shared library is missing or a call fails, an exception is raised.
 """
 from __future__ import annotations
 
+import collections
 import ctypes
 import os
 from dataclasses import dataclass
@@ -308,6 +309,7 @@ class Graph:
         self._ctx = ctx
         self._H = 0
         self._K = 0
+        self._held = collections.deque()  # (event, host targets whose copy it follows)
 
     # -- lifetime --------------------------------------------------------------
     def close(self):
@@ -329,17 +331,38 @@ class Graph:
 
     # -- calls -------------------------------------------------------------------
     def prepare(self, targets, fanouts, seed: int, first_minibatch_id: int = 0, stream=None):
-        """Enqueues one hyperbatch.  targets: [H, B] int32 (CUDA or CPU tensor)."""
+        """Enqueues one hyperbatch.  targets: [H, B] int32 (CUDA or CPU tensor),
+        read in stream order: a CPU tensor in pinned memory must keep its
+        values until the stream has come past the call."""
         if targets.dtype != torch.int32 or targets.dim() != 2 or not targets.is_contiguous():
             raise TypeError("targets must be a contiguous [H, B] int32 tensor")
         fan = (ctypes.c_int32 * len(fanouts))(*fanouts)
         H, B = targets.shape
-        self._targets = targets  # keep alive until the copy has run
+        self._targets = targets
         rc = lib().agnes_prepare_hyperbatch(self._ctx, targets.data_ptr(), H, B, fan, len(fanouts),
                                             seed & (2**64 - 1), first_minibatch_id,
                                             _stream_handle(stream, self.device))
+        if not targets.is_cuda:
+            self._hold_until_copied(targets, stream)
         _check(rc, self._ctx)
         self._H, self._K = H, len(fanouts)
+
+    def _hold_until_copied(self, targets, stream):
+        """Keeps host targets alive until their copy, which anything later on
+        the caller's stream follows, has run: the host may reuse their memory
+        at once.  (In a capture nothing has run yet: the caller keeps them.)"""
+        while self._held and self._held[0][0].query():
+            self._held.popleft()
+        if stream is None:
+            stream = torch.cuda.current_stream(self.device)
+        elif not isinstance(stream, torch.cuda.Stream):
+            stream = torch.cuda.ExternalStream(int(stream), self.device)
+        with torch.cuda.stream(stream):
+            if torch.cuda.is_current_stream_capturing():
+                return
+            event = torch.cuda.Event()
+            event.record()
+        self._held.append((event, targets))
 
     def fetch(self, j: int) -> MinibatchView:
         v = _View()

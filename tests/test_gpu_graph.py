@@ -222,6 +222,33 @@ def test_pipelined_targets_may_be_overwritten_after_the_call(cuda_device, depth)
     g.close()
 
 
+@pytest.mark.parametrize("depth", [1, 2])
+def test_host_targets_live_until_they_are_copied(cuda_device, depth):
+    """Pinned targets that the program drops right after the call are not
+    given back while their copy is still to come, and are once it has run."""
+    off, ind, feats = make(30000, 12, seed=51, dim=32)
+    og = oracle.Graph(off.numpy(), ind.numpy(), feats.numpy())
+    g = load(off, ind, feats, ADJ, FEAT)
+    g.set_pipeline_depth(depth)
+    pool = torch.arange(30000, dtype=torch.int32)
+    tgts = [synth.hyperbatch_targets(pool, 6, 200, 53, s) for s in range(3)]
+    for _ in range(depth):  # every set has its workspace
+        g.prepare(tgts[0], [4, 3], 7, 0)
+    torch.cuda.synchronize()
+    torch.cuda._sleep(50_000_000)  # some 25 ms of the caller's stream
+    pinned = [t.pin_memory() for t in tgts[1:]]
+    ptr = {p.data_ptr() for p in pinned}
+    for s in (1, 2):
+        g.prepare(pinned.pop(0), [4, 3], 7, 100 * s)
+    others = [torch.full_like(t, -1).pin_memory() for t in tgts]
+    assert not ptr & {o.data_ptr() for o in others}
+    compare(g, og, tgts[2].numpy(), [4, 3], 7, 200, ADJ, FEAT)
+    torch.cuda.synchronize()
+    g.prepare(tgts[0], [4, 3], 7, 0)
+    assert len(g._held) == 1
+    g.close()
+
+
 def test_pipeline_depth_two_needs_a_resident_graph(cuda_device):
     off, ind, feats = make(3000, 6, seed=52)
     dev = torch.device("cuda:0")
