@@ -15,6 +15,7 @@
 // the scatter and the compaction with the fix-up; the cells are resolved in
 // dedup_cells.cu.
 #include "common.cuh"
+#include "compact_index.h"
 #include "internal.h"
 
 namespace agnes {
@@ -62,11 +63,7 @@ dedup_scatter_kernel(const int32_t* __restrict__ nbr, const int32_t* __restrict_
   }
 }
 
-constexpr int kCellThreads = 128;  // threads per CTA of the compaction
-constexpr int kCompactIlp = 2;     // bucket entries per thread and round of the compaction (4 and 8 measured slower)
-constexpr int kCompactOversplit = 2;    // the compaction's (group, slice) items per resident CTA
-constexpr int kCompactMaxSlices = 256;
-constexpr int kCompactRound = kCompactIlp * kCellThreads;
+constexpr int kCompactOversplit = 2;  // the compaction's (group, slice) items per resident CTA
 constexpr int kGroupCells = kCellThreads;
 
 // ---- compaction and fix-up (after the scans) --------------------------------------
@@ -142,7 +139,8 @@ __global__ void __launch_bounds__(kCellThreads) dedup_compact_kernel(CompactArgs
   grid_dep_wait();
   if (failed(a.status)) return;
   __shared__ int32_t s_nfo[kGroupCells + 1];
-  __shared__ int32_t s_src[kGroupCells];   // source base in fb (>= 0) or ~base in tmp
+  __shared__ uint32_t s_src[kGroupCells];  // the cell's first entry in fb or in tmp
+  __shared__ bool s_tmp[kGroupCells];      // which of the two
   __shared__ int32_t s_row[kGroupCells];   // j * capK + |dst_h| + newbase
   const int tid = threadIdx.x;
   const int64_t ngroups = (a.ncells + kGroupCells - 1) / kGroupCells;
@@ -159,37 +157,40 @@ __global__ void __launch_bounds__(kCellThreads) dedup_compact_kernel(CompactArgs
       const int32_t sn = a.soff[cell + 1] - so;
       const int32_t j = (int32_t)((uint32_t)cell % (uint32_t)a.H);
       s_nfo[tid] = a.nfcell_off[cell];
-      s_src[tid] = sn == 0 && !a.sampled ? fo : ~(fo + so);
+      const bool from_tmp = sn > 0 || a.sampled;
+      s_tmp[tid] = from_tmp;
+      s_src[tid] = from_tmp ? tmp_base(fo, so) : (uint32_t)fo;
       s_row[tid] = (int32_t)((int64_t)j * a.capK +
                              (a.sampled ? a.noutbase[cell] : a.nsz_prev[j] + a.newbase[cell]));
     }
     if (tid == 0) s_nfo[last - c0] = a.nfcell_off[last];
     __syncthreads();
-    const int32_t k0 = s_nfo[0], k1 = s_nfo[last - c0];
+    const int32_t k0 = s_nfo[0];
+    const uint32_t k1 = (uint32_t)s_nfo[last - c0];
     // kCompactIlp entries per thread and round: their loads in flight before the stores
-    for (int32_t kb = k0 + slice * kCompactRound + tid; kb < k1; kb += a.slices * kCompactRound) {
+    for (uint32_t kb = compact_first(k0, slice, tid); kb < k1; kb = compact_next(kb, a.slices)) {
       int32_t cl[kCompactIlp], r[kCompactIlp], id[kCompactIlp], pos[kCompactIlp];
       bool in[kCompactIlp];
 #pragma unroll
       for (int u = 0; u < kCompactIlp; ++u) {
-        const int32_t k = kb + u * kCellThreads;
+        const uint32_t k = kb + u * kCellThreads;
         in[u] = k < k1;
         int32_t lo = 0, hi = (int32_t)(last - c0);  // last cell with nfo <= k
         while (hi - lo > 1) {
           const int32_t mid = (lo + hi) >> 1;
-          if (s_nfo[mid] <= k) lo = mid; else hi = mid;
+          if ((uint32_t)s_nfo[mid] <= k) lo = mid; else hi = mid;
         }
         cl[u] = lo;
-        r[u] = k - s_nfo[lo];
+        r[u] = (int32_t)(k - (uint32_t)s_nfo[lo]);
         id[u] = 0;
         pos[u] = 0;
         if (in[u]) {
-          const int32_t src = s_src[lo];
-          if (src >= 0) {
-            id[u] = a.fb_id[src + r[u]];
-            pos[u] = a.fb_pos[src + r[u]];
+          const uint32_t src = s_src[lo] + (uint32_t)r[u];
+          if (!s_tmp[lo]) {
+            id[u] = a.fb_id[src];
+            pos[u] = a.fb_pos[src];
           } else {
-            const int2 e = a.tmp[~src + r[u]];
+            const int2 e = a.tmp[src];
             id[u] = e.x;
             pos[u] = e.y;
           }
@@ -198,8 +199,8 @@ __global__ void __launch_bounds__(kCellThreads) dedup_compact_kernel(CompactArgs
 #pragma unroll
       for (int u = 0; u < kCompactIlp; ++u) {
         if (!in[u]) continue;
-        const int32_t k = kb + u * kCellThreads;
-        if (s_src[cl[u]] < 0) {
+        const uint32_t k = kb + u * kCellThreads;
+        if (s_tmp[cl[u]]) {
           if (a.sampled) {
             pos[u] = s_row[cl[u]] + r[u];
             a.nodes[pos[u]] = id[u];
