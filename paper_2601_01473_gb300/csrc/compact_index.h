@@ -4,7 +4,9 @@
 //
 // A hyperbatch may have up to 2^31 - 1 frontier entries and as many sampled
 // ones, so a place in tmp (frontier and sampled entries before it) and the
-// first entry of a CTA's next round can pass 2^31: both are unsigned.
+// first entry of a CTA's next round can pass 2^31: the one is kept in 64 bits,
+// where its complement can mark it as one in tmp (a 32-bit place and a flag of its
+// own cost 1 x 1024 targets on 10M nodes 219 -> 224 us), the other is unsigned.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -19,8 +21,8 @@ constexpr int kCompactRound = kCompactIlp * kCellThreads;
 
 // Where a cell's next-frontier entries start in tmp: behind its `fo` frontier
 // and `so` sampled predecessors.
-__host__ __device__ inline uint32_t tmp_base(int32_t fo, int32_t so) {
-  return (uint32_t)fo + (uint32_t)so;
+__host__ __device__ inline int64_t tmp_base(int32_t fo, int32_t so) {
+  return (int64_t)fo + so;
 }
 
 // A thread's first entry of a group that starts at k0, and of its next round.

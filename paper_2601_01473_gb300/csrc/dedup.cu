@@ -139,8 +139,7 @@ __global__ void __launch_bounds__(kCellThreads) dedup_compact_kernel(CompactArgs
   grid_dep_wait();
   if (failed(a.status)) return;
   __shared__ int32_t s_nfo[kGroupCells + 1];
-  __shared__ uint32_t s_src[kGroupCells];  // the cell's first entry in fb or in tmp
-  __shared__ bool s_tmp[kGroupCells];      // which of the two
+  __shared__ int64_t s_src[kGroupCells];   // the cell's first entry in fb, or ~ that in tmp
   __shared__ int32_t s_row[kGroupCells];   // j * capK + |dst_h| + newbase
   const int tid = threadIdx.x;
   const int64_t ngroups = (a.ncells + kGroupCells - 1) / kGroupCells;
@@ -157,9 +156,7 @@ __global__ void __launch_bounds__(kCellThreads) dedup_compact_kernel(CompactArgs
       const int32_t sn = a.soff[cell + 1] - so;
       const int32_t j = (int32_t)((uint32_t)cell % (uint32_t)a.H);
       s_nfo[tid] = a.nfcell_off[cell];
-      const bool from_tmp = sn > 0 || a.sampled;
-      s_tmp[tid] = from_tmp;
-      s_src[tid] = from_tmp ? tmp_base(fo, so) : (uint32_t)fo;
+      s_src[tid] = sn == 0 && !a.sampled ? (int64_t)fo : ~tmp_base(fo, so);
       s_row[tid] = (int32_t)((int64_t)j * a.capK +
                              (a.sampled ? a.noutbase[cell] : a.nsz_prev[j] + a.newbase[cell]));
     }
@@ -185,12 +182,12 @@ __global__ void __launch_bounds__(kCellThreads) dedup_compact_kernel(CompactArgs
         id[u] = 0;
         pos[u] = 0;
         if (in[u]) {
-          const uint32_t src = s_src[lo] + (uint32_t)r[u];
-          if (!s_tmp[lo]) {
-            id[u] = a.fb_id[src];
-            pos[u] = a.fb_pos[src];
+          const int64_t src = s_src[lo];
+          if (src >= 0) {
+            id[u] = a.fb_id[src + r[u]];
+            pos[u] = a.fb_pos[src + r[u]];
           } else {
-            const int2 e = a.tmp[src];
+            const int2 e = a.tmp[~src + r[u]];
             id[u] = e.x;
             pos[u] = e.y;
           }
@@ -200,7 +197,7 @@ __global__ void __launch_bounds__(kCellThreads) dedup_compact_kernel(CompactArgs
       for (int u = 0; u < kCompactIlp; ++u) {
         if (!in[u]) continue;
         const uint32_t k = kb + u * kCellThreads;
-        if (s_tmp[cl[u]]) {
+        if (s_src[cl[u]] < 0) {
           if (a.sampled) {
             pos[u] = s_row[cl[u]] + r[u];
             a.nodes[pos[u]] = id[u];
