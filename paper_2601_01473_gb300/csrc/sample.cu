@@ -78,40 +78,126 @@ targets_scatter_kernel(const int32_t* __restrict__ nodes, int64_t capK, int32_t 
   }
 }
 
+// A cell of up to kWalkMax targets is ordered by a thread per target, a larger
+// one by a CTA on a bitmap.
+constexpr int32_t kWalkMax = 64;
+
+// The n targets of a large cell, at o of the bucket, in id order: ranks from a
+// bitmap over the tile (base: its first id), by the whole CTA.
+__device__ __forceinline__ void place_large_cell(int32_t o, int32_t n, int32_t base,
+                                                 uint32_t* s_bits, int32_t* s_below,
+                                                 const int32_t* __restrict__ tmp_id,
+                                                 const int32_t* __restrict__ tmp_pos,
+                                                 int32_t* __restrict__ fb_id,
+                                                 int32_t* __restrict__ fb_pos, int32_t* status) {
+  const int tid = threadIdx.x;
+  constexpr int kBatch = 4;  // loads in flight per thread
+  __syncthreads();
+  if (tid < kTileWords) s_bits[tid] = 0;
+  __syncthreads();
+  for (int32_t i0 = tid; i0 < n; i0 += kBatch * kThreads) {
+    int32_t v[kBatch];
+#pragma unroll
+    for (int q = 0; q < kBatch; ++q)
+      v[q] = i0 + q * kThreads < n ? tmp_id[o + i0 + q * kThreads] - base : -1;
+#pragma unroll
+    for (int q = 0; q < kBatch; ++q) {
+      const uint32_t bit = 1u << (v[q] & 31);
+      if (v[q] >= 0 && (atomicOr(s_bits + (v[q] >> 5), bit) & bit)) atomicOr(status, kErrTargetDup);
+    }
+  }
+  __syncthreads();
+  if (tid < 32) {  // ids below each word: a lane takes four words
+    const uint4 w = reinterpret_cast<const uint4*>(s_bits)[tid];
+    const int32_t c0 = __popc(w.x), c1 = __popc(w.y), c2 = __popc(w.z);
+    const int32_t own = c0 + c1 + c2 + __popc(w.w);
+    const int32_t ex = warp_incl_scan(own) - own;
+    reinterpret_cast<int4*>(s_below)[tid] = make_int4(ex, ex + c0, ex + c0 + c1, ex + c0 + c1 + c2);
+  }
+  __syncthreads();
+  for (int32_t i0 = tid; i0 < n; i0 += kBatch * kThreads) {
+    int32_t v[kBatch], pos[kBatch];
+#pragma unroll
+    for (int q = 0; q < kBatch; ++q) {
+      const int32_t i = i0 + q * kThreads;
+      v[q] = i < n ? tmp_id[o + i] - base : -1;
+      pos[q] = i < n ? tmp_pos[o + i] : 0;
+    }
+#pragma unroll
+    for (int q = 0; q < kBatch; ++q) {
+      if (v[q] < 0) continue;
+      const int32_t w = v[q] >> 5;
+      const int32_t at = o + s_below[w] + __popc(s_bits[w] & ((1u << (v[q] & 31)) - 1u));
+      fb_id[at] = base + v[q];
+      fb_pos[at] = pos[q];
+    }
+  }
+}
+
 // Orders each cell's targets by id and flags a target repeated within a
-// minibatch: a thread per slot counts the smaller ids of its cell.  Neighbouring
-// slots share a cell, so its ids are read from L1, and the work is spread over
-// the whole grid however few cells hold the targets.  A cell with more entries
-// than a tile has ids repeats one, and is not walked.  (A warp per 32 cells,
-// sorting them one after another, took 5 us of a hyperbatch of 16 x 1024 targets
-// on 10M nodes, 623 -> 619 us.)
+// minibatch.  In a cell of up to kWalkMax targets a thread per slot counts the
+// smaller ids: neighbouring slots share a cell, so its ids are read from L1, and
+// the work is spread over the whole grid however few cells hold the targets.  (A
+// warp per 32 cells, sorting them one after another, took 5 us of a hyperbatch of
+// 16 x 1024 targets on 10M nodes, 623 -> 619 us.)  That work grows with the square
+// of a cell, so a larger cell is placed by the CTA that holds its first slot.  A
+// cell with more entries than a tile has ids repeats one, and is not placed.
+// Bucketing of 4 x 65536 consecutive targets: walked 340 us, a warp per 32 cells
+// 184, like this 29; 4 x 2M random ones on 2M nodes 9.7, 2.0 and 0.9 ms.  With a
+// limit of 32, 64, 128, 256, 512: 8 x 8192 on 100k nodes 31, 31, 33, 35, 41 us,
+// 64 x 500 consecutive ones 17, 17, 19, 21, 31, 8 x 1024 on 100k nodes 19, 17, 17,
+// 16, 17.
 __global__ void __launch_bounds__(kThreads)
 targets_place_kernel(const int32_t* __restrict__ fcell_off, int64_t total, int64_t capK, int32_t H,
                      TileMap tm, const int32_t* __restrict__ tmp_id,
                      const int32_t* __restrict__ tmp_pos, int32_t* __restrict__ fb_id,
                      int32_t* __restrict__ fb_pos, int32_t* status) {
   grid_dep_wait();
-  if (failed(status)) return;
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < total; s += stride) {
-    const int32_t v = tmp_id[s];
-    const int32_t pos = tmp_pos[s];
-    const int64_t cell = (int64_t)tile_of(tm, v) * H + (uint32_t)pos / (uint32_t)capK;
-    const int32_t o = fcell_off[cell], e = fcell_off[cell + 1];
-    if (e - o > kTileSpan) {
-      atomicOr(status, kErrTargetDup);
-      continue;
-    }
-    int32_t smaller = 0, same = 0;
+  if (cta_failed(status)) return;
+  __shared__ __align__(16) uint32_t s_bits[kTileWords];
+  __shared__ __align__(16) int32_t s_below[kTileWords];
+  __shared__ int32_t s_large;
+  __shared__ int3 s_cell[kThreads / kWalkMax + 1];  // large cells that start in the chunk
+  const int tid = threadIdx.x;
+  const int64_t stride = (int64_t)gridDim.x * kThreads;
+  for (int64_t s0 = (int64_t)blockIdx.x * kThreads; s0 < total; s0 += stride) {
+    const int64_t s = s0 + tid;
+    bool starts = false;  // the slot is the first of a large cell
+    int3 large = make_int3(0, 0, 0);
+    if (s < total) {
+      const int32_t v = tmp_id[s];
+      const int32_t pos = tmp_pos[s];
+      const int32_t t = tile_of(tm, v);
+      const int64_t cell = (int64_t)t * H + (uint32_t)pos / (uint32_t)capK;
+      const int32_t o = fcell_off[cell], e = fcell_off[cell + 1];
+      if (e - o > kTileSpan) {
+        atomicOr(status, kErrTargetDup);
+      } else if (e - o > kWalkMax) {
+        starts = s == o;
+        large = make_int3(o, e - o, __ldg(tm.tile_first + t));
+      } else {
+        int32_t smaller = 0, same = 0;
 #pragma unroll 4
-    for (int32_t q = o; q < e; ++q) {
-      const int32_t u = tmp_id[q];
-      smaller += u < v;
-      same += u == v;
+        for (int32_t q = o; q < e; ++q) {
+          const int32_t u = tmp_id[q];
+          smaller += u < v;
+          same += u == v;
+        }
+        if (same > 1) atomicOr(status, kErrTargetDup);
+        fb_id[o + smaller] = v;
+        fb_pos[o + smaller] = pos;
+      }
     }
-    if (same > 1) atomicOr(status, kErrTargetDup);
-    fb_id[o + smaller] = v;
-    fb_pos[o + smaller] = pos;
+    if (!__syncthreads_or(starts)) continue;
+    if (tid == 0) s_large = 0;
+    __syncthreads();
+    if (starts) s_cell[atomicAdd(&s_large, 1)] = large;
+    __syncthreads();
+    const int32_t n = s_large;
+    for (int32_t c = 0; c < n; ++c)
+      place_large_cell(s_cell[c].x, s_cell[c].y, s_cell[c].z, s_bits, s_below, tmp_id, tmp_pos,
+                       fb_id, fb_pos, status);
+    __syncthreads();  // the list is rewritten by the next chunk
   }
 }
 

@@ -68,6 +68,33 @@ def test_hyperbatch_shapes(cuda_device, H, B, block):
     g.close()
 
 
+@pytest.mark.parametrize("H,first,B", [
+    (5, 0, 64), (5, 0, 65),          # cells at the walk's limit and past it
+    (2, 0, 255), (2, 100, 257), (1, 0, 513),
+    (3, 4096, 4095), (2, 4096, 4096),  # all of a tile's ids but one, and all
+    (2, 4000, 9000),                 # several large cells in a minibatch
+    (70, 4090, 70),                  # cells of 6 and of 64
+])
+def test_targets_in_dense_cells(cuda_device, H, first, B):
+    """Consecutive targets in random order, so that a (tile, minibatch) cell
+    holds many; then one of them twice."""
+    N, block = 20_000, 1 << 20  # one block: the tiles are the 4096-id chunks
+    g, og, *_ = _graph(N, 6, 16, 5, block, bits=32)
+    gen = torch.Generator().manual_seed(B)
+    t = torch.stack([first + torch.randperm(B, generator=gen) for _ in range(H)]).to(torch.int32)
+    bad = t.clone()
+    bad[H - 1, B - 1] = bad[H - 1, 0]
+    for targets in (t, bad, t):
+        g.prepare(targets.to(cuda_device), [2], 4, 1)
+        if targets is bad:
+            with pytest.raises(AgnesError) as e:
+                g.fetch_all()
+            assert e.value.status == 1
+        else:
+            compare(g, og, t.numpy(), [2], 4, 1, block, block)
+    g.close()
+
+
 @pytest.mark.parametrize("shift", [1, 2])
 def test_targets_at_any_device_address(cuda_device, shift):
     """Device targets that are not aligned to their four bytes go through a copy."""
