@@ -23,6 +23,10 @@ constexpr int kThreads = 256;
 // two hyperbatches are in flight.
 constexpr int kGatherCtasPerSm = 3;
 constexpr int kU = 8;
+// Vectors from which a row has a warp of its own, and whole numbers of which take
+// the kernel for whole rows.
+constexpr int kWideRow = 176;
+constexpr int kWideWhole = 128;
 
 // LPR lanes per row, row = LPR 16-byte vectors, U rows in flight per lane.
 template <int LPR, int U>
@@ -103,6 +107,58 @@ gather_any_kernel(const uint4* __restrict__ feats, uint32_t vecs, int32_t R, uin
 #pragma unroll
       for (int u = 0; u < U; ++u)
         if (to[u] >= 0) __stcs(out + to[u], v[u]);
+    }
+  }
+}
+
+// Rows of 176 vectors and more have a warp each.  A warp's range of
+// gather_any_kernel is one such row, in rounds of 8 loads and 8 stores a lane, and
+// takes longer.  438k rows, us (any / whole / odd kernel): 144 vectors 329 / 336 /
+// 333, 176: 391 / 416 / 348, 224: 493 / 492 / 411, 255: 590 / 657 / 469, 256: 559 /
+// 502 / 536, 257: 642 / 610 / 548, 384: 825 / 745 / 802, 512: 1114 / 997 / 1073, 513:
+// 1228 / 1178 / 1069, 625: 1462 / 1608 / 1252, 1024: 2233 / 1995 / 2156.
+
+// A whole number of kWideWhole vectors: the compiler's own unrolling of one
+// vector a lane.
+__global__ void __launch_bounds__(kThreads)
+gather_whole_rows_kernel(const uint4* __restrict__ feats, int64_t vecs,
+                         const int32_t* __restrict__ fb_id, const int32_t* __restrict__ fb_pos,
+                         const int32_t* total_ptr, uint4* __restrict__ out,
+                         const int32_t* status) {
+  grid_dep_wait();
+  if (failed(status)) return;
+  const int64_t total = *total_ptr;
+  const int lane = lane_id();
+  const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  for (int64_t i = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; i < total; i += nwarps) {
+    const int64_t src = (int64_t)__ldg(fb_id + i) * vecs;
+    const int64_t dst = (int64_t)__ldg(fb_pos + i) * vecs;
+    for (int64_t c = lane; c < vecs; c += 32) __stcs(out + dst + c, __ldg(feats + src + c));
+  }
+}
+
+// Any other number: rounds of U loads a lane, the last of them in part.
+template <int U>
+__global__ void __launch_bounds__(kThreads)
+gather_odd_rows_kernel(const uint4* __restrict__ feats, int64_t vecs,
+                       const int32_t* __restrict__ fb_id, const int32_t* __restrict__ fb_pos,
+                       const int32_t* total_ptr, uint4* __restrict__ out, const int32_t* status) {
+  grid_dep_wait();
+  if (failed(status)) return;
+  const int64_t total = *total_ptr;
+  const int lane = lane_id();
+  const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  for (int64_t i = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; i < total; i += nwarps) {
+    const uint4* src = feats + (int64_t)__ldg(fb_id + i) * vecs;
+    uint4* dst = out + (int64_t)__ldg(fb_pos + i) * vecs;
+    for (int64_t c0 = lane; c0 < vecs; c0 += 32 * U) {
+      uint4 v[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        if (c0 + 32 * u < vecs) v[u] = __ldg(src + c0 + 32 * u);
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        if (c0 + 32 * u < vecs) __stcs(dst + c0 + 32 * u, v[u]);
     }
   }
 }
@@ -278,6 +334,12 @@ cudaError_t launch_gather(const void* feats, int64_t feats_bytes, int64_t row_by
   else if (vecs == 32)
     gather_vec_kernel<32, kU><<<AGNES_GRID((gather_vec_kernel<32, kU>))>>>(f, fb_id, fb_pos, total,
                                                                            o, status);
+  else if (vecs >= kWideRow && vecs % kWideWhole == 0)
+    gather_whole_rows_kernel<<<AGNES_GRID(gather_whole_rows_kernel)>>>(f, vecs, fb_id, fb_pos, total,
+                                                                       o, status);
+  else if (vecs >= kWideRow)
+    gather_odd_rows_kernel<4><<<AGNES_GRID(gather_odd_rows_kernel<4>)>>>(f, vecs, fb_id, fb_pos,
+                                                                         total, o, status);
   else
     gather_any_kernel<kU><<<AGNES_GRID(gather_any_kernel<kU>)>>>(
         f, (uint32_t)vecs, R, inverse_of(vecs), fb_id, fb_pos, total, o, status);

@@ -141,7 +141,9 @@ def test_bad_targets_leave_no_counts_behind(cuda_device, H, B, kind):
 @pytest.mark.parametrize("dtype", [torch.float16, torch.float32])
 @pytest.mark.parametrize("dim,shift", [(1, 0), (2, 0), (3, 0), (7, 1), (8, 1), (16, 0), (25, 0),
                                        (50, 0), (96, 0), (100, 0), (127, 3), (128, 0), (130, 0),
-                                       (256, 0), (301, 0), (602, 2), (1030, 0)])
+                                       (256, 0), (301, 0), (602, 2), (1030, 0),
+                                       (1024, 0), (1032, 0), (1400, 0), (1408, 0), (2040, 0),
+                                       (2048, 0), (2056, 0), (3072, 0)])
 def test_rows_of_any_width(cuda_device, dtype, dim, shift):
     """Rows of every alignment, from a matrix that starts `shift` elements past
     an aligned address: the first and last rows are read at the matrix's ends."""
