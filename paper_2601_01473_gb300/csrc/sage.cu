@@ -12,8 +12,8 @@
 //                   contiguous run of col) in a ring of shared-memory slots, so
 //                   that the chain indptr -> col -> row costs the producers one
 //                   trip per round of neighbours, not three, and ask for the
-//                   tile's rows in L2 while they are at it, so that the trip ends
-//                   there;
+//                   tile's rows in L2 while they are at it (as far as L2 holds them),
+//                   so that the trip ends there;
 //   producer warps  form the update's input A = [x_i | mean_i]: an item (row,
 //                   8-feature chunk) per thread, its neighbours' chunks summed
 //                   in fp32 with several loads in flight, rounded to fp16 into
@@ -71,6 +71,11 @@ struct IdxHead {
   int32_t ptr[kM + 4];
 };
 static_assert(sizeof(IdxHead) % 16 == 0, "the slots stay 16-byte aligned");
+// Neighbours' rows on their way to L2 (129 MB) ahead of the producers at most, by
+// the mean: 0.7 of it.  Further ahead they push one another out before they are
+// used.  786k dst rows, d_in = d_out = 128 in fp16, with / without: 73 MB ahead 344 /
+// 361 us, 146 MB 699 / 556; d_in = 64: 75 MB 310 / 300, 112 MB 443 / 388.
+constexpr double kSageAheadBytes = 91e6;
 // Every CTA asks for at least this much shared memory, so no two CTAs
 // share an SM (and its 512 tensor-memory columns).
 constexpr size_t kSageMinSmem = 120 * 1024;
@@ -244,6 +249,7 @@ struct SageArgs {
   int64_t out_stride;
   int32_t stages;             // A stages in shared memory
   int32_t idx_cap;            // neighbour positions an index slot holds
+  bool ahead;                 // neighbours' rows are asked for in L2 ahead
   int32_t* err;
 };
 
@@ -374,8 +380,10 @@ __device__ __forceinline__ bool sage_index_warp(const SageArgs& a, const SageTil
         for (int u = 0; u < 8; ++u)
           if (i + 32 * u < n) {
             cols[i + 32 * u] = v[u];
-            const char* row = x + (size_t)v[u] * row_bytes;
-            for (uint32_t b = 0; b < row_bytes; b += 128) prefetch_l2(row + b);
+            if (a.ahead) {
+              const char* row = x + (size_t)v[u] * row_bytes;
+              for (uint32_t b = 0; b < row_bytes; b += 128) prefetch_l2(row + b);
+            }
           }
       }
     }
@@ -776,6 +784,12 @@ extern "C" agnes_status agnes_sage_mean_layer(agnes_ctx* ctx, int32_t hop, const
   }
   const int H = v.H;
   const int32_t* dst_size = v.node_size + (size_t)hop * H;
+  int64_t dsts_all = 0, srcs_all = 0, edges_all = 0;
+  for (int j = 0; j < H; ++j) {
+    dsts_all += dst_size[j];
+    srcs_all += v.src_size[(size_t)hop * H + j];
+    edges_all += v.edges[(size_t)hop * H + j];
+  }
   // rows per tile: 128 (the MMA's M), halved down to 32 while that leaves SMs
   // without a tile -- a small layer is bound by the latency of its producers'
   // loads, and the MMA costs the same for fewer rows
@@ -889,6 +903,13 @@ extern "C" agnes_status agnes_sage_mean_layer(agnes_ctx* ctx, int32_t hop, const
     a.out_stride = staged ? max_dst : out_stride_rows;
     a.stages = stages;
     a.idx_cap = idx_cap;
+    // the rows ahead: the edges' of the tiles in the slots, or, where fewer, all
+    // rows of the minibatches that those tiles lie in
+    const double rows_ahead =
+        (double)(tiles < g.num_sms ? tiles : g.num_sms) * kIdxSlots * tile_rows;
+    const double edges_ahead = rows_ahead * edges_all / dsts_all;
+    const double near = (rows_ahead * H / dsts_all + 1) * srcs_all / H;
+    a.ahead = (edges_ahead < near ? edges_ahead : near) * x_row <= kSageAheadBytes;
     a.err = d_err;
     if (x_dtype == AGNES_F16)
       e = out_dtype == AGNES_F32 ? launch_sage<__half, float>(a, inl, g.num_sms, st)
