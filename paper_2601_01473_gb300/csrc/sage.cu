@@ -7,7 +7,7 @@
 //
 // One persistent, warp-specialised kernel, one CTA per SM.  The dst rows of
 // minibatch j form ceil(|dst_h| / R) tiles of R rows, R = 128 (the MMA's M) or
-// less where that gives every SM a tile.  Per tile of a CTA:
+// less where that gives every SM a tile or the rows are heavy.  Per tile of a CTA:
 //   index warps     stage the tile's indptr and neighbour positions (one
 //                   contiguous run of col) in a ring of shared-memory slots, so
 //                   that the chain indptr -> col -> row costs the producers one
@@ -27,7 +27,8 @@
 // timeout the kernel records an error, frees its tensor memory and returns.
 //
 // Bound by the neighbour rows' loads and the instructions that sum them (61% of
-// the issue slots, the tensor pipe nearly idle), so most warps are producers.
+// the issue slots, the tensor pipe nearly idle), so most warps are producers, and
+// how much L1 their loads in flight find matters as much (sage_shape).
 // Measured against a gather kernel that wrote A to memory and a GEMM that read
 // it back: 24 x 8192 rows of up to 15 neighbours, d_in = d_out = 128 in fp16,
 // 241 -> 160 us a call; 128 x 1024 targets at [15, 10, 5] on 40M nodes with
@@ -38,7 +39,7 @@
 // rows asked for in L2 ahead: the model's outermost layer (3.4M rows, 16M
 // edges) 1.15 -> 1.01 ms, 5.2 TB/s; four or five index slots, further ahead,
 // lose that again.  With this and the steps noted below the 24 x 8192 layer takes
-// 127 us and the model 4.05 ms.
+// 128 us and the model 4.03 ms.
 #include <cuda_fp16.h>
 
 #include "../../include/agnes.h"
@@ -58,7 +59,6 @@ constexpr int kIdxWarp0 = kMmaWarp + 1;
 constexpr int kProdWarp0 = kIdxWarp0 + kIdxWarps;
 constexpr int kProdWarps = 24;
 constexpr int kSageThreads = 32 * (kProdWarp0 + kProdWarps);
-constexpr int kBarBytes = 128;       // mbarriers + TMEM address slot
 // Index slots: row, validity and col facts of a tile, its indptr relative to
 // the tile's first edge, and up to idx_cap neighbour positions.
 constexpr int kIdxSlots = 3;
@@ -71,10 +71,15 @@ struct IdxHead {
   int32_t ptr[kM + 4];
 };
 static_assert(sizeof(IdxHead) % 16 == 0, "the slots stay 16-byte aligned");
+// Shared memory that leaves L1 about 60 KB, which the producers' loads in flight
+// take (24 warps, 5 x 512 bytes each): the next larger split of the SM's 256 KB
+// leaves 28.
+constexpr size_t kSageL1Smem = 195 * 1024;
 // Neighbours' rows on their way to L2 (129 MB) ahead of the producers at most, by
 // the mean: 0.7 of it.  Further ahead they push one another out before they are
 // used.  786k dst rows, d_in = d_out = 128 in fp16, with / without: 73 MB ahead 344 /
-// 361 us, 146 MB 699 / 556; d_in = 64: 75 MB 310 / 300, 112 MB 443 / 388.
+// 361 us, 146 MB 699 / 556; d_in = 64: 75 MB 310 / 300, 112 MB 443 / 388; 160 -> 192:
+// 47 MB 419 / 489, 93 MB 784 / 771.
 constexpr double kSageAheadBytes = 91e6;
 // Every CTA asks for at least this much shared memory, so no two CTAs
 // share an SM (and its 512 tensor-memory columns).
@@ -93,10 +98,10 @@ __host__ __device__ __forceinline__ uint32_t kmajor_off(int r, int k, int rows) 
 }
 
 // Byte offset of the 16-byte chunk c (elements 8 c .. 8 c + 7) of row r in a
-// K-major operand of kM rows with 128-byte swizzle: blocks of 64 elements
-// (kM rows of 128 bytes each), a row's eight chunks permuted by the row.
-__device__ __forceinline__ uint32_t swizzled_off(int r, int c) {
-  return (uint32_t)((c >> 3) * (kM * 128) + r * 128 + (((c & 7) ^ (r & 7)) << 4));
+// K-major operand of `rows` rows with 128-byte swizzle: blocks of 64 elements
+// (`rows` rows of 128 bytes each), a row's eight chunks permuted by the row.
+__device__ __forceinline__ uint32_t swizzled_off(int r, int c, int rows) {
+  return (uint32_t)((c >> 3) * (rows * 128) + r * 128 + (((c & 7) ^ (r & 7)) << 4));
 }
 
 // tcgen05 shared-memory matrix descriptor, no swizzle: start address, the
@@ -248,8 +253,8 @@ struct SageArgs {
   void* out;                  // minibatch j's dst rows at out + (j * out_stride + i) * d_out
   int64_t out_stride;
   int32_t stages;             // A stages in shared memory
-  int32_t idx_cap;            // neighbour positions an index slot holds
   bool ahead;                 // neighbours' rows are asked for in L2 ahead
+  int32_t idx_cap;            // neighbour positions an index slot holds
   int32_t* err;
 };
 
@@ -288,7 +293,10 @@ __device__ __forceinline__ SageTile sage_tile(const SageArgs& a, const SageTiles
   return r;
 }
 
-// Shared memory: W, the A stages, the index slots, the mbarriers.
+// Shared memory: the A stages, W, the index slots, the mbarriers.  The MMA reads kM
+// rows of every stage.  Where a stage has fewer, the others are whatever lies behind
+// it, the next stage or W (8 KB at most, and W has as much: d_in > 64), and fill
+// accumulator rows that nobody reads.
 struct SageSmem {
   uint8_t* w;
   uint8_t* a;
@@ -301,12 +309,13 @@ __host__ __device__ __forceinline__ uint32_t idx_slot_bytes(int32_t idx_cap) {
   return (uint32_t)sizeof(IdxHead) + 4u * (uint32_t)idx_cap;  // idx_cap: a multiple of 4
 }
 
+template <int kRows>
 __device__ __forceinline__ SageSmem sage_smem(uint8_t* smem, const SageArgs& a) {
   const uint32_t KT = 2 * a.d_in;
   SageSmem m;
-  m.w = smem;
-  m.a = m.w + (size_t)a.d_out * KT * 2;
-  m.idx = m.a + (size_t)a.stages * kM * KT * 2;
+  m.a = smem;
+  m.w = m.a + (size_t)a.stages * kRows * KT * 2;
+  m.idx = m.w + (size_t)a.d_out * KT * 2;
   m.idx_bytes = idx_slot_bytes(a.idx_cap);
   m.bars = (uint64_t*)(m.idx + (size_t)kIdxSlots * m.idx_bytes);
   return m;
@@ -332,11 +341,22 @@ struct SageBars {
 constexpr int kBars = 2 * kMaxStages + 4 + 2 * kIdxSlots + 1;
 constexpr int kBarBytesNeeded = 8 * kBars + 8;  // and the TMEM address slot
 
-// Whether use k (from 0) of a ring of n slots may start: use k - n has been
-// released.
-__device__ __forceinline__ bool ring_free(uint32_t bar, int k, int n) {
-  return k < n || mbar_wait(bar, (uint32_t)((k / n - 1) & 1));
-}
+// A walk around a ring of n slots: the slot of the current use, and its round.
+struct Ring {
+  int slot = 0, round = 0;
+  __device__ void next(int n) {
+    if (++slot == n) {
+      slot = 0;
+      ++round;
+    }
+  }
+  // the parity of the phase that this use completes
+  __device__ uint32_t parity() const { return (uint32_t)(round & 1); }
+  // Whether this use may start: the use a round earlier has been released.
+  __device__ bool free(uint32_t bar) const {
+    return round == 0 || mbar_wait(bar, parity() ^ 1u);
+  }
+};
 
 __device__ __forceinline__ void prefetch_l2(const void* p) {
   asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
@@ -348,11 +368,13 @@ __device__ __forceinline__ bool sage_index_warp(const SageArgs& a, const SageTil
                                                 const SageSmem& m,
                                                 const SageBars& bar, int w, int lane,
                                                 int total_tiles) {
+  Ring ring;
+  for (int k = 0; k < w; ++k) ring.next(kIdxSlots);
   for (int k = w;; k += kIdxWarps) {
     const int tile = (int)blockIdx.x + k * (int)gridDim.x;
     if (tile >= total_tiles) return true;
-    const int q = k % kIdxSlots;
-    if (!__all_sync(0xffffffffu, ring_free(bar.iempty(q), k, kIdxSlots))) return false;
+    const int q = ring.slot;
+    if (!__all_sync(0xffffffffu, ring.free(bar.iempty(q)))) return false;
     IdxHead* h = (IdxHead*)(m.idx + (size_t)q * m.idx_bytes);
     int32_t* cols = (int32_t*)(h + 1);
     const SageTile st = sage_tile(a, tiles, tile);
@@ -396,32 +418,32 @@ __device__ __forceinline__ bool sage_index_warp(const SageArgs& a, const SageTil
     }
     __syncwarp();
     if (lane == 0) mbar_arrive(bar.ifull(q));
+    for (int i = 0; i < kIdxWarps; ++i) ring.next(kIdxSlots);
   }
 }
 
 // A producer warp: groups of 32 items of every tile of the CTA.
-template <typename T, bool kSwizzle>
+template <typename T, bool kSwizzle, int kRows>
 __device__ __forceinline__ bool sage_producer_warp(const SageArgs& a, const SageSmem& m,
                                                    const SageBars& bar, int w, int lane,
                                                    int total_tiles) {
   constexpr int kER = sizeof(T) == 2 ? 5 : 3;  // neighbours in flight per item
   const int chunks = a.d_in / 8;
   const int groups = a.tile_rows * chunks / 32;
-  const size_t stage_bytes = (size_t)kM * 2 * a.d_in * 2;
+  const uint32_t stage_bytes = (uint32_t)(kRows * 4 * a.d_in);
   int first = w;  // the warp's first group, rotated from tile to tile so that a
                   // remainder of groups falls to every warp in turn
-  for (int k = 0;; ++k) {
-    const int tile = (int)blockIdx.x + k * (int)gridDim.x;
-    if (tile >= total_tiles) return true;
-    const int q = k % kIdxSlots, s = k % a.stages;
-    const bool ready = mbar_wait(bar.ifull(q), (uint32_t)((k / kIdxSlots) & 1)) &&
-                       ring_free(bar.empty(s), k, a.stages);
+  Ring stage, slot;
+  for (int tile = blockIdx.x; tile < total_tiles; tile += gridDim.x) {
+    const int q = slot.slot;
+    const bool ready =
+        mbar_wait(bar.ifull(q), slot.parity()) && stage.free(bar.empty(stage.slot));
     if (!__all_sync(0xffffffffu, ready)) return false;
     const IdxHead* h = (const IdxHead*)(m.idx + (size_t)q * m.idx_bytes);
     const int32_t* cl = h->staged ? (const int32_t*)(h + 1) : h->col;
     const T* x = (const T*)a.x + (size_t)h->j * a.x_stride * a.d_in;
     const int32_t i0 = h->i0, rows = h->rows;
-    uint8_t* A = m.a + (size_t)s * stage_bytes;
+    uint8_t* A = m.a + stage.slot * stage_bytes;
     for (int g = first; g < groups; g += kProdWarps) {
       // the chunks fastest: the 8 lanes of a quarter warp, which one wavefront
       // serves, read one 128-byte line of a row
@@ -467,39 +489,44 @@ __device__ __forceinline__ bool sage_producer_warp(const SageArgs& a, const Sage
         }
       }
       if constexpr (kSwizzle) {
-        *(uint4*)(A + swizzled_off(r, c)) = self;
-        *(uint4*)(A + swizzled_off(r, chunks + c)) = mean;
+        *(uint4*)(A + swizzled_off(r, c, kRows)) = self;
+        *(uint4*)(A + swizzled_off(r, chunks + c, kRows)) = mean;
       } else {
-        *(uint4*)(A + kmajor_off(r, c * 8, kM)) = self;
-        *(uint4*)(A + kmajor_off(r, a.d_in + c * 8, kM)) = mean;
+        *(uint4*)(A + kmajor_off(r, c * 8, kRows)) = self;
+        *(uint4*)(A + kmajor_off(r, a.d_in + c * 8, kRows)) = mean;
       }
     }
     first = (first + kProdWarps - groups % kProdWarps) % kProdWarps;
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     __syncwarp();
     if (lane == 0) {
-      mbar_arrive(bar.full(s));
+      mbar_arrive(bar.full(stage.slot));
       mbar_arrive(bar.iempty(q));
     }
+    stage.next(a.stages);
+    slot.next(kIdxSlots);
   }
+  return true;
 }
 
 // kSwizzle: A with 128-byte swizzle, where its rows are whole 64-element blocks
 // (d_in a multiple of 32): a quarter warp's 8 chunks of one row then go to 8
 // different bank groups.  Otherwise without swizzle, where they share one.
-template <typename T, typename OutT, bool kSwizzle>
-__global__ void __launch_bounds__(kSageThreads, 1) sage_kernel(SageArgs a, const __grid_constant__ SageTiles tiles) {
+// kRows: the rows of a stage, tile_rows or more.
+template <typename T, typename OutT, bool kSwizzle, int kRows>
+__global__ void __launch_bounds__(kSageThreads, 1)
+sage_kernel(SageArgs a, const __grid_constant__ SageTiles tiles) {
   extern __shared__ __align__(1024) uint8_t smem[];
   const int KT = 2 * a.d_in;
   const int N = a.d_out;
-  const SageSmem m = sage_smem(smem, a);
+  const SageSmem m = sage_smem<kRows>(smem, a);
   const SageBars bar{smem_u32(m.bars)};
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const uint32_t ncols = 2 * N <= 64 ? 64 : (2 * N <= 128 ? 128 : (2 * N <= 256 ? 256 : 512));
   uint32_t* tmem_slot = (uint32_t*)(m.bars + kBars);
 
   // the swizzle's atoms are 1024-byte aligned: dynamic shared memory starts on
-  // such a boundary, and W is a multiple of that long
+  // such a boundary, and a stage is a multiple of that long
   if (kSwizzle && (smem_u32(smem) & 1023u) != 0) {
     if (tid == 0) *(volatile int32_t*)a.err = kSageTimeout;
     return;
@@ -536,21 +563,22 @@ __global__ void __launch_bounds__(kSageThreads, 1) sage_kernel(SageArgs a, const
   const bool wide_out = ((uintptr_t)a.out & 31) == 0;  // rows are whole 32-byte sectors
 
   if (warp >= kProdWarp0) {
-    ok = sage_producer_warp<T, kSwizzle>(a, m, bar, warp - kProdWarp0, lane, total_tiles);
+    ok = sage_producer_warp<T, kSwizzle, kRows>(a, m, bar, warp - kProdWarp0, lane, total_tiles);
   } else if (warp >= kIdxWarp0) {
     ok = sage_index_warp<T>(a, tiles, m, bar, warp - kIdxWarp0, lane, total_tiles);
   } else if (warp == kMmaWarp) {
-    // MMA issuer: tile k from stage k % stages into accumulator k % 2
+    // MMA issuer: each tile from the next stage into the next accumulator
     if (lane == 0) {
       const uint32_t idesc = idesc_f16(kM, N);
       const uint32_t w_addr = smem_u32(m.w);
-      const uint32_t stage_bytes = (uint32_t)kM * KT * 2;
+      constexpr uint32_t kBlockBytes = kRows * 128;  // a swizzled 64-element block
+      constexpr uint32_t kColBytes = kRows * 16;     // a core-matrix column
+      const uint32_t stage_bytes = (uint32_t)(kRows * KT * 2);
       ok = mbar_wait(bar.w(), 0);
-      int k = 0;
-      for (int tile = blockIdx.x; ok && tile < total_tiles; tile += gridDim.x, ++k) {
-        const int s = k % a.stages, d = k & 1;
-        if (!mbar_wait(bar.full(s), (uint32_t)((k / a.stages) & 1)) ||
-            !ring_free(bar.dempty(d), k, 2)) {
+      Ring stage, acc;
+      for (int tile = blockIdx.x; ok && tile < total_tiles; tile += gridDim.x) {
+        const int s = stage.slot, d = acc.slot;
+        if (!mbar_wait(bar.full(s), stage.parity()) || !acc.free(bar.dempty(d))) {
           ok = false;
           break;
         }
@@ -560,16 +588,17 @@ __global__ void __launch_bounds__(kSageThreads, 1) sage_kernel(SageArgs a, const
         // K step t covers K columns [16 t, 16 t + 16): core-matrix columns 2t, 2t+1
         for (int t = 0; t < KT / 16; ++t) {
           const uint64_t da =
-              kSwizzle ? smem_desc_swizzled(a_addr + (uint32_t)(t >> 2) * (kM * 128) +
+              kSwizzle ? smem_desc_swizzled(a_addr + (uint32_t)(t >> 2) * kBlockBytes +
                                             (uint32_t)(t & 3) * 32)
-                       : smem_desc(a_addr + (uint32_t)(2 * t) * (kM / 8) * 128, (kM / 8) * 128,
-                                   128);
+                       : smem_desc(a_addr + (uint32_t)(2 * t) * kColBytes, kColBytes, 128);
           const uint64_t dw = smem_desc(w_addr + (uint32_t)(2 * t) * (uint32_t)(N / 8) * 128,
                                         (uint32_t)(N / 8) * 128, 128);
           mma_f16(dcol, da, dw, idesc, t > 0 ? 1u : 0u);
         }
         mma_commit(bar.empty(s));  // the stage is free once these MMAs have read it
         mma_commit(bar.dfull(d));  // and the accumulator is complete
+        stage.next(a.stages);
+        acc.next(2);
       }
     }
   } else {
@@ -669,18 +698,19 @@ sage_place_kernel(SageArgs a, const __grid_constant__ SageTiles tiles, int32_t r
 
 // Shared memory of the kernel with `stages` A stages and index slots of
 // idx_cap neighbour positions.
-size_t sage_smem_bytes(int64_t d_in, int64_t d_out, int stages, int32_t idx_cap) {
-  return (size_t)d_out * 2 * d_in * 2 + (size_t)stages * kM * 2 * d_in * 2 +
+size_t sage_smem_bytes(int64_t d_in, int64_t d_out, int stages, int stage_rows, int32_t idx_cap) {
+  return (size_t)d_out * 2 * d_in * 2 + (size_t)stages * stage_rows * 2 * d_in * 2 +
          (size_t)kIdxSlots * idx_slot_bytes(idx_cap) + kBarBytesNeeded;
 }
 
-// What the entry point's limit counts: W, one stage and kBarBytes.  The largest
+// What the entry point's limit counts: W, kM rows of A and 128 bytes.  The largest
 // accepted shapes (d_in a multiple of 8, d_out of 32) leave 2048 bytes of the
 // limit or more, so the heads of the index slots (kIdxSlots * sizeof(IdxHead)
-// = 1680 bytes) and the mbarriers always fit beside them.
+// = 1680 bytes) and the mbarriers with the TMEM address slot always fit beside them.
 size_t stated_smem_bytes(int64_t d_in, int64_t d_out) {
-  return (size_t)d_out * 2 * d_in * 2 + (size_t)kM * 2 * d_in * 2 + kBarBytes;
+  return (size_t)d_out * 2 * d_in * 2 + (size_t)kM * 2 * d_in * 2 + 128;
 }
+static_assert(kIdxSlots * sizeof(IdxHead) + kBarBytesNeeded <= 2048, "the largest shapes fit");
 
 bool is_device_ptr(const void* p) {
   cudaPointerAttributes attr;
@@ -696,12 +726,12 @@ bool ranges_overlap(const void* a, size_t na, const void* b, size_t nb) {
   return a && b && (uintptr_t)a < (uintptr_t)b + nb && (uintptr_t)b < (uintptr_t)a + na;
 }
 
-template <typename T, typename OutT, bool kSwizzle>
+template <typename T, typename OutT, bool kSwizzle, int kRows>
 cudaError_t launch_sage_typed(const SageArgs& a, const SageTiles& t, int num_sms,
                               cudaStream_t st) {
-  size_t smem = sage_smem_bytes(a.d_in, a.d_out, a.stages, a.idx_cap);
+  size_t smem = sage_smem_bytes(a.d_in, a.d_out, a.stages, kRows, a.idx_cap);
   if (smem < kSageMinSmem) smem = kSageMinSmem;
-  const auto kernel = sage_kernel<T, OutT, kSwizzle>;
+  const auto kernel = sage_kernel<T, OutT, kSwizzle, kRows>;
   cudaError_t e =
       cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
@@ -711,26 +741,89 @@ cudaError_t launch_sage_typed(const SageArgs& a, const SageTiles& t, int num_sms
 }
 
 template <typename T, typename OutT>
-cudaError_t launch_sage(const SageArgs& a, const SageTiles& t, int num_sms, cudaStream_t st) {
-  return a.d_in % 32 == 0 ? launch_sage_typed<T, OutT, true>(a, t, num_sms, st)
-                          : launch_sage_typed<T, OutT, false>(a, t, num_sms, st);
+cudaError_t launch_sage(const SageArgs& a, const SageTiles& t, int stage_rows, int num_sms,
+                        cudaStream_t st) {
+  const bool swizzle = a.d_in % 32 == 0;
+  const auto launch =
+      stage_rows == kM ? (swizzle ? launch_sage_typed<T, OutT, true, kM>
+                                  : launch_sage_typed<T, OutT, false, kM>)
+                       : (swizzle ? launch_sage_typed<T, OutT, true, kM / 2>
+                                  : launch_sage_typed<T, OutT, false, kM / 2>);
+  return launch(a, t, num_sms, st);
 }
 
-// A stages and index slot size: the slots hold a tile of `edges` edges where
-// there is room, and at least half of it where that leaves two stages or more.
-bool sage_shape(int64_t d_in, int64_t d_out, int64_t edges, int32_t* stages, int32_t* idx_cap) {
-  const int32_t want = (int32_t)((edges < kIdxCapMax ? edges : kIdxCapMax) + 3) & ~3;
-  for (int s = kMaxStages; s >= 1; --s) {
-    const size_t base = sage_smem_bytes(d_in, d_out, s, 0);
-    if (base > AGNES_SAGE_MAX_SMEM) continue;
-    const int32_t room =
-        (int32_t)((AGNES_SAGE_MAX_SMEM - base) / (sizeof(int32_t) * kIdxSlots)) & ~3;
-    if (s > 1 && room < want / 2) continue;
-    *stages = s;
-    *idx_cap = room < want ? room : want;
-    return true;
+// How a layer is cut into tiles and uses its shared memory.
+struct SageShape {
+  int tile_rows, stages, stage_rows;
+  int32_t idx_cap;
+};
+
+// What decides it.
+struct SageLoad {
+  int64_t d_in, d_out;
+  int64_t row_bytes;  // of x
+  double degree;      // mean edges per dst row
+  int64_t fanout;     // the most
+};
+
+// Neighbour positions for which an index slot has room beside the rest, in `bytes`
+// of shared memory (negative: the rest does not fit).
+int32_t idx_room(const SageLoad& l, const SageShape& s, size_t bytes) {
+  const size_t base = sage_smem_bytes(l.d_in, l.d_out, s.stages, s.stage_rows, 0);
+  if (base > bytes) return -1;
+  return (int32_t)((bytes - base) / (sizeof(int32_t) * kIdxSlots)) & ~3;
+}
+
+// The shape for tiles of up to tile_rows rows.
+//
+// What shared memory takes is not L1's, and the producers' loads in flight need L1,
+// so more stages, rows in a stage and staged indices pay only up to a point, and
+// that point depends on what a dst row costs the producers: the bytes of its own
+// row and its neighbours', (1 + degree) * row_bytes.
+//  - Light rows: tiles of 128, as the epilogue and the MMA cost the same for fewer.
+//  - Heavy rows: tiles of 64 in two stages of 64 rows, which take what one stage of
+//    128 does, so that they always fit.
+//  - One stage of 128 rows, where two do not fit, only for light rows: the
+//    producers wait for every tile's MMA.
+//  - Up to 64 features two stages of 128 rows are small: always those.
+// 786k dst rows of equal degree, us, tiles of 128 / 64 rows.  d_in = d_out = 128 in
+// fp16: degree 3 262 / 298, 5 343 / 345, 8 485 / 414, 20 926 / 780; 3.5M rows of
+// degree 4.75 on 40M nodes 1122 / 1260.  In fp32: degree 2 321 / 314, 3 436 / 354.
+// 128 -> 192, whose two stages leave no room to stage indices: 3 311 / 333, 5 416 /
+// 361.  128 -> 256, one stage: 1 335 / 371, 2 374 / 370, 3 424 / 392, 8 641 / 457.
+// 64 -> 64: 3 199 / 237, 20 475 / 498.
+// The same layers with up to three stages of 128 rows whatever the degree, before,
+// and with two kernels, an aggregation at full occupancy and a GEMM, before that:
+// 128 -> 128 at degree 12 882 and 835 (now 557), at 20 1337 and 1149 (781); 256 -> 64
+// at 12 1776 and 1450 (1051); fp32 128 -> 128 at 12 1598 and 1160 (903).
+SageShape sage_shape(const SageLoad& l, int32_t tile_rows) {
+  SageShape s{tile_rows, 2, kM, 0};
+  if (l.d_in > 64) {
+    const int32_t room = idx_room(l, s, AGNES_SAGE_MAX_SMEM);
+    const bool f32 = l.row_bytes > 2 * l.d_in;  // its loads take a fifth more of L1
+    const double heavy = room < 0                 ? 2.4 * l.d_out
+                         : room < kM * l.degree ? 1000
+                         : f32                  ? 1300
+                                                : 1800;
+    if ((1 + l.degree) * l.row_bytes >= heavy) {
+      s.stage_rows = kM / 2;
+      s.tile_rows = tile_rows < kM / 2 ? tile_rows : kM / 2;
+    } else if (room < 0) {
+      s.stages = 1;
+    }
   }
-  return false;
+  // The slots stage twice a tile's mean of edges.
+  const double most = 2 * l.degree + 1 < l.fanout ? 2 * l.degree + 1 : l.fanout;
+  const int32_t want =
+      (int32_t)(s.tile_rows * most < kIdxCapMax ? s.tile_rows * most + 3 : kIdxCapMax) & ~3;
+  if (s.stages == 2) {  // a third stage, as long as L1 keeps its share
+    SageShape more = s;
+    more.stages = 3;
+    if (idx_room(l, more, kSageL1Smem) >= want) s = more;
+  }
+  const int32_t room = idx_room(l, s, AGNES_SAGE_MAX_SMEM);
+  s.idx_cap = room < want ? room : want;
+  return s;
 }
 
 }  // namespace
@@ -784,12 +877,6 @@ extern "C" agnes_status agnes_sage_mean_layer(agnes_ctx* ctx, int32_t hop, const
   }
   const int H = v.H;
   const int32_t* dst_size = v.node_size + (size_t)hop * H;
-  int64_t dsts_all = 0, srcs_all = 0, edges_all = 0;
-  for (int j = 0; j < H; ++j) {
-    dsts_all += dst_size[j];
-    srcs_all += v.src_size[(size_t)hop * H + j];
-    edges_all += v.edges[(size_t)hop * H + j];
-  }
   // rows per tile: 128 (the MMA's M), halved down to 32 while that leaves SMs
   // without a tile -- a small layer is bound by the latency of its producers'
   // loads, and the MMA costs the same for fewer rows
@@ -799,18 +886,20 @@ extern "C" agnes_status agnes_sage_mean_layer(agnes_ctx* ctx, int32_t hop, const
     return n;
   };
   int32_t tile_rows = kM;
-  int64_t tiles = tiles_of(tile_rows);
-  while (tile_rows > 32 && tiles < g.num_sms) {
-    tile_rows /= 2;
-    tiles = tiles_of(tile_rows);
-  }
-  int32_t stages = 1, idx_cap = 0;
+  while (tile_rows > 32 && tiles_of(tile_rows) < g.num_sms) tile_rows /= 2;
   const int64_t fanout = v.col_stride[hop] / (v.indptr_stride[hop] - 1);
-  if (!sage_shape(d_in, d_out, tile_rows * fanout, &stages, &idx_cap)) {
-    ctx_set_error(ctx, "d_in %lld with d_out %d does not fit shared memory", (long long)d_in,
-                  d_out);
-    return AGNES_ERANGE;
+  const size_t x_row = (size_t)d_in * (x_dtype == AGNES_F32 ? 4 : 2);
+  int64_t dsts_all = 0, srcs_all = 0, edges_all = 0;
+  for (int j = 0; j < H; ++j) {
+    dsts_all += dst_size[j];
+    srcs_all += v.src_size[(size_t)hop * H + j];
+    edges_all += v.edges[(size_t)hop * H + j];
   }
+  const double degree = dsts_all > 0 ? (double)edges_all / dsts_all : 0;
+  const SageShape shape =
+      sage_shape(SageLoad{d_in, d_out, (int64_t)x_row, degree, fanout}, tile_rows);
+  tile_rows = shape.tile_rows;
+  int64_t tiles = tiles_of(tile_rows);
   int64_t max_src = 0, max_dst = 0;
   const bool inline_tiles = H <= kInlineH;
   // pinned staging: error word (16 bytes; the kernel writes it in place), then,
@@ -857,7 +946,6 @@ extern "C" agnes_status agnes_sage_mean_layer(agnes_ctx* ctx, int32_t hop, const
   // Tiles are stored while other CTAs still read the inputs, so an output that
   // shares memory with any of them (a layer in place) is formed in scratch and
   // placed once the kernel has read everything.
-  const size_t x_row = (size_t)d_in * (x_dtype == AGNES_F32 ? 4 : 2);
   const size_t out_row = (size_t)d_out * (out_dtype == AGNES_F32 ? 4 : 2);
   const size_t out_span = ((size_t)(H - 1) * out_stride_rows + max_dst) * out_row;
   auto out_meets = [&](const void* p, size_t bytes) {
@@ -901,22 +989,20 @@ extern "C" agnes_status agnes_sage_mean_layer(agnes_ctx* ctx, int32_t hop, const
     a.bias = bias;
     a.out = staged ? (char*)scratch + tab_room : out;
     a.out_stride = staged ? max_dst : out_stride_rows;
-    a.stages = stages;
-    a.idx_cap = idx_cap;
+    a.stages = shape.stages;
+    const int64_t ctas = tiles < g.num_sms ? tiles : g.num_sms;
     // the rows ahead: the edges' of the tiles in the slots, or, where fewer, all
     // rows of the minibatches that those tiles lie in
-    const double rows_ahead =
-        (double)(tiles < g.num_sms ? tiles : g.num_sms) * kIdxSlots * tile_rows;
-    const double edges_ahead = rows_ahead * edges_all / dsts_all;
+    const double rows_ahead = (double)ctas * kIdxSlots * tile_rows;
     const double near = (rows_ahead * H / dsts_all + 1) * srcs_all / H;
-    a.ahead = (edges_ahead < near ? edges_ahead : near) * x_row <= kSageAheadBytes;
+    a.ahead = (rows_ahead * degree < near ? rows_ahead * degree : near) * x_row <= kSageAheadBytes;
+    a.idx_cap = shape.idx_cap;
     a.err = d_err;
-    if (x_dtype == AGNES_F16)
-      e = out_dtype == AGNES_F32 ? launch_sage<__half, float>(a, inl, g.num_sms, st)
-                                 : launch_sage<__half, __half>(a, inl, g.num_sms, st);
-    else
-      e = out_dtype == AGNES_F32 ? launch_sage<float, float>(a, inl, g.num_sms, st)
-                                 : launch_sage<float, __half>(a, inl, g.num_sms, st);
+    const auto launch =
+        x_dtype == AGNES_F16
+            ? (out_dtype == AGNES_F32 ? launch_sage<__half, float> : launch_sage<__half, __half>)
+            : (out_dtype == AGNES_F32 ? launch_sage<float, float> : launch_sage<float, __half>);
+    e = launch(a, inl, shape.stage_rows, g.num_sms, st);
     if (e == cudaSuccess && staged) {
       sage_place_kernel<<<fitted_grid((const void*)sage_place_kernel, 256, g.num_sms, tiles), 256,
                           0, st>>>(a, inl, (int32_t)(out_row / 16), (uint4*)out, out_stride_rows);

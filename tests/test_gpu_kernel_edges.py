@@ -181,6 +181,10 @@ def test_rows_of_any_width(cuda_device, dtype, dim, shift):
     (64, 256, torch.float16, [300], 2, 60),     # more edges in a tile than are staged
     (64, 64, torch.float16, [4], 256, 3),       # the most minibatches whose tiles travel along
     (64, 64, torch.float16, [4], 257, 3),       # one more: tables on the device
+    (96, 32, torch.float16, [200], 6, 8000),    # heavy rows: tiles of 64, the smallest W behind
+    (104, 256, torch.float16, [200], 3, 5000),  # the same without swizzle
+    (128, 256, torch.float16, [1], 4, 6000),    # light rows, one stage of 128
+    (128, 256, torch.float32, [60], 6, 8000),   # heavy ones, two of 64, more tiles than stages
 ])
 def test_sage_layer_shapes(cuda_device, d_in, d_out, dtype, fan, H, B):
     N = 30_000
