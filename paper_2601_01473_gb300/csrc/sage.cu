@@ -61,9 +61,10 @@ constexpr int kProdWarps = 24;
 constexpr int kSageThreads = 32 * (kProdWarp0 + kProdWarps);
 // Index slots: row, validity and col facts of a tile, its indptr relative to
 // the tile's first edge, and up to idx_cap neighbour positions.
-constexpr int kIdxSlots = 3;
+constexpr int kIdxSlots = 3;  // of most layers, with two or three stages (sage_shape)
 constexpr int kIdxCapMax = 4096;
-constexpr int kMaxStages = 3;
+constexpr int kMaxSlots = 6;
+constexpr int kMaxStages = 6;
 struct IdxHead {
   int32_t i0, rows, j, staged;
   const int32_t* col;  // the tile's first edge's neighbour position, in global memory
@@ -253,6 +254,7 @@ struct SageArgs {
   void* out;                  // minibatch j's dst rows at out + (j * out_stride + i) * d_out
   int64_t out_stride;
   int32_t stages;             // A stages in shared memory
+  int32_t slots;              // index slots
   bool ahead;                 // neighbours' rows are asked for in L2 ahead
   int32_t idx_cap;            // neighbour positions an index slot holds
   int32_t* err;
@@ -317,7 +319,7 @@ __device__ __forceinline__ SageSmem sage_smem(uint8_t* smem, const SageArgs& a) 
   m.w = m.a + (size_t)a.stages * kRows * KT * 2;
   m.idx = m.w + (size_t)a.d_out * KT * 2;
   m.idx_bytes = idx_slot_bytes(a.idx_cap);
-  m.bars = (uint64_t*)(m.idx + (size_t)kIdxSlots * m.idx_bytes);
+  m.bars = (uint64_t*)(m.idx + (size_t)a.slots * m.idx_bytes);
   return m;
 }
 
@@ -332,13 +334,13 @@ struct SageBars {
   __device__ uint32_t dempty(int d) const { return base + 8u * (uint32_t)(2 * kMaxStages + 2 + d); }
   __device__ uint32_t ifull(int q) const { return base + 8u * (uint32_t)(2 * kMaxStages + 4 + q); }
   __device__ uint32_t iempty(int q) const {
-    return base + 8u * (uint32_t)(2 * kMaxStages + 4 + kIdxSlots + q);
+    return base + 8u * (uint32_t)(2 * kMaxStages + 4 + kMaxSlots + q);
   }
   __device__ uint32_t w() const {
-    return base + 8u * (uint32_t)(2 * kMaxStages + 4 + 2 * kIdxSlots);
+    return base + 8u * (uint32_t)(2 * kMaxStages + 4 + 2 * kMaxSlots);
   }
 };
-constexpr int kBars = 2 * kMaxStages + 4 + 2 * kIdxSlots + 1;
+constexpr int kBars = 2 * kMaxStages + 4 + 2 * kMaxSlots + 1;
 constexpr int kBarBytesNeeded = 8 * kBars + 8;  // and the TMEM address slot
 
 // A walk around a ring of n slots: the slot of the current use, and its round.
@@ -369,7 +371,7 @@ __device__ __forceinline__ bool sage_index_warp(const SageArgs& a, const SageTil
                                                 const SageBars& bar, int w, int lane,
                                                 int total_tiles) {
   Ring ring;
-  for (int k = 0; k < w; ++k) ring.next(kIdxSlots);
+  for (int k = 0; k < w; ++k) ring.next(a.slots);
   for (int k = w;; k += kIdxWarps) {
     const int tile = (int)blockIdx.x + k * (int)gridDim.x;
     if (tile >= total_tiles) return true;
@@ -388,7 +390,7 @@ __device__ __forceinline__ bool sage_index_warp(const SageArgs& a, const SageTil
     const int32_t* col = a.col + (size_t)j * a.col_stride + e0;
     const bool staged = n <= a.idx_cap;
     // the rows the tile reads -- its own, one after another, and its neighbours'
-    // -- on their way to L2, up to kIdxSlots tiles ahead of the producers
+    // -- on their way to L2, up to `slots` tiles ahead of the producers
     const uint32_t row_bytes = (uint32_t)a.d_in * (uint32_t)sizeof(T);
     const char* x = (const char*)a.x + (size_t)j * a.x_stride * row_bytes;
     for (uint32_t b = 128u * lane; b < (uint32_t)rows * row_bytes; b += 4096)
@@ -418,7 +420,7 @@ __device__ __forceinline__ bool sage_index_warp(const SageArgs& a, const SageTil
     }
     __syncwarp();
     if (lane == 0) mbar_arrive(bar.ifull(q));
-    for (int i = 0; i < kIdxWarps; ++i) ring.next(kIdxSlots);
+    for (int i = 0; i < kIdxWarps; ++i) ring.next(a.slots);
   }
 }
 
@@ -504,7 +506,7 @@ __device__ __forceinline__ bool sage_producer_warp(const SageArgs& a, const Sage
       mbar_arrive(bar.iempty(q));
     }
     stage.next(a.stages);
-    slot.next(kIdxSlots);
+    slot.next(a.slots);
   }
   return true;
 }
@@ -547,7 +549,7 @@ sage_kernel(SageArgs a, const __grid_constant__ SageTiles tiles) {
       mbar_init(bar.dfull(d), 1);
       mbar_init(bar.dempty(d), 4);  // one arrival per epilogue warp
     }
-    for (int q = 0; q < kIdxSlots; ++q) {
+    for (int q = 0; q < kMaxSlots; ++q) {
       mbar_init(bar.ifull(q), 1);
       mbar_init(bar.iempty(q), kProdWarps);
     }
@@ -698,9 +700,10 @@ sage_place_kernel(SageArgs a, const __grid_constant__ SageTiles tiles, int32_t r
 
 // Shared memory of the kernel with `stages` A stages and index slots of
 // idx_cap neighbour positions.
-size_t sage_smem_bytes(int64_t d_in, int64_t d_out, int stages, int stage_rows, int32_t idx_cap) {
+size_t sage_smem_bytes(int64_t d_in, int64_t d_out, int stages, int stage_rows, int slots,
+                       int32_t idx_cap) {
   return (size_t)d_out * 2 * d_in * 2 + (size_t)stages * stage_rows * 2 * d_in * 2 +
-         (size_t)kIdxSlots * idx_slot_bytes(idx_cap) + kBarBytesNeeded;
+         (size_t)slots * idx_slot_bytes(idx_cap) + kBarBytesNeeded;
 }
 
 // What the entry point's limit counts: W, kM rows of A and 128 bytes.  The largest
@@ -729,7 +732,7 @@ bool ranges_overlap(const void* a, size_t na, const void* b, size_t nb) {
 template <typename T, typename OutT, bool kSwizzle, int kRows>
 cudaError_t launch_sage_typed(const SageArgs& a, const SageTiles& t, int num_sms,
                               cudaStream_t st) {
-  size_t smem = sage_smem_bytes(a.d_in, a.d_out, a.stages, kRows, a.idx_cap);
+  size_t smem = sage_smem_bytes(a.d_in, a.d_out, a.stages, kRows, a.slots, a.idx_cap);
   if (smem < kSageMinSmem) smem = kSageMinSmem;
   const auto kernel = sage_kernel<T, OutT, kSwizzle, kRows>;
   cudaError_t e =
@@ -754,7 +757,7 @@ cudaError_t launch_sage(const SageArgs& a, const SageTiles& t, int stage_rows, i
 
 // How a layer is cut into tiles and uses its shared memory.
 struct SageShape {
-  int tile_rows, stages, stage_rows;
+  int tile_rows, stages, stage_rows, slots;
   int32_t idx_cap;
 };
 
@@ -769,9 +772,9 @@ struct SageLoad {
 // Neighbour positions for which an index slot has room beside the rest, in `bytes`
 // of shared memory (negative: the rest does not fit).
 int32_t idx_room(const SageLoad& l, const SageShape& s, size_t bytes) {
-  const size_t base = sage_smem_bytes(l.d_in, l.d_out, s.stages, s.stage_rows, 0);
+  const size_t base = sage_smem_bytes(l.d_in, l.d_out, s.stages, s.stage_rows, s.slots, 0);
   if (base > bytes) return -1;
-  return (int32_t)((bytes - base) / (sizeof(int32_t) * kIdxSlots)) & ~3;
+  return (int32_t)((bytes - base) / (sizeof(int32_t) * s.slots)) & ~3;
 }
 
 // The shape for tiles of up to tile_rows rows.
@@ -797,7 +800,7 @@ int32_t idx_room(const SageLoad& l, const SageShape& s, size_t bytes) {
 // 128 -> 128 at degree 12 882 and 835 (now 557), at 20 1337 and 1149 (781); 256 -> 64
 // at 12 1776 and 1450 (1051); fp32 128 -> 128 at 12 1598 and 1160 (903).
 SageShape sage_shape(const SageLoad& l, int32_t tile_rows) {
-  SageShape s{tile_rows, 2, kM, 0};
+  SageShape s{tile_rows, 2, kM, kIdxSlots, 0};
   if (l.d_in > 64) {
     const int32_t room = idx_room(l, s, AGNES_SAGE_MAX_SMEM);
     const bool f32 = l.row_bytes > 2 * l.d_in;  // its loads take a fifth more of L1
@@ -812,13 +815,24 @@ SageShape sage_shape(const SageLoad& l, int32_t tile_rows) {
       s.stages = 1;
     }
   }
-  // The slots stage twice a tile's mean of edges.
-  const double most = 2 * l.degree + 1 < l.fanout ? 2 * l.degree + 1 : l.fanout;
-  const int32_t want =
-      (int32_t)(s.tile_rows * most < kIdxCapMax ? s.tile_rows * most + 3 : kIdxCapMax) & ~3;
-  if (s.stages == 2) {  // a third stage, as long as L1 keeps its share
+  // The slots stage twice a tile's mean of edges.  Rows of up to 48 bytes are read by
+  // a thread or two an edge: staging costs the two index warps more than it saves
+  // (8 -> 32 at degree 30: 474 us staged, 235 not; two kernels 292).
+  int32_t want = 0;
+  if (l.row_bytes > 48) {
+    const double most = 2 * l.degree + 1 < l.fanout ? 2 * l.degree + 1 : l.fanout;
+    want = (int32_t)(s.tile_rows * most < kIdxCapMax ? s.tile_rows * most + 3 : kIdxCapMax) & ~3;
+  }
+  // More stages and slots as long as L1 keeps its share: six where a tile is work
+  // for a third of the producer warps, so that three tiles are in the making (8 -> 32
+  // at degree 20: 224 -> 186 us), four up to 64 features (64 -> 64 on a skewed graph,
+  // fanouts 15 and 50: 241 -> 232, 404 -> 383), else three.
+  const int rings[][2] = {{6, 6}, {4, 4}, {3, kIdxSlots}};  // stages, slots
+  const int groups = s.tile_rows * (int)l.d_in / 8 / 32;
+  for (int i = 3 * groups <= kProdWarps ? 0 : l.d_in <= 64 ? 1 : 2; s.stages == 2 && i < 3; ++i) {
     SageShape more = s;
-    more.stages = 3;
+    more.stages = rings[i][0];
+    more.slots = rings[i][1];
     if (idx_room(l, more, kSageL1Smem) >= want) s = more;
   }
   const int32_t room = idx_room(l, s, AGNES_SAGE_MAX_SMEM);
@@ -990,10 +1004,11 @@ extern "C" agnes_status agnes_sage_mean_layer(agnes_ctx* ctx, int32_t hop, const
     a.out = staged ? (char*)scratch + tab_room : out;
     a.out_stride = staged ? max_dst : out_stride_rows;
     a.stages = shape.stages;
+    a.slots = shape.slots;
     const int64_t ctas = tiles < g.num_sms ? tiles : g.num_sms;
     // the rows ahead: the edges' of the tiles in the slots, or, where fewer, all
     // rows of the minibatches that those tiles lie in
-    const double rows_ahead = (double)ctas * kIdxSlots * tile_rows;
+    const double rows_ahead = (double)ctas * shape.slots * tile_rows;
     const double near = (rows_ahead * H / dsts_all + 1) * srcs_all / H;
     a.ahead = (rows_ahead * degree < near ? rows_ahead * degree : near) * x_row <= kSageAheadBytes;
     a.idx_cap = shape.idx_cap;
