@@ -144,7 +144,6 @@ agnes_status agnes_free(agnes_ctx* ctx) {
   free_spare_state(ctx);
   if (ctx->pipe_st) cudaStreamDestroy(ctx->pipe_st);
   if (ctx->pipe_in) cudaEventDestroy(ctx->pipe_in);
-  if (ctx->pipe_read) cudaEventDestroy(ctx->pipe_read);
   free_block_tables(&ctx->bt);
   if (ctx->own_offsets) cudaFree(ctx->offsets);
   if (ctx->own_indices) cudaFree(ctx->indices);

@@ -178,7 +178,6 @@ struct agnes_ctx {
   int32_t pipe_depth = 1;
   cudaStream_t pipe_st = nullptr;  // the active set's internal stream (depth > 1)
   cudaEvent_t pipe_in = nullptr;   // orders an internal stream after the caller's
-  cudaEvent_t pipe_read = nullptr;  // orders the caller's stream after the targets' read
   struct Spare {
     agnes::Workspace ws;
     LaunchGraph lg;

@@ -264,10 +264,9 @@ agnes_status make_spare_state(agnes_ctx* ctx, int32_t depth) {
   const unsigned f = cudaEventDisableTiming;
   if ((!ctx->pipe_st && cudaStreamCreateWithFlags(&ctx->pipe_st, cudaStreamNonBlocking) !=
                             cudaSuccess) ||
-      (!ctx->pipe_in && cudaEventCreateWithFlags(&ctx->pipe_in, f) != cudaSuccess) ||
-      (!ctx->pipe_read && cudaEventCreateWithFlags(&ctx->pipe_read, f) != cudaSuccess)) {
+      (!ctx->pipe_in && cudaEventCreateWithFlags(&ctx->pipe_in, f) != cudaSuccess)) {
     cudaGetLastError();
-    set_err(ctx, "creating the pipeline's stream or events failed");
+    set_err(ctx, "creating the pipeline's stream or event failed");
     return AGNES_ECUDA;
   }
   return AGNES_OK;
@@ -641,19 +640,13 @@ agnes_status agnes_prepare_hyperbatch(agnes_ctx* ctx, const int32_t* targets, in
     set_err(ctx, "cudaSetDevice(%d) failed", ctx->device);
     return AGNES_ECUDA;
   }
-  cudaStream_t st = (cudaStream_t)cuda_stream;
-  const bool capturing = stream_capturing(st);
+  const cudaStream_t caller = (cudaStream_t)cuda_stream;
+  const bool capturing = stream_capturing(caller);
   const bool resident = !ctx->features_on_host && !ctx->topo.on;
   const bool pipelined = ctx->pipe_depth > 1 && resident && !capturing;
-  if (pipelined) {
-    // the least recently used set of per-hyperbatch state: its internal
-    // stream starts once the caller's stream reaches this call, and is
-    // already ordered after the set's previous hyperbatch
-    rotate_hyperbatch_state(ctx);
-    CK(ctx, cudaEventRecord(ctx->pipe_in, st));
-    CK(ctx, cudaStreamWaitEvent(ctx->pipe_st, ctx->pipe_in, 0));
-    st = ctx->pipe_st;
-  }
+  // the least recently used set of per-hyperbatch state
+  if (pipelined) rotate_hyperbatch_state(ctx);
+  const cudaStream_t st = pipelined ? ctx->pipe_st : caller;
   agnes_status rc = ensure_workspace(ctx, H, B, fanouts, K, cap);
   if (rc != AGNES_OK) return rc;
   Workspace& w = ctx->ws;
@@ -668,16 +661,18 @@ agnes_status agnes_prepare_hyperbatch(agnes_ctx* ctx, const int32_t* targets, in
   ctx->n_phases[ring] = 0;
   // a prepare on another stream than the last one on these buffers still runs
   // after it (a caller's own capture orders its replays itself)
-  if (ctx->n_prepared > 0 && !capturing) CK(ctx, cudaStreamWaitEvent(st, ctx->done, 0));
+  if (ctx->n_prepared > 0 && !capturing) CK(ctx, cudaStreamWaitEvent(caller, ctx->done, 0));
   if (!capturing) {
-    rc = update_topology_cache(ctx, st);
+    rc = update_topology_cache(ctx, caller);
     if (rc != AGNES_OK) return rc;
   }
+  // the targets are read on the caller's stream, whatever the hyperbatch runs on:
+  // what the stream does next may overwrite or free them
   BeginArgs b;
   b.targets = device_can_read(targets, ctx->device) ? targets : nullptr;
   if (!b.targets)
     CK(ctx, cudaMemcpy2DAsync(w.nodes, sizeof(int32_t) * w.capK, targets, sizeof(int32_t) * B,
-                              sizeof(int32_t) * B, H, cudaMemcpyDefault, st));
+                              sizeof(int32_t) * B, H, cudaMemcpyDefault, caller));
   b.nodes = w.nodes;
   b.capK = w.capK;
   b.H = H;
@@ -689,13 +684,11 @@ agnes_status agnes_prepare_hyperbatch(agnes_ctx* ctx, const int32_t* targets, in
   b.back_words = (int64_t)(w.back_bytes / sizeof(int32_t));
   const int64_t most = b.back_words > (int64_t)H * B ? b.back_words : (int64_t)H * B;
   begin_kernel<<<fitted_grid((const void*)begin_kernel, 256, ctx->num_sms, (most + 255) / 256), 256,
-                 0, st>>>(b);
+                 0, caller>>>(b);
   CK(ctx, cudaGetLastError());
   if (pipelined) {
-    // the targets have been read by then: what the caller's stream does next
-    // may overwrite or free them
-    CK(ctx, cudaEventRecord(ctx->pipe_read, st));
-    CK(ctx, cudaStreamWaitEvent((cudaStream_t)cuda_stream, ctx->pipe_read, 0));
+    CK(ctx, cudaEventRecord(ctx->pipe_in, caller));
+    CK(ctx, cudaStreamWaitEvent(st, ctx->pipe_in, 0));
   }
   int n_marks = 0;
   if (resident && ctx->lg.mode != AGNES_LAUNCH_DIRECT && !capturing)
