@@ -257,13 +257,12 @@ cudaError_t build_block_tables(const void* d_offsets, int offsets_bits, int64_t 
 
   BT_CHECK(cudaMalloc(&flags, N));
   BT_CHECK(cudaMalloc(&rank, sizeof(int32_t) * (N + 1)));
-  BT_CHECK(cudaMalloc(&scratch, sizeof(int64_t) * scan_scratch_elems(1, N)));
-  BT_CHECK(cudaMemsetAsync(scratch, 0, sizeof(int64_t) * scan_scratch_elems(1, N), st));
+  BT_CHECK(cudaMalloc(&scratch, sizeof(int64_t) * scan_scratch_elems(N)));
+  BT_CHECK(cudaMemsetAsync(scratch, 0, sizeof(int64_t) * scan_scratch_elems(N), st));
   tile_flags_kernel<<<grid, 256, 0, st>>>(flags, N, rows_per_feat_block);
   tile_flag_starts_kernel<<<grid, 256, 0, st>>>(flags, bt->start_node, bt->n_starts);
   BT_CHECK(cudaGetLastError());
-  BT_CHECK((seg_scan<uint8_t, int32_t>(flags, 0, rank, 0, nullptr, N, 1, N, true, nullptr,
-                                       scratch, nullptr, st)));
+  BT_CHECK(scan(flags, rank, N, scratch, nullptr, st));
   BT_CHECK(cudaMemcpyAsync(&T32, rank + N, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
   BT_CHECK(cudaStreamSynchronize(st));
   bt->T = T32;

@@ -73,7 +73,7 @@ struct Workspace {
   uint64_t* flat_scratch = nullptr;  // single-pass scans of the cell counts (zero between scans)
   int64_t flat_elems = 0;
   void* feats_out = nullptr;
-  int64_t* scan_scratch = nullptr;
+  int64_t* scan_scratch = nullptr;  // the scan of the tiles' distinct rows (row I/O)
   int32_t* cols_scratch = nullptr;  // column scans' chunk sums
   unsigned long long* distinct = nullptr;
   uint64_t* key = nullptr;  // sampling key {seed, first minibatch id}

@@ -230,7 +230,7 @@ cudaError_t launch_dedup(const HopArgs& a, const DedupBufs& d, int num_sms, cuda
   const int64_t gx = (num_sms * 8 + a.H - 1) / a.H, fill = (a.ecap + kThreads - 1) / kThreads;
   const dim3 egrid((unsigned)(gx < fill ? gx : fill), (unsigned)a.H);
   cudaError_t e =
-      flat_scan(d.scnt, d.soff, ncells, true, nullptr, true, d.flat_scratch, a.status, st);
+      flat_scan(d.scnt, d.soff, ncells, true, d.flat_scratch, a.status, st);
   if (e != cudaSuccess) return e;
   dedup_scatter_kernel<<<egrid, kThreads, 0, st>>>(d.nbr, d.ecnt, a.ecap, d.scell, d.srank,
                                                    d.soff, d.sb, a.sb_packed, d.q_ctl,

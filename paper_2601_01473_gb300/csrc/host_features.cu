@@ -236,8 +236,7 @@ static agnes_status gather_rows_io(agnes_ctx* ctx, int cur, int32_t n, int64_t* 
   // distinct requested rows per tile, and their total (for the staging size)
   CK(ctx, launch_tile_bitmaps(w.fb_id[cur], w.fcell_off[cur], ctx->bt.tile_first, T, w.H,
                               ctx->rm_bitmap, ctx->rm_wpref, ctx->rm_dcnt, w.status, st));
-  CK(ctx, (seg_scan<int32_t, int32_t>(ctx->rm_dcnt, 0, ctx->rm_doff, 0, nullptr, T, 1, T, true,
-                                      nullptr, w.scan_scratch, w.status, st)));
+  CK(ctx, scan(ctx->rm_dcnt, ctx->rm_doff, T, w.scan_scratch, w.status, st));
   int32_t* h_total = (int32_t*)ctx->h_rm;
   CK(ctx, cudaMemcpyAsync(h_total, ctx->rm_doff + T, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
   CK(ctx, cudaStreamSynchronize(st));

@@ -22,29 +22,22 @@ inline int fitted_grid(const void* kernel, int threads, int num_sms, int64_t cta
   return ctas < 1 ? 1 : ctas < resident ? (int)ctas : resident;
 }
 
-// Exclusive scan of nseg segments.  Segment s reads in[s*in_stride + i] for
-// i < len(s) and writes out[s*out_stride + i]; len(s) = d_len[s] when d_len is
-// non-null, else const_len.  With write_end, out[s*out_stride + len(s)] gets
-// the segment total; seg_total (if non-null) gets it too.  max_len bounds
-// every len(s).  scratch needs scan_scratch_elems(nseg, max_len) int64s,
-// zeroed once before first use (the scan leaves its tickets at zero again).
-int64_t scan_scratch_elems(int64_t nseg, int64_t max_len);
-
-template <typename InT, typename OutT>
-cudaError_t seg_scan(const InT* in, int64_t in_stride, OutT* out, int64_t out_stride,
-                     const int32_t* d_len, int64_t const_len, int32_t nseg, int64_t max_len,
-                     bool write_end, int32_t* seg_total, int64_t* scratch,
-                     const int32_t* status, cudaStream_t st);
+// Exclusive scan of n values, out[n] = the total, in two launches without waits
+// between blocks.  scratch needs scan_scratch_elems(n) int64s, the first zero
+// before first use (the scan leaves it zero again).
+int64_t scan_scratch_elems(int64_t n);
+template <typename InT>
+cudaError_t scan(const InT* in, int32_t* out, int64_t n, int64_t* scratch, const int32_t* status,
+                 cudaStream_t st);
 
 // Single-pass exclusive scan of n int32 values (decoupled look-back): out[i]
-// = sum of in[i'] for i' < i; with write_end out[n] = the total; total_out
-// (if non-null) gets it too; with clear the counts are left zero.  in and out
-// are 16-byte aligned.  scratch needs flat_scan_scratch_elems(n) uint64s,
+// = sum of in[i'] for i' < i, out[n] = the total; with clear the counts are left
+// zero.  in and out are 16-byte aligned.  scratch needs flat_scan_scratch_elems(n) uint64s,
 // zero before first use (the scan leaves it zero again).  Scans sharing a
 // scratch must be ordered on one stream.
 int64_t flat_scan_scratch_elems(int64_t max_n);
-cudaError_t flat_scan(int32_t* in, int32_t* out, int64_t n, bool write_end, int32_t* total_out,
-                      bool clear, uint64_t* scratch, int32_t* status, cudaStream_t st);
+cudaError_t flat_scan(int32_t* in, int32_t* out, int64_t n, bool clear, uint64_t* scratch,
+                      int32_t* status, cudaStream_t st);
 
 // Exclusive scan down each column of a row-major [rows x cols] matrix:
 // out[r*cols + c] = sum of in[r'*cols + c] over r' < r; total[i][c] (where

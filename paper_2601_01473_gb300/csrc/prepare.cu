@@ -132,9 +132,7 @@ static agnes_status ensure_workspace(agnes_ctx* ctx, int32_t H, int32_t B, const
   const int64_t cells = T * H;
   const int64_t rows = (int64_t)H * w.capK;
   const int64_t edges = (int64_t)H * w.ecap_max;
-  int64_t scratch = scan_scratch_elems(1, cells);
-  const int64_t s2 = scan_scratch_elems(1, ctx->N);
-  if (s2 > scratch) scratch = s2;
+  const int64_t scan_elems = scan_scratch_elems(T);
 
 #define WA(p, n)                                                                             \
   do {                                                                                       \
@@ -200,7 +198,7 @@ static agnes_status ensure_workspace(agnes_ctx* ctx, int32_t H, int32_t B, const
     WA(f, rows * ctx->row_bytes);
     w.feats_out = f;
   }
-  WA(w.scan_scratch, scratch);
+  WA(w.scan_scratch, scan_elems);
   WA(w.cols_scratch, cell_scans_scratch_elems(T, H));
   WA(w.distinct, 1);
   WA(w.key, 2);
@@ -212,7 +210,7 @@ static agnes_status ensure_workspace(agnes_ctx* ctx, int32_t H, int32_t B, const
     set_err(ctx, "out of pinned host memory");
     return AGNES_ENOMEM;
   }
-  if (cudaMemset(w.scan_scratch, 0, sizeof(int64_t) * scratch) != cudaSuccess ||
+  if (cudaMemset(w.scan_scratch, 0, sizeof(int64_t) * scan_elems) != cudaSuccess ||
       cudaMemset(w.indptr_scratch, 0, sizeof(uint64_t) * indptr_elems) != cudaSuccess ||
       cudaMemset(w.fcnt, 0, sizeof(int32_t) * cells) != cudaSuccess ||
       cudaMemset(w.scnt, 0, sizeof(int32_t) * cells) != cudaSuccess ||

@@ -792,7 +792,7 @@ cudaError_t launch_bucket_targets(int32_t* nodes, int64_t capK, int32_t H, int32
   targets_count_kernel<<<grid((const void*)targets_count_kernel), kThreads, 0, st>>>(
       nodes, capK, H, B, N, tm, fcnt, rank, status);
   cudaError_t e =
-      flat_scan(fcnt, fcell_off, ncells, true, nullptr, true, flat_scratch, status, st);
+      flat_scan(fcnt, fcell_off, ncells, true, flat_scratch, status, st);
   if (e != cudaSuccess) return e;
   targets_scatter_kernel<<<grid((const void*)targets_scatter_kernel), kThreads, 0, st>>>(
       nodes, capK, H, B, tm, fcell_off, rank, tmp_id, tmp_pos, status);

@@ -2,8 +2,8 @@
 //
 // The cell offsets of the bucket matrix (single pass), the per-minibatch
 // offsets of the new nodes of each (tile, minibatch) cell (column scans), and
-// the segmented scan of the tile compaction at load time and of the staged
-// rows (two launches, no waiting between blocks).
+// the scan of the tile compaction at load time and of the staged rows (two
+// launches, no waiting between blocks).
 #include <mutex>
 #include <unordered_map>
 
@@ -17,15 +17,7 @@ namespace {
 constexpr int kThreads = 256;
 constexpr int kItems = 8;
 constexpr int kChunk = kThreads * kItems;  // elements per block and chunk
-// Scratch layout shared by every scan: one ticket per segment (at most
-// kMaxSegments) first, kept at zero between scans, then the chunk sums.
-constexpr int64_t kMaxSegments = 65536;
-constexpr int64_t kTicketElems = kMaxSegments / 2;  // int64 slots holding the uint32 tickets
-constexpr int64_t kGridBlocks = 2048;  // blocks of a segmented scan (at least one per segment)
-
-__device__ __forceinline__ int64_t seg_len(const int32_t* d_len, int64_t const_len, int s) {
-  return d_len ? (int64_t)d_len[s] : const_len;
-}
+constexpr int64_t kGridBlocks = 2048;      // blocks of a two-launch scan at most
 
 // Exclusive block-wide scan of one int64 per thread; *total gets the sum.
 __device__ __forceinline__ int64_t block_excl_scan(int64_t v, int64_t* total) {
@@ -48,20 +40,16 @@ __device__ __forceinline__ int64_t block_excl_scan(int64_t v, int64_t* total) {
   return out;
 }
 
-// In-place exclusive scan of n int64 values at p (element i at p[i * stride])
-// by one CTA: each pass loads kItems consecutive values per thread before
+// In-place exclusive scan of n int64 values, written by other blocks of the
+// launch, by one CTA: each pass loads kItems consecutive values per thread before
 // scanning them, so a pass costs one memory round trip.  Returns the total.
-__device__ __forceinline__ int64_t cta_scan_inplace(int64_t* p, int64_t n, int64_t stride,
-                                                   bool volatile_loads) {
+__device__ __forceinline__ int64_t cta_scan_inplace(int64_t* p, int64_t n) {
   int64_t carry = 0;
   for (int64_t base = 0; base < n; base += (int64_t)kThreads * kItems) {
     const int64_t i0 = base + (int64_t)threadIdx.x * kItems;
     int64_t v[kItems];
 #pragma unroll
-    for (int k = 0; k < kItems; ++k) {
-      const int64_t i = i0 + k;
-      v[k] = i < n ? (volatile_loads ? *(volatile int64_t*)(p + i * stride) : p[i * stride]) : 0;
-    }
+    for (int k = 0; k < kItems; ++k) v[k] = i0 + k < n ? *(volatile int64_t*)(p + i0 + k) : 0;
     int64_t run = 0;
 #pragma unroll
     for (int k = 0; k < kItems; ++k) {
@@ -72,70 +60,55 @@ __device__ __forceinline__ int64_t cta_scan_inplace(int64_t* p, int64_t n, int64
     int64_t tot;
     const int64_t ex = block_excl_scan(run, &tot);
 #pragma unroll
-    for (int k = 0; k < kItems; ++k) {
-      const int64_t i = i0 + k;
-      if (i < n) p[i * stride] = carry + ex + v[k];
-    }
+    for (int k = 0; k < kItems; ++k)
+      if (i0 + k < n) p[i0 + k] = carry + ex + v[k];
     carry += tot;
   }
   return carry;
 }
 
-// Chunk sums; the last chunk of a segment to finish (atomic ticket after a
-// fence, no waiting) then scans the segment's chunk sums in place, writes
-// the segment total, and resets the ticket for the next scan.  Only the
-// chunks that hold elements of the segment take part (at least one, which
-// writes the total of an empty segment); a block takes chunks blockIdx.x,
-// blockIdx.x + gridDim.x, ... so the grid need not cover a segment's whole
-// capacity.
-template <typename InT, typename OutT>
+// Chunk sums; the last chunk to finish (atomic ticket after a fence, no waiting)
+// then scans them in place, writes the total to out[n], and resets the ticket for
+// the next scan.  A block takes chunks blockIdx.x, blockIdx.x + gridDim.x, ...
+template <typename InT>
 __global__ void __launch_bounds__(kThreads)
-scan_reduce_kernel(const InT* __restrict__ in, int64_t in_stride, const int32_t* d_len,
-                   int64_t const_len, int64_t chunks, int64_t* __restrict__ partial,
-                   unsigned int* __restrict__ tickets, OutT* __restrict__ out, int64_t out_stride,
-                   bool write_end, int32_t* seg_total, const int32_t* status) {
+scan_reduce_kernel(const InT* __restrict__ in, int64_t n, int64_t chunks,
+                   int64_t* __restrict__ partial, unsigned int* __restrict__ ticket,
+                   int32_t* __restrict__ out, const int32_t* status) {
   grid_dep_wait();
   if (status && failed(status)) return;
-  const int s = blockIdx.y;
-  const int64_t len = seg_len(d_len, const_len, s);
-  int64_t nvalid = len > 0 ? (len + kChunk - 1) / kChunk : 1;
-  if (nvalid > chunks) nvalid = chunks;
   __shared__ int64_t wsum[kThreads / 32];
   __shared__ bool last;
-  for (int64_t c = blockIdx.x; c < nvalid; c += gridDim.x) {
+  for (int64_t c = blockIdx.x; c < chunks; c += gridDim.x) {
     const int64_t begin = c * kChunk;
     int64_t sum = 0;
-    if (begin < len) {  // all of the thread's loads in flight at once
-      const InT* p = in + (int64_t)s * in_stride;
-      InT v[kItems];
+    InT v[kItems];  // all of the thread's loads in flight at once
 #pragma unroll
-      for (int k = 0; k < kItems; ++k) {
-        const int64_t i = begin + k * kThreads + threadIdx.x;
-        v[k] = i < len ? p[i] : (InT)0;
-      }
-#pragma unroll
-      for (int k = 0; k < kItems; ++k) sum += (int64_t)v[k];
+    for (int k = 0; k < kItems; ++k) {
+      const int64_t i = begin + k * kThreads + threadIdx.x;
+      v[k] = i < n ? in[i] : (InT)0;
     }
+#pragma unroll
+    for (int k = 0; k < kItems; ++k) sum += (int64_t)v[k];
     sum = warp_sum(sum);
     if ((threadIdx.x & 31) == 0) wsum[threadIdx.x >> 5] = sum;
     __syncthreads();
     if (threadIdx.x < 32) {
-      int64_t v = threadIdx.x < kThreads / 32 ? wsum[threadIdx.x] : 0;
-      v = warp_sum(v);
+      int64_t w = threadIdx.x < kThreads / 32 ? wsum[threadIdx.x] : 0;
+      w = warp_sum(w);
       if (threadIdx.x == 0) {
-        partial[(int64_t)s * chunks + c] = v;
+        partial[c] = w;
         __threadfence();
-        last = atomicAdd(tickets + s, 1u) == (unsigned)(nvalid - 1);
+        last = atomicAdd(ticket, 1u) == (unsigned)(chunks - 1);
       }
     }
     __syncthreads();
-    if (last) {  // the segment's final chunk: no later chunk of this block remains
+    if (last) {  // the final chunk: no later chunk of this block remains
       __threadfence();
-      const int64_t carry = cta_scan_inplace(partial + (int64_t)s * chunks, nvalid, 1, true);
+      const int64_t carry = cta_scan_inplace(partial, chunks);
       if (threadIdx.x == 0) {
-        if (write_end) out[(int64_t)s * out_stride + len] = (OutT)carry;
-        if (seg_total) seg_total[s] = (int32_t)carry;
-        tickets[s] = 0;
+        out[n] = (int32_t)carry;
+        *ticket = 0;
       }
     }
     __syncthreads();  // wsum and last are rewritten by the next chunk
@@ -144,27 +117,22 @@ scan_reduce_kernel(const InT* __restrict__ in, int64_t in_stride, const int32_t*
 
 // Each warp scans 256 consecutive elements as 8 coalesced 32-wide slices
 // (carry passed slice to slice), then the warps' totals are scanned.
-template <typename InT, typename OutT>
+template <typename InT>
 __global__ void __launch_bounds__(kThreads)
-scan_down_kernel(const InT* __restrict__ in, int64_t in_stride, OutT* __restrict__ out,
-                 int64_t out_stride, const int32_t* d_len, int64_t const_len, int64_t chunks,
+scan_down_kernel(const InT* __restrict__ in, int32_t* __restrict__ out, int64_t n,
                  const int64_t* __restrict__ partial, const int32_t* status) {
   grid_dep_wait();
   if (status && failed(status)) return;
-  const int s = blockIdx.y;
-  const int64_t len = seg_len(d_len, const_len, s);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const InT* p = in + (int64_t)s * in_stride;
-  OutT* q = out + (int64_t)s * out_stride;
   __shared__ int64_t wtot[kThreads / 32];
-  for (int64_t c = blockIdx.x; c * kChunk < len; c += gridDim.x) {
+  for (int64_t c = blockIdx.x; c * kChunk < n; c += gridDim.x) {
     const int64_t wbase = c * kChunk + (int64_t)warp * (32 * kItems);
-    const int64_t chunk_off = partial[(int64_t)s * chunks + c];  // issued with the loads below
+    const int64_t chunk_off = partial[c];  // issued with the loads below
     int64_t v[kItems];
 #pragma unroll
     for (int k = 0; k < kItems; ++k) {
       const int64_t i = wbase + k * 32 + lane;
-      v[k] = i < len ? (int64_t)p[i] : 0;
+      v[k] = i < n ? (int64_t)in[i] : 0;
     }
     int64_t carry = 0;
 #pragma unroll
@@ -186,7 +154,7 @@ scan_down_kernel(const InT* __restrict__ in, int64_t in_stride, OutT* __restrict
 #pragma unroll
     for (int k = 0; k < kItems; ++k) {
       const int64_t i = wbase + k * 32 + lane;
-      if (i < len) q[i] = (OutT)(off + v[k]);
+      if (i < n) out[i] = (int32_t)(off + v[k]);
     }
     __syncthreads();  // wtot is rewritten by the next chunk
   }
@@ -218,8 +186,7 @@ __device__ __forceinline__ unsigned long long flag_load(const unsigned long long
 }
 
 __device__ __forceinline__ void flat_scan_cta(int32_t* __restrict__ in, int32_t* __restrict__ out,
-                                              int64_t n, int64_t ntiles, bool write_end,
-                                              int32_t* total_out, bool clear,
+                                              int64_t n, int64_t ntiles, bool clear,
                                               unsigned long long* scratch, int32_t* status) {
   // no early return on a failed status: every CTA takes its tile and counts
   // itself finished, so the scratch is left zero for the next scan
@@ -305,10 +272,7 @@ __device__ __forceinline__ void flat_scan_cta(int32_t* __restrict__ in, int32_t*
     }
     if (lane == 0) {
       s_excl = excl;
-      if (tile == ntiles - 1) {
-        if (write_end) out[n] = (int32_t)(excl + agg);
-        if (total_out) *total_out = (int32_t)(excl + agg);
-      }
+      if (tile == ntiles - 1) out[n] = (int32_t)(excl + agg);
     }
   }
   __syncthreads();
@@ -342,10 +306,10 @@ __device__ __forceinline__ void flat_scan_cta(int32_t* __restrict__ in, int32_t*
 }
 
 __global__ void __launch_bounds__(kThreads)
-flat_scan_kernel(int32_t* __restrict__ in, int32_t* __restrict__ out, int64_t n, bool write_end,
-                 int32_t* total_out, bool clear, unsigned long long* scratch, int32_t* status) {
+flat_scan_kernel(int32_t* __restrict__ in, int32_t* __restrict__ out, int64_t n, bool clear,
+                 unsigned long long* scratch, int32_t* status) {
   grid_dep_wait();
-  flat_scan_cta(in, out, n, gridDim.x, write_end, total_out, clear, scratch, status);
+  flat_scan_cta(in, out, n, gridDim.x, clear, scratch, status);
 }
 
 // ---- the scans between a hop's cells and its compaction -----------------------------
@@ -462,8 +426,7 @@ struct CellScansArgs {
 __global__ void __launch_bounds__(kThreads) cell_scans_kernel(CellScansArgs a) {
   grid_dep_wait();
   if ((int32_t)blockIdx.x < a.flat_tiles) {
-    flat_scan_cta(a.flat_in, a.flat_out, a.flat_n, a.flat_tiles, true, nullptr, false,
-                  a.flat_scratch, a.status);
+    flat_scan_cta(a.flat_in, a.flat_out, a.flat_n, a.flat_tiles, false, a.flat_scratch, a.status);
     return;
   }
   if (cta_failed(a.status)) return;
@@ -573,58 +536,39 @@ int resident_grid(const void* kernel, int threads, int num_sms) {
   return per_sm * num_sms;
 }
 
-int64_t scan_scratch_elems(int64_t nseg, int64_t max_len) {
-  int64_t chunks = (max_len + kChunk - 1) / kChunk;
-  if (chunks < 1) chunks = 1;
-  return kTicketElems + nseg * chunks;
+int64_t scan_scratch_elems(int64_t n) {
+  return 1 + (n > 0 ? (n + kChunk - 1) / kChunk : 1);  // the ticket, then the chunk sums
 }
 
 int64_t flat_scan_scratch_elems(int64_t max_n) {
   return 2 + (max_n + kFlatTile - 1) / kFlatTile + 1;
 }
 
-cudaError_t flat_scan(int32_t* in, int32_t* out, int64_t n, bool write_end, int32_t* total_out,
-                      bool clear, uint64_t* scratch, int32_t* status, cudaStream_t st) {
+cudaError_t flat_scan(int32_t* in, int32_t* out, int64_t n, bool clear, uint64_t* scratch,
+                      int32_t* status, cudaStream_t st) {
   if ((uintptr_t)in % 16 != 0 || (uintptr_t)out % 16 != 0) return cudaErrorInvalidValue;
   const int64_t ntiles = n > 0 ? (n + kFlatTile - 1) / kFlatTile : 1;
   if (ntiles > 0x7fffffff) return cudaErrorInvalidValue;
   flat_scan_kernel<<<(unsigned)ntiles, kThreads, 0, st>>>(
-      in, out, n, write_end, total_out, clear, reinterpret_cast<unsigned long long*>(scratch),
-      status);
+      in, out, n, clear, reinterpret_cast<unsigned long long*>(scratch), status);
   return cudaGetLastError();
 }
 
-template <typename InT, typename OutT>
-cudaError_t seg_scan(const InT* in, int64_t in_stride, OutT* out, int64_t out_stride,
-                     const int32_t* d_len, int64_t const_len, int32_t nseg, int64_t max_len,
-                     bool write_end, int32_t* seg_total, int64_t* scratch,
-                     const int32_t* status, cudaStream_t st) {
-  if (nseg <= 0) return cudaSuccess;
-  int64_t chunks = (max_len + kChunk - 1) / kChunk;
-  if (chunks < 1) chunks = 1;
-  // Segments of a per-minibatch scan are usually far shorter than their
-  // capacity max_len: about kGridBlocks blocks in all, each looping over its
-  // segment's chunks, instead of a block per chunk of capacity.
-  int64_t gx = kGridBlocks / nseg;
-  if (gx < 1) gx = 1;
-  if (gx > chunks) gx = chunks;
-  const dim3 grid((unsigned)gx, (unsigned)nseg);
-  if (nseg > kMaxSegments) return cudaErrorInvalidValue;
-  unsigned int* tickets = (unsigned int*)scratch;
-  int64_t* partial = scratch + kTicketElems;
-  scan_reduce_kernel<InT, OutT><<<grid, kThreads, 0, st>>>(in, in_stride, d_len, const_len, chunks,
-                                                           partial, tickets, out, out_stride,
-                                                           write_end, seg_total, status);
-  scan_down_kernel<InT, OutT><<<grid, kThreads, 0, st>>>(in, in_stride, out, out_stride, d_len,
-                                                         const_len, chunks, partial, status);
+template <typename InT>
+cudaError_t scan(const InT* in, int32_t* out, int64_t n, int64_t* scratch, const int32_t* status,
+                 cudaStream_t st) {
+  const int64_t chunks = scan_scratch_elems(n) - 1;
+  const unsigned grid = (unsigned)(chunks < kGridBlocks ? chunks : kGridBlocks);
+  int64_t* partial = scratch + 1;
+  scan_reduce_kernel<InT><<<grid, kThreads, 0, st>>>(in, n, chunks, partial,
+                                                     (unsigned int*)scratch, out, status);
+  scan_down_kernel<InT><<<grid, kThreads, 0, st>>>(in, out, n, partial, status);
   return cudaGetLastError();
 }
 
-template cudaError_t seg_scan<int32_t, int32_t>(const int32_t*, int64_t, int32_t*, int64_t,
-                                                const int32_t*, int64_t, int32_t, int64_t, bool,
-                                                int32_t*, int64_t*, const int32_t*, cudaStream_t);
-template cudaError_t seg_scan<uint8_t, int32_t>(const uint8_t*, int64_t, int32_t*, int64_t,
-                                                const int32_t*, int64_t, int32_t, int64_t, bool,
-                                                int32_t*, int64_t*, const int32_t*, cudaStream_t);
+template cudaError_t scan<int32_t>(const int32_t*, int32_t*, int64_t, int64_t*, const int32_t*,
+                                   cudaStream_t);
+template cudaError_t scan<uint8_t>(const uint8_t*, int32_t*, int64_t, int64_t*, const int32_t*,
+                                   cudaStream_t);
 
 }  // namespace agnes
