@@ -126,26 +126,15 @@ class ClockSampler:
                 "sm_max_mhz": max(mx) if mx else None, "reasons": reasons, "samples": len(rows)}
 
 
-def kernel_launches_per_step(K: int) -> int:
-    """Passes of a hyperbatch in the one-kernel-per-pass plan (60 at K = 3): the
-    sampling-key write and the dst-size fill 2; target bucketing 4 (count,
-    single-pass scan, scatter, sort); per hop 16 (count, 2-pass segmented scan,
-    fill, single-pass scan, scatter, the cells' lane pass, queue offsets, queue
-    copy, tile pass, 3-pass column scan, single-pass scan, col fix-up,
-    compaction); after the last hop 3 (feature-block marks, their count, gather)
-    and K counts of touched topology blocks. libagnes runs several of them in
-    one launch: launches_per_hyperbatch has the number of its kernels."""
-    return 2 + 4 + 16 * K + 3 + K
-
-
-def launches_per_hyperbatch(K: int) -> int:
-    """Kernels libagnes launches per hyperbatch with the graph in HBM and more
-    than 256 targets (33 at K = 3): the setup 1; target bucketing 4 (count,
-    single-pass scan, scatter, place); per hop 9 (indptr, fill, single-pass
-    scan, scatter with the counts of touched topology blocks, the cells' lane
-    and tile kernels, the two launches of the scans after them, compaction with
-    the col fix-up and the count of touched feature blocks); the gather 1."""
-    return 1 + 4 + 9 * K + 1
+def launches_per_hyperbatch(K: int, targets: int, cells: int) -> int:
+    """Kernels libagnes launches per hyperbatch of H x B `targets` with the graph in
+    HBM (33 at K = 3): the setup 1; target bucketing 4 (count, single-pass scan,
+    scatter, place), or 1 for at most 256 targets on at most 8192 (tile,
+    minibatch) cells; per hop 9 (indptr, fill, single-pass scan, scatter with the
+    counts of touched topology blocks, the cells' lane and tile kernels, the two
+    launches of the scans after them, compaction with the col fix-up and the count
+    of touched feature blocks); the gather 1."""
+    return 1 + (1 if targets <= 256 and cells <= 8192 else 4) + 9 * K + 1
 
 
 def algorithmic_bytes(c: dict, off_bytes: int) -> dict:
@@ -559,7 +548,7 @@ def main():
             "topology_streaming": topo,
             # counted for the HBM-resident path; the host-resident modes add per-batch
             # loads and gathers
-            "gpu_launches": launches_per_hyperbatch(K) * args.steps
+            "gpu_launches": launches_per_hyperbatch(K, w.H * w.B, w.H * info["tiles"]) * args.steps
             if not (args.stream or args.stream_topology) else None,
             "clocks": clocks,
             "phases_ms": {"names": ["bucket_targets"] + [f"hop{h + 1}_{p}" for h in range(K)

@@ -23,11 +23,20 @@ def test_algorithmic_bytes_by_hand():
     assert got == {"sampling": hop1 + hop2, "gather": gather, "total": hop1 + hop2 + gather}
 
 
-def test_launch_count_per_step():
-    # key + size fill, 4 for the targets, 16 per hop, mark + count + gather, one count per hop;
-    # 60 at K = 3 is the count of the ncu launch list of one rmat100m hyperbatch
-    assert bench.kernel_launches_per_step(3) == 60
-    assert bench.kernel_launches_per_step(1) == 2 + 4 + 16 + 3 + 1
+def test_launches_per_hyperbatch_are_the_ones_in_the_sources():
+    """setup, 4 for the targets, 9 per hop, gather: 33 at K = 3, the count of the
+    ncu launch list of one rmat100m hyperbatch; and one CTA for few targets up to
+    the sampler's limits."""
+    f = bench.launches_per_hyperbatch
+    assert f(3, 128 * 1024, 10**6) == 33
+    assert f(1, 257, 100) == f(1, 100, 8193) == 1 + 4 + 9 + 1
+    assert f(1, 256, 8192) == 1 + 1 + 9 + 1
+    src = open(os.path.join(ROOT, "paper_2601_01473_gb300", "csrc", "sample.cu")).read()
+    assert "constexpr int kThreads = 256;" in src and "constexpr int kFewTargets = kThreads;" in src
+    assert "constexpr int kFewItems = 32;" in src  # cells per thread
+    listing = open(os.path.join(ROOT, "profiles", "step_rmat100m_launches.md")).read()
+    block = listing.split("```")[1].strip().splitlines()
+    assert len(block) == 33
 
 
 def test_profiled_traffic_only_for_its_workload_and_source():
