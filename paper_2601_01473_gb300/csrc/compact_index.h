@@ -16,7 +16,9 @@ namespace agnes {
 
 constexpr int kCellThreads = 128;  // threads per CTA of the compaction
 constexpr int kCompactIlp = 2;  // bucket entries per thread and round (4 and 8 measured slower)
-constexpr int kCompactMaxSlices = 256;
+constexpr int kCompactMaxSlices = 256;  // of a group, binding where a graph has a few tiles:
+                                        // hop 2 of 32 x 1024 targets on 20k nodes with 64,
+                                        // 256, 1024: dedup 351, 344, 344 us
 constexpr int kCompactRound = kCompactIlp * kCellThreads;
 
 // Where a cell's next-frontier entries start in tmp: behind its `fo` frontier

@@ -304,7 +304,8 @@ targets_few_kernel(const int32_t* __restrict__ nodes, int64_t capK, int32_t H, i
 // Scratch (uint64, zero on entry; the hop's scatter clears it): [0] the
 // counter, [1 + j * tiles + t] flag of minibatch j's tile t = state << 62 |
 // value, state 1 = the tile's sum, 2 = the inclusive prefix through it.
-constexpr int kIndptrItems = 8;
+constexpr int kIndptrItems = 8;  // rows per thread; hop 3 of 64 x 1024 targets on 40M nodes
+                                 // with 4, 8, 16: 31, 27, 35 us; 16 x 1024 on 10M: 16, 18, 26
 constexpr int kIndptrTile = kThreads * kIndptrItems;
 constexpr unsigned long long kFlagAgg = 1ull << 62;
 constexpr unsigned long long kFlagInc = 2ull << 62;
