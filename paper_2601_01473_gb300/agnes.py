@@ -309,7 +309,10 @@ class Graph:
         self._ctx = ctx
         self._H = 0
         self._K = 0
-        self._held = collections.deque()  # (event, host targets whose copy it follows)
+        self._prepares = 0
+        self._copying = collections.deque()  # (prepare, host targets), copied on _copy_stream
+        self._copy_stream = None
+        self._held = collections.deque()  # (event, host targets whose copies it follows)
 
     # -- lifetime --------------------------------------------------------------
     def close(self):
@@ -339,34 +342,43 @@ class Graph:
         fan = (ctypes.c_int32 * len(fanouts))(*fanouts)
         H, B = targets.shape
         self._targets = targets
-        rc = lib().agnes_prepare_hyperbatch(self._ctx, targets.data_ptr(), H, B, fan, len(fanouts),
-                                            seed & (2**64 - 1), first_minibatch_id,
-                                            _stream_handle(stream, self.device))
+        handle = _stream_handle(stream, self.device)
         if not targets.is_cuda:
-            self._hold_until_copied(targets, stream)
+            self._hold_until_copied(targets, handle)
+        rc = lib().agnes_prepare_hyperbatch(self._ctx, targets.data_ptr(), H, B, fan, len(fanouts),
+                                            seed & (2**64 - 1), first_minibatch_id, handle)
         _check(rc, self._ctx)
+        self._prepares += 1
         self._H, self._K = H, len(fanouts)
 
-    def _hold_until_copied(self, targets, stream):
-        """Keeps host targets alive until their copy, which anything later on
-        the caller's stream follows, has run: the host may reuse their memory
-        at once.  (In a capture nothing has run yet: the caller keeps them.)"""
-        while self._held and self._held[0][0].query():
-            self._held.popleft()
-        if stream is None:
-            stream = torch.cuda.current_stream(self.device)
-        elif not isinstance(stream, torch.cuda.Stream):
-            stream = torch.cuda.ExternalStream(int(stream), self.device)
-        with torch.cuda.stream(stream):
-            if torch.cuda.is_current_stream_capturing():
-                return
-            event = torch.cuda.Event()
-            event.record()
-        self._held.append((event, targets))
+    def _hold_until_copied(self, targets, handle):
+        """Keeps host targets alive until their copy has run: the host may
+        reuse their memory at once.  The copies run in order on the caller's
+        stream, so a hyperbatch that has been fetched is behind all earlier
+        ones (_copied); for a program that does not fetch, or changes streams,
+        an event follows every 64 of them."""
+        if self._copying and (handle != self._copy_stream or len(self._copying) >= 64):
+            stream = torch.cuda.ExternalStream(self._copy_stream or 0, self.device)
+            with torch.cuda.stream(stream):
+                if not torch.cuda.is_current_stream_capturing():
+                    event = torch.cuda.Event()
+                    event.record()
+                    self._held.append((event, self._copying))
+                    self._copying = collections.deque()
+            while self._held and self._held[0][0].query():
+                self._held.popleft()
+        self._copy_stream = handle
+        self._copying.append((self._prepares, targets))
+
+    def _copied(self, ago=0):
+        """The hyperbatch `ago` prepares before the last one has run."""
+        while self._copying and self._copying[0][0] < self._prepares - ago:
+            self._copying.popleft()
 
     def fetch(self, j: int) -> MinibatchView:
         v = _View()
         _check(lib().agnes_fetch_minibatch(self._ctx, j, ctypes.byref(v)), self._ctx)
+        self._copied()
         hops = []
         for h in range(v.K):
             nd, ns, ne = v.num_dst[h], v.num_src[h], v.num_edges[h]
@@ -382,6 +394,7 @@ class Graph:
         workspace stays where it is (same hyperbatch shape)."""
         v = _HyperbatchView()
         _check(lib().agnes_fetch_hyperbatch(self._ctx, ctypes.byref(v)), self._ctx)
+        self._copied()
         key = bytes(v)  # every address, stride and shape
         cached = getattr(self, "_hv_cache", None)
         hv = HyperbatchView(v, self.device, cached[1] if cached and cached[0] == key else None)
@@ -410,6 +423,7 @@ class Graph:
         (agnes_fetch_previous_hyperbatch)."""
         v = _HyperbatchView()
         _check(lib().agnes_fetch_previous_hyperbatch(self._ctx, ctypes.byref(v)), self._ctx)
+        self._copied(1)
         return HyperbatchView(v, self.device)
 
     def fetch_earlier(self, ago: int) -> HyperbatchView:
@@ -418,6 +432,7 @@ class Graph:
         v = _HyperbatchView()
         _check(lib().agnes_fetch_earlier_hyperbatch(self._ctx, int(ago), ctypes.byref(v)),
                self._ctx)
+        self._copied(int(ago))
         return HyperbatchView(v, self.device)
 
     def set_pipeline_depth(self, depth: int) -> None:

@@ -243,9 +243,14 @@ def test_host_targets_live_until_they_are_copied(cuda_device, depth):
     others = [torch.full_like(t, -1).pin_memory() for t in tgts]
     assert not ptr & {o.data_ptr() for o in others}
     compare(g, og, tgts[2].numpy(), [4, 3], 7, 200, ADJ, FEAT)
-    torch.cuda.synchronize()
-    g.prepare(tgts[0], [4, 3], 7, 0)
-    assert len(g._held) == 1
+    other = torch.cuda.Stream(cuda_device)
+    for s in range(100):  # they are let go as the copies run, whatever the stream
+        g.prepare(tgts[s % 3], [4, 3], 7, 0, other if s % 40 == 39 else None)
+        if s % 20 == 19:
+            torch.cuda.synchronize()
+    assert len(g._copying) + sum(len(h) for _, h in g._held) <= 128
+    g.fetch_all()
+    assert not g._copying
     g.close()
 
 
