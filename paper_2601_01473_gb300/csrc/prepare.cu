@@ -645,11 +645,11 @@ agnes_status agnes_prepare_hyperbatch(agnes_ctx* ctx, const int32_t* targets, in
   // the least recently used set of per-hyperbatch state
   if (pipelined) rotate_hyperbatch_state(ctx);
   const cudaStream_t st = pipelined ? ctx->pipe_st : caller;
+  ctx->prepared = false;  // also if the workspace cannot be allocated: the last one is gone
+  ctx->synced = false;
   agnes_status rc = ensure_workspace(ctx, H, B, fanouts, K, cap);
   if (rc != AGNES_OK) return rc;
   Workspace& w = ctx->ws;
-  ctx->prepared = false;
-  ctx->synced = false;
   if (ctx->profiling && !ctx->ev_created) {
     for (int r = 0; r < kEventRing; ++r)
       for (int i = 0; i <= kMaxPhases; ++i) CK(ctx, cudaEventCreate(&ctx->ev[r][i]));

@@ -254,6 +254,30 @@ def test_host_targets_live_until_they_are_copied(cuda_device, depth):
     g.close()
 
 
+def test_a_workspace_that_does_not_fit_leaves_nothing_to_fetch(cuda_device):
+    """ENOMEM (a terabyte of gathered rows) drops the previous hyperbatch: fetch
+    says so, and the next prepare works again."""
+    from paper_2601_01473_gb300 import AgnesError
+    N, block = 1000, 1 << 18
+    off, ind, _ = make(N, 12, seed=58)
+    feats = torch.zeros((N, 8192), dtype=torch.float16)
+    og = oracle.Graph(off.numpy(), ind.numpy(), feats.numpy())
+    g = load(off, ind, feats, block, block)
+    t = synth.hyperbatch_targets(torch.arange(N, dtype=torch.int32), 2, 20, 3, 0)
+    g.prepare(t.to(cuda_device), [3], 1, 0)
+    g.fetch_all()
+    many = torch.zeros((65535, 1), dtype=torch.int32, device=cuda_device)
+    with pytest.raises(AgnesError) as e:
+        g.prepare(many, [999], 1, 0)
+    assert e.value.status == 3
+    with pytest.raises(AgnesError) as e:
+        g.fetch_all()
+    assert e.value.status == 5
+    g.prepare(t.to(cuda_device), [3], 1, 0)
+    compare(g, og, t.numpy(), [3], 1, 0, block, block)
+    g.close()
+
+
 def test_pipeline_depth_two_needs_a_resident_graph(cuda_device):
     off, ind, feats = make(3000, 6, seed=52)
     dev = torch.device("cuda:0")
