@@ -185,7 +185,7 @@ def test_rows_of_any_width(cuda_device, dtype, dim, shift):
     (104, 256, torch.float16, [200], 3, 5000),  # the same without swizzle
     (128, 256, torch.float16, [1], 4, 6000),    # light rows, one stage of 128
     (128, 256, torch.float32, [60], 6, 8000),   # heavy ones, two of 64, more tiles than stages
-    (8, 32, torch.float16, [30], 8, 25000),     # nothing staged, six stages, several rounds
+    (8, 32, torch.float16, [30], 8, 25000),     # nothing staged; six stages, all used again
     (24, 64, torch.float16, [5], 8, 15000),     # the last width that is not staged, four
     (16, 32, torch.float32, [9], 8, 25000),     # staged, six stages
 ])
