@@ -295,10 +295,10 @@ __device__ __forceinline__ SageTile sage_tile(const SageArgs& a, const SageTiles
   return r;
 }
 
-// Shared memory: the A stages, W, the index slots, the mbarriers.  The MMA reads kM
+// Shared memory: W and the A stages, the index slots, the mbarriers.  The MMA reads kM
 // rows of every stage.  Where a stage has fewer, the others are whatever lies behind
 // it, the next stage or W (8 KB at most, and W has as much: d_in > 64), and fill
-// accumulator rows that nobody reads.
+// accumulator rows that nobody reads.  Stages of kM rows lie behind W.
 struct SageSmem {
   uint8_t* w;
   uint8_t* a;
@@ -315,9 +315,15 @@ template <int kRows>
 __device__ __forceinline__ SageSmem sage_smem(uint8_t* smem, const SageArgs& a) {
   const uint32_t KT = 2 * a.d_in;
   SageSmem m;
-  m.a = smem;
-  m.w = m.a + (size_t)a.stages * kRows * KT * 2;
-  m.idx = m.w + (size_t)a.d_out * KT * 2;
+  if (kRows == kM) {
+    m.w = smem;
+    m.a = m.w + (size_t)a.d_out * KT * 2;
+    m.idx = m.a + (size_t)a.stages * kRows * KT * 2;
+  } else {
+    m.a = smem;
+    m.w = m.a + (size_t)a.stages * kRows * KT * 2;
+    m.idx = m.w + (size_t)a.d_out * KT * 2;
+  }
   m.idx_bytes = idx_slot_bytes(a.idx_cap);
   m.bars = (uint64_t*)(m.idx + (size_t)a.slots * m.idx_bytes);
   return m;
@@ -435,11 +441,17 @@ __device__ __forceinline__ bool sage_producer_warp(const SageArgs& a, const Sage
   const uint32_t stage_bytes = (uint32_t)(kRows * 4 * a.d_in);
   int first = w;  // the warp's first group, rotated from tile to tile so that a
                   // remainder of groups falls to every warp in turn
+  // fp32's loads in flight leave no registers for the tile's and the slot's place,
+  // which are computed anew (64 -> 128 on a skewed graph, fanouts 30 and 50, with this
+  // and W first: 403 -> 389, 561 -> 543 us); in fp16 keeping them is faster
+  constexpr bool kAnew = sizeof(T) == 4;
   Ring stage, slot;
-  for (int tile = blockIdx.x; tile < total_tiles; tile += gridDim.x) {
-    const int q = slot.slot;
-    const bool ready =
-        mbar_wait(bar.ifull(q), slot.parity()) && stage.free(bar.empty(stage.slot));
+  for (int k = 0, kept = blockIdx.x;; ++k, kept += kAnew ? 0 : gridDim.x, stage.next(a.stages)) {
+    const int tile = kAnew ? (int)blockIdx.x + k * (int)gridDim.x : kept;
+    if (tile >= total_tiles) return true;
+    const int q = kAnew ? k % a.slots : slot.slot;
+    const uint32_t parity = kAnew ? (uint32_t)((k / a.slots) & 1) : slot.parity();
+    const bool ready = mbar_wait(bar.ifull(q), parity) && stage.free(bar.empty(stage.slot));
     if (!__all_sync(0xffffffffu, ready)) return false;
     const IdxHead* h = (const IdxHead*)(m.idx + (size_t)q * m.idx_bytes);
     const int32_t* cl = h->staged ? (const int32_t*)(h + 1) : h->col;
@@ -505,10 +517,8 @@ __device__ __forceinline__ bool sage_producer_warp(const SageArgs& a, const Sage
       mbar_arrive(bar.full(stage.slot));
       mbar_arrive(bar.iempty(q));
     }
-    stage.next(a.stages);
-    slot.next(a.slots);
+    if (!kAnew) slot.next(a.slots);
   }
-  return true;
 }
 
 // kSwizzle: A with 128-byte swizzle, where its rows are whole 64-element blocks
@@ -528,7 +538,7 @@ sage_kernel(SageArgs a, const __grid_constant__ SageTiles tiles) {
   uint32_t* tmem_slot = (uint32_t*)(m.bars + kBars);
 
   // the swizzle's atoms are 1024-byte aligned: dynamic shared memory starts on
-  // such a boundary, and a stage is a multiple of that long
+  // such a boundary, and W and a stage are multiples of that long
   if (kSwizzle && (smem_u32(smem) & 1023u) != 0) {
     if (tid == 0) *(volatile int32_t*)a.err = kSageTimeout;
     return;
